@@ -191,7 +191,7 @@ sb_status sb_sgd_step(sb_model* m, float lr, float momentum, void* stream);
  * algorithm (the FC weights move between sub-iterations).  sb_loss afterwards returns the mean of the R*b row
  * losses.  Needs SB_FLAG_MODULO_SCHEDULE at creation (SB_ERR_STATE otherwise).  Arguments as for sb_forward /
  * sb_sgd_step; runs on `stream`, asynchronous; like sb_graph_step the second call captures the iteration as a CUDA
- * graph and later calls with the same pointers and hyper-parameters replay it.  Afterwards SB_T_ROW_LOSS and the FC activation tensors hold their
+ * graph and later calls with the same pointers replay it.  Afterwards SB_T_ROW_LOSS and the FC activation tensors hold their
  * rows in sub-iteration order (position k*(R*b/K) + r*(b/K) + i = example k*(b/K) + i of replica r), the FC
  * activations as left by the sub-iteration that wrote them; sb_backward needs a new sb_forward.
  */
@@ -201,9 +201,9 @@ sb_status sb_modulo_step(sb_model* m, const void* const* x, const int32_t* const
 /*
  * One whole iteration (sb_forward + sb_backward + sb_sgd_step on device-resident inputs) replayed as a CUDA
  * graph: the first call runs the three passes directly, the second captures them on `stream` (thread-local
- * capture mode) and every later call with the same input pointers, lr and momentum is one graph launch, which
- * removes the per-kernel launch cost that dominates at small batch sizes.  Different pointers or
- * hyper-parameters re-capture.  `stream` must not be the legacy default stream (NULL runs the passes directly).
+ * capture mode) and every later call with the same input pointers is one graph launch, which
+ * removes the per-kernel launch cost that dominates at small batch sizes.  Other pointers are captured into the same
+ * graph (updated in place); lr and momentum may change on every call.  `stream` must not be the legacy default stream (NULL runs the passes directly).
  * Arguments as for sb_forward / sb_sgd_step.  Parameters, momentum, activations and loss are identical to the
  * three separate calls.  SB_T_GRAD_W / SB_T_GRAD_B are unspecified afterwards (here and after
  * sb_modulo_step / sb_train_step_host): where a weight gradient is summed from split partial copies, the ordered
@@ -225,8 +225,8 @@ sb_status sb_loss(sb_model* m, void* stream, float* host_loss);
  * end-to-end call.  host_x: [B,H,W,C] in the activation dtype, rows r*b..(r+1)*b-1 = replica r;
  * host_labels: int32 [B].  Both are copied host->device on `stream` into staging space inside
  * the arena (pinned host memory makes the copies asynchronous).  Synchronises `stream`.  From the second call on,
- * the copies, the iteration and the read-back of the loss are replayed as one CUDA graph keyed by the two host
- * pointers, lr and momentum (the host buffers must then stay at the same addresses; new addresses re-capture).
+ * the iteration and the read-back of the loss are replayed as one CUDA graph behind the copies; host buffers, lr and momentum
+ * may change on every call.
  */
 sb_status sb_train_step_host(sb_model* m, const void* host_x, const int32_t* host_labels,
                              float lr, float momentum, void* stream, float* host_loss);

@@ -99,13 +99,16 @@ struct sb_model {
     unsigned int* counter = nullptr;
     uint32_t* status = nullptr;
     uint32_t* drop_state = nullptr;   // dropout: {seed lo, seed hi, iteration, 0} (device words, kept between calls)
+    float* hyper = nullptr;           // {learning rate, momentum} of the captured iterations (device words), and what they hold once the
+    float hyper_lr = 0.f, hyper_mu = 0.f;   // stream has reached this point (zero after creation)
+    bool hyper_words = false;         // they have changed from one captured iteration to the next: captures read the words
     int last_dropout = -1;            // index of the network's last dropout layer: its forward kernel is followed by the iteration bump
     bool st_clean = false;     // the chain stream's last kernel belongs to the current forward / backward pass (it cannot have written weights)
     int pooled_by_conv = -1;   // index of the pool layer whose output the conv kernel just before it has already written (same forward call)
     // Set by the multi-stream backward pass while it enqueues the weight side of one conv layer: the layer's split
     // reduces then apply the update themselves (launch_reduce_sgd) once `ev` (the layer's input-gradient kernel, which
     // reads the weights) has passed; `covered` counts the parameters updated that way.
-    struct { bool on = false; float lr = 0.f, mu = 0.f; cudaEvent_t ev = nullptr; bool waited = false; size_t covered = 0; } fuse;
+    struct { bool on = false; Hyper hy{}; cudaEvent_t ev = nullptr; bool waited = false; size_t covered = 0; } fuse;
     char* stage_x = nullptr;
     int32_t* stage_labels = nullptr;
     // Input prefetch (sb_prefetch_host): a second staging area, so that the copy of the next iteration's inputs runs on a
@@ -124,7 +127,7 @@ struct sb_model {
     int n_flights = 0;
     bool slot_busy[2] = {false, false};
     cudaEvent_t ev_done[2] = {nullptr, nullptr};
-    uint32_t* host_res = nullptr;      // pinned host memory: [3][2] words (areas 0, 1; 2 = the call that copies its inputs itself)
+    uint32_t* host_res = nullptr;      // pinned host memory: [2][2] words (areas 0, 1)
     char* input_grad = nullptr;
     PtrTab x_tab{}, label_tab{};
     bool have_x = false, have_labels = false, have_fwd = false;
@@ -137,18 +140,17 @@ struct sb_model {
     bool sub_active = false;
     int sub_row0 = 0, full_B = 0;
     int64_t launches = 0, last_step_launches = 0;
-    // CUDA graphs of a whole iteration (sb_graph_step, sb_train_step_host), re-captured when their key changes
+    // CUDA graphs of a whole iteration (sb_graph_step, sb_modulo_step, sb_train_step_host)
     struct StepGraph {
         cudaGraphExec_t exec = nullptr;
         PtrTab x{}, labels{};
-        const void* host_x = nullptr;
-        const void* host_labels = nullptr;
-        float* host_loss = nullptr;
-        float lr = 0.f, mu = 0.f;
+        Hyper hy{};            // captured with these values, or with the device words
         bool warmed = false;
+        bool fits(float lr, float mu) const { return hy.dev || (hy.lr == lr && hy.mu == mu); }
     };
-    StepGraph g_dev, g_host, g_mod;
-    StepGraph g_pre[2];      // sb_train_step_host on inputs staged by sb_prefetch_host: one graph per staging area
+    StepGraph g_dev, g_mod;
+    StepGraph g_host[2];     // iterations from host buffers: one graph per staging area
+    bool host_warmed = false;
     // Debug aids that stand in for a memory checker: every arena region is followed by a 256-byte guard holding a fixed
     // pattern (sb_debug_check_guards), and the regions a step overwrites are listed so that they can be filled with NaN
     // bit patterns before a step (sb_debug_poison).
@@ -182,10 +184,9 @@ struct sb_model {
         if (ev_join) cudaEventDestroy(ev_join);
         for (int k = 0; k < MAX_WSTREAMS; ++k) { if (wstreams[k]) cudaStreamDestroy(wstreams[k]); if (ev_wjoin[k]) cudaEventDestroy(ev_wjoin[k]); }
         if (g_dev.exec) cudaGraphExecDestroy(g_dev.exec);
-        if (g_host.exec) cudaGraphExecDestroy(g_host.exec);
         if (g_mod.exec) cudaGraphExecDestroy(g_mod.exec);
         for (int k = 0; k < 2; ++k) {
-            if (g_pre[k].exec) cudaGraphExecDestroy(g_pre[k].exec);
+            if (g_host[k].exec) cudaGraphExecDestroy(g_host[k].exec);
             if (ev_staged[k]) cudaEventDestroy(ev_staged[k]);
             if (ev_done[k]) cudaEventDestroy(ev_done[k]);
         }
@@ -351,6 +352,7 @@ sb_status plan(const sb_layer* layers, int n, const sb_config* cfg, sb_model* m,
     m->status = base ? (uint32_t*)(m->loss + 1) : nullptr;
     m->counter = (unsigned int*)take(256);
     m->drop_state = (uint32_t*)take(256);
+    m->hyper = (float*)take(256);
     m->stage_x = take(B * m->in_per_img * m->esz);
     m->stage_labels = (int32_t*)take(B * 4);
     m->stage_xb[0] = m->stage_x; m->stage_lb[0] = m->stage_labels;
@@ -566,7 +568,7 @@ sb_status backward_layer(sb_model* m, int i, cudaStream_t st, int part = SIDE_BO
             // fused pass: the update is applied by the weight-gradient kernel's epilogue (after the layer's input-gradient
             // kernel, which reads the weights); the gradient itself is never stored
             if (!m->fuse.waited) { CU_TRY(cudaStreamWaitEvent(st, m->fuse.ev, 0)); m->fuse.waited = true; }
-            U_TRY("fc_wgrad_umma", flops, act_bytes + (double)(l.n_w + l.n_b) * (m->bf16 ? 18.0 : 16.0), umma_fc_wgrad_update(m, i, m->fuse.lr, m->fuse.mu, st));
+            U_TRY("fc_wgrad_umma", flops, act_bytes + (double)(l.n_w + l.n_b) * (m->bf16 ? 18.0 : 16.0), umma_fc_wgrad_update(m, i, m->fuse.hy, st));
             ++m->launches;
             m->fuse.covered = l.n_w + l.n_b;
         } else if (l.um.wgrad.enabled) {
@@ -639,9 +641,9 @@ sb_status backward_layer(sb_model* m, int i, cudaStream_t st, int part = SIDE_BO
             __nv_bfloat16* sh = m->Sm ? m->Sm + goff : nullptr;
             if (reduce)
                 L_TRY("split_reduce_sgd", 0.0, (double)n * (4.0 * S + (m->bf16 ? 18.0 : 16.0)),
-                      launch_reduce_sgd(src, stride, n, S, m->Wm + goff, m->Vm + goff, sh, m->fuse.lr, m->fuse.mu, st));
+                      launch_reduce_sgd(src, stride, n, S, m->Wm + goff, m->Vm + goff, sh, m->fuse.hy, st));
             else
-                L_TRY("sgd", 0.0, (double)n * (m->bf16 ? 22.0 : 20.0), launch_sgd(m->Wm + goff, m->Vm + goff, m->Gm + goff, sh, n, m->fuse.lr, m->fuse.mu, st));
+                L_TRY("sgd", 0.0, (double)n * (m->bf16 ? 22.0 : 20.0), launch_sgd(m->Wm + goff, m->Vm + goff, m->Gm + goff, sh, n, m->fuse.hy, st));
             m->fuse.covered += n;
             return SB_OK;
         };
@@ -1037,7 +1039,7 @@ static sb_status weight_side(sb_model* m, int i, cudaStream_t wst, bool classic)
 // stream as soon as that layer's gradients are complete and its input gradient (which reads the weights) has
 // been computed, so the bandwidth-bound update overlaps the rest of the backward pass.  Element for element the
 // update is the one sb_sgd_step does.  Returns *updated = true if the update was done here.
-static sb_status backward_pass(sb_model* m, cudaStream_t st, bool fuse_update, float lr, float mu, bool* updated, int hi = -1, int lo = 0)
+static sb_status backward_pass(sb_model* m, cudaStream_t st, bool fuse_update, Hyper hy, bool* updated, int hi = -1, int lo = 0)
 {
     if (hi < 0) hi = m->n_layers - 1;     // layers hi .. lo, top down
     // The weight-gradient work of a layer (and its split reduce) only has to be finished before the update,
@@ -1079,7 +1081,7 @@ static sb_status backward_pass(sb_model* m, cudaStream_t st, bool fuse_update, f
                 s = chain_bwd(m, i, st, SIDE_D);
                 if (s != SB_OK) return s;
                 CU_TRY(cudaEventRecord(m->ev_dgrad[i], st));
-                m->fuse.on = true; m->fuse.lr = lr; m->fuse.mu = mu; m->fuse.ev = m->ev_dgrad[i]; m->fuse.waited = false; m->fuse.covered = 0;
+                m->fuse.on = true; m->fuse.hy = hy; m->fuse.ev = m->ev_dgrad[i]; m->fuse.waited = false; m->fuse.covered = 0;
                 s = weight_side(m, i, wst, classic);
                 m->fuse.on = false;
                 if (s != SB_OK) return s;
@@ -1104,7 +1106,7 @@ static sb_status backward_pass(sb_model* m, cudaStream_t st, bool fuse_update, f
                     cudaStream_t st = m->ustream;   // the launch bracket below records on the stream it launches on
                     m->cur_layer = i;
                     L_TRY("sgd", 0.0, (double)cnt * (m->bf16 ? 22.0 : 20.0),
-                          launch_sgd(m->Wm + off, m->Vm + off, m->Gm + off, m->Sm ? m->Sm + off : nullptr, cnt, lr, mu, st));
+                          launch_sgd(m->Wm + off, m->Vm + off, m->Gm + off, m->Sm ? m->Sm + off : nullptr, cnt, hy, st));
                 }
             }
         } else {
@@ -1134,18 +1136,25 @@ sb_status sb_backward(sb_model* m, void* stream)
 {
     if (!m) return fail(SB_ERR_INVALID_ARG, "null model");
     if (!m->have_fwd) return fail(SB_ERR_STATE, "sb_backward needs a preceding sb_forward");
-    return backward_pass(m, (cudaStream_t)stream, false, 0.f, 0.f, nullptr);
+    return backward_pass(m, (cudaStream_t)stream, false, Hyper{}, nullptr);
 }
 
 // forward + backward + update of one iteration, with the update folded into the backward pass when possible
-static sb_status whole_step(sb_model* m, const void* const* x, const int32_t* const* labels, float lr, float mu, void* stream)
+static sb_status update_all(sb_model* m, Hyper hy, cudaStream_t st)
+{
+    m->cur_layer = -1;
+    L_TRY("sgd", 0.0, (double)m->P * (m->bf16 ? 22.0 : 20.0), launch_sgd(m->Wm, m->Vm, m->Gm, m->Sm, m->P, hy, st));
+    m->last_step_launches = m->launches;
+    return SB_OK;
+}
+static sb_status whole_step(sb_model* m, const void* const* x, const int32_t* const* labels, Hyper hy, void* stream)
 {
     sb_status s = sb_forward(m, x, labels, stream);
     if (s != SB_OK) return s;
     bool updated = false;
-    s = backward_pass(m, (cudaStream_t)stream, true, lr, mu, &updated);
+    s = backward_pass(m, (cudaStream_t)stream, true, hy, &updated);
     if (s != SB_OK) return s;
-    if (!updated) s = sb_sgd_step(m, lr, mu, stream);
+    if (!updated) s = update_all(m, hy, (cudaStream_t)stream);
     return s;
 }
 
@@ -1154,7 +1163,7 @@ static sb_status whole_step(sb_model* m, const void* const* x, const int32_t* co
 // -> rows k*B/K + r*b/K ...); the FC stack then runs K sub-iterations (forward, loss with 1/B per row, backward,
 // SGD update of the FC parameters), each on B/K rows; the input gradients are copied back into row order and the
 // conv-side stack back-propagates once and takes its update.  Everything runs on the caller's stream.
-static sb_status modulo_step_direct(sb_model* m, const void* const* x, const int32_t* const* labels, float lr, float momentum, void* stream)
+static sb_status modulo_step_direct(sb_model* m, const void* const* x, const int32_t* const* labels, Hyper hy, void* stream)
 {
     if (!m) return fail(SB_ERR_INVALID_ARG, "null model");
     if (!(m->cfg.flags & SB_FLAG_MODULO_SCHEDULE)) return fail(SB_ERR_STATE, "the model was created without SB_FLAG_MODULO_SCHEDULE");
@@ -1191,7 +1200,7 @@ static sb_status modulo_step_direct(sb_model* m, const void* const* x, const int
         if (s != SB_OK) return s;
         m->cur_layer = -1;
         L_TRY("sgd", 0.0, (double)fc_cnt * (m->bf16 ? 22.0 : 20.0),
-              launch_sgd(m->Wm + fc_off, m->Vm + fc_off, m->Gm + fc_off, m->Sm ? m->Sm + fc_off : nullptr, fc_cnt, lr, momentum, st));
+              launch_sgd(m->Wm + fc_off, m->Vm + fc_off, m->Gm + fc_off, m->Sm ? m->Sm + fc_off : nullptr, fc_cnt, hy, st));
     }
     m->cur_layer = ff;
     {
@@ -1200,10 +1209,10 @@ static sb_status modulo_step_direct(sb_model* m, const void* const* x, const int
     }
     // conv-side stack: the multi-stream backward pass with the per-layer updates folded in, as in the synchronous step
     bool updated = false;
-    s = backward_pass(m, st, true, lr, momentum, &updated, ff - 1, 0);
+    s = backward_pass(m, st, true, hy, &updated, ff - 1, 0);
     if (s != SB_OK) return s;
     m->cur_layer = -1;
-    if (!updated) L_TRY("sgd", 0.0, (double)fc_off * (m->bf16 ? 22.0 : 20.0), launch_sgd(m->Wm, m->Vm, m->Gm, m->Sm, fc_off, lr, momentum, st));
+    if (!updated) L_TRY("sgd", 0.0, (double)fc_off * (m->bf16 ? 22.0 : 20.0), launch_sgd(m->Wm, m->Vm, m->Gm, m->Sm, fc_off, hy, st));
     m->have_fwd = false;   // the FC activations hold the last sub-iteration only: sb_backward has nothing consistent to use
     m->last_step_launches = m->launches;
     return SB_OK;
@@ -1212,11 +1221,7 @@ static sb_status modulo_step_direct(sb_model* m, const void* const* x, const int
 sb_status sb_sgd_step(sb_model* m, float lr, float momentum, void* stream)
 {
     if (!m) return fail(SB_ERR_INVALID_ARG, "null model");
-    cudaStream_t st = (cudaStream_t)stream;
-    m->cur_layer = -1;
-    L_TRY("sgd", 0.0, (double)m->P * (m->bf16 ? 22.0 : 20.0), launch_sgd(m->Wm, m->Vm, m->Gm, m->Sm, m->P, lr, momentum, st));
-    m->last_step_launches = m->launches;
-    return SB_OK;
+    return update_all(m, Hyper{lr, momentum, nullptr}, (cudaStream_t)stream);
 }
 
 sb_status sb_refresh_shadow(sb_model* m, void* stream)
@@ -1268,9 +1273,43 @@ static void abandon_capture(cudaStream_t st)
     cudaGetLastError();
 }
 
+// What was captured on `st` becomes G's executable graph.  An executable graph that is there already is updated in place where
+// the two have the same shape (other input pointers): 0.2 ms where destroying and instantiating it takes 2 ms at VGG-16 size.
+static sb_status end_capture(sb_model::StepGraph& G, cudaStream_t st)
+{
+    cudaGraph_t graph = nullptr;
+    CU_TRY(cudaStreamEndCapture(st, &graph));
+    cudaError_t e = cudaErrorUnknown;
+    if (G.exec) {
+        cudaGraphExecUpdateResultInfo info{};
+        e = cudaGraphExecUpdate(G.exec, graph, &info);
+        if (e != cudaSuccess) { cudaGetLastError(); cudaGraphExecDestroy(G.exec); G.exec = nullptr; }
+    }
+    if (e != cudaSuccess) e = cudaGraphInstantiate(&G.exec, graph, 0);
+    cudaGraphDestroy(graph);
+    if (e != cudaSuccess) { G.exec = nullptr; return fail(SB_ERR_CUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(e)); }
+    return SB_OK;
+}
+
+// What the capture of an iteration is to use for its hyper-parameters.
+static Hyper capture_hyper(sb_model* m, const sb_model::StepGraph& G, float lr, float momentum)
+{
+    if (G.exec && !G.fits(lr, momentum)) m->hyper_words = true;
+    return Hyper{lr, momentum, m->hyper_words ? m->hyper : nullptr};
+}
+static sb_status launch_graph(sb_model* m, const sb_model::StepGraph& G, float lr, float momentum, cudaStream_t st)
+{
+    if (G.hy.dev && (m->hyper_lr != lr || m->hyper_mu != momentum)) {
+        CU_TRY(launch_hyper(m->hyper, lr, momentum, st));
+        m->hyper_lr = lr; m->hyper_mu = momentum;
+    }
+    CU_TRY(cudaGraphLaunch(G.exec, st));
+    return SB_OK;
+}
+
 // An iteration on device-resident inputs replayed as a CUDA graph: the first call runs `step` directly, the second
-// captures it, later calls with the same pointers and hyper-parameters are one graph launch.
-typedef sb_status (*StepFn)(sb_model*, const void* const*, const int32_t* const*, float, float, void*);
+// captures it, later calls with the same pointers are one graph launch; other pointers are captured into the same graph.
+typedef sb_status (*StepFn)(sb_model*, const void* const*, const int32_t* const*, Hyper, void*);
 static sb_status graph_replay(sb_model* m, sb_model::StepGraph& G, StepFn step, const void* const* x, const int32_t* const* labels,
                               float lr, float momentum, void* stream)
 {
@@ -1282,25 +1321,21 @@ static sb_status graph_replay(sb_model* m, sb_model::StepGraph& G, StepFn step, 
     const bool eager = m->profiling || m->debug_sync || !G.warmed || st == nullptr;
     if (eager) {
         // first use (one-time function attributes are set by the first launches), or a mode that needs every launch visible
-        sb_status s = step(m, x, labels, lr, momentum, stream);
+        sb_status s = step(m, x, labels, Hyper{lr, momentum, nullptr}, stream);
         if (s == SB_OK) G.warmed = true;
         return s;
     }
-    const bool hit = G.exec && same_ptrs(G.x, xt, m->cfg.R) && same_ptrs(G.labels, lt, m->cfg.R) && G.lr == lr && G.mu == momentum;
+    const bool hit = G.exec && same_ptrs(G.x, xt, m->cfg.R) && same_ptrs(G.labels, lt, m->cfg.R) && G.fits(lr, momentum);
     if (!hit) {
-        if (G.exec) { cudaGraphExecDestroy(G.exec); G.exec = nullptr; }
+        const Hyper hy = capture_hyper(m, G, lr, momentum);
         CU_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-        sb_status s = step(m, x, labels, lr, momentum, stream);
+        sb_status s = step(m, x, labels, hy, stream);
         if (s != SB_OK) { abandon_capture(st); return s; }
-        cudaGraph_t graph = nullptr;
-        CU_TRY(cudaStreamEndCapture(st, &graph));
-        cudaError_t e = cudaGraphInstantiate(&G.exec, graph, 0);
-        cudaGraphDestroy(graph);
-        if (e != cudaSuccess) { G.exec = nullptr; return fail(SB_ERR_CUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(e)); }
-        G.x = xt; G.labels = lt; G.lr = lr; G.mu = momentum;
+        s = end_capture(G, st);
+        if (s != SB_OK) return s;
+        G.x = xt; G.labels = lt; G.hy = hy;
     }
-    CU_TRY(cudaGraphLaunch(G.exec, st));
-    return SB_OK;
+    return launch_graph(m, G, lr, momentum, st);
 }
 
 sb_status sb_graph_step(sb_model* m, const void* const* x, const int32_t* const* labels, float lr, float momentum, void* stream)
@@ -1325,8 +1360,8 @@ namespace {
 sb_status host_step_objects(sb_model* m)
 {
     if (m->host_res) return SB_OK;
-    CU_TRY(cudaHostAlloc((void**)&m->host_res, 6 * sizeof(uint32_t), cudaHostAllocDefault));
-    memset(m->host_res, 0, 6 * sizeof(uint32_t));
+    CU_TRY(cudaHostAlloc((void**)&m->host_res, 4 * sizeof(uint32_t), cudaHostAllocDefault));
+    memset(m->host_res, 0, 4 * sizeof(uint32_t));
     CU_TRY(cudaStreamCreateWithFlags(&m->cpstream, cudaStreamNonBlocking));
     for (int k = 0; k < 2; ++k) {
         CU_TRY(cudaEventCreateWithFlags(&m->ev_staged[k], cudaEventDisableTiming));
@@ -1391,7 +1426,7 @@ static sb_status host_step(sb_model* m, const void* host_x, const int32_t* host_
         if (m->n_flights > 0) return fail(SB_ERR_STATE, "iterations are in flight: only staged batches may be launched behind them");
         m->stage_next = 1;      // (this call copies into staging area 0 itself: the next prefetch goes to area 1)
     }
-    const int slot = pre ? buf : 2;
+    const int slot = buf;
     const void* xp[MAX_PARTS];
     const int32_t* lp[MAX_PARTS];
     const int b = m->cfg.batch_per_replica;
@@ -1399,49 +1434,40 @@ static sb_status host_step(sb_model* m, const void* host_x, const int32_t* host_
         xp[r] = m->stage_xb[buf] + (size_t)r * b * m->in_per_img * m->esz;
         lp[r] = m->stage_lb[buf] + (size_t)r * b;
     }
-    sb_model::StepGraph& G = pre ? m->g_pre[buf] : m->g_host;
-    const bool eager = m->profiling || m->debug_sync || !m->g_host.warmed || st == nullptr;
+    sb_model::StepGraph& G = m->g_host[buf];
+    const bool eager = m->profiling || m->debug_sync || !m->host_warmed || st == nullptr;
     sb_status s = SB_OK;
     bool finished = false;
     float loss = 0.f;
+    if (!pre) {
+        CU_TRY(cudaMemcpyAsync(m->stage_x, host_x, xb, cudaMemcpyHostToDevice, st));
+        CU_TRY(cudaMemcpyAsync(m->stage_labels, host_labels, (size_t)m->B * 4, cudaMemcpyHostToDevice, st));
+    }
     if (eager) {
-        if (!pre) {
-            CU_TRY(cudaMemcpyAsync(m->stage_x, host_x, xb, cudaMemcpyHostToDevice, st));
-            CU_TRY(cudaMemcpyAsync(m->stage_labels, host_labels, (size_t)m->B * 4, cudaMemcpyHostToDevice, st));
-        }
-        s = whole_step(m, xp, lp, lr, momentum, stream);
+        s = whole_step(m, xp, lp, Hyper{lr, momentum, nullptr}, stream);
         if (s != SB_OK) return s;
-        m->g_host.warmed = true;
+        m->host_warmed = true;
         if (pre) CU_TRY(cudaEventRecord(m->ev_done[buf], st));
         s = sb_loss(m, stream, &loss);       // (synchronises: the direct path is the first call and the diagnostic modes)
         finished = true;
     } else {
-        // One graph per (host buffers, lr, momentum): H2D copies (unless staged beforehand), the whole iteration, and the
-        // loss / status read-back.  A staged batch has one graph per staging area, keyed by lr and momentum only.
-        const bool hit = G.exec && (pre || (G.host_x == host_x && G.host_labels == (const void*)host_labels)) && G.lr == lr && G.mu == momentum;
-        if (!hit) {
-            if (G.exec) { cudaGraphExecDestroy(G.exec); G.exec = nullptr; }
+        // One graph per staging area: the whole iteration and the loss / status read-back.  The input copies stay outside, so that
+        // the graph does not depend on the host buffers (a loader hands out another one every step) or the hyper-parameters.
+        if (!G.exec || !G.fits(lr, momentum)) {
+            const Hyper hy = capture_hyper(m, G, lr, momentum);
             CU_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-            cudaError_t e = cudaSuccess;
-            if (!pre) {
-                e = cudaMemcpyAsync(m->stage_x, host_x, xb, cudaMemcpyHostToDevice, st);
-                if (e == cudaSuccess) e = cudaMemcpyAsync(m->stage_labels, host_labels, (size_t)m->B * 4, cudaMemcpyHostToDevice, st);
-            }
-            s = e == cudaSuccess ? SB_OK : fail(SB_ERR_CUDA, "capturing the input copies: %s", cudaGetErrorString(e));
-            if (s == SB_OK) s = whole_step(m, xp, lp, lr, momentum, stream);
+            s = whole_step(m, xp, lp, hy, stream);
             if (s == SB_OK) {
-                e = cudaMemcpyAsync(&m->host_res[2 * slot], m->loss, 8, cudaMemcpyDeviceToHost, st);      // loss and status word
+                const cudaError_t e = cudaMemcpyAsync(&m->host_res[2 * slot], m->loss, 8, cudaMemcpyDeviceToHost, st);      // loss and status word
                 if (e != cudaSuccess) s = fail(SB_ERR_CUDA, "capturing the read-back: %s", cudaGetErrorString(e));
             }
             if (s != SB_OK) { abandon_capture(st); return s; }
-            cudaGraph_t graph = nullptr;
-            CU_TRY(cudaStreamEndCapture(st, &graph));
-            e = cudaGraphInstantiate(&G.exec, graph, 0);
-            cudaGraphDestroy(graph);
-            if (e != cudaSuccess) { G.exec = nullptr; return fail(SB_ERR_CUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(e)); }
-            G.host_x = host_x; G.host_labels = host_labels; G.lr = lr; G.mu = momentum;
+            s = end_capture(G, st);
+            if (s != SB_OK) return s;
+            G.hy = hy;
         }
-        CU_TRY(cudaGraphLaunch(G.exec, st));
+        s = launch_graph(m, G, lr, momentum, st);
+        if (s != SB_OK) return s;
         if (pre) CU_TRY(cudaEventRecord(m->ev_done[buf], st));
         m->have_fwd = true;
         if (wait || !pre) {

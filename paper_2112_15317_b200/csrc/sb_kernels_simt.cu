@@ -782,11 +782,12 @@ __device__ __forceinline__ void sgd_apply(float4& ww, float4& vv, const float4& 
 // all give the same step time, and confined to 32 or 64 blocks the update overlaps but is itself too slow;
 // streaming (evict-first) loads and stores make no difference either.  SB_SGD_BLOCKS_PER_SM changes the grid.)
 template <bool SHADOW>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 4)
 sgd_kernel(float4* __restrict__ w, float4* __restrict__ v, const float4* __restrict__ g,
-           uint2* __restrict__ shadow, size_t n4, float lr, float mu)
+           uint2* __restrict__ shadow, size_t n4, Hyper hy)
 {
     pdl_prologue();
+    const float lr = hy.rate(), mu = hy.decay();
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     for (; i + 3 * stride < n4; i += 4 * stride) {
@@ -813,9 +814,10 @@ sgd_kernel(float4* __restrict__ w, float4* __restrict__ v, const float4* __restr
 template <bool SHADOW>
 __global__ void __launch_bounds__(256)
 reduce_sgd4_kernel(const float4* __restrict__ part, size_t stride4, int splits, float4* __restrict__ w, float4* __restrict__ v,
-                   uint2* __restrict__ shadow, size_t n4, float lr, float mu)
+                   uint2* __restrict__ shadow, size_t n4, Hyper hy)
 {
     pdl_prologue();
+    const float lr = hy.rate(), mu = hy.decay();
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
         float4 ww = w[i], vv = v[i];
         float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -842,9 +844,10 @@ __device__ __forceinline__ void sgd_apply_scalar(float* w, float* v, float g, __
 template <int LANES>
 __global__ void __launch_bounds__(32 * LANES)
 reduce_sgd_many_kernel(const float* __restrict__ part, size_t stride, int splits, float* __restrict__ w, float* __restrict__ v,
-                       __nv_bfloat16* __restrict__ shadow, size_t n, float lr, float mu)
+                       __nv_bfloat16* __restrict__ shadow, size_t n, Hyper hy)
 {
     pdl_prologue();
+    const float lr = hy.rate(), mu = hy.decay();
     __shared__ float s[LANES][33];
     const int e = threadIdx.x % 32, lane = threadIdx.x / 32;
     const size_t i = blockIdx.x * 32ull + e;
@@ -859,9 +862,10 @@ reduce_sgd_many_kernel(const float* __restrict__ part, size_t stride, int splits
 }
 __global__ void __launch_bounds__(256)
 reduce_sgd_kernel(const float* __restrict__ part, size_t stride, int splits, float* __restrict__ w, float* __restrict__ v,
-                  __nv_bfloat16* __restrict__ shadow, size_t n, float lr, float mu)
+                  __nv_bfloat16* __restrict__ shadow, size_t n, Hyper hy)
 {
     pdl_prologue();
+    const float lr = hy.rate(), mu = hy.decay();
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         float t = 0.f;
         for (int sp = 0; sp < splits; ++sp) t += part[(size_t)sp * stride + i];
@@ -869,35 +873,47 @@ reduce_sgd_kernel(const float* __restrict__ part, size_t stride, int splits, flo
     }
 }
 cudaError_t launch_reduce_sgd(const float* part, size_t stride, size_t n, int splits, float* w, float* v, __nv_bfloat16* shadow,
-                              float lr, float mu, cudaStream_t st)
+                              Hyper hy, cudaStream_t st)
 {
     // (the same case split as launch_reduce_partials: each case sums in the same order there and here)
     if (splits >= 128 && n <= (1u << 20)) {
-        SB_LAUNCH((reduce_sgd_many_kernel<32>), cdiv((long)n, 32), 1024, 0, st, part, stride, splits, w, v, shadow, n, lr, mu);
+        SB_LAUNCH((reduce_sgd_many_kernel<32>), cdiv((long)n, 32), 1024, 0, st, part, stride, splits, w, v, shadow, n, hy);
     } else if (splits >= 32 && n <= (1u << 20)) {
-        SB_LAUNCH((reduce_sgd_many_kernel<8>), cdiv((long)n, 32), 256, 0, st, part, stride, splits, w, v, shadow, n, lr, mu);
+        SB_LAUNCH((reduce_sgd_many_kernel<8>), cdiv((long)n, 32), 256, 0, st, part, stride, splits, w, v, shadow, n, hy);
     } else if (n % 4 == 0 && stride % 4 == 0 && (((uintptr_t)part | (uintptr_t)w | (uintptr_t)v) & 15) == 0 && (((uintptr_t)shadow) & 7) == 0) {
         int blocks = cdiv((long)(n / 4), 256);
         if (blocks > 148 * 8) blocks = 148 * 8;
-        if (shadow) SB_LAUNCH((reduce_sgd4_kernel<true>), blocks, 256, 0, st, (const float4*)part, stride / 4, splits, (float4*)w, (float4*)v, (uint2*)shadow, n / 4, lr, mu);
-        else SB_LAUNCH((reduce_sgd4_kernel<false>), blocks, 256, 0, st, (const float4*)part, stride / 4, splits, (float4*)w, (float4*)v, nullptr, n / 4, lr, mu);
+        if (shadow) SB_LAUNCH((reduce_sgd4_kernel<true>), blocks, 256, 0, st, (const float4*)part, stride / 4, splits, (float4*)w, (float4*)v, (uint2*)shadow, n / 4, hy);
+        else SB_LAUNCH((reduce_sgd4_kernel<false>), blocks, 256, 0, st, (const float4*)part, stride / 4, splits, (float4*)w, (float4*)v, nullptr, n / 4, hy);
     } else {
         int blocks = cdiv((long)n, 256);
         if (blocks > 148 * 8) blocks = 148 * 8;
-        SB_LAUNCH((reduce_sgd_kernel), blocks, 256, 0, st, part, stride, splits, w, v, shadow, n, lr, mu);
+        SB_LAUNCH((reduce_sgd_kernel), blocks, 256, 0, st, part, stride, splits, w, v, shadow, n, hy);
     }
     return cudaGetLastError();
 }
 
-cudaError_t launch_sgd(float* w, float* v, const float* g, __nv_bfloat16* shadow, size_t n, float lr, float mu, cudaStream_t st)
+// hyper-parameter words of the replayed iterations (see Hyper)
+__global__ void hyper_kernel(float* dev, float lr, float mu)
+{
+    pdl_prologue();
+    if (threadIdx.x == 0) { dev[0] = lr; dev[1] = mu; }
+}
+cudaError_t launch_hyper(float* dev, float lr, float mu, cudaStream_t st)
+{
+    SB_LAUNCH((hyper_kernel), 1, 32, 0, st, dev, lr, mu);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sgd(float* w, float* v, const float* g, __nv_bfloat16* shadow, size_t n, Hyper hy, cudaStream_t st)
 {
     size_t n4 = n / 4;
     static const int per_sm = (int)tune("SB_SGD_BLOCKS_PER_SM", 16);
     long blocks = ((long)n4 + 255) / 256;
     if (blocks > 148L * per_sm) blocks = 148L * per_sm;
     if (blocks < 1) blocks = 1;
-    if (shadow) SB_LAUNCH((sgd_kernel<true>), (int)blocks, 256, 0, st, (float4*)w, (float4*)v, (const float4*)g, (uint2*)shadow, n4, lr, mu);
-    else SB_LAUNCH((sgd_kernel<false>), (int)blocks, 256, 0, st, (float4*)w, (float4*)v, (const float4*)g, nullptr, n4, lr, mu);
+    if (shadow) SB_LAUNCH((sgd_kernel<true>), (int)blocks, 256, 0, st, (float4*)w, (float4*)v, (const float4*)g, (uint2*)shadow, n4, hy);
+    else SB_LAUNCH((sgd_kernel<false>), (int)blocks, 256, 0, st, (float4*)w, (float4*)v, (const float4*)g, nullptr, n4, hy);
     return cudaGetLastError();
 }
 

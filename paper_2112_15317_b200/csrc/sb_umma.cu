@@ -84,7 +84,7 @@ struct UmmaParams {
     // the tile's offsets (same element offsets as in `out`) and refreshes their bf16 copy instead of storing g
     float *sgd_w, *sgd_v;
     __nv_bfloat16* sgd_s;
-    float sgd_lr, sgd_mu;
+    Hyper sgd_hy;
     // Reciprocals for the divisions on the CTAs' start-up and epilogue paths (filled by launch_op from the fields above):
     // q = n / d as __umulhi(n, mul) with mul = 2^32 / d + 1, exact while n * d < 2^32; mul = 0 stands for d = 1.
     uint32_t rcp_tiles_w, rcp_tiles_wh, rcp_bw, rcp_bwbh, rcp_wb, rcp_wbhb;   // (wb, hb = bw / 2, bh / 2: the pooled box)
@@ -220,7 +220,7 @@ __device__ __forceinline__ void upd_request_slab(const CUtensorMap* mapW, const 
 template <int BN>
 __device__ __forceinline__ bool wgrad_sweep_update_epilogue(const UmmaParams& p, const CUtensorMap* mapW, const CUtensorMap* mapV, uint32_t taddr,
                                                              uint8_t* stage, uint8_t* slab_buf, uint64_t* slab_bar, int row, int m0, int m_hi, int n0,
-                                                             int n_hi, size_t tile_off)
+                                                             int n_hi, size_t tile_off, float lr, float mu)
 {
     const uint32_t slab_s = smem_u32(slab_buf);
     const int t128 = threadIdx.x - 64, q = t128 >> 5, lane = t128 & 31;
@@ -258,8 +258,8 @@ __device__ __forceinline__ bool wgrad_sweep_update_epilogue(const UmmaParams& p,
                              : "r"(buf_s + (uint32_t)rr * 256u + ((uint32_t)hl << 4)));
                 asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
                              : "r"(buf_s + 32768u + (uint32_t)rr * 256u + ((uint32_t)hl << 4)));
-                v.x = fmaf(p.sgd_mu, v.x, g.x); v.y = fmaf(p.sgd_mu, v.y, g.y); v.z = fmaf(p.sgd_mu, v.z, g.z); v.w = fmaf(p.sgd_mu, v.w, g.w);
-                w.x = fmaf(-p.sgd_lr, v.x, w.x); w.y = fmaf(-p.sgd_lr, v.y, w.y); w.z = fmaf(-p.sgd_lr, v.z, w.z); w.w = fmaf(-p.sgd_lr, v.w, w.w);
+                v.x = fmaf(mu, v.x, g.x); v.y = fmaf(mu, v.y, g.y); v.z = fmaf(mu, v.z, g.z); v.w = fmaf(mu, v.w, g.w);
+                w.x = fmaf(-lr, v.x, w.x); w.y = fmaf(-lr, v.y, w.y); w.z = fmaf(-lr, v.z, w.z); w.w = fmaf(-lr, v.w, w.w);
                 const size_t off = tile_off + (size_t)rr * p.ldc + c0 + 4 * hl;
                 __stcs((float4*)(p.sgd_v + off), v);
                 __stcs((float4*)(p.sgd_w + off), w);
@@ -870,7 +870,9 @@ umma_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         // where this thread's accumulator row goes (computed while the main loop runs)
         bool row_ok;
         size_t row_off;
+        float lr = 0.f, mu = 0.f;      // (update folded in: fetched while the main loop runs)
         if (MODE == MODE_WGRAD) {
+            if (p.sgd_w != nullptr) { lr = p.sgd_hy.rate(); mu = p.sgd_hy.decay(); }
             row_ok = (m0 + row) < m_hi;
             row_off = (size_t)split * p.split_stride + (size_t)(m0 + row) * p.ldc + (size_t)tap_fixed * p.w_cols;
             if (p.sgd_w != nullptr && threadIdx.x == 64) {
@@ -911,7 +913,7 @@ umma_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
             if (ok && (m0 + row) < m_hi) {
                 const size_t bo = (size_t)split * p.split_stride + p.bias_off + m0 + row;
                 if (p.sgd_w != nullptr) {
-                    const float vb = fmaf(p.sgd_mu, p.sgd_v[bo], bsum), wb = fmaf(-p.sgd_lr, vb, p.sgd_w[bo]);
+                    const float vb = fmaf(mu, p.sgd_v[bo], bsum), wb = fmaf(-lr, vb, p.sgd_w[bo]);
                     p.sgd_v[bo] = vb;
                     p.sgd_w[bo] = wb;
                     if (p.sgd_s != nullptr) p.sgd_s[bo] = __float2bfloat16_rn(wb);
@@ -935,7 +937,7 @@ umma_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16);
                 if (p.sgd_w != nullptr) {
                     if (!wgrad_sweep_update_epilogue<BN>(p, &mapC, &mapD, taddr, smem, slab_buf, slab_bar, row, m0, m_hi, n0, n_hi,
-                                                         (size_t)split * p.split_stride + (size_t)m0 * p.ldc + (size_t)tap_fixed * p.w_cols + n0) && lane == 0) {
+                                                         (size_t)split * p.split_stride + (size_t)m0 * p.ldc + (size_t)tap_fixed * p.w_cols + n0, lr, mu) && lane == 0) {
                         *abort_flag = 1; atomicMax(p.status, (uint32_t)DEV_TIMEOUT_EPI);
                     }
                 } else if (BN == 192 && p.hn_order)      // slab j = tap row j of filter column tap_fixed / 3: gradient columns (3 j + column) * Cin ..
@@ -2204,7 +2206,7 @@ void umma_set_timing_buffer(void* dev_ptr) { g_timing = (unsigned long long*)dev
 void umma_set_trace_buffer(void* dev_ptr) { g_trace = (unsigned long long*)dev_ptr; }
 #endif
 
-struct SgdFuse { float *w, *v; __nv_bfloat16* s; float lr, mu; };
+struct SgdFuse { float *w, *v; __nv_bfloat16* s; Hyper hy; };
 static bool wgrad_sweep_ok(const OpBlock* b)
 {
     const UmmaParams& pp = b->p;
@@ -2224,7 +2226,7 @@ static sb_status launch_op(const UmmaOp& op, cudaStream_t st, int64_t* launches 
             snprintf(g_umma_err, sizeof(g_umma_err), "weight gradient with folded update asked for an op that cannot carry it");
             return SB_ERR_CUDA;
         }
-        pp.sgd_w = fuse->w; pp.sgd_v = fuse->v; pp.sgd_s = fuse->s; pp.sgd_lr = fuse->lr; pp.sgd_mu = fuse->mu;
+        pp.sgd_w = fuse->w; pp.sgd_v = fuse->v; pp.sgd_s = fuse->s; pp.sgd_hy = fuse->hy;
     }
     if (pp.mode == MODE_WGRAD && !b->pair) {
         pp.wg_sweep = wgrad_sweep_ok(b) ? 1 : 0;
@@ -3023,11 +3025,11 @@ bool umma_fc_wgrad_can_update(sb_model* m, int layer)
     return b->p.mode == MODE_WGRAD && b->upd_maps && !b->pair && b->p.ntaps == 1 && b->bn != 192 && b->p.splits == 1 && b->p.bias_fused && wgrad_sweep_ok(b) &&
            (lv.p_w & 3) == 0 && (lv.in_f % 64) == 0 && smem <= 227 * 1024 && (long)b->grid.x * b->grid.y * b->grid.z >= min_ctas;
 }
-sb_status umma_fc_wgrad_update(sb_model* m, int layer, float lr, float mu, cudaStream_t st)
+sb_status umma_fc_wgrad_update(sb_model* m, int layer, Hyper hy, cudaStream_t st)
 {
     const ModelView mv = model_view(m);
     const LayerView lv = layer_view(m, layer);
-    SgdFuse f{mv.Wm + lv.p_w, mv.Vm + lv.p_w, mv.Sm ? mv.Sm + lv.p_w : nullptr, lr, mu};
+    SgdFuse f{mv.Wm + lv.p_w, mv.Vm + lv.p_w, mv.Sm ? mv.Sm + lv.p_w : nullptr, hy};
     return launch_op(lv.um->wgrad, st, nullptr, &f);
 }
 

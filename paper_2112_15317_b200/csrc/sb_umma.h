@@ -79,7 +79,7 @@ sb_status umma_fc_wgrad(sb_model* m, int layer, cudaStream_t st);
 // FC weight gradient with the SGD-momentum update applied in the kernel's epilogue (gradient never stored): possible when
 // umma_fc_wgrad_can_update says so (unsplit reduction, staged epilogue, bias gradient in the same kernel)
 bool umma_fc_wgrad_can_update(sb_model* m, int layer);
-sb_status umma_fc_wgrad_update(sb_model* m, int layer, float lr, float mu, cudaStream_t st);
+sb_status umma_fc_wgrad_update(sb_model* m, int layer, Hyper hy, cudaStream_t st);
 
 // Input-layer convolution (1, 3 or 4 input channels, 64 output channels, bf16) on the tensor cores.
 bool conv_in_umma_supported(int Cin, int Cout);
