@@ -55,10 +55,10 @@ struct UmmaParams {
     int kchunks, w_cols;
     // output columns
     int n_total;          // valid output columns (FWD: Cout, DGRAD: Cin, WGRAD: Cin)
-    int shards, tiles_per_shard;  // N-tile enumeration per model shard (FWD of a sharded FC layer); shards=1 otherwise
+    int n_tiles;          // N tiles.  (The K column shards of an FC layer lie one after another in its [out][in] matrix and in its output
+                          // rows, so the tiles run over the whole width: one that spans two shards computes the same elements.)
     // WGRAD
     int m_total;          // rows of the weight gradient (Cout / out-features)
-    int m_shards, m_tiles_per_shard;
     int tap_group;        // WGRAD: filter taps per CTA: 1, 3 (one filter row; Cin = 64, N tile = 3 x 64 columns) or 2 (Cin = 128,
                           // N tile = 2 x 128 columns; the fifth group holds tap 8 alone)
     int splits, chunks_per_split, total_chunks;   // split of the reduction (k-iterations) over blockIdx.z
@@ -614,24 +614,15 @@ umma_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         n_hi = p.n_total;                                     // tap_group = 3: 3 x Cin (the taps' columns are adjacent)
         if (p.tap_group == 2) n_hi = min(p.n_total, (9 - tap_fixed) * p.w_cols);   // the last pair of taps has one member
     } else {
-        if (p.shards == 1) {
-            n0 = n_idx * BN;
-            n_hi = p.n_total;
-        } else {
-            const int sh = n_idx / p.tiles_per_shard, t = n_idx % p.tiles_per_shard;
-            const int lo = (int)(((long)sh * p.n_total) / p.shards), hi = (int)(((long)(sh + 1) * p.n_total) / p.shards);
-            n0 = lo + t * BN;
-            n_hi = hi;
-        }
+        n0 = n_idx * BN;
+        n_hi = p.n_total;
         if (n0 >= n_hi) return;   // uniform over the CTA, before any barrier or TMEM allocation
     }
-    // FWD/DGRAD: the M tile is one pixel box; WGRAD: the M tile is 128 gradient rows of one shard
+    // FWD/DGRAD: the M tile is one pixel box; WGRAD: the M tile is 128 gradient rows
     int pw0 = 0, ph0 = 0, pn0 = 0, m0 = 0, m_hi = 0;
     if (MODE == MODE_WGRAD) {
-        const int sh = m_idx / p.m_tiles_per_shard, t = m_idx % p.m_tiles_per_shard;
-        const int lo = (int)(((long)sh * p.m_total) / p.m_shards), hi = (int)(((long)(sh + 1) * p.m_total) / p.m_shards);
-        m0 = lo + t * 128;
-        m_hi = hi;
+        m0 = m_idx * 128;
+        m_hi = p.m_total;
         if (m0 >= m_hi) return;
     } else {
         const int q1 = fast_div_exact(m_idx, p.rcp_tiles_w, p.tiles_w), q2 = fast_div_exact(m_idx, p.rcp_tiles_wh, p.tiles_w * p.tiles_h);
@@ -1366,7 +1357,7 @@ umma_halo_persist_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_
     SB_TRACE_BEGIN();
     SB_TLOG(threadIdx.x == 0, 6, clock64());
     const int m_tiles = p.tiles_w * p.tiles_h * p.tiles_n;
-    const int n_tiles_total = m_tiles * p.tiles_per_shard;       // (tiles_per_shard = N tiles; conv layers have one shard)
+    const int n_tiles_total = m_tiles * p.n_tiles;
     const int n_groups = p.total_chunks;                         // 3 * kchunks groups per tile
     const uint32_t smem0 = smem_u32(smem), bring0 = smem_u32(b_ring);
 
@@ -1709,7 +1700,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
     const bool leader = rank == 0;
 
     // ---- tile coordinates (the pair shares blockIdx.y / blockIdx.z; its M tiles are 2j and 2j+1) ----
-    // FWD / DGRAD: M tile = a 128-pixel box, N tile inside a shard.  WGRAD (conv layers, one tap per CTA, unsharded): M
+    // FWD / DGRAD: M tile = a 128-pixel box, N tile = BN columns.  WGRAD (conv layers, one tap per CTA, unsharded): M
     // tile = 128 gradient rows (output channels), N tile = BN input channels, blockIdx.z = tap * splits + split.
     const int m_idx = blockIdx.x, n_idx = blockIdx.y;
     int split = blockIdx.z, tap_fixed = 0, n0, n_hi, m0 = 0, m_hi = 0;
@@ -1719,15 +1710,8 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
         n0 = n_idx * BN; n_hi = p.n_total;
         m0 = m_idx * 128; m_hi = p.m_total;
     } else {
-        if (p.shards == 1) {
-            n0 = n_idx * BN;
-            n_hi = p.n_total;
-        } else {
-            const int sh = n_idx / p.tiles_per_shard, t = n_idx % p.tiles_per_shard;
-            const int lo = (int)(((long)sh * p.n_total) / p.shards);
-            n_hi = (int)(((long)(sh + 1) * p.n_total) / p.shards);
-            n0 = lo + t * BN;
-        }
+        n0 = n_idx * BN;
+        n_hi = p.n_total;
     }
     if (n0 >= n_hi) return;   // uniform over the pair, before any barrier or TMEM allocation
     // an M index past the last tile (odd tile count) lands wholly out of bounds: zero loads, no stores
@@ -2334,33 +2318,33 @@ static int cohabit_stages(int bn) { return bn >= 192 ? 2 : (bn >= 128 ? 3 : 4); 
 //   * a CTA carries ~3 us of fixed work (start, first loads, drain, epilogue);
 //   * a split reduction costs a second kernel (~4 us) plus ~0.5 us per MB of float partial sums written and read back
 //     (8.4 MB -> 7 us, 16.8 MB -> 9 us, 33.5 MB -> 27 us measured).
-static double plan_cost(int bn, int s, int n_cols_per_shard, int shards, long m_tiles, int k_iters)
+static double plan_cost(int bn, int s, int n_cols, long m_tiles, int k_iters)
 {
-    const long ctas = m_tiles * cdiv_i(n_cols_per_shard, bn) * shards * s;
+    const long ctas = m_tiles * cdiv_i(n_cols, bn) * s;
     const double per_sm = (bn < 256 && ctas >= 296) ? 2.0 : 1.0;
     const double waves = (double)cdiv_i(ctas, (long)(148 * per_sm));
     const double t_iter = bn >= 256 ? 0.38 : (bn >= 128 ? 0.315 : 0.245);
-    const double partial_mb = (double)s * (double)m_tiles * 128.0 * (double)n_cols_per_shard * shards * 4.0 / 1.0e6;
+    const double partial_mb = (double)s * (double)m_tiles * 128.0 * (double)n_cols * 4.0 / 1.0e6;
     const double mb_us = 0.5;
     return waves * (cdiv_i(k_iters, s) * t_iter * (per_sm > 1.0 ? 1.6 : 1.0) + 3.0) + (s > 1 ? 4.0 + mb_us * partial_mb : 0.0);
 }
-static TilePlan plan_tiles(int n_cols_per_shard, int shards, long m_tiles, int k_iters, bool backward, bool force_pair)
+static TilePlan plan_tiles(int n_cols, long m_tiles, int k_iters, bool backward, bool force_pair)
 {
     TilePlan t;
     int best_bn = 64, best_s = 1;
     {
         double best = 1e300;
         for (int bn = 64; bn <= 256; bn *= 2) {
-            if (bn > 64 && bn / 2 >= n_cols_per_shard) break;      // never wider than the columns need
-            if (force_pair && bn < 256 && bn < n_cols_per_shard) continue;   // forced pairs: the widest tile only
+            if (bn > 64 && bn / 2 >= n_cols) break;      // never wider than the columns need
+            if (force_pair && bn < 256 && bn < n_cols) continue;   // forced pairs: the widest tile only
             for (int s = 1; s <= 32 && (s == 1 || k_iters / s >= 4); s *= 2) {
-                const double c = plan_cost(bn, s, n_cols_per_shard, shards, m_tiles, k_iters);
+                const double c = plan_cost(bn, s, n_cols, m_tiles, k_iters);
                 if (c < best - 1e-9) { best = c; best_bn = bn; best_s = s; }
             }
         }
     }
     t.bn = best_bn;
-    const long tiles = m_tiles * cdiv_i(n_cols_per_shard, t.bn) * shards;
+    const long tiles = m_tiles * cdiv_i(n_cols, t.bn);
     t.cps = cdiv_i(k_iters, best_s);
     t.splits = cdiv_i(k_iters, t.cps);
     const int fit = t.bn >= 256 ? 4 : (t.bn >= 128 ? 6 : 8);
@@ -2412,7 +2396,7 @@ static TilePlan plan_tiles(int n_cols_per_shard, int shards, long m_tiles, int k
         t.stages = pst < 1 ? 1 : pst;
     }
     static const bool verbose = tune("SB_PLAN_VERBOSE", 0) != 0;
-    if (verbose) fprintf(stderr, "plan: N/shard=%d shards=%d m_tiles=%ld k_iters=%d -> bn=%d splits=%d stages=%d pair=%d\n", n_cols_per_shard, shards, m_tiles, k_iters, t.bn, t.splits, t.stages, t.pair);
+    if (verbose) fprintf(stderr, "plan: N=%d m_tiles=%ld k_iters=%d -> bn=%d splits=%d stages=%d pair=%d\n", n_cols, m_tiles, k_iters, t.bn, t.splits, t.stages, t.pair);
     return t;
 }
 
@@ -2643,8 +2627,8 @@ static ConvGeom conv_geom(const LayerView& lv, int B, bool force_pair, bool no_h
         choose_box(lv.W, lv.H, B, 128, &g.bw, &g.bh, &g.bn);
         g.tw = cdiv_i(lv.W, g.bw); g.th = cdiv_i(lv.H, g.bh); g.tn = cdiv_i(B, g.bn);
         g.m_tiles = (long)g.tw * g.th * g.tn;
-        g.fwd = plan_tiles(lv.Cout, 1, g.m_tiles, 9 * (lv.Cin / 64), false, force_pair);
-        g.dgrad = plan_tiles(lv.Cin, 1, g.m_tiles, 9 * (lv.Cout / 64), true, force_pair);
+        g.fwd = plan_tiles(lv.Cout, g.m_tiles, 9 * (lv.Cin / 64), false, force_pair);
+        g.dgrad = plan_tiles(lv.Cin, g.m_tiles, 9 * (lv.Cout / 64), true, force_pair);
     }
     choose_box(lv.W, lv.H, B, 64, &g.cw, &g.ch, &g.cn);
     g.ctw = cdiv_i(lv.W, g.cw); g.cth = cdiv_i(lv.H, g.ch); g.ctn = cdiv_i(B, g.cn);
@@ -2686,12 +2670,12 @@ struct FcGeom {
     int m_tiles;
     TilePlan fwd, dgrad;
 };
-static FcGeom fc_geom(const LayerView& lv, int B, int K, bool force_pair)
+static FcGeom fc_geom(const LayerView& lv, int B, bool force_pair)
 {
     FcGeom g;
     g.m_tiles = cdiv_i(B, 128);
-    g.fwd = plan_tiles(cdiv_i(lv.out_f, K), K, g.m_tiles, lv.in_f / 64, false, force_pair);
-    g.dgrad = plan_tiles(lv.in_f, 1, g.m_tiles, cdiv_i(lv.out_f, 64), true, force_pair);
+    g.fwd = plan_tiles(lv.out_f, g.m_tiles, lv.in_f / 64, false, force_pair);
+    g.dgrad = plan_tiles(lv.in_f, g.m_tiles, cdiv_i(lv.out_f, 64), true, force_pair);
     return g;
 }
 
@@ -2709,7 +2693,7 @@ sb_status umma_plan_scratch(sb_model* m, size_t* floats)
             if (g.fwd.splits > 1) upd((size_t)g.fwd.splits * pix * lv.Cout);
             if (g.dgrad.splits > 1) upd((size_t)g.dgrad.splits * pix * lv.Cin);
         } else if ((lv.kind == SB_FC_RELU || lv.kind == SB_FC) && fc_umma_ok(mv, lv, i)) {
-            FcGeom g = fc_geom(lv, mv.B, lv.K, (mv.cfg->flags & SB_FLAG_FORCE_PAIR) != 0);
+            FcGeom g = fc_geom(lv, mv.B, (mv.cfg->flags & SB_FLAG_FORCE_PAIR) != 0);
             if (g.fwd.splits > 1) upd((size_t)g.fwd.splits * mv.B * lv.out_f);
             if (g.dgrad.splits > 1) upd((size_t)g.dgrad.splits * mv.B * lv.in_f);
         }
@@ -2743,15 +2727,14 @@ static void apply_plan(OpBlock* b, const TilePlan& t, int k_iters, long m_tiles,
 }
 
 // TMA-store epilogue of a FWD / DGRAD op: possible when the output is bf16, the reduction is not split, every N tile
-// ends on a 64-column slab boundary inside its shard, and the idle operand ring can hold the staged tile.
+// ends on a 64-column slab boundary, and the idle operand ring can hold the staged tile.
 // SB_TMA_OUT=0 keeps the direct row stores.
-static bool tma_out_ok(const OpBlock* b, int cols_per_shard, int shards)
+static bool tma_out_ok(const OpBlock* b)
 {
     static const bool off = tune("SB_TMA_OUT", 1) == 0;
     const UmmaParams& p = b->p;
     if (off || p.out_f32 || p.splits > 1 || p.epi == UEPI_F32) return false;
     if (p.n_total % 64 != 0 || p.ldc % 64 != 0) return false;
-    if (shards > 1 && (cols_per_shard % b->bn != 0 || p.n_total % shards != 0)) return false;
     if (b->halo && b->persist) return true;
     if (b->halo) return (long)p.a_stages * (p.bh + 2) * p.bw * p.bn * 128 + (long)p.stages * b->bn * 128 >= (long)(b->bn / 64) * 16384;
     const long stage_bytes = b->pair ? 16384 + b->bn * 64 : 16384 + b->bn * 128;
@@ -2786,16 +2769,16 @@ sb_status umma_plan_layers(sb_model* m, int first_layer)
                 UmmaParams& p = b->p;
                 p.mode = MODE_FWD; p.ntaps = 9; p.bw = g.bw; p.bh = g.bh; p.bn = g.bn; p.W = lv.W; p.H = lv.H; p.N = B;
                 p.tiles_w = g.tw; p.tiles_h = g.th; p.tiles_n = g.tn; p.kchunks = lv.Cin / 64; p.w_cols = lv.Cin;
-                p.n_total = lv.Cout; p.shards = 1;
-                p.tiles_per_shard = cdiv_i(lv.Cout, g.fwd.bn);
+                p.n_total = lv.Cout;
+                p.n_tiles = cdiv_i(lv.Cout, g.fwd.bn);
                 p.epi = UEPI_BIAS_ACT; p.relu = 1; p.out_f32 = 0; p.out = lv.act; p.ldc = lv.Cout; p.bias = mv.Wm + lv.p_b;
                 p.status = mv.status;
-                apply_plan(b, g.fwd, g.halo ? 3 * p.kchunks : 9 * p.kchunks, g.m_tiles, p.tiles_per_shard, mv.ws, pix);
+                apply_plan(b, g.fwd, g.halo ? 3 * p.kchunks : 9 * p.kchunks, g.m_tiles, p.n_tiles, mv.ws, pix);
                 if (g.halo) {
                     if (!act_map_hn(&um.fwd.mapA, lv.in_act, B, lv.H, lv.W, lv.Cin, g.bw, g.bh + 2, g.bn)) return fail_plan();
                 } else if (!act_map(&um.fwd.mapA, lv.in_act, B, lv.H, lv.W, lv.Cin, g.bw, g.bh, g.bn)) return fail_plan();
                 if (!mat_map(&um.fwd.mapB, mv.Sm + lv.p_w, lv.Cout, 9L * lv.Cin, b->pair ? b->bn / 2 : b->bn)) return fail_plan();
-                if (tma_out_ok(b, lv.Cout, 1)) {
+                if (tma_out_ok(b)) {
                     if (g.halo) {
                         if (!act_map_hn(&um.fwd.mapC, lv.act, B, lv.H, lv.W, lv.Cout, g.bw, g.bh, g.bn)) return fail_plan();
                     } else if (!act_map(&um.fwd.mapC, lv.act, B, lv.H, lv.W, lv.Cout, g.bw, g.bh, g.bn)) return fail_plan();
@@ -2821,17 +2804,17 @@ sb_status umma_plan_layers(sb_model* m, int first_layer)
                 UmmaParams& p = b->p;
                 p.mode = MODE_DGRAD; p.ntaps = 9; p.bw = g.bw; p.bh = g.bh; p.bn = g.bn; p.W = lv.W; p.H = lv.H; p.N = B;
                 p.tiles_w = g.tw; p.tiles_h = g.th; p.tiles_n = g.tn; p.kchunks = lv.Cout / 64; p.w_cols = lv.Cin;
-                p.n_total = lv.Cin; p.shards = 1;
-                p.tiles_per_shard = cdiv_i(lv.Cin, g.dgrad.bn);
+                p.n_total = lv.Cin;
+                p.n_tiles = cdiv_i(lv.Cin, g.dgrad.bn);
                 p.epi = UEPI_MASK; p.out = lv.d_below; p.ldc = lv.Cin;
                 p.ref = lv.below_relu ? (const __nv_bfloat16*)lv.in_act : nullptr;
                 p.status = mv.status;
-                apply_plan(b, g.dgrad, g.halo ? 3 * p.kchunks : 9 * p.kchunks, g.m_tiles, p.tiles_per_shard, mv.ws, pix);
+                apply_plan(b, g.dgrad, g.halo ? 3 * p.kchunks : 9 * p.kchunks, g.m_tiles, p.n_tiles, mv.ws, pix);
                 if (g.halo) {
                     if (!act_map_hn(&um.dgrad.mapA, lv.dact, B, lv.H, lv.W, lv.Cout, g.bw, g.bh + 2, g.bn)) return fail_plan();
                 } else if (!act_map(&um.dgrad.mapA, lv.dact, B, lv.H, lv.W, lv.Cout, g.bw, g.bh, g.bn)) return fail_plan();
                 if (!mat_map(&um.dgrad.mapB, mv.Sm + lv.p_w, lv.Cout, 9L * lv.Cin, 64)) return fail_plan();
-                if (tma_out_ok(b, lv.Cin, 1)) {
+                if (tma_out_ok(b)) {
                     if (g.halo) {
                         if (!act_map_hn(&um.dgrad.mapC, lv.d_below, B, lv.H, lv.W, lv.Cin, g.bw, g.bh, g.bn)) return fail_plan();
                     } else if (!act_map(&um.dgrad.mapC, lv.d_below, B, lv.H, lv.W, lv.Cin, g.bw, g.bh, g.bn)) return fail_plan();
@@ -2847,8 +2830,8 @@ sb_status umma_plan_layers(sb_model* m, int first_layer)
                 p.mode = MODE_WGRAD; p.ntaps = 9; p.bw = g.cw; p.bh = g.ch; p.bn = g.cn; p.W = lv.W; p.H = lv.H; p.N = B;
                 p.tiles_w = g.ctw; p.tiles_h = g.cth; p.tiles_n = g.ctn;
                 p.total_chunks = g.total_chunks;
-                p.w_cols = lv.Cin; p.n_total = lv.Cin * g.wg_tap_group; p.shards = 1; p.tiles_per_shard = 1;
-                p.m_total = lv.Cout; p.m_shards = 1; p.m_tiles_per_shard = g.wg_m_tiles;
+                p.w_cols = lv.Cin; p.n_total = lv.Cin * g.wg_tap_group;
+                p.m_total = lv.Cout;
                 p.tap_group = g.wg_tap_group;
                 b->bn = g.wg_bn;
                 p.splits = g.wg_splits;
@@ -2860,7 +2843,7 @@ sb_status umma_plan_layers(sb_model* m, int first_layer)
                 {
                     // grids of fewer than ~100 CTAs leave the other streams whole SMs: no need to keep the ring shallow (measured: -1.5 % step)
                     static const long wg_cohabit_min = (long)tune("SB_WG_COHABIT_MIN_CTAS", 100);
-                    const long ctas = (long)p.m_tiles_per_shard * g.wg_n_tiles * ((9 + p.tap_group - 1) / p.tap_group) * p.splits;
+                    const long ctas = (long)g.wg_m_tiles * g.wg_n_tiles * ((9 + p.tap_group - 1) / p.tap_group) * p.splits;
                     // (the filter-row kernel keeps its whole five-stage ring: with two slots per round the deeper ring is worth more
                     // than a neighbour on the SM -- steps -0.2 to -1.6 % against a ring cut to two or three 40 KB stages)
                     const int cap = b->bn == 192 ? 5 : cohabit_stages(b->bn);
@@ -2892,7 +2875,7 @@ sb_status umma_plan_layers(sb_model* m, int first_layer)
                 }
                 p.out = p.splits > 1 ? (void*)mv.ws_wk[mv.n_wstreams > 0 ? i % mv.n_wstreams : 0] : (void*)(mv.Gm + lv.p_w);
                 p.status = mv.status;
-                b->grid = dim3((unsigned)p.m_tiles_per_shard, (unsigned)g.wg_n_tiles, (unsigned)((9 + p.tap_group - 1) / p.tap_group * p.splits));
+                b->grid = dim3((unsigned)g.wg_m_tiles, (unsigned)g.wg_n_tiles, (unsigned)((9 + p.tap_group - 1) / p.tap_group * p.splits));
                 if ((size_t)p.splits * (lv.n_w + lv.n_b) > mv.ws_floats && p.splits > 1) return SB_ERR_ARENA_TOO_SMALL;
                 // 64 input channels: one filter COLUMN per CTA instead of one filter row -- the three taps then share one
                 // activation box with a halo row above and below (the three N panels of the MMA are windows into it) instead
@@ -2910,27 +2893,26 @@ sb_status umma_plan_layers(sb_model* m, int first_layer)
                 um.wgrad.enabled = true;
             }
         } else if ((lv.kind == SB_FC_RELU || lv.kind == SB_FC) && fc_umma_ok(mv, lv, i)) {
-            const int K = lv.K;
-            const FcGeom g = fc_geom(lv, B, K, (mv.cfg->flags & SB_FLAG_FORCE_PAIR) != 0);
+            const FcGeom g = fc_geom(lv, B, (mv.cfg->flags & SB_FLAG_FORCE_PAIR) != 0);
             const int m_tiles = g.m_tiles;
             if (i == 0) lv.in_act = mv.stage_x;   // placeholder; rebound to the caller's input by umma_bind_input
             const bool fc_in_grad = i > 0 || (mv.cfg->flags & SB_FLAG_INPUT_GRAD);
-            // ---- forward: Y[:, shard j] = X W_j^T + b_j ; N tiles enumerated per shard ----
+            // ---- forward: Y = X W^T + b over the shards' concatenated columns ----
             {
                 OpBlock* b = blk(um.fwd);
                 memset(b, 0, sizeof(*b));
                 UmmaParams& p = b->p;
                 p.mode = MODE_FWD; p.ntaps = 1; p.bw = 1; p.bh = 1; p.bn = 128; p.W = 1; p.H = 1; p.N = B;
                 p.tiles_w = 1; p.tiles_h = 1; p.tiles_n = m_tiles; p.kchunks = lv.in_f / 64; p.w_cols = lv.in_f;
-                p.n_total = lv.out_f; p.shards = K;
-                p.tiles_per_shard = cdiv_i(cdiv_i(lv.out_f, K), g.fwd.bn);
+                p.n_total = lv.out_f;
+                p.n_tiles = cdiv_i(lv.out_f, g.fwd.bn);
                 p.epi = UEPI_BIAS_ACT; p.relu = lv.relu ? 1 : 0; p.out_f32 = lv.kind == SB_FC; p.out = lv.act; p.ldc = lv.out_f;
                 p.bias = mv.Wm + lv.p_b; p.status = mv.status;
-                apply_plan(b, g.fwd, p.kchunks, m_tiles, p.tiles_per_shard * K, mv.ws, (size_t)B);
+                apply_plan(b, g.fwd, p.kchunks, m_tiles, p.n_tiles, mv.ws, (size_t)B);
                 if (p.splits > 1 && (size_t)p.splits * (size_t)p.split_stride > mv.ws_floats) return SB_ERR_ARENA_TOO_SMALL;
                 if (!act_map(&um.fwd.mapA, lv.in_act, B, 1, 1, lv.in_f, 1, 1, 128)) return fail_plan();
                 if (!mat_map(&um.fwd.mapB, mv.Sm + lv.p_w, lv.out_f, lv.in_f, b->pair ? b->bn / 2 : b->bn)) return fail_plan();
-                if (tma_out_ok(b, cdiv_i(lv.out_f, K), K)) {
+                if (tma_out_ok(b)) {
                     if (!act_map(&um.fwd.mapC, lv.act, B, 1, 1, lv.out_f, 1, 1, 128)) return fail_plan();
                     p.tma_out = 1;
                 }
@@ -2943,33 +2925,31 @@ sb_status umma_plan_layers(sb_model* m, int first_layer)
                 UmmaParams& p = b->p;
                 p.mode = MODE_DGRAD; p.ntaps = 1; p.bw = 1; p.bh = 1; p.bn = 128; p.W = 1; p.H = 1; p.N = B;
                 p.tiles_w = 1; p.tiles_h = 1; p.tiles_n = m_tiles; p.kchunks = cdiv_i(lv.out_f, 64); p.w_cols = lv.in_f;
-                p.n_total = lv.in_f; p.shards = 1;
-                p.tiles_per_shard = cdiv_i(lv.in_f, g.dgrad.bn);
+                p.n_total = lv.in_f;
+                p.n_tiles = cdiv_i(lv.in_f, g.dgrad.bn);
                 p.epi = UEPI_MASK; p.out = lv.d_below; p.ldc = lv.in_f;
                 p.ref = lv.below_relu ? (const __nv_bfloat16*)lv.in_act : nullptr;
                 p.status = mv.status;
-                apply_plan(b, g.dgrad, p.kchunks, m_tiles, p.tiles_per_shard, mv.ws, (size_t)B);
+                apply_plan(b, g.dgrad, p.kchunks, m_tiles, p.n_tiles, mv.ws, (size_t)B);
                 if (p.splits > 1 && (size_t)p.splits * (size_t)p.split_stride > mv.ws_floats) return SB_ERR_ARENA_TOO_SMALL;
                 if (!act_map(&um.dgrad.mapA, lv.dact, B, 1, 1, lv.out_f, 1, 1, 128)) return fail_plan();
                 if (!mat_map(&um.dgrad.mapB, mv.Sm + lv.p_w, lv.out_f, lv.in_f, 64)) return fail_plan();
-                if (tma_out_ok(b, lv.in_f, 1)) {
+                if (tma_out_ok(b)) {
                     if (!act_map(&um.dgrad.mapC, lv.d_below, B, 1, 1, lv.in_f, 1, 1, 128)) return fail_plan();
                     p.tma_out = 1;
                 }
                 um.dgrad.enabled = true;
             }
-            // ---- weight gradient: dW_j = dY_j^T X ; M tiles enumerated per shard (needs 16-byte aligned shard starts) ----
-            bool aligned = true;
-            for (int j = 0; j <= K; ++j) aligned = aligned && ((((long)j * lv.out_f) / K) % 8 == 0);
-            if (aligned) {
+            // ---- weight gradient: dW = dY^T X over the shards' concatenated rows ----
+            {
                 OpBlock* b = blk(um.wgrad);
                 memset(b, 0, sizeof(*b));
                 UmmaParams& p = b->p;
                 p.mode = MODE_WGRAD; p.ntaps = 1; p.bw = 1; p.bh = 1; p.bn = 64; p.W = 1; p.H = 1; p.N = B;
                 p.tiles_w = 1; p.tiles_h = 1; p.tiles_n = cdiv_i(B, 64);
                 p.total_chunks = p.tiles_n;
-                p.w_cols = lv.in_f; p.n_total = lv.in_f; p.shards = 1; p.tiles_per_shard = 1;
-                p.m_total = lv.out_f; p.m_shards = K; p.m_tiles_per_shard = cdiv_i(cdiv_i(lv.out_f, K), 128);
+                p.w_cols = lv.in_f; p.n_total = lv.in_f;
+                p.m_total = lv.out_f;
                 p.tap_group = 1;
                 b->bn = lv.in_f >= 256 ? 256 : (lv.in_f >= 128 ? 128 : 64);
                 const int n_tiles = cdiv_i(lv.in_f, b->bn);
@@ -2980,7 +2960,7 @@ sb_status umma_plan_layers(sb_model* m, int first_layer)
                 p.bias_fused = 1; p.bias_off = (long)lv.n_w;
                 p.out = (void*)(mv.Gm + lv.p_w);
                 p.status = mv.status;
-                b->grid = dim3((unsigned)(p.m_tiles_per_shard * K), (unsigned)n_tiles, 1);
+                b->grid = dim3((unsigned)cdiv_i(lv.out_f, 128), (unsigned)n_tiles, 1);
                 if (!act_map(&um.wgrad.mapA, lv.dact, B, 1, 1, lv.out_f, 1, 1, 64)) return fail_plan();
                 if (!act_map(&um.wgrad.mapB, lv.in_act, B, 1, 1, lv.in_f, 1, 1, 64)) return fail_plan();
                 // float maps over the master weights and the momentum buffer, for the weight gradient with the update folded in
