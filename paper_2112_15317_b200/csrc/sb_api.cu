@@ -8,7 +8,7 @@
 //    the same buffer shape *is* the scatter back to the replicas (modulo layer, backward).
 //  * an FC weight is [out, in]; shard j is the row block [c_j, c_{j+1}), c_j = floor(j*out/K),
 //    and owns the output columns with the same indices (shard layer, forward = column concat by
-//    addressing).  The FC kernels take (shard_dim, K) and never let a tile straddle two shards.
+//    addressing).  The FC kernels' tiles run over the concatenated shards.
 #include "../../include/splitbrain.h"
 #include "sb_internal.h"
 #include "sb_umma.h"
@@ -52,12 +52,11 @@ struct Layer {
     char* act = nullptr;                        // [B, out_per_img] activation dtype (float for the logits layer)
     char* dact = nullptr;                       // same shape, activation dtype
     uint8_t* idx = nullptr;                     // pool argmax
-    int wg_splits = 1;                          // conv wgrad pixel-range splits (CUDA-core kernel)
-    int bg_splits = 1;                          // conv bias-gradient row splits
     bool thin_input = false;                    // conv with Cin of 1/3/4: dedicated input-layer kernels
     bool narrow = false;                        // FC with out <= 16: dedicated narrow kernels
     int K = 1;                                  // FC: column shards of this layer (the model's K, or 1 for a layer kept whole)
     int act_dt = SB_DT_F32;
+    ContractPlan cplan[3];                      // forward / data gradient / weight gradient on CUDA cores, where these run there
     UmmaLayer um;                               // tensor-core plan of this layer (tcgen05 path)
     // Sub-batch copies of the first FC layer (modulo schedule): where its input comes from and where its input
     // gradient goes, instead of the layer below's buffers
@@ -197,6 +196,39 @@ struct sb_model {
 
 namespace {
 
+inline bool has_weights(const Layer& l) { return l.kind == SB_CONV3X3_RELU || l.kind == SB_FC_RELU || l.kind == SB_FC; }
+
+// Shape, plan and layer input of layer i as a CUDA-core contraction (the FC layers' K column shards lie one after another in the
+// weight matrix and in the output rows, so they are one contraction over the whole width).
+ContractArgs contract_args(sb_model* m, int i, int mode)
+{
+    const Layer& l = m->L[i];
+    const bool conv = l.kind == SB_CONV3X3_RELU;
+    ContractArgs a{};
+    a.mode = mode; a.taps = conv ? 9 : 1; a.B = m->B;
+    a.H = conv ? l.H : 1; a.W = conv ? l.W : 1;
+    a.Cin = conv ? l.Cin : l.in_f; a.Cout = conv ? l.Cout : l.out_f;
+    a.plan = l.cplan[mode];
+    a.act = l.in_override ? l.in_override : (i > 0 ? m->L[i - 1].act : nullptr);
+    if (i == 0) { a.tab = &m->x_tab; a.tab_imgs = m->cfg.batch_per_replica; }
+    return a;
+}
+
+// Plans the CUDA-core passes of layer i for the model's current batch; returns the scratch floats they need.
+size_t contract_plan_layer(sb_model* m, int i, size_t max_part_floats)
+{
+    Layer& l = m->L[i];
+    size_t need = 0;
+    if (!has_weights(l) || l.narrow || umma_layer_ok(m, i)) return 0;
+    for (int mode : {CMODE_FWD, CMODE_DGRAD, CMODE_WGRAD}) {
+        const ContractArgs a = contract_args(m, i, mode);
+        l.cplan[mode] = contract_plan(mode, a.B, a.H, a.W, a.taps, a.Cin, a.Cout, max_part_floats);
+        const size_t result = mode == CMODE_WGRAD ? l.n_w + l.n_b : (size_t)a.B * a.H * a.W * (mode == CMODE_FWD ? a.Cout : a.Cin);
+        if (l.cplan[mode].splits > 1) need = std::max(need, l.cplan[mode].splits * result);
+    }
+    return need;
+}
+
 // Walks the layer list, fills shapes, and assigns arena offsets (relative to base, which may be
 // null for a pure size computation).  Returns SB_OK and the total size.
 sb_status plan(const sb_layer* layers, int n, const sb_config* cfg, sb_model* m, char* base, size_t* total)
@@ -318,18 +350,6 @@ sb_status plan(const sb_layer* layers, int n, const sb_config* cfg, sb_model* m,
         if (l.kind == SB_MAXPOOL2) l.idx = (uint8_t*)take(B * l.out_per_img);
         if (l.kind == SB_FC_RELU || l.kind == SB_FC) l.narrow = fc_narrow_supported(l.out_f, (int)B);
         if (l.kind == SB_CONV3X3_RELU) {
-            // pixel-range splits of the weight gradient: enough blocks to fill the machine, each
-            // split a whole number of images
-            long tiles = (long)((l.Cout + 31) / 32) * ((l.Cin + 31) / 32) * 9;
-            int s = 1;
-            while (tiles * s < 148 * 4 && s * 2 <= (int)B && B % (s * 2) == 0) s *= 2;
-            l.wg_splits = s;
-            size_t need = (size_t)s * l.n_w;
-            if (need > ws_floats) ws_floats = need;
-            int sb_ = 1;
-            while (sb_ * 2 <= (int)B && B % (sb_ * 2) == 0 && (long)sb_ * ((l.Cout + 31) / 32) < 148 * 2) sb_ *= 2;
-            l.bg_splits = sb_;
-            if ((size_t)sb_ * l.n_b > ws_floats) ws_floats = (size_t)sb_ * l.n_b;
             l.thin_input = conv_in_supported(l.Cin, l.Cout);
             if (l.thin_input) {
                 const int nblk = std::max(conv_in_wgrad_blocks((int)B, l.H, l.W), conv_in_umma_wgrad_blocks((long)B * l.H * l.W));
@@ -338,6 +358,8 @@ sb_status plan(const sb_layer* layers, int n, const sb_config* cfg, sb_model* m,
             }
         }
     }
+    // CUDA-core layers: partial sums of split reductions, 64 MB at most
+    for (int i = 0; i < n; ++i) ws_floats = std::max(ws_floats, contract_plan_layer(m, i, (size_t)16 << 20));
     size_t um_ws = 0;
     sb_status us = umma_plan_scratch(m, &um_ws);
     if (us != SB_OK) return us;
@@ -408,6 +430,31 @@ inline int shard_lo(int j, int total, int K) { return (int)(((long)j * total) / 
 // Which buffer holds the input of layer i: the previous layer's output, or the caller's images.
 inline const char* layer_input(const sb_model* m, int i) { return m->L[i].in_override ? m->L[i].in_override : (i > 0 ? m->L[i - 1].act : nullptr); }
 
+const void* weights_of(const sb_model* m, const Layer& l) { return m->bf16 ? (const void*)(m->Sm + l.p_w) : (const void*)(m->Wm + l.p_w); }
+
+// CUDA-core passes of one layer
+sb_status contract_forward(sb_model* m, int i, const char* tag, double flops, double bytes, cudaStream_t st)
+{
+    const Layer& l = m->L[i];
+    ContractArgs a = contract_args(m, i, CMODE_FWD);
+    a.wt = weights_of(m, l); a.bias = m->Wm + l.p_b; a.relu = l.relu;
+    if (l.act_dt == SB_DT_F32) a.out32 = (float*)l.act; else a.out = l.act;
+    a.part = m->ws; a.split_stride = (long)a.B * a.H * a.W * a.Cout;
+    L_TRY(tag, flops, bytes, launch_contract(a, m->bf16, st));
+    if (a.plan.splits > 1) ++m->launches;
+    return SB_OK;
+}
+sb_status contract_dgrad(sb_model* m, int i, const char* tag, double flops, double bytes, void* dx, const void* ref, cudaStream_t st)
+{
+    const Layer& l = m->L[i];
+    ContractArgs a = contract_args(m, i, CMODE_DGRAD);
+    a.wt = weights_of(m, l); a.dy = l.dact; a.out = dx; a.ref = ref;
+    a.part = m->ws; a.split_stride = (long)a.B * a.H * a.W * a.Cin;
+    L_TRY(tag, flops, bytes, launch_contract(a, m->bf16, st));
+    if (a.plan.splits > 1) ++m->launches;
+    return SB_OK;
+}
+
 sb_status forward_layer(sb_model* m, int i, cudaStream_t st)
 {
     Layer& l = m->L[i];
@@ -429,13 +476,14 @@ sb_status forward_layer(sb_model* m, int i, cudaStream_t st)
             if (l.um.pool_fused) m->pooled_by_conv = i + 1;
             break;
         }
+        sb_status fs = SB_OK;
         ConvSimtArgs a{};
         a.in = layer_input(m, i); a.tab = i == 0 ? &m->x_tab : nullptr; a.b_per_rep = b;
-        a.w = wts; a.bias = m->Wm + l.p_b; a.out = l.act; a.mask_ref = nullptr;
-        a.B = B; a.H = l.H; a.W = l.W; a.Cin = l.Cin; a.Cout = l.Cout; a.dgrad = 0; a.relu = 1;
+        a.w = wts; a.bias = m->Wm + l.p_b; a.out = l.act;
+        a.B = B; a.H = l.H; a.W = l.W; a.Cin = l.Cin; a.Cout = l.Cout; a.relu = 1;
         if (l.thin_input && l.um.conv_in) L_TRY("conv_in_fwd_umma", flops, bytes, launch_conv_in_fwd_umma(a, &l.um.fwd.mapA, m->status, st));
         else if (l.thin_input) L_TRY("conv_in_fwd", flops, bytes, launch_conv_in_fwd(a, bf, st));
-        else L_TRY("conv_fwd_simt", flops, bytes, launch_conv_simt(a, bf, st));
+        else if ((fs = contract_forward(m, i, "conv_fwd_simt", flops, bytes, st)) != SB_OK) return fs;
         break;
     }
     case SB_MAXPOOL2: {
@@ -481,15 +529,8 @@ sb_status forward_layer(sb_model* m, int i, cudaStream_t st)
             L_TRY("fc_narrow_fwd", flops, bytes, launch_fc_narrow(a, bf, st));
             break;
         }
-        GemmSimtArgs a{};
-        a.A = layer_input(m, i); a.sAm = l.in_f; a.sAk = 1;
-        a.B = wts; a.sBn = l.in_f; a.sBk = 1;
-        a.M = B; a.N = l.out_f; a.K = l.in_f;
-        a.epi = EPI_BIAS_ACT; a.ldc = l.out_f; a.bias = m->Wm + l.p_b; a.relu = l.relu;
-        if (l.kind == SB_FC) { a.C = nullptr; a.C32 = (float*)l.act; } else { a.C = l.act; a.C32 = nullptr; }
-        a.shard_dim = 1; a.shards = l.K;
-        if (i == 0) { a.tab = &m->x_tab; a.tab_mode = 1; a.tab_b = b; }
-        L_TRY("fc_fwd_simt", flops, bytes, launch_gemm_simt(a, bf, st));
+        const sb_status fs = contract_forward(m, i, "fc_fwd_simt", flops, bytes, st);
+        if (fs != SB_OK) return fs;
         break;
     }
     case SB_DROPOUT: {
@@ -543,6 +584,46 @@ sb_status backward_layer(sb_model* m, int i, cudaStream_t st, int part = SIDE_BO
     // this layer's weight-side scratch: one region per weight stream, so two layers that share a region are
     // ordered by the stream they share
     float* const ws_w = m->ws_wk[m->n_wstreams > 0 ? i % m->n_wstreams : 0];
+    // End of a gradient range [goff, goff + n) of this layer: S > 1 partial copies at `src` are reduced in order into
+    // the gradient arena -- or, when the backward pass folds the update in, reduced and applied in one kernel (S = 1:
+    // the gradient is already in the arena and takes a plain update).
+    const bool fuse = m->fuse.on && (part & SIDE_W) && !(part & SIDE_D) && l.n_w % 4 == 0 && l.n_b % 4 == 0 && l.p_w % 4 == 0 && l.p_b % 4 == 0;
+    // (in_place: with S = 1 the kernel wrote the gradient into the arena itself; the input-layer kernels always write
+    // partial buffers, so a single one still has to be carried over)
+    auto finish = [&](const float* src, size_t stride, size_t goff, size_t n, int S, bool in_place = true) -> sb_status {
+        const bool reduce = S > 1 || !in_place;
+        if (!fuse) {
+            if (reduce) L_TRY("split_reduce", 0.0, (double)n * 4.0 * (S + 1), launch_reduce_partials(src, stride, m->Gm + goff, n, S, st));
+            return SB_OK;
+        }
+        if (!m->fuse.waited) { CU_TRY(cudaStreamWaitEvent(st, m->fuse.ev, 0)); m->fuse.waited = true; }
+        __nv_bfloat16* sh = m->Sm ? m->Sm + goff : nullptr;
+        if (reduce)
+            L_TRY("split_reduce_sgd", 0.0, (double)n * (4.0 * S + (m->bf16 ? 18.0 : 16.0)),
+                  launch_reduce_sgd(src, stride, n, S, m->Wm + goff, m->Vm + goff, sh, m->fuse.hy, st));
+        else
+            L_TRY("sgd", 0.0, (double)n * (m->bf16 ? 22.0 : 20.0), launch_sgd(m->Wm + goff, m->Vm + goff, m->Gm + goff, sh, n, m->fuse.hy, st));
+        m->fuse.covered += n;
+        return SB_OK;
+    };
+    // weights and bias gradient of a CUDA-core contraction: S > 1 copies of [n_w][n_b] at `src`
+    auto finish_both = [&](const float* src, int S) -> sb_status {
+        const size_t stride = l.n_w + l.n_b;
+        if (l.p_b == l.p_w + l.n_w) return finish(src, stride, l.p_w, stride, S);
+        const sb_status s = finish(src, stride, l.p_w, l.n_w, S);
+        return s != SB_OK ? s : finish(src + l.n_w, stride, l.p_b, l.n_b, S);
+    };
+    auto contract_wgrad = [&](const char* tag, double flops, double bytes, int* S) -> sb_status {
+        ContractArgs a = contract_args(m, i, CMODE_WGRAD);
+        a.dy = l.dact;
+        *S = a.plan.splits;
+        a.part = *S > 1 ? ws_w : m->Gm + l.p_w;
+        a.split_stride = (long)(l.n_w + l.n_b);
+        a.bias_off = *S > 1 ? (long)l.n_w : (long)(l.p_b - l.p_w);
+        L_TRY(tag, flops, bytes, launch_contract(a, bf, st));
+        return SB_OK;
+    };
+    sb_status fs = SB_OK;
     switch (l.kind) {
     case SB_SOFTMAX_XENT:
         break;  // dZ was produced by the forward loss kernel
@@ -575,17 +656,10 @@ sb_status backward_layer(sb_model* m, int i, cudaStream_t st, int part = SIDE_BO
             U_TRY("fc_wgrad_umma", flops, act_bytes + (double)l.n_w * 4.0, umma_fc_wgrad(m, i, st));
             ++m->launches;
         } else {
-            GemmSimtArgs a{};
-            a.A = l.dact; a.sAm = 1; a.sAk = l.out_f;
-            a.B = layer_input(m, i); a.sBn = 1; a.sBk = l.in_f;
-            a.M = l.out_f; a.N = l.in_f; a.K = B;
-            a.epi = EPI_F32; a.C = m->Gm + l.p_w; a.ldc = l.in_f;
-            a.shard_dim = 3; a.shards = l.K;
-            if (i == 0) { a.tab = &m->x_tab; a.tab_mode = 2; a.tab_b = b; }
-            L_TRY("fc_wgrad_simt", flops, act_bytes + (double)l.n_w * 4.0, launch_gemm_simt(a, bf, st));
+            int S = 1;
+            if ((fs = contract_wgrad("fc_wgrad_simt", flops, act_bytes + (double)l.n_w * 4.0, &S)) != SB_OK) return fs;
+            if ((fs = finish_both(ws_w, S)) != SB_OK) return fs;
         }
-        if (!l.um.wgrad.enabled && (part & SIDE_W))   // the tensor-core weight-gradient kernel also produces the bias gradient
-            L_TRY("bias_grad", 0.0, (double)B * l.out_f * e + 4.0 * l.out_f, launch_colsum(l.dact, bf, m->Gm + l.p_b, B, l.out_f, 1, st));
         if (want_in_grad && (part & SIDE_D)) {
             // shard-layer / modulo-layer backward: dX = sum_j dY_j W_j, rows stay with their replica
             const double bytes = act_bytes + (double)l.n_w * e + (below_relu ? (double)B * l.in_f * e : 0.0);
@@ -593,14 +667,7 @@ sb_status backward_layer(sb_model* m, int i, cudaStream_t st, int part = SIDE_BO
                 U_TRY("fc_dgrad_umma", flops, bytes, umma_fc_dgrad(m, i, st));
                 ++m->launches;
             } else {
-                GemmSimtArgs a{};
-                a.A = l.dact; a.sAm = l.out_f; a.sAk = 1;
-                a.B = wts; a.sBn = 1; a.sBk = l.in_f;
-                a.M = B; a.N = l.in_f; a.K = l.out_f;
-                a.epi = EPI_MASK; a.C = d_below; a.ldc = l.in_f;
-                a.ref = below_relu ? layer_input(m, i) : nullptr; a.ldref = l.in_f;
-                a.shard_dim = 2; a.shards = l.K;
-                L_TRY("fc_dgrad_simt", flops, bytes, launch_gemm_simt(a, bf, st));
+                if ((fs = contract_dgrad(m, i, "fc_dgrad_simt", flops, bytes, d_below, below_relu ? layer_input(m, i) : nullptr, st)) != SB_OK) return fs;
             }
         }
         break;
@@ -625,29 +692,6 @@ sb_status backward_layer(sb_model* m, int i, cudaStream_t st, int part = SIDE_BO
         if (i == 0 && !m->have_x) return fail(SB_ERR_STATE, "layer 0 needs input pointers");
         const double pix = (double)B * l.H * l.W;
         const double flops = 2.0 * pix * l.Cout * 9.0 * l.Cin;
-        // End of a gradient range [goff, goff + n) of this layer: S > 1 partial copies at `src` are reduced in order into
-        // the gradient arena -- or, when the backward pass folds the update in, reduced and applied in one kernel (S = 1:
-        // the gradient is already in the arena and takes a plain update).
-        const bool fuse = m->fuse.on && (part & SIDE_W) && !(part & SIDE_D) && l.n_w % 4 == 0 && l.n_b % 4 == 0 && l.p_w % 4 == 0 && l.p_b % 4 == 0;
-        // (in_place: with S = 1 the kernel wrote the gradient into the arena itself; the input-layer kernels always write
-        // partial buffers, so a single one still has to be carried over)
-        auto finish = [&](const float* src, size_t stride, size_t goff, size_t n, int S, bool in_place = true) -> sb_status {
-            const bool reduce = S > 1 || !in_place;
-            if (!fuse) {
-                if (reduce) L_TRY("split_reduce", 0.0, (double)n * 4.0 * (S + 1), launch_reduce_partials(src, stride, m->Gm + goff, n, S, st));
-                return SB_OK;
-            }
-            if (!m->fuse.waited) { CU_TRY(cudaStreamWaitEvent(st, m->fuse.ev, 0)); m->fuse.waited = true; }
-            __nv_bfloat16* sh = m->Sm ? m->Sm + goff : nullptr;
-            if (reduce)
-                L_TRY("split_reduce_sgd", 0.0, (double)n * (4.0 * S + (m->bf16 ? 18.0 : 16.0)),
-                      launch_reduce_sgd(src, stride, n, S, m->Wm + goff, m->Vm + goff, sh, m->fuse.hy, st));
-            else
-                L_TRY("sgd", 0.0, (double)n * (m->bf16 ? 22.0 : 20.0), launch_sgd(m->Wm + goff, m->Vm + goff, m->Gm + goff, sh, n, m->fuse.hy, st));
-            m->fuse.covered += n;
-            return SB_OK;
-        };
-        sb_status fs = SB_OK;
         // weight gradient over all replicas' pixels (the DP reduce is the sum over image ranges)
         if (!(part & SIDE_W)) {
         } else if (l.thin_input) {
@@ -681,29 +725,22 @@ sb_status backward_layer(sb_model* m, int i, cudaStream_t st, int part = SIDE_BO
                 else if ((fs = finish(part, l.n_w + l.n_b, l.p_w, l.n_w, S)) != SB_OK) return fs;
             }
         } else {
-            const int S = l.wg_splits;
-            WgradSimtArgs a{};
-            a.x = layer_input(m, i); a.tab = i == 0 ? &m->x_tab : nullptr; a.b_per_rep = b;
-            a.dy = l.dact; a.part = S > 1 ? ws_w : m->Gm + l.p_w;
-            a.B = B; a.H = l.H; a.W = l.W; a.Cin = l.Cin; a.Cout = l.Cout; a.splits = S;
-            L_TRY("conv_wgrad_simt", flops, pix * (l.Cin + l.Cout) * e + (double)l.n_w * 4.0, launch_wgrad_simt(a, bf, st));
-            if ((fs = finish(ws_w, l.n_w, l.p_w, l.n_w, S)) != SB_OK) return fs;
+            int S = 1;
+            if ((fs = contract_wgrad("conv_wgrad_simt", flops, pix * (l.Cin + l.Cout) * e + (double)l.n_w * 4.0, &S)) != SB_OK) return fs;
+            if ((fs = finish_both(ws_w, S)) != SB_OK) return fs;
         }
-        if (!l.thin_input && (part & SIDE_W) && (!l.um.wgrad.enabled || !umma_wgrad_bias_fused(m, i))) {
+        if (!l.thin_input && (part & SIDE_W) && l.um.wgrad.enabled && !umma_wgrad_bias_fused(m, i)) {
             // bias gradient: column sums of dY over image-range splits, then the same ordered reduce
             const long M = (long)B * l.H * l.W;
             // (stream order makes it safe to reuse the scratch the weight-gradient reduce just read)
-            int S = l.bg_splits;
-            if (bf && l.Cout % 8 == 0) {
-                // the vectorised column-sum kernel covers 256 columns per block column: split the rows finely enough to
-                // fill the machine (its splits need not be whole images), within the scratch
-                long want = 592 / ((l.Cout / 8 + 31) / 32);
-                if (want > M / 64) want = M / 64;
-                if (want > (long)(m->ws_floats / l.n_b)) want = (long)(m->ws_floats / l.n_b);
-                S = want < 1 ? 1 : (int)want;
-            }
+            // (the column-sum kernel covers 256 columns per block column: split the rows finely enough to fill the machine, within
+            // the scratch)
+            long want = 592 / ((l.Cout / 8 + 31) / 32);
+            if (want > M / 64) want = M / 64;
+            if (want > (long)(m->ws_floats / l.n_b)) want = (long)(m->ws_floats / l.n_b);
+            const int S = want < 1 ? 1 : (int)want;
             float* part = S > 1 ? ws_w : m->Gm + l.p_b;
-            L_TRY("bias_grad", 0.0, pix * l.Cout * e, launch_colsum(l.dact, bf, part, (int)M, l.Cout, S, st));
+            L_TRY("bias_grad", 0.0, pix * l.Cout * e, launch_colsum(l.dact, part, (int)M, l.Cout, S, st));
             if ((fs = finish(part, l.n_b, l.p_b, l.n_b, S)) != SB_OK) return fs;
         }
         if (want_in_grad && (part & SIDE_D)) {
@@ -712,12 +749,7 @@ sb_status backward_layer(sb_model* m, int i, cudaStream_t st, int part = SIDE_BO
                 U_TRY("conv_dgrad_umma", flops, bytes, umma_conv_dgrad(m, i, st));
                 ++m->launches;
             } else {
-                ConvSimtArgs a{};
-                a.in = l.dact; a.tab = nullptr; a.b_per_rep = b;
-                a.w = wts; a.bias = nullptr; a.out = d_below;
-                a.mask_ref = below_relu ? m->L[i - 1].act : nullptr;
-                a.B = B; a.H = l.H; a.W = l.W; a.Cin = l.Cin; a.Cout = l.Cout; a.dgrad = 1; a.relu = 0;
-                L_TRY("conv_dgrad_simt", flops, bytes, launch_conv_simt(a, bf, st));
+                if ((fs = contract_dgrad(m, i, "conv_dgrad_simt", flops, bytes, d_below, below_relu ? m->L[i - 1].act : nullptr, st)) != SB_OK) return fs;
             }
         }
         break;
@@ -936,6 +968,7 @@ sb_status sb_model_create(const sb_layer* layers, int32_t n, const sb_config* cf
             std::swap(m->L, m->mod_L[k]);
             m->B = Bk;
             s = umma_plan_layers(m, m->first_fc);
+            for (int i = m->first_fc; i < m->n_layers; ++i) contract_plan_layer(m, i, m->ws_floats);
             m->B = m->full_B;
             std::swap(m->L, m->mod_L[k]);
         }
@@ -1074,7 +1107,7 @@ static sb_status backward_pass(sb_model* m, cudaStream_t st, bool fuse_update, H
             static const bool reduce_updates = tune("SB_REDUCE_SGD", 1) != 0;
             // FC layers whose weight-gradient kernel can carry the update take the same order (SB_FC_WGRAD_UPDATE=0: separate update)
             static const bool fc_wgrad_update = tune("SB_FC_WGRAD_UPDATE", 1) != 0;
-            const bool in_reduce = fuse && ((reduce_updates && l.kind == SB_CONV3X3_RELU) ||
+            const bool in_reduce = fuse && ((reduce_updates && (l.kind == SB_CONV3X3_RELU || (!l.narrow && !l.um.wgrad.enabled))) ||
                                             (fc_wgrad_update && l.kind != SB_CONV3X3_RELU && !l.narrow && umma_fc_wgrad_can_update(m, i)));
             sb_status s = SB_OK;
             if (in_reduce) {

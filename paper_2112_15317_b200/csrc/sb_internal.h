@@ -94,29 +94,41 @@ enum : uint32_t { DEV_OK = 0, DEV_TIMEOUT_TMA = 1, DEV_TIMEOUT_MMA = 2, DEV_TIME
 // ---------------------------------------------------------------------------------------------
 
 struct ConvSimtArgs {
-    const void* in;       // [B,H,W,Cred] activation dtype (ignored when tab != nullptr)
+    const void* in;       // [B,H,W,Cin] activation dtype (ignored when tab != nullptr)
     const PtrTab* tab;    // optional: R per-replica input pointers (host pointer to the table)
     int b_per_rep;
     const void* w;        // [Cout,3,3,Cin] activation dtype (float master or bf16 shadow)
-    const float* bias;    // [Cout] (forward only)
-    void* out;            // [B,H,W,Cres] activation dtype
-    const void* mask_ref; // dgrad only, optional: zero the result where mask_ref <= 0 ([B,H,W,Cres])
+    const float* bias;    // [Cout]
+    void* out;            // [B,H,W,Cout] activation dtype
     int B, H, W, Cin, Cout;
-    int dgrad;            // 0: forward (+bias, ReLU if relu) ; 1: data gradient
     int relu;
 };
-cudaError_t launch_conv_simt(const ConvSimtArgs& a, bool bf16, cudaStream_t st);
-
 struct WgradSimtArgs {
     const void* x;        // [B,H,W,Cin] (ignored when tab != nullptr)
     const PtrTab* tab;
     int b_per_rep;
     const void* dy;       // [B,H,W,Cout]
-    float* part;          // [splits][Cout*9*Cin] partial sums (or the gradient itself if splits==1)
+    float* part;          // partial sums
     int B, H, W, Cin, Cout;
-    int splits;           // pixel-range splits; split s covers images [s*B/splits, (s+1)*B/splits)
 };
-cudaError_t launch_wgrad_simt(const WgradSimtArgs& a, bool bf16, cudaStream_t st);
+
+// 3x3 convolution (taps = 9) or fully-connected layer (taps = 1, H = W = 1) on CUDA cores: sb_contract_simt.cu.
+enum { CMODE_FWD = 0, CMODE_DGRAD = 1, CMODE_WGRAD = 2 };
+struct ContractPlan { int bm = 64, bn = 64, iters = 0, splits = 1; };     // block tile, reduction steps per split, splits
+// max_part_floats: room for split partial sums ([splits][result], for WGRAD with the bias gradient behind each)
+ContractPlan contract_plan(int mode, int B, int H, int W, int taps, int Cin, int Cout, size_t max_part_floats);
+struct ContractArgs {
+    int mode, taps, B, H, W, Cin, Cout;
+    const void *act, *wt, *dy;             // layer input (or tab), weights [Cout][taps][Cin], output gradient, in the activation dtype
+    const PtrTab* tab; int tab_imgs;       // optional: the layer input as per-replica buffers of tab_imgs images
+    ContractPlan plan;
+    float* part; long split_stride;        // splits > 1: partial sums.  WGRAD: always where the gradient (or its splits) goes,
+    long bias_off;                         // and the bias gradient's place relative to it
+    void* out; float* out32;               // FWD / DGRAD result (out32: float instead of the activation dtype)
+    const float* bias; int relu;           // FWD
+    const void* ref;                       // DGRAD: zero where ref <= 0
+};
+cudaError_t launch_contract(const ContractArgs& a, bool bf16, cudaStream_t st);
 
 // Input-layer convolution (Cin of 1, 3 or 4; Cout a multiple of 8): dedicated forward and weight+bias
 // gradient kernels.  The gradient kernel writes conv_in_wgrad_blocks() partial buffers of
@@ -139,8 +151,8 @@ struct FcNarrowArgs {
 bool fc_narrow_supported(int out_f, int B);
 cudaError_t launch_fc_narrow(const FcNarrowArgs& a, bool bf16, cudaStream_t st);
 
-// part[s][n] = sum over the rows of split s of in[row][n];  rows split evenly (M % splits == 0).
-cudaError_t launch_colsum(const void* in, bool bf16, float* part, int M, int N, int splits, cudaStream_t st);
+// part[s][n] = sum over the rows of split s of in[row][n] (bf16, N a multiple of 8).
+cudaError_t launch_colsum(const void* in, float* part, int M, int N, int splits, cudaStream_t st);
 // out[i] = sum_{s<splits} part[s*stride + i], s ascending.
 cudaError_t launch_reduce_partials(const float* part, size_t stride, float* out, size_t n, int splits, cudaStream_t st);
 // the same ordered sum, consumed at once by the SGD step of the n parameters at w / v (shadow: their bf16 copies or nullptr)
@@ -209,35 +221,15 @@ cudaError_t launch_sgd(float* w, float* v, const float* g, __nv_bfloat16* shadow
 cudaError_t launch_hyper(float* dev, float lr, float mu, cudaStream_t st);
 cudaError_t launch_to_bf16(const float* w, __nv_bfloat16* shadow, size_t n, cudaStream_t st);
 
-enum { EPI_BIAS_ACT = 0, EPI_MASK = 1, EPI_F32 = 2 };
+enum { EPI_BIAS_ACT = 0, EPI_MASK = 1 };
 // Ordered sum of split-reduction partial sums [split][rows][N] followed by the GEMM epilogue
-// (epi = EPI_BIAS_ACT or EPI_MASK below); N must be a multiple of 4.
+// (epi = EPI_BIAS_ACT or EPI_MASK below).
 struct SplitKEpiArgs {
     const float* part; size_t split_stride; int splits;
     long rows; int N;
     int epi; const float* bias; int relu; const void* ref;
     void* out; int out_f32;
 };
-cudaError_t launch_splitk_epilogue(const SplitKEpiArgs& a, cudaStream_t st);
-
-// Strided GEMM  C[m,n] = sum_k A(m,k) * B(n,k)  with A(m,k) = A[m*sAm + k*sAk], B(n,k) = B[n*sBn + k*sBk].
-struct GemmSimtArgs {
-    const void* A; long sAm, sAk;
-    const void* B; long sBn, sBk;
-    int M, N, K;
-    int epi;
-    void* C; long ldc;        // activation dtype (EPI_BIAS_ACT, EPI_MASK) or float (EPI_F32)
-    float* C32;               // EPI_BIAS_ACT: optional float copy of the result (logits), same ldc
-    const float* bias;        // EPI_BIAS_ACT: [N]
-    int relu;
-    const void* ref; long ldref;  // EPI_MASK: optional, zero where ref <= 0
-    // Model-shard partition of one GEMM dimension: 0 none, 1 = N (forward: each shard owns its
-    // output columns), 2 = K (dgrad: sum over shards), 3 = M (wgrad: each shard owns its rows).
-    int shard_dim, shards;
-    // Optional replica gather by addressing: the rows of the activation matrix live in R separate
-    // caller buffers of tab_b rows each.  tab_mode 1: A's m index is the row; 2: B's k index is.
-    const PtrTab* tab; int tab_mode, tab_b;
-};
-cudaError_t launch_gemm_simt(const GemmSimtArgs& a, bool bf16, cudaStream_t st);
+cudaError_t launch_splitk_epilogue(const SplitKEpiArgs& a, bool bf16, cudaStream_t st);
 
 }  // namespace sb

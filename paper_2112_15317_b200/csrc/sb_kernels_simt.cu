@@ -2,10 +2,7 @@
 //
 //  * bandwidth-bound steps that every mode uses: 2x2 max-pool forward/backward, softmax
 //    cross-entropy, SGD with momentum, column sums (bias gradients) and split reductions;
-//  * float-accumulating FFMA versions of the contractions (3x3 conv forward / dgrad / wgrad and
-//    a strided GEMM for the sharded FC layers).  They are the float mode, serve layers whose
-//    channel count does not fit the tensor-core tiles (e.g. the 3-channel input layer), and are
-//    the on-device cross-check of the tcgen05 kernels.
+//  * the input layer's convolution and the narrow FC layers, which no contraction tile fits.
 //
 // T is the activation dtype (float or __nv_bfloat16); all sums are carried in float.
 #include "sb_internal.h"
@@ -39,226 +36,8 @@ __device__ __forceinline__ void store8(__nv_bfloat16* p, const float (&v)[8])
 static inline int cdiv(long a, long b) { return (int)((a + b - 1) / b); }
 
 // =============================================================================================
-// 3x3 convolution, forward and data gradient (direct, tiled through shared memory).
-//   forward: y[n,h,w,o] = act(bias[o] + sum_{r,s,i} x[n,h+r-1,w+s-1,i] * W[o,r,s,i])
-//   dgrad  : dx[n,h,w,o] = mask * sum_{r,s,i} dy[n,h-r+1,w-s+1,i] * W[i,r,s,o]
-// Block: 8x8 output pixels x 32 output channels, 128 threads, 4 pixels x 4 channels per thread.
-// =============================================================================================
-constexpr int CV_TP = 8, CV_TC = 32, CV_CK = 16;
-
-template <typename T, bool DGRAD, bool TAB>
-__global__ void __launch_bounds__(128)
-conv3x3_simt_kernel(const T* __restrict__ in, PtrTab tab, int b_per_rep, const T* __restrict__ wt,
-                    const float* __restrict__ bias, T* __restrict__ out, const T* __restrict__ mask_ref,
-                    int H, int W, int Cred, int Cres, int Cin, int relu)
-{
-    pdl_prologue();
-    __shared__ float s_in[CV_TP + 2][CV_TP + 2][CV_CK + 1];
-    __shared__ float s_w[9][CV_CK][CV_TC];
-    const int tiles_w = (W + CV_TP - 1) / CV_TP;
-    const int h0 = (blockIdx.x / tiles_w) * CV_TP, w0 = (blockIdx.x % tiles_w) * CV_TP;
-    const int n = blockIdx.y;
-    const int o0 = blockIdx.z * CV_TC;
-    const int tid = threadIdx.x;
-    const int cg = tid / 16, pg = tid % 16;
-    const int prow = pg / 2, pcol = (pg % 2) * 4;
-    const T* img = TAB ? (const T*)tab.p[n / b_per_rep] + (size_t)(n % b_per_rep) * H * W * Cred
-                       : in + (size_t)n * H * W * Cred;
-    float acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-
-    for (int c0 = 0; c0 < Cred; c0 += CV_CK) {
-        for (int e = tid; e < (CV_TP + 2) * (CV_TP + 2) * CV_CK; e += 128) {
-            int c = e % CV_CK, q = e / CV_CK;
-            int ww = q % (CV_TP + 2), hh = q / (CV_TP + 2);
-            int gh = h0 + hh - 1, gw = w0 + ww - 1, gc = c0 + c;
-            float v = 0.f;
-            if (gh >= 0 && gh < H && gw >= 0 && gw < W && gc < Cred) v = ldf(img + ((size_t)gh * W + gw) * Cred + gc);
-            s_in[hh][ww][c] = v;
-        }
-        for (int e = tid; e < 9 * CV_CK * CV_TC; e += 128) {
-            int o = e % CV_TC, q = e / CV_TC;
-            int c = q % CV_CK, t = q / CV_CK;
-            int go = o0 + o, gc = c0 + c;
-            float v = 0.f;
-            if (go < Cres && gc < Cred) {
-                // weight tensor is [Cout][9][Cin]; forward: out=o, in=c ; dgrad: out index is Cin, reduce index is Cout
-                size_t wi = DGRAD ? (((size_t)gc * 9 + t) * Cin + go) : (((size_t)go * 9 + t) * Cin + gc);
-                v = ldf(wt + wi);
-            }
-            s_w[t][c][o] = v;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int t = 0; t < 9; ++t) {
-            const int r = t / 3, s = t % 3;
-            const int dr = DGRAD ? (2 - r) : r, ds = DGRAD ? (2 - s) : s;
-#pragma unroll 4
-            for (int c = 0; c < CV_CK; ++c) {
-                float xv[4], wv[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) xv[i] = s_in[prow + dr][pcol + i + ds][c];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) wv[j] = s_w[t][c][cg * 4 + j];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(xv[i], wv[j], acc[i][j]);
-            }
-        }
-        __syncthreads();
-    }
-    const int gh = h0 + prow;
-    if (gh >= H) return;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        int gw = w0 + pcol + i;
-        if (gw >= W) continue;
-        size_t pix = ((size_t)n * H + gh) * W + gw;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            int go = o0 + cg * 4 + j;
-            if (go >= Cres) continue;
-            float v = acc[i][j];
-            if (!DGRAD) {
-                v += bias[go];
-                if (relu && !(v > 0.f)) v = 0.f;
-            } else if (mask_ref != nullptr) {
-                if (!(ldf(mask_ref + pix * Cres + go) > 0.f)) v = 0.f;
-            }
-            stf(out + pix * Cres + go, v);
-        }
-    }
-}
-
-template <typename T>
-static cudaError_t launch_conv_simt_t(const ConvSimtArgs& a, cudaStream_t st)
-{
-    const int Cred = a.dgrad ? a.Cout : a.Cin, Cres = a.dgrad ? a.Cin : a.Cout;
-    dim3 grid(cdiv(a.H, CV_TP) * cdiv(a.W, CV_TP), a.B, cdiv(Cres, CV_TC));
-    PtrTab tab{};
-    if (a.tab) tab = *a.tab;
-    if (a.dgrad)
-        SB_LAUNCH((conv3x3_simt_kernel<T, true, false>), grid, 128, 0, st, (const T*)a.in, tab, a.b_per_rep, (const T*)a.w, a.bias,
-                                                                  (T*)a.out, (const T*)a.mask_ref, a.H, a.W, Cred, Cres, a.Cin, 0);
-    else if (a.tab)
-        SB_LAUNCH((conv3x3_simt_kernel<T, false, true>), grid, 128, 0, st, nullptr, tab, a.b_per_rep, (const T*)a.w, a.bias,
-                                                                  (T*)a.out, nullptr, a.H, a.W, Cred, Cres, a.Cin, a.relu);
-    else
-        SB_LAUNCH((conv3x3_simt_kernel<T, false, false>), grid, 128, 0, st, (const T*)a.in, tab, a.b_per_rep, (const T*)a.w, a.bias,
-                                                                   (T*)a.out, nullptr, a.H, a.W, Cred, Cres, a.Cin, a.relu);
-    return cudaGetLastError();
-}
-cudaError_t launch_conv_simt(const ConvSimtArgs& a, bool bf16, cudaStream_t st)
-{
-    return bf16 ? launch_conv_simt_t<__nv_bfloat16>(a, st) : launch_conv_simt_t<float>(a, st);
-}
-
-// =============================================================================================
-// 3x3 convolution weight gradient: part[s][k,t,c] = sum over split s's pixels of
-// dy[pix,k] * x[pix shifted by tap t, c].  Block: 32 (k) x 32 (c) outputs of one tap, 256 threads.
-// =============================================================================================
-template <typename T, bool TAB>
-__global__ void __launch_bounds__(256)
-conv3x3_wgrad_simt_kernel(const T* __restrict__ x, PtrTab tab, int b_per_rep, const T* __restrict__ dy,
-                          float* __restrict__ part, int B, int H, int W, int Cin, int Cout, int splits)
-{
-    pdl_prologue();
-    __shared__ float s_dy[32][33];
-    __shared__ float s_x[32][33];
-    const int k0 = blockIdx.x * 32;
-    const int ctiles = (Cin + 31) / 32;
-    const int c0 = (blockIdx.y % ctiles) * 32, t = blockIdx.y / ctiles;
-    const int r = t / 3, s = t % 3;
-    const int sp = blockIdx.z;
-    const int imgs = B / splits;
-    const long pix_begin = (long)sp * imgs * H * W, pix_end = pix_begin + (long)imgs * H * W;
-    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-    float acc[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
-    for (long p0 = pix_begin; p0 < pix_end; p0 += 32) {
-        for (int e = tid; e < 32 * 32; e += 256) {
-            int j = e % 32, pp = e / 32;
-            long pix = p0 + pp;
-            float vd = 0.f, vx = 0.f;
-            if (pix < pix_end) {
-                if (k0 + j < Cout) vd = ldf(dy + pix * Cout + k0 + j);
-                int w_ = (int)(pix % W);
-                long q = pix / W;
-                int h_ = (int)(q % H), n_ = (int)(q / H);
-                int hh = h_ + r - 1, ww = w_ + s - 1;
-                if (hh >= 0 && hh < H && ww >= 0 && ww < W && c0 + j < Cin) {
-                    const T* img = TAB ? (const T*)tab.p[n_ / b_per_rep] + (size_t)(n_ % b_per_rep) * H * W * Cin
-                                       : x + (size_t)n_ * H * W * Cin;
-                    vx = ldf(img + ((size_t)hh * W + ww) * Cin + c0 + j);
-                }
-            }
-            s_dy[pp][j] = vd;
-            s_x[pp][j] = vx;
-        }
-        __syncthreads();
-#pragma unroll 8
-        for (int pp = 0; pp < 32; ++pp) {
-            float a0 = s_dy[pp][ty * 2], a1 = s_dy[pp][ty * 2 + 1];
-            float b0 = s_x[pp][tx * 2], b1 = s_x[pp][tx * 2 + 1];
-            acc[0][0] = fmaf(a0, b0, acc[0][0]);
-            acc[0][1] = fmaf(a0, b1, acc[0][1]);
-            acc[1][0] = fmaf(a1, b0, acc[1][0]);
-            acc[1][1] = fmaf(a1, b1, acc[1][1]);
-        }
-        __syncthreads();
-    }
-    float* dst = part + (size_t)sp * Cout * 9 * Cin;
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            int k = k0 + ty * 2 + i, c = c0 + tx * 2 + j;
-            if (k < Cout && c < Cin) dst[((size_t)k * 9 + t) * Cin + c] = acc[i][j];
-        }
-}
-
-cudaError_t launch_wgrad_simt(const WgradSimtArgs& a, bool bf16, cudaStream_t st)
-{
-    dim3 grid(cdiv(a.Cout, 32), cdiv(a.Cin, 32) * 9, a.splits);
-    PtrTab tab{};
-    if (a.tab) tab = *a.tab;
-#define SB_WG(T, TABF)                                                                                         \
-    SB_LAUNCH((conv3x3_wgrad_simt_kernel<T, TABF>), grid, 256, 0, st, (const T*)a.x, tab, a.b_per_rep, (const T*)a.dy, \
-                                                            a.part, a.B, a.H, a.W, a.Cin, a.Cout, a.splits)
-    if (bf16) { if (a.tab) SB_WG(__nv_bfloat16, true); else SB_WG(__nv_bfloat16, false); }
-    else      { if (a.tab) SB_WG(float, true); else SB_WG(float, false); }
-#undef SB_WG
-    return cudaGetLastError();
-}
-
-// =============================================================================================
 // Column sums (bias gradients) and the reduction of split partial sums.
 // =============================================================================================
-template <typename T>
-__global__ void __launch_bounds__(256)
-colsum_kernel(const T* __restrict__ in, float* __restrict__ part, int M, int N, int splits)
-{
-    pdl_prologue();
-    __shared__ float s[8][33];
-    const int col = blockIdx.x * 32 + threadIdx.x % 32;
-    const int lane_row = threadIdx.x / 32;
-    const int sp = blockIdx.y;
-    const long rows = M / splits, r0 = (long)sp * rows;
-    float acc = 0.f;
-    if (col < N)
-        for (long r = lane_row; r < rows; r += 8) acc += ldf(in + (r0 + r) * N + col);
-    s[lane_row][threadIdx.x % 32] = acc;
-    __syncthreads();
-    if (lane_row == 0 && col < N) {
-        float t = 0.f;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) t += s[i][threadIdx.x];
-        part[(size_t)sp * N + col] = t;
-    }
-}
 // bf16, N a multiple of 8: a thread owns 8 adjacent columns (one 16-byte load per row), 8 row lanes per block take rows
 // r0 + lane_row, + 8, ... with four independent loads in flight and are combined in lane order (deterministic).
 __global__ void __launch_bounds__(256)
@@ -306,16 +85,10 @@ colsum_vec_kernel(const uint4* __restrict__ in, float* __restrict__ part, int M,
         }
     }
 }
-cudaError_t launch_colsum(const void* in, bool bf16, float* part, int M, int N, int splits, cudaStream_t st)
+cudaError_t launch_colsum(const void* in, float* part, int M, int N, int splits, cudaStream_t st)
 {
-    if (bf16 && N % 8 == 0 && (((uintptr_t)in) & 15) == 0) {
-        dim3 vgrid(cdiv(N / 8, 32), splits);
-        SB_LAUNCH((colsum_vec_kernel), vgrid, 256, 0, st, (const uint4*)in, part, M, N, splits);
-        return cudaGetLastError();
-    }
-    dim3 grid(cdiv(N, 32), splits);
-    if (bf16) SB_LAUNCH((colsum_kernel<__nv_bfloat16>), grid, 256, 0, st, (const __nv_bfloat16*)in, part, M, N, splits);
-    else SB_LAUNCH((colsum_kernel<float>), grid, 256, 0, st, (const float*)in, part, M, N, splits);
+    if (N % 8 != 0 || (((uintptr_t)in) & 15) != 0) return cudaErrorInvalidValue;
+    SB_LAUNCH((colsum_vec_kernel), dim3(cdiv(N / 8, 32), splits), 256, 0, st, (const uint4*)in, part, M, N, splits);
     return cudaGetLastError();
 }
 
@@ -402,10 +175,10 @@ cudaError_t launch_reduce_partials(const float* part, size_t stride, float* out,
 // Split-reduction epilogue of the tensor-core GEMMs: out = epi(sum_s part[s]) with the splits added in
 // order; epi = bias + ReLU (-> bf16 or float) or the ReLU mask (-> bf16).  Four columns per thread.
 // =============================================================================================
-template <int EPI>
+template <typename T, int EPI>
 __global__ void __launch_bounds__(256)
 splitk_epilogue_kernel(const float* __restrict__ part, size_t split_stride, int splits, size_t n4, int N,
-                       const float* __restrict__ bias, int relu, const __nv_bfloat16* __restrict__ ref,
+                       const float* __restrict__ bias, int relu, const T* __restrict__ ref,
                        void* __restrict__ out, int out_f32)
 {
     pdl_prologue();
@@ -431,14 +204,15 @@ splitk_epilogue_kernel(const float* __restrict__ part, size_t split_stride, int 
                 if (!(t.w > 0.f)) t.w = 0.f;
             }
         } else if (ref != nullptr) {
-            const uint2 r = *(const uint2*)(ref + e);
-            const __nv_bfloat16* rb = (const __nv_bfloat16*)&r;
-            if (!(__bfloat162float(rb[0]) > 0.f)) t.x = 0.f;
-            if (!(__bfloat162float(rb[1]) > 0.f)) t.y = 0.f;
-            if (!(__bfloat162float(rb[2]) > 0.f)) t.z = 0.f;
-            if (!(__bfloat162float(rb[3]) > 0.f)) t.w = 0.f;
+            __align__(16) T r[4];
+            if (sizeof(T) == 2) *(uint2*)r = *(const uint2*)(ref + e);
+            else *(float4*)r = *(const float4*)(ref + e);
+            if (!(ldf(r) > 0.f)) t.x = 0.f;
+            if (!(ldf(r + 1) > 0.f)) t.y = 0.f;
+            if (!(ldf(r + 2) > 0.f)) t.z = 0.f;
+            if (!(ldf(r + 3) > 0.f)) t.w = 0.f;
         }
-        if (out_f32) {
+        if (sizeof(T) == 4 || out_f32) {
             *(float4*)((float*)out + e) = t;
         } else {
             __nv_bfloat162 lo = __floats2bfloat162_rn(t.x, t.y), hi = __floats2bfloat162_rn(t.z, t.w);
@@ -449,17 +223,41 @@ splitk_epilogue_kernel(const float* __restrict__ part, size_t split_stride, int 
         }
     }
 }
-cudaError_t launch_splitk_epilogue(const SplitKEpiArgs& a, cudaStream_t st)
+// widths that are not multiples of four
+template <typename T, int EPI>
+__global__ void __launch_bounds__(256)
+splitk_epilogue1_kernel(const float* __restrict__ part, size_t split_stride, int splits, size_t n, int N,
+                        const float* __restrict__ bias, int relu, const T* __restrict__ ref, void* __restrict__ out, int out_f32)
 {
-    if (a.N % 4 != 0) return cudaErrorInvalidValue;
-    const size_t n4 = (size_t)a.rows * a.N / 4;
-    int blocks = cdiv((long)n4, 256);
+    pdl_prologue();
+    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
+        float t = 0.f;
+        for (int s = 0; s < splits; ++s) t += part[(size_t)s * split_stride + e];
+        if (EPI == EPI_BIAS_ACT) {
+            t += bias[e % (size_t)N];
+            if (relu && !(t > 0.f)) t = 0.f;
+        } else if (ref != nullptr) {
+            if (!(ldf(ref + e) > 0.f)) t = 0.f;
+        }
+        if (out_f32) ((float*)out)[e] = t;
+        else stf((T*)out + e, t);
+    }
+}
+template <typename T, int EPI>
+static cudaError_t launch_splitk_t(const SplitKEpiArgs& a, cudaStream_t st)
+{
+    const size_t total = (size_t)a.rows * a.N;
+    const bool vec = a.N % 4 == 0;
+    int blocks = cdiv((long)(vec ? total / 4 : total), 256);
     if (blocks > 148 * 8) blocks = 148 * 8;
-    if (a.epi == EPI_BIAS_ACT)
-        SB_LAUNCH((splitk_epilogue_kernel<EPI_BIAS_ACT>), blocks, 256, 0, st, a.part, a.split_stride, a.splits, n4, a.N, a.bias, a.relu, nullptr, a.out, a.out_f32);
-    else
-        SB_LAUNCH((splitk_epilogue_kernel<EPI_MASK>), blocks, 256, 0, st, a.part, a.split_stride, a.splits, n4, a.N, nullptr, 0, (const __nv_bfloat16*)a.ref, a.out, 0);
+    if (vec) SB_LAUNCH((splitk_epilogue_kernel<T, EPI>), blocks, 256, 0, st, a.part, a.split_stride, a.splits, total / 4, a.N, a.bias, a.relu, (const T*)a.ref, a.out, a.out_f32);
+    else SB_LAUNCH((splitk_epilogue1_kernel<T, EPI>), blocks, 256, 0, st, a.part, a.split_stride, a.splits, total, a.N, a.bias, a.relu, (const T*)a.ref, a.out, a.out_f32);
     return cudaGetLastError();
+}
+cudaError_t launch_splitk_epilogue(const SplitKEpiArgs& a, bool bf16, cudaStream_t st)
+{
+    if (a.epi == EPI_BIAS_ACT) return bf16 ? launch_splitk_t<__nv_bfloat16, EPI_BIAS_ACT>(a, st) : launch_splitk_t<float, EPI_BIAS_ACT>(a, st);
+    return bf16 ? launch_splitk_t<__nv_bfloat16, EPI_MASK>(a, st) : launch_splitk_t<float, EPI_MASK>(a, st);
 }
 
 // =============================================================================================
@@ -1400,125 +1198,6 @@ static cudaError_t launch_fc_narrow_t(const FcNarrowArgs& a, cudaStream_t st)
 cudaError_t launch_fc_narrow(const FcNarrowArgs& a, bool bf16, cudaStream_t st)
 {
     return bf16 ? launch_fc_narrow_t<__nv_bfloat16>(a, st) : launch_fc_narrow_t<float>(a, st);
-}
-
-// =============================================================================================
-// Strided FFMA GEMM for the sharded FC layers:  C[m,n] = sum_k A(m,k) * B(n,k).
-// 64x64 tile, BK = 16, 256 threads, 4x4 outputs per thread.  blockIdx.z = shard for the
-// partitions that own outputs; the K-partition (dgrad) walks the shards one after another.
-// =============================================================================================
-__device__ __forceinline__ int shard_lo(int j, int total, int shards) { return (int)(((long)j * total) / shards); }
-
-template <typename T, int EPI>
-__global__ void __launch_bounds__(256)
-gemm_simt_kernel(const T* __restrict__ A, long sAm, long sAk, const T* __restrict__ Bm, long sBn, long sBk,
-                 int M, int N, int K, void* __restrict__ Cv, long ldc, float* __restrict__ C32,
-                 const float* __restrict__ bias, int relu, const T* __restrict__ ref, long ldref,
-                 int shard_dim, int shards, PtrTab tab, int tab_mode, int tab_b)
-{
-    pdl_prologue();
-    __shared__ float As[16][65];
-    __shared__ float Bs[16][65];
-    int m_lo = 0, m_hi = M, n_lo = 0, n_hi = N;
-    if (shard_dim == 1) { n_lo = shard_lo(blockIdx.z, N, shards); n_hi = shard_lo(blockIdx.z + 1, N, shards); }
-    if (shard_dim == 3) { m_lo = shard_lo(blockIdx.z, M, shards); m_hi = shard_lo(blockIdx.z + 1, M, shards); }
-    const int m0 = m_lo + blockIdx.y * 64, n0 = n_lo + blockIdx.x * 64;
-    if (m0 >= m_hi || n0 >= n_hi) return;
-    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-    float acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-    const int kparts = (shard_dim == 2) ? shards : 1;
-    for (int kp = 0; kp < kparts; ++kp) {
-        const int k_lo = (shard_dim == 2) ? shard_lo(kp, K, shards) : 0;
-        const int k_hi = (shard_dim == 2) ? shard_lo(kp + 1, K, shards) : K;
-        for (int k0 = k_lo; k0 < k_hi; k0 += 16) {
-            for (int e = tid; e < 64 * 16; e += 256) {
-                int mm, kk;
-                if (sAk == 1) { kk = e % 16; mm = e / 16; } else { mm = e % 64; kk = e / 64; }
-                float v = 0.f;
-                if (m0 + mm < m_hi && k0 + kk < k_hi) {
-                    const int m = m0 + mm;
-                    v = (tab_mode == 1) ? ldf((const T*)tab.p[m / tab_b] + (long)(m % tab_b) * sAm + (long)(k0 + kk) * sAk)
-                                        : ldf(A + (long)m * sAm + (long)(k0 + kk) * sAk);
-                }
-                As[kk][mm] = v;
-                int nn;
-                if (sBk == 1) { kk = e % 16; nn = e / 16; } else { nn = e % 64; kk = e / 64; }
-                v = 0.f;
-                if (n0 + nn < n_hi && k0 + kk < k_hi) {
-                    const int k = k0 + kk;
-                    v = (tab_mode == 2) ? ldf((const T*)tab.p[k / tab_b] + (long)(n0 + nn) * sBn + (long)(k % tab_b) * sBk)
-                                        : ldf(Bm + (long)(n0 + nn) * sBn + (long)k * sBk);
-                }
-                Bs[kk][nn] = v;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int kk = 0; kk < 16; ++kk) {
-                float a[4], b[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-            }
-            __syncthreads();
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        int m = m0 + ty * 4 + i;
-        if (m >= m_hi) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            int n = n0 + tx * 4 + j;
-            if (n >= n_hi) continue;
-            float v = acc[i][j];
-            if (EPI == EPI_BIAS_ACT) {
-                v += bias[n];
-                if (relu && !(v > 0.f)) v = 0.f;
-                if (C32) C32[(long)m * ldc + n] = v;
-                if (Cv) stf((T*)Cv + (long)m * ldc + n, v);
-            } else if (EPI == EPI_MASK) {
-                if (ref != nullptr && !(ldf(ref + (long)m * ldref + n) > 0.f)) v = 0.f;
-                stf((T*)Cv + (long)m * ldc + n, v);
-            } else {
-                ((float*)Cv)[(long)m * ldc + n] = v;
-            }
-        }
-    }
-}
-
-template <typename T>
-static cudaError_t launch_gemm_simt_t(const GemmSimtArgs& a, cudaStream_t st)
-{
-    int shards = a.shard_dim ? a.shards : 1;
-    int Mmax = a.M, Nmax = a.N, gz = 1;
-    if (a.shard_dim == 1) { Nmax = cdiv(a.N, shards); gz = shards; }
-    if (a.shard_dim == 3) { Mmax = cdiv(a.M, shards); gz = shards; }
-    dim3 grid(cdiv(Nmax, 64), cdiv(Mmax, 64), gz);
-    PtrTab tab{};
-    if (a.tab) tab = *a.tab;
-    const int tab_mode = a.tab ? a.tab_mode : 0;
-#define SB_GM(E)                                                                                                    \
-    SB_LAUNCH((gemm_simt_kernel<T, E>), grid, 256, 0, st, (const T*)a.A, a.sAm, a.sAk, (const T*)a.B, a.sBn, a.sBk, a.M, a.N, a.K, \
-                                                 a.C, a.ldc, a.C32, a.bias, a.relu, (const T*)a.ref, a.ldref, a.shard_dim, shards, \
-                                                 tab, tab_mode, a.tab_b > 0 ? a.tab_b : 1)
-    if (a.epi == EPI_BIAS_ACT) SB_GM(EPI_BIAS_ACT);
-    else if (a.epi == EPI_MASK) SB_GM(EPI_MASK);
-    else SB_GM(EPI_F32);
-#undef SB_GM
-    return cudaGetLastError();
-}
-cudaError_t launch_gemm_simt(const GemmSimtArgs& a, bool bf16, cudaStream_t st)
-{
-    return bf16 ? launch_gemm_simt_t<__nv_bfloat16>(a, st) : launch_gemm_simt_t<float>(a, st);
 }
 
 }  // namespace sb

@@ -2257,7 +2257,7 @@ static sb_status launch_op(const UmmaOp& op, cudaStream_t st, int64_t* launches 
         a.rows = b->rows; a.N = b->p.n_total;
         a.epi = b->p.epi == UEPI_BIAS_ACT ? EPI_BIAS_ACT : EPI_MASK;
         a.bias = b->p.bias; a.relu = b->p.relu; a.ref = b->p.ref; a.out = b->p.out; a.out_f32 = b->p.out_f32;
-        e = launch_splitk_epilogue(a, st);
+        e = launch_splitk_epilogue(a, true, st);
         if (launches) ++*launches;
     }
     if (e != cudaSuccess) {
@@ -2566,6 +2566,13 @@ static bool fc_umma_ok(const ModelView& mv, const LayerView& lv, int layer)
     // TMA needs 16-byte row strides: in and out multiples of 8; the reduce dims multiples of 64 keep every box row in bounds
     (void)layer;   // a first-layer FC reads the network input through a tensor map bound at forward time
     return mv.bf16 && !(mv.cfg->flags & SB_FLAG_FORCE_SIMT) && lv.in_f % 64 == 0 && lv.out_f % 8 == 0 && lv.out_f > 16;
+}
+
+bool umma_layer_ok(sb_model* m, int layer)
+{
+    const ModelView mv = model_view(m);
+    const LayerView lv = layer_view(m, layer);
+    return lv.kind == SB_CONV3X3_RELU ? conv_umma_ok(mv, lv, layer) : fc_umma_ok(mv, lv, layer);
 }
 
 // Geometry shared by the scratch sizing pass and the real planning pass.

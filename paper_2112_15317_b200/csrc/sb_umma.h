@@ -61,6 +61,8 @@ int64_t* launch_counter(sb_model* m);
 // Scratch floats the tensor-core path needs (split partial sums); called during planning,
 // before the arena exists (pointers in the views are null or unset).
 sb_status umma_plan_scratch(sb_model* m, size_t* floats);
+// Whether layer i's passes run on tensor-core tiles (the input layer's im2col kernels aside).
+bool umma_layer_ok(sb_model* m, int layer);
 // Encodes tensor maps and decides, per layer and pass, whether the tensor-core kernel runs (layers first_layer..).
 sb_status umma_plan_layers(sb_model* m, int first_layer);
 
