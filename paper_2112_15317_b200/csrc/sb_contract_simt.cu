@@ -353,11 +353,12 @@ contract_kernel(const __grid_constant__ ContractParams p)
 }
 
 // ---- tile and split choice -----------------------------------------------------------------------------------------------
-// Cost model in microseconds: a reduction step of BK costs an SM 1.1 us per 128 x 128 outputs at the FFMA rate; smaller tiles
-// have less of it per shared-memory word; blocks of few warps do not fill an SM's pipes by themselves.  A split reduction adds
-// a kernel and its float partial sums at about 2 TB/s.
-struct TileShape { int bm, bn; double eff; };
-static const TileShape shapes[] = {{128, 128, 0.85}, {128, 64, 0.75}, {64, 128, 0.75}, {64, 64, 0.65}, {128, 32, 0.55}, {32, 128, 0.55}};
+// Cost model in microseconds, fitted to a sweep of every shape and 1 to 128 splits over the layers of a 7-conv / 3-FC net.  One
+// reduction step of BK costs the n blocks that share an SM lone + more * n, up to `resident` of them together, the rest in further
+// rounds (128 x 128: 1.7 us alone, 2.95 for two = 53 TFLOP/s).  A split reduction adds a kernel and its float partial sums.
+struct TileShape { int bm, bn, resident; double lone, more; };
+static const TileShape shapes[] = {{128, 128, 2, 0.45, 1.25}, {128, 64, 4, 0.75, 0.65}, {64, 128, 4, 0.75, 0.63},
+                                   {64, 64, 6, 0.62, 0.30},   {128, 32, 6, 0.85, 0.30}, {32, 128, 6, 0.85, 0.30}};
 
 static bool vec_ok(int Cin, int Cout) { return Cin % 4 == 0 && Cout % 4 == 0; }
 static long contract_iters(int mode, int B, int H, int W, int taps, int Cin, int Cout)
@@ -376,17 +377,14 @@ ContractPlan contract_plan(int mode, int B, int H, int W, int taps, int Cin, int
     for (const TileShape& s : shapes) {
         if (!vec_ok(Cin, Cout) && (s.bm != 64 || s.bn != 64)) continue;      // (odd channel counts: one shape)
         const long tiles = ((M + s.bm - 1) / s.bm) * ((N + s.bn - 1) / s.bn);
-        const double step = 1.1 * s.bm * s.bn / (128.0 * 128.0) / s.eff;
-        for (int split = 1; split <= 256 && (split == 1 || iters / split >= 4); split = split < 8 ? split + 1 : split + split / 4) {
+        for (int split = 1; split <= 256 && (split == 1 || iters / split >= 3); split = split < 8 ? split + 1 : split + split / 4) {
             const long per = (iters + split - 1) / split;
             const int real = (int)((iters + per - 1) / per);
             if (real > 1 && (size_t)real * M * (N + (mode == CMODE_WGRAD ? 1 : 0)) > max_part_floats) break;
-            const double ctas = (double)tiles * real;
-            const double on_sm = std::max(1.0, ctas / 148.0);                      // blocks per SM over the launch
-            const double waves = on_sm < 6.0 ? (double)((long)((ctas + 147.0) / 148.0)) : on_sm;
-            const double warps = (s.bm * s.bn / 64 / 32) * std::min(on_sm, 16.0);     // of them resident together, at most
-            double t = waves * per * step * std::max(1.0, 8.0 / warps) + 4.0;
-            if (real > 1) t += 3.0 + (double)real * M * N * 8.0 / 2.0e6;
+            const long n = (tiles * real + 147) / 148, rest = n % s.resident;        // blocks of the fullest SM
+            const double step = (double)(n / s.resident) * (s.lone + s.more * s.resident) + (rest ? s.lone + s.more * rest : 0.0);
+            double t = per * step * (mode == CMODE_WGRAD ? 1.08 : 1.0) + 3.0;
+            if (real > 1) t += 3.0 + (double)real * M * N * 8.0 / 7.0e6;
             if (t < best_t) { best_t = t; best = ContractPlan{s.bm, s.bn, (int)per, real}; }
         }
     }
@@ -395,11 +393,23 @@ ContractPlan contract_plan(int mode, int B, int H, int W, int taps, int Cin, int
 
 static uint32_t rcp_of(int d) { return d <= 1 ? 0u : (uint32_t)(0x100000000ull / (uint32_t)d) + 1u; }
 
+// A grid of n blocks per SM is kept to n of them on any SM by the shared memory each asks for: left alone, the hardware puts two
+// of 100 to 148 blocks on some SMs while others stay empty (144 blocks of 128 x 128: 301 us, 72 blocks of twice the length: 349).
+template <typename T, int MODE, int BM, int BN, bool VEC>
+static cudaError_t launch_one(const ContractParams& p, cudaStream_t st)
+{
+    constexpr int STATIC = (int)(2 * BK * (BM + 4 + BN + 4) * sizeof(float)), MOST = 224 * 1024;
+    static const cudaError_t attr = cudaFuncSetAttribute(contract_kernel<T, MODE, BM, BN, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, MOST - STATIC);
+    if (attr != cudaSuccess) return attr;
+    const dim3 grid((unsigned)((p.M + BM - 1) / BM), (unsigned)((p.N + BN - 1) / BN), (unsigned)p.splits);
+    const long n = ((long)grid.x * grid.y * grid.z + 147) / 148;
+    const int share = n <= 4 ? (int)(MOST / n) - 2048 - STATIC : 0;
+    return pdl_launch(contract_kernel<T, MODE, BM, BN, VEC>, grid, dim3(BM * BN / 64), share > 0 ? (size_t)share / 1024 * 1024 : 0, st, p);
+}
 template <typename T, int MODE, bool VEC>
 static cudaError_t launch_shape(const ContractPlan& c, const ContractParams& p, cudaStream_t st)
 {
-    const dim3 grid((unsigned)((p.M + c.bm - 1) / c.bm), (unsigned)((p.N + c.bn - 1) / c.bn), (unsigned)p.splits);
-#define SB_SHAPE(BM, BN) if (c.bm == BM && c.bn == BN) return pdl_launch(contract_kernel<T, MODE, BM, BN, VEC>, grid, dim3(BM * BN / 64), 0, st, p)
+#define SB_SHAPE(BM, BN) if (c.bm == BM && c.bn == BN) return launch_one<T, MODE, BM, BN, VEC>(p, st)
     SB_SHAPE(64, 64);
     if constexpr (VEC) {
         SB_SHAPE(128, 128);
