@@ -248,7 +248,7 @@ conv_in_fwd_umma_kernel(const __grid_constant__ CUtensorMap mapY, int tma_out, c
                     pk[j] = *(uint32_t*)&t;
                 }
                 if (tma_out) {
-                    // output row r = 128 bytes (64 channels), staged in the A tile's buffer (the MMA has consumed it) in
+                    // output row r = up to 128 bytes (64 channels), staged in the A tile's buffer (the MMA has consumed it) in
                     // the same 128-byte swizzle, so that one TMA store writes the tile's 16 KB in full lines
                     const int j0 = c0 >> 3;
                     *(uint4*)(sA + r * 128 + (((j0) ^ (r & 7)) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
@@ -284,15 +284,14 @@ conv_in_fwd_umma_kernel(const __grid_constant__ CUtensorMap mapY, int tma_out, c
 template <int CIN, bool TAB>
 __global__ void __launch_bounds__(CI_THREADS)
 conv_in_wgrad_umma_kernel(const __grid_constant__ CUtensorMap mapDy, const __nv_bfloat16* __restrict__ x, PtrTab tab, int b_per_rep,
-                          float* __restrict__ part, long npix, int H, int W, long stride_floats, long n_chunks, long chunks_per_cta,
+                          float* __restrict__ part, long npix, int H, int W, int Cout, long stride_floats, long n_chunks, long chunks_per_cta,
                           uint32_t* status)
 {
-    constexpr int COUT = 64;
     constexpr int NK = 9 * CIN;                       // weight columns; column NK is the bias gradient
     constexpr int CHUNKS = (NK + 1 + 7) / 8;          // 16-byte chunks per row that hold data
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    // stage s: [dy tile: 64 pixel rows x 128 B (64 couts)] [patch tile: 64 pixel rows x 128 B]; the MMA's second
+    // stage s: [dy tile: 64 pixel rows x 128 B (64 couts, zeros past the last one)] [patch tile: 64 pixel rows x 128 B]; the MMA's second
     // 64-row block of A (couts 64..127, unused) aliases the patch tile, which always holds finite values
     uint8_t* stage0 = smem;
     uint64_t* full = (uint64_t*)(smem + 2 * 16384);   // [2] dy tile landed
@@ -411,13 +410,13 @@ conv_in_wgrad_umma_kernel(const __grid_constant__ CUtensorMap mapDy, const __nv_
             const uint32_t taddr = tmem_base + ((uint32_t)(warp * 32) << 16);
             const int cout = warp * 32 + lane;               // accumulator row; rows 64.. are the unused block
             float* pw = part + (size_t)blockIdx.x * stride_floats + (size_t)cout * NK;
-            float* pb = part + (size_t)blockIdx.x * stride_floats + (size_t)COUT * NK + cout;
+            float* pb = part + (size_t)blockIdx.x * stride_floats + (size_t)Cout * NK + cout;
 #pragma unroll
             for (int c0 = 0; c0 < 8 * CHUNKS; c0 += 16) {
                 uint32_t v[16];
                 tmem_ld16(taddr + c0, v);                    // warp-collective
                 tmem_ld_wait();
-                if (cout < COUT) {
+                if (cout < Cout) {
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
                         if (c0 + j < NK) pw[c0 + j] = __uint_as_float(v[j]);
@@ -449,7 +448,7 @@ uint32_t pow2_cols(int n)
 
 }  // namespace
 
-bool conv_in_umma_supported(int Cin, int Cout) { return (Cin == 1 || Cin == 3 || Cin == 4) && Cout == 64; }
+bool conv_in_umma_supported(int Cin, int Cout) { return (Cin == 1 || Cin == 3 || Cin == 4) && Cout <= 64 && Cout % 16 == 0; }
 
 int conv_in_umma_wgrad_blocks(long npix)
 {
@@ -475,9 +474,9 @@ static cudaError_t launch_fwd_t(const ConvSimtArgs& a, const CUtensorMap* mapY, 
     PtrTab tab{};
     if (a.tab) tab = *a.tab;
     const uint32_t cols = pow2_cols(a.Cout);
-    // the output goes out by TMA store when the caller made a tensor map for it (64 channels: one 128-byte row per pixel)
+    // the output goes out by TMA store when the caller made a tensor map for it (rows of up to 64 channels, clipped at the last)
     static const bool no_tma_out = tune("SB_CONV_IN_TMA_OUT", 1) == 0;
-    const int tma_out = (mapY && a.Cout == 64 && !no_tma_out) ? 1 : 0;
+    const int tma_out = (mapY && !no_tma_out) ? 1 : 0;
     CUtensorMap dummy{};
     const CUtensorMap& my = tma_out ? *mapY : dummy;
     // persistent CTAs, as many as are resident at once (7 per SM for 64 output channels; their TMEM columns also fit:
@@ -518,9 +517,9 @@ static cudaError_t launch_wgrad_t(const WgradSimtArgs& a, const CUtensorMap& map
     if (a.tab) tab = *a.tab;
     if (a.tab)
         return pdl_launch(conv_in_wgrad_umma_kernel<CIN, true>, dim3(grid), dim3(CI_THREADS), smem, st, mapDy, (const __nv_bfloat16*)nullptr, tab,
-                          a.b_per_rep, a.part, npix, a.H, a.W, stride, chunks, cpc, status);
+                          a.b_per_rep, a.part, npix, a.H, a.W, a.Cout, stride, chunks, cpc, status);
     return pdl_launch(conv_in_wgrad_umma_kernel<CIN, false>, dim3(grid), dim3(CI_THREADS), smem, st, mapDy, (const __nv_bfloat16*)a.x, tab,
-                      a.b_per_rep, a.part, npix, a.H, a.W, stride, chunks, cpc, status);
+                      a.b_per_rep, a.part, npix, a.H, a.W, a.Cout, stride, chunks, cpc, status);
 }
 
 cudaError_t launch_conv_in_wgrad_umma(const WgradSimtArgs& a, const CUtensorMap& mapDy, uint32_t* status, cudaStream_t st)

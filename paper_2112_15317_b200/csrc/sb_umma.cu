@@ -331,7 +331,7 @@ __device__ __forceinline__ void store_row(const UmmaParams& p, uint32_t taddr, b
             tmem_ld16(taddr + c0, v[0]);     // warp-collective; two loads per wait
             tmem_ld16(taddr + c0 + 16, v[1]);
             tmem_ld_wait();
-            if (n0 + c0 >= n_hi) continue;            // (uniform: whole 64-column slabs)
+            if (n0 + c0 >= n_hi) continue;            // (uniform)
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int c = c0 + 16 * h;
@@ -356,7 +356,7 @@ __device__ __forceinline__ void store_row(const UmmaParams& p, uint32_t taddr, b
     }
     if (MODE != MODE_WGRAD && stage != nullptr) {
         // Staged bf16 tile for the TMA store (the planner only selects it for unsplit bf16 outputs whose columns end on
-        // 64-column slabs): every decision is taken once, outside the loop -- an epilogue warp runs alone on its
+        // 16-column chunks): every decision is taken once, outside the loop -- an epilogue warp runs alone on its
         // scheduler, so every branch and every dependent instruction in the loop costs its full latency.
         const bool bias_act = p.epi == UEPI_BIAS_ACT, relu = p.relu != 0;
         const __nv_bfloat16* refrow = (p.epi == UEPI_MASK && p.ref != nullptr && row_ok) ? p.ref + row_off + n0 : nullptr;
@@ -369,10 +369,11 @@ __device__ __forceinline__ void store_row(const UmmaParams& p, uint32_t taddr, b
             tmem_ld16(taddr + c0, v[0]);     // warp-collective; two loads per wait
             tmem_ld16(taddr + c0 + 16, v[1]);
             tmem_ld_wait();
-            if (n0 + c0 >= n_hi) continue;            // (uniform: whole 64-column slabs)
+            if (n0 + c0 >= n_hi) continue;            // (uniform: whole 16-column chunks)
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int c = c0 + 16 * h;
+                if (h == 1 && n0 + c >= n_hi) break;
                 float f[16];
 #pragma unroll
                 for (int j = 0; j < 16; ++j) f[j] = __uint_as_float(v[h][j]);
@@ -2559,13 +2560,15 @@ static int wgrad_splits(long ctas_without_split, int total_chunks, int bn, size_
 
 static bool conv_umma_ok(const ModelView& mv, const LayerView& lv, int layer)
 {
-    return mv.bf16 && !(mv.cfg->flags & SB_FLAG_FORCE_SIMT) && layer > 0 && lv.Cin % 64 == 0 && lv.Cout % 64 == 0;
+    // Channel counts need not fill the 64-wide boxes: the activation (or dy) box reads zeros past the last channel, which cancels
+    // whatever the weight box holds there (the next tap's columns), and columns past the last one are not stored.
+    return mv.bf16 && !(mv.cfg->flags & SB_FLAG_FORCE_SIMT) && layer > 0 && lv.Cin % 16 == 0 && lv.Cout % 16 == 0;
 }
 static bool fc_umma_ok(const ModelView& mv, const LayerView& lv, int layer)
 {
-    // TMA needs 16-byte row strides: in and out multiples of 8; the reduce dims multiples of 64 keep every box row in bounds
+    // TMA needs 16-byte row strides; reduction tails past the last column read as zeros in both operands
     (void)layer;   // a first-layer FC reads the network input through a tensor map bound at forward time
-    return mv.bf16 && !(mv.cfg->flags & SB_FLAG_FORCE_SIMT) && lv.in_f % 64 == 0 && lv.out_f % 8 == 0 && lv.out_f > 16;
+    return mv.bf16 && !(mv.cfg->flags & SB_FLAG_FORCE_SIMT) && lv.in_f % 16 == 0 && lv.out_f % 8 == 0 && lv.out_f > 16;
 }
 
 bool umma_layer_ok(sb_model* m, int layer)
@@ -2620,22 +2623,22 @@ static ConvGeom conv_geom(const LayerView& lv, int B, bool force_pair, bool no_h
         g.m_tiles = (long)g.tw * g.th * g.tn;
         const int a_slot = (g.bh + 2) * g.bw * g.bn * 128;
         if (persist) {
-            g.fwd = plan_tiles_halo_persist(lv.Cout, g.m_tiles, lv.Cin / 64, a_slot);
-            g.dgrad = plan_tiles_halo_persist(lv.Cin, g.m_tiles, lv.Cout / 64, a_slot);
+            g.fwd = plan_tiles_halo_persist(lv.Cout, g.m_tiles, cdiv_i(lv.Cin, 64), a_slot);
+            g.dgrad = plan_tiles_halo_persist(lv.Cin, g.m_tiles, cdiv_i(lv.Cout, 64), a_slot);
             if (force_persist) {      // (tests at small sizes: few CTAs, so that each walks several tiles and reuses both accumulators)
                 if (g.fwd.persist_ctas > 3) g.fwd.persist_ctas = 3;
                 if (g.dgrad.persist_ctas > 3) g.dgrad.persist_ctas = 3;
             }
         } else {
-            g.fwd = plan_tiles_halo(lv.Cout, g.m_tiles, lv.Cin / 64, a_slot, false);
-            g.dgrad = plan_tiles_halo(lv.Cin, g.m_tiles, lv.Cout / 64, a_slot, true);
+            g.fwd = plan_tiles_halo(lv.Cout, g.m_tiles, cdiv_i(lv.Cin, 64), a_slot, false);
+            g.dgrad = plan_tiles_halo(lv.Cin, g.m_tiles, cdiv_i(lv.Cout, 64), a_slot, true);
         }
     } else {
         choose_box(lv.W, lv.H, B, 128, &g.bw, &g.bh, &g.bn);
         g.tw = cdiv_i(lv.W, g.bw); g.th = cdiv_i(lv.H, g.bh); g.tn = cdiv_i(B, g.bn);
         g.m_tiles = (long)g.tw * g.th * g.tn;
-        g.fwd = plan_tiles(lv.Cout, g.m_tiles, 9 * (lv.Cin / 64), false, force_pair);
-        g.dgrad = plan_tiles(lv.Cin, g.m_tiles, 9 * (lv.Cout / 64), true, force_pair);
+        g.fwd = plan_tiles(lv.Cout, g.m_tiles, 9 * cdiv_i(lv.Cin, 64), false, force_pair);
+        g.dgrad = plan_tiles(lv.Cin, g.m_tiles, 9 * cdiv_i(lv.Cout, 64), true, force_pair);
     }
     choose_box(lv.W, lv.H, B, 64, &g.cw, &g.ch, &g.cn);
     g.ctw = cdiv_i(lv.W, g.cw); g.cth = cdiv_i(lv.H, g.ch); g.ctn = cdiv_i(B, g.cn);
@@ -2681,7 +2684,7 @@ static FcGeom fc_geom(const LayerView& lv, int B, bool force_pair)
 {
     FcGeom g;
     g.m_tiles = cdiv_i(B, 128);
-    g.fwd = plan_tiles(lv.out_f, g.m_tiles, lv.in_f / 64, false, force_pair);
+    g.fwd = plan_tiles(lv.out_f, g.m_tiles, cdiv_i(lv.in_f, 64), false, force_pair);
     g.dgrad = plan_tiles(lv.in_f, g.m_tiles, cdiv_i(lv.out_f, 64), true, force_pair);
     return g;
 }
@@ -2733,15 +2736,15 @@ static void apply_plan(OpBlock* b, const TilePlan& t, int k_iters, long m_tiles,
     b->rows = (long)rows;
 }
 
-// TMA-store epilogue of a FWD / DGRAD op: possible when the output is bf16, the reduction is not split, every N tile
-// ends on a 64-column slab boundary, and the idle operand ring can hold the staged tile.
+// TMA-store epilogue of a FWD / DGRAD op: possible when the output is bf16, the reduction is not split, the columns
+// end on a 16-column chunk (the store clips the rest of a slab), and the idle operand ring can hold the staged tile.
 // SB_TMA_OUT=0 keeps the direct row stores.
 static bool tma_out_ok(const OpBlock* b)
 {
     static const bool off = tune("SB_TMA_OUT", 1) == 0;
     const UmmaParams& p = b->p;
     if (off || p.out_f32 || p.splits > 1 || p.epi == UEPI_F32) return false;
-    if (p.n_total % 64 != 0 || p.ldc % 64 != 0) return false;
+    if (p.n_total % 16 != 0 || p.ldc % 16 != 0) return false;
     if (b->halo && b->persist) return true;
     if (b->halo) return (long)p.a_stages * (p.bh + 2) * p.bw * p.bn * 128 + (long)p.stages * b->bn * 128 >= (long)(b->bn / 64) * 16384;
     const long stage_bytes = b->pair ? 16384 + b->bn * 64 : 16384 + b->bn * 128;
@@ -2775,7 +2778,7 @@ sb_status umma_plan_layers(sb_model* m, int first_layer)
                 memset(b, 0, sizeof(*b));
                 UmmaParams& p = b->p;
                 p.mode = MODE_FWD; p.ntaps = 9; p.bw = g.bw; p.bh = g.bh; p.bn = g.bn; p.W = lv.W; p.H = lv.H; p.N = B;
-                p.tiles_w = g.tw; p.tiles_h = g.th; p.tiles_n = g.tn; p.kchunks = lv.Cin / 64; p.w_cols = lv.Cin;
+                p.tiles_w = g.tw; p.tiles_h = g.th; p.tiles_n = g.tn; p.kchunks = cdiv_i(lv.Cin, 64); p.w_cols = lv.Cin;
                 p.n_total = lv.Cout;
                 p.n_tiles = cdiv_i(lv.Cout, g.fwd.bn);
                 p.epi = UEPI_BIAS_ACT; p.relu = 1; p.out_f32 = 0; p.out = lv.act; p.ldc = lv.Cout; p.bias = mv.Wm + lv.p_b;
@@ -2810,7 +2813,7 @@ sb_status umma_plan_layers(sb_model* m, int first_layer)
                 memset(b, 0, sizeof(*b));
                 UmmaParams& p = b->p;
                 p.mode = MODE_DGRAD; p.ntaps = 9; p.bw = g.bw; p.bh = g.bh; p.bn = g.bn; p.W = lv.W; p.H = lv.H; p.N = B;
-                p.tiles_w = g.tw; p.tiles_h = g.th; p.tiles_n = g.tn; p.kchunks = lv.Cout / 64; p.w_cols = lv.Cin;
+                p.tiles_w = g.tw; p.tiles_h = g.th; p.tiles_n = g.tn; p.kchunks = cdiv_i(lv.Cout, 64); p.w_cols = lv.Cin;
                 p.n_total = lv.Cin;
                 p.n_tiles = cdiv_i(lv.Cin, g.dgrad.bn);
                 p.epi = UEPI_MASK; p.out = lv.d_below; p.ldc = lv.Cin;
@@ -2910,7 +2913,7 @@ sb_status umma_plan_layers(sb_model* m, int first_layer)
                 memset(b, 0, sizeof(*b));
                 UmmaParams& p = b->p;
                 p.mode = MODE_FWD; p.ntaps = 1; p.bw = 1; p.bh = 1; p.bn = 128; p.W = 1; p.H = 1; p.N = B;
-                p.tiles_w = 1; p.tiles_h = 1; p.tiles_n = m_tiles; p.kchunks = lv.in_f / 64; p.w_cols = lv.in_f;
+                p.tiles_w = 1; p.tiles_h = 1; p.tiles_n = m_tiles; p.kchunks = cdiv_i(lv.in_f, 64); p.w_cols = lv.in_f;
                 p.n_total = lv.out_f;
                 p.n_tiles = cdiv_i(lv.out_f, g.fwd.bn);
                 p.epi = UEPI_BIAS_ACT; p.relu = lv.relu ? 1 : 0; p.out_f32 = lv.kind == SB_FC; p.out = lv.act; p.ldc = lv.out_f;

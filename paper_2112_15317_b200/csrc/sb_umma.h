@@ -83,7 +83,7 @@ sb_status umma_fc_wgrad(sb_model* m, int layer, cudaStream_t st);
 bool umma_fc_wgrad_can_update(sb_model* m, int layer);
 sb_status umma_fc_wgrad_update(sb_model* m, int layer, Hyper hy, cudaStream_t st);
 
-// Input-layer convolution (1, 3 or 4 input channels, 64 output channels, bf16) on the tensor cores.
+// Input-layer convolution (1, 3 or 4 input channels, 16, 32, 48 or 64 output channels, bf16) on the tensor cores.
 bool conv_in_umma_supported(int Cin, int Cout);
 // Partial buffers the weight-gradient kernel writes ([blocks][Cout*9*Cin + Cout] floats, reduced in block order).
 int conv_in_umma_wgrad_blocks(long npix);
