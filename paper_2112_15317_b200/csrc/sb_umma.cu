@@ -136,7 +136,7 @@ __device__ __forceinline__ int fast_div_exact(int n, uint32_t mul, int d)
 constexpr int UMMA_THREADS = 192;
 constexpr int A_STAGE_BYTES = 16384;   // 128 rows x 128 B (K-major) or 2 boxes of 64 rows x 128 B (MN-major)
 
-constexpr int CTRL_BYTES = 2048;       // [0,512) barriers + flags, [512,1536) bias (FWD)
+constexpr int CTRL_BYTES = 2048;       // [0,512) barriers + flags, [512,1536) bias (FWD), [512,2048) partial bias gradients (WGRAD)
 constexpr int MAX_STAGES = 8;
 template <int MODE, int BN> struct Cfg {
     static constexpr int B_STAGE_BYTES = BN * 128;
@@ -882,38 +882,62 @@ umma_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
             row_off = (((size_t)n * p.H + h) * p.W + w) * p.ldc;
         }
         if (MODE == MODE_WGRAD && do_bias) {
-            // Bias gradient: thread `row` sums dy[pixel, m0 + row] over this CTA's pixel chunks, reading the A
-            // stage (64 pixel rows of 128 bytes per 64-channel box, 16-byte chunks XOR-swizzled by row % 8)
-            // while the MMA consumes it; pixel order is fixed, so the sum is deterministic.
-            float bsum = 0.f;
-            const uint32_t box_off = (uint32_t)(row / 64) * 8192u, c = (uint32_t)(row % 64);
-            for (int it = 0; it < n_iters && ok; ++it) {
-                const int s = it % STAGES;
-                const uint32_t ph = (uint32_t)((it / STAGES) & 1);
-                if (lane == 0) ok = mbar_wait(&full[s], ph);
-                ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+            // Bias gradient: the sum of dy[pixel, m0 + ..] over this CTA's pixel chunks, read from the A stage (64 pixel rows of 128
+            // bytes per 64-channel box, 16-byte pieces XOR-swizzled by row % 8) while the MMA consumes it.  A thread takes one piece
+            // (8 channels) of every eighth row, so that the swizzle is a constant of the thread and a quarter-warp reads a whole
+            // 128-byte row; fixed order, so the sum is deterministic.  (One thread per channel, 64 two-byte loads and a chain of 64
+            // additions per chunk, took 1.1 us a chunk where the MMAs take 0.25: the few CTAs with the bias paced every launch --
+            // 512 -> 512 channels at 4x4, batch 128: 37 us alone.)
+            const int piece = row % 16, rg = row / 16;
+            const uint32_t at0 = smem0 + (uint32_t)(piece / 8) * 8192u + (uint32_t)rg * 128u + (uint32_t)(((piece % 8) ^ rg) << 4);
+            float bs[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            int s = 0;
+            uint32_t ph = 0, at = at0;
+            for (int it = 0; it < n_iters; ++it) {
+                ok = __all_sync(0xffffffffu, mbar_wait(&full[s], ph) ? 1 : 0) != 0;
                 if (!ok) break;
-                const uint8_t* sa = smem + s * C::STAGE_BYTES + box_off;
-#pragma unroll 8
-                for (uint32_t k = 0; k < 64; ++k) {
-                    const uint32_t off = k * 128u + (((c >> 3) ^ (k & 7u)) << 4) + (c & 7u) * 2u;
-                    bsum += __bfloat162float(*(const __nv_bfloat16*)(sa + off));
-                }
+                uint32_t v[8][4];
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v[i][0]), "=r"(v[i][1]), "=r"(v[i][2]), "=r"(v[i][3]) : "r"(at + 1024u * i));
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        bs[2 * j] += __uint_as_float(v[i][j] << 16);
+                        bs[2 * j + 1] += __uint_as_float(v[i][j] & 0xffff0000u);
+                    }
                 __syncwarp();
-                if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&empty[s])) : "memory");
-            }
-            if (ok && (m0 + row) < m_hi) {
-                const size_t bo = (size_t)split * p.split_stride + p.bias_off + m0 + row;
-                if (p.sgd_w != nullptr) {
-                    const float vb = fmaf(mu, p.sgd_v[bo], bsum), wb = fmaf(-lr, vb, p.sgd_w[bo]);
-                    p.sgd_v[bo] = vb;
-                    p.sgd_w[bo] = wb;
-                    if (p.sgd_s != nullptr) p.sgd_s[bo] = __float2bfloat16_rn(wb);
-                } else {
-                    ((float*)p.out)[bo] = bsum;
-                }
+                if (lane == 0) mbar_arrive(smem_u32(&empty[s]));
+                at += (uint32_t)C::STAGE_BYTES;
+                if (++s == STAGES) { s = 0; ph ^= 1u; at = at0; }
             }
             if (!ok && lane == 0) { *abort_flag = 1; atomicMax(p.status, (uint32_t)DEV_TIMEOUT_EPI); }
+            // row groups 2q, 2q + 1 of warp q, then the four warps in order
+#pragma unroll
+            for (int j = 0; j < 8; ++j) bs[j] += __shfl_down_sync(0xffffffffu, bs[j], 16);
+            if (q > 0 && lane < 16) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) s_bias[(q - 1) * 128 + piece * 8 + j] = bs[j];
+            }
+            epi_bar_sync();
+            if (ok && q == 0 && lane < 16) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int c = piece * 8 + j;
+                    if (m0 + c >= m_hi) break;
+                    const float bsum = ((bs[j] + s_bias[c]) + s_bias[128 + c]) + s_bias[256 + c];
+                    const size_t bo = (size_t)split * p.split_stride + p.bias_off + m0 + c;
+                    if (p.sgd_w != nullptr) {
+                        const float vb = fmaf(mu, p.sgd_v[bo], bsum), wb = fmaf(-lr, vb, p.sgd_w[bo]);
+                        p.sgd_v[bo] = vb;
+                        p.sgd_w[bo] = wb;
+                        if (p.sgd_s != nullptr) p.sgd_s[bo] = __float2bfloat16_rn(wb);
+                    } else {
+                        ((float*)p.out)[bo] = bsum;
+                    }
+                }
+            }
         }
         uint4 refq[MODE == MODE_DGRAD ? MaskRow<BN>::SLOTS : 1];
         const bool have_refq = prefetch_mask_row<MODE, BN>(p, row_ok, row_off, n0, n_hi, refq);
