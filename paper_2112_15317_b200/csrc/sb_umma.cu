@@ -2630,11 +2630,11 @@ static ConvGeom conv_geom(const LayerView& lv, int B, bool force_pair, bool no_h
         const int widest = lv.Cout < lv.Cin ? lv.Cout : lv.Cin;
         const long tiles = mt * cdiv_i(widest, widest >= 128 ? 128 : 64);
         if (tiles > halo_max_tiles || force_persist) {
-            // Four or more tiles per SM: the persistent variant (layers up to 128 channels wide; wider ones do better on the
+            // Three or more tiles per SM: the persistent variant (layers up to 128 channels wide; wider ones do better on the
             // per-tap kernel's CTA pairs with 256-column tiles).  Measured at CIFAR size, batch 128: the 1024-tile layer
             // 20.3 -> 16.3 us, the 256-tile layers 7.3 -> 9.0 and 12.8 -> 13.5 us (one or two tiles per CTA do not repay the
-            // second accumulator's set-up); ImageNet-size step -3.6 %, batch 256 -2 %.
-            static const long persist_min_tiles = (long)tune("SB_PERSIST_MIN_TILES", 4 * 148);
+            // second accumulator's set-up); ImageNet-size step -3.6 %, batch 256 -2 %, its 512-tile layers a further -1.5 %.
+            static const long persist_min_tiles = (long)tune("SB_PERSIST_MIN_TILES", 3 * 148);
             persist = persist_on && (tiles >= persist_min_tiles || force_persist) && lv.Cout <= persist_max_width && lv.Cin <= persist_max_width &&
                       lv.Cout % 64 == 0 && lv.Cin % 64 == 0;
             if (!persist) halo = false;
@@ -2875,13 +2875,11 @@ sb_status umma_plan_layers(sb_model* m, int first_layer)
                     p.stages = g.wg_cps < fit ? g.wg_cps : fit;
                 }
                 {
-                    // grids of fewer than ~100 CTAs leave the other streams whole SMs: no need to keep the ring shallow (measured: -1.5 % step)
-                    static const long wg_cohabit_min = (long)tune("SB_WG_COHABIT_MIN_CTAS", 100);
-                    const long ctas = (long)g.wg_m_tiles * g.wg_n_tiles * ((9 + p.tap_group - 1) / p.tap_group) * p.splits;
                     // (the filter-row kernel keeps its whole five-stage ring: with two slots per round the deeper ring is worth more
                     // than a neighbour on the SM -- steps -0.2 to -1.6 % against a ring cut to two or three 40 KB stages)
                     const int cap = b->bn == 192 ? 5 : cohabit_stages(b->bn);
-                    if (bwd_cohabit() && ctas >= wg_cohabit_min && p.stages > cap) p.stages = cap;
+                    // (grids that leave SMs idle too: whole rings for those of fewer than 100 CTAs cost the step 1.2 % at CIFAR size, batch 128)
+                    if (bwd_cohabit() && p.stages > cap) p.stages = cap;
                 }
                 p.epi = UEPI_F32; p.ldc = 9L * lv.Cin;
                 // the bias gradient rides along: in the parameter arena the bias vector directly follows the
@@ -2893,10 +2891,10 @@ sb_status umma_plan_layers(sb_model* m, int first_layer)
                     // activation tile (a smaller stage, a deeper ring in the same shared memory).  The pair kernel
                     // does not sum dy on the side, so the bias gradient is taken by a column-sum kernel (wgrad_pair).
                     static const bool wg_pair = tune("SB_WG_PAIR", 1) != 0;
-                    // (long reductions only: below ~160 pixel chunks the pair's two cluster barriers and the separate column-sum
-                    // kernel cost more than the halved activation fetch saves: CIFAR shape at batch 128 -1.4 % step with pairs,
-                    // batch 256 +0.4 %, ImageNet shape +1.9 %)
-                    static const int wg_pair_min_chunks = (int)tune("SB_WG_PAIR_MIN_CHUNKS", 160);
+                    // (long reductions only: below 320 pixel chunks the pair's two cluster barriers and the separate column-sum
+                    // kernel cost more than the halved activation fetch saves: from 64 chunks up CIFAR shape at batch 128 +0.7 % step,
+                    // from 160 up batch 256 +0.7 %; never at ImageNet shape +1.2 %)
+                    static const int wg_pair_min_chunks = (int)tune("SB_WG_PAIR_MIN_CHUNKS", 320);
                     if (wg_pair && (g.total_chunks >= wg_pair_min_chunks || (mv.cfg->flags & SB_FLAG_FORCE_PAIR)) && p.tap_group == 1 && (b->bn == 128 || b->bn == 256) && g.wg_m_tiles % 2 == 0 && lv.Cout % 128 == 0) {
                         b->pair = 1;
                         p.bias_fused = 0;
