@@ -162,7 +162,8 @@ sb_status sb_model_destroy(sb_model* m);
  *   labels : HOST array of R DEVICE pointers; labels[r] = int32 [b], values in [0, classes).
  * Row g = r*b + i of every FC-side tensor belongs to replica r (the owner rule of the modulo layer:
  * a batch row's index divided by the rows per worker) [Modulo Layer].  Computes the per-row and mean loss and the gradient
- * of the loss w.r.t. the logits.  The input buffers must stay valid until sb_backward has run.
+ * of the loss w.r.t. the logits.  The input buffers must stay valid until sb_backward has run.  Called several times in a
+ * row with the same buffers on a stream other than the legacy default stream, this pass and sb_backward are replayed as CUDA graphs.
  */
 sb_status sb_forward(sb_model* m, const void* const* x, const int32_t* const* labels, void* stream);
 

@@ -150,6 +150,13 @@ struct sb_model {
     StepGraph g_dev, g_mod;
     StepGraph g_host[2];     // iterations from host buffers: one graph per staging area
     bool host_warmed = false;
+    // Graphs of the single passes (sb_forward, sb_backward), captured once the same input buffers have come `need` times in a row
+    struct PassGraph : StepGraph {
+        PtrTab last_x{}, last_labels{};
+        int same = 0, need = 3;
+        int64_t launches = 0;
+    };
+    PassGraph g_fwd, g_bwd;
     // Debug aids that stand in for a memory checker: every arena region is followed by a 256-byte guard holding a fixed
     // pattern (sb_debug_check_guards), and the regions a step overwrites are listed so that they can be filled with NaN
     // bit patterns before a step (sb_debug_poison).
@@ -183,6 +190,8 @@ struct sb_model {
         if (ev_join) cudaEventDestroy(ev_join);
         for (int k = 0; k < MAX_WSTREAMS; ++k) { if (wstreams[k]) cudaStreamDestroy(wstreams[k]); if (ev_wjoin[k]) cudaEventDestroy(ev_wjoin[k]); }
         if (g_dev.exec) cudaGraphExecDestroy(g_dev.exec);
+        if (g_fwd.exec) cudaGraphExecDestroy(g_fwd.exec);
+        if (g_bwd.exec) cudaGraphExecDestroy(g_bwd.exec);
         if (g_mod.exec) cudaGraphExecDestroy(g_mod.exec);
         for (int k = 0; k < 2; ++k) {
             if (g_host[k].exec) cudaGraphExecDestroy(g_host[k].exec);
@@ -1039,24 +1048,103 @@ sb_status sb_backward_layers(sb_model* m, int32_t last, int32_t first, void* str
     return SB_OK;
 }
 
-sb_status sb_forward(sb_model* m, const void* const* x, const int32_t* const* labels, void* stream)
+static bool same_ptrs(const PtrTab& a, const PtrTab& b, int n)
+{
+    for (int i = 0; i < n; ++i)
+        if (a.p[i] != b.p[i]) return false;
+    return true;
+}
+
+// Ends a capture that failed half-way so that the stream is usable again.
+static void abandon_capture(cudaStream_t st)
+{
+    cudaGraph_t g = nullptr;
+    cudaStreamEndCapture(st, &g);
+    if (g) cudaGraphDestroy(g);
+    cudaGetLastError();
+}
+
+// What was captured on `st` becomes G's executable graph.  An executable graph that is there already is updated in place where
+// the two have the same shape (other input pointers): 0.2 ms where destroying and instantiating it takes 2 ms at VGG-16 size.
+static sb_status end_capture(sb_model::StepGraph& G, cudaStream_t st)
+{
+    cudaGraph_t graph = nullptr;
+    CU_TRY(cudaStreamEndCapture(st, &graph));
+    cudaError_t e = cudaErrorUnknown;
+    if (G.exec) {
+        cudaGraphExecUpdateResultInfo info{};
+        e = cudaGraphExecUpdate(G.exec, graph, &info);
+        if (e != cudaSuccess) { cudaGetLastError(); cudaGraphExecDestroy(G.exec); G.exec = nullptr; }
+    }
+    if (e != cudaSuccess) e = cudaGraphInstantiate(&G.exec, graph, 0);
+    cudaGraphDestroy(graph);
+    if (e != cudaSuccess) { G.exec = nullptr; return fail(SB_ERR_CUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(e)); }
+    return SB_OK;
+}
+
+// One pass on the model's current inputs, replayed as a CUDA graph where that pays: enqueued kernel by kernel a pass costs the host 2
+// to 3.5 us a launch (more than the kernels of a small network take), the graph 2.5 us in all.  It is captured once the
+// same buffers have come several times in a row (each capture that later buffers make useless doubles that number), so a
+// caller whose buffers change from call to call never pays for one.
+}  // extern "C"
+template <typename Pass>
+static sb_status pass_replay(sb_model* m, sb_model::PassGraph& G, cudaStream_t st, Pass pass)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    // (a network that begins with an FC layer binds its input into tensor maps: kernel by kernel)
+    if (m->profiling || m->debug_sync || st == nullptr || m->first_fc == 0 || cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
+        return pass();
+    const int R = m->cfg.R;
+    if (G.same > 0 && same_ptrs(G.last_x, m->x_tab, R) && same_ptrs(G.last_labels, m->label_tab, R)) {
+        if (G.same < G.need) ++G.same;
+    } else {
+        G.last_x = m->x_tab; G.last_labels = m->label_tab; G.same = 1;
+    }
+    if (!(G.exec && same_ptrs(G.x, m->x_tab, R) && same_ptrs(G.labels, m->label_tab, R))) {
+        if (G.same < G.need) return pass();
+        CU_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+        const int64_t l0 = m->launches;
+        sb_status s = pass();
+        if (s != SB_OK) { abandon_capture(st); return s; }
+        G.launches = m->launches - l0;
+        m->launches = l0;
+        s = end_capture(G, st);
+        if (s != SB_OK) return s;
+        G.x = m->x_tab; G.labels = m->label_tab;
+        if (G.need < (1 << 20)) G.need *= 2;
+    }
+    m->launches += G.launches;
+    CU_TRY(cudaGraphLaunch(G.exec, st));
+    return SB_OK;
+}
+
+extern "C" {
+static sb_status forward_pass(sb_model* m, cudaStream_t st)
+{
+    m->pooled_by_conv = -1;
+    m->st_clean = false;
+    for (int i = 0; i < m->n_layers; ++i) {
+        const sb_status s = chain_fwd(m, i, st);
+        if (s != SB_OK) return s;
+    }
+    m->st_clean = false;
+    m->pooled_by_conv = -1;
+    return SB_OK;
+}
+
+// sb_forward / whole iterations: inputs, then the pass (by itself: replayed where that pays)
+static sb_status forward_on(sb_model* m, const void* const* x, const int32_t* const* labels, cudaStream_t st, bool by_itself)
 {
     if (!m) return fail(SB_ERR_INVALID_ARG, "null model");
     if (!x || !labels) return fail(SB_ERR_INVALID_ARG, "x or labels is null");
     sb_status s = set_inputs(m, x, labels);
     if (s != SB_OK) return s;
     m->launches = 0;
-    m->pooled_by_conv = -1;
-    m->st_clean = false;
-    for (int i = 0; i < m->n_layers; ++i) {
-        s = chain_fwd(m, i, (cudaStream_t)stream);
-        if (s != SB_OK) return s;
-    }
-    m->st_clean = false;
-    m->pooled_by_conv = -1;
-    m->have_fwd = true;
-    return SB_OK;
+    s = by_itself ? pass_replay(m, m->g_fwd, st, [&] { return forward_pass(m, st); }) : forward_pass(m, st);
+    if (s == SB_OK) m->have_fwd = true;
+    return s;
 }
+sb_status sb_forward(sb_model* m, const void* const* x, const int32_t* const* labels, void* stream) { return forward_on(m, x, labels, (cudaStream_t)stream, true); }
 
 // The weight-side work of layer i (weight / bias gradient, split reduces, folded update) on `wst`; classic = without the
 // programmatic-dependent-launch attribute.
@@ -1175,7 +1263,8 @@ sb_status sb_backward(sb_model* m, void* stream)
 {
     if (!m) return fail(SB_ERR_INVALID_ARG, "null model");
     if (!m->have_fwd) return fail(SB_ERR_STATE, "sb_backward needs a preceding sb_forward");
-    return backward_pass(m, (cudaStream_t)stream, false, Hyper{}, nullptr);
+    cudaStream_t st = (cudaStream_t)stream;
+    return pass_replay(m, m->g_bwd, st, [&] { return backward_pass(m, st, false, Hyper{}, nullptr); });
 }
 
 // forward + backward + update of one iteration, with the update folded into the backward pass when possible
@@ -1188,7 +1277,7 @@ static sb_status update_all(sb_model* m, Hyper hy, cudaStream_t st)
 }
 static sb_status whole_step(sb_model* m, const void* const* x, const int32_t* const* labels, Hyper hy, void* stream)
 {
-    sb_status s = sb_forward(m, x, labels, stream);
+    sb_status s = forward_on(m, x, labels, (cudaStream_t)stream, false);
     if (s != SB_OK) return s;
     bool updated = false;
     s = backward_pass(m, (cudaStream_t)stream, true, hy, &updated);
@@ -1308,40 +1397,6 @@ sb_status sb_loss(sb_model* m, void* stream, float* host_loss)
         cudaStreamSynchronize((cudaStream_t)stream);
         return fail(SB_ERR_TIMEOUT, "a kernel gave up on a bounded wait (device status %u)", r.status);
     }
-    return SB_OK;
-}
-
-static bool same_ptrs(const PtrTab& a, const PtrTab& b, int n)
-{
-    for (int i = 0; i < n; ++i)
-        if (a.p[i] != b.p[i]) return false;
-    return true;
-}
-
-// Ends a capture that failed half-way so that the stream is usable again.
-static void abandon_capture(cudaStream_t st)
-{
-    cudaGraph_t g = nullptr;
-    cudaStreamEndCapture(st, &g);
-    if (g) cudaGraphDestroy(g);
-    cudaGetLastError();
-}
-
-// What was captured on `st` becomes G's executable graph.  An executable graph that is there already is updated in place where
-// the two have the same shape (other input pointers): 0.2 ms where destroying and instantiating it takes 2 ms at VGG-16 size.
-static sb_status end_capture(sb_model::StepGraph& G, cudaStream_t st)
-{
-    cudaGraph_t graph = nullptr;
-    CU_TRY(cudaStreamEndCapture(st, &graph));
-    cudaError_t e = cudaErrorUnknown;
-    if (G.exec) {
-        cudaGraphExecUpdateResultInfo info{};
-        e = cudaGraphExecUpdate(G.exec, graph, &info);
-        if (e != cudaSuccess) { cudaGetLastError(); cudaGraphExecDestroy(G.exec); G.exec = nullptr; }
-    }
-    if (e != cudaSuccess) e = cudaGraphInstantiate(&G.exec, graph, 0);
-    cudaGraphDestroy(graph);
-    if (e != cudaSuccess) { G.exec = nullptr; return fail(SB_ERR_CUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(e)); }
     return SB_OK;
 }
 

@@ -39,3 +39,31 @@ def test_other_inputs_and_learning_rates_every_step(call):
             assert np.array_equal(p["w"], q["w"]) and np.array_equal(p["b"], q["b"])
     a.close()
     b.close()
+
+
+def test_passes_replayed_on_repeated_buffers():
+    """sb_forward / sb_backward on buffers that repeat (captured), then change, then come back: the same bits as a model that
+    runs every pass kernel by kernel (on the legacy default stream)."""
+    import torch
+
+    from paper_2112_15317_b200 import binding as sb
+    wl = si.config(0)
+    params = si.make_params(wl, bias_std=0.1)
+    a, b = tu.gpu_model(wl, params, sb.SB_BF16), tu.gpu_model(wl, params, sb.SB_BF16)
+    dev = [tu.device_batch(wl, *si.make_batch(wl, seed=40 + k), True) for k in range(2)]
+    side = torch.cuda.Stream()
+    for k in [0] * 5 + [1, 0, 1] + [1] * 6 + [0] * 2:
+        a.forward(*dev[k])
+        a.backward()
+        a.sgd_step(0.01, 0.9)
+        with torch.cuda.stream(side):
+            b.forward(*dev[k])
+            b.backward()
+            b.sgd_step(0.01, 0.9)
+            assert b.loss() == a.loss() and a.launch_count() == b.launch_count(), k
+    for what in ((sb.SB_T_WEIGHT, sb.SB_T_BIAS), (sb.SB_T_GRAD_W, sb.SB_T_GRAD_B)):
+        for p, q in zip(a.gather_params(*what), b.gather_params(*what)):
+            if p is not None:
+                assert np.array_equal(p["w"], q["w"]) and np.array_equal(p["b"], q["b"])
+    a.close()
+    b.close()
