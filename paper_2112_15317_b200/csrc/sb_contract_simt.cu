@@ -399,8 +399,8 @@ template <typename T, int MODE, int BM, int BN, bool VEC>
 static cudaError_t launch_one(const ContractParams& p, cudaStream_t st)
 {
     constexpr int STATIC = (int)(2 * BK * (BM + 4 + BN + 4) * sizeof(float)), MOST = 224 * 1024;
-    static const cudaError_t attr = cudaFuncSetAttribute(contract_kernel<T, MODE, BM, BN, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, MOST - STATIC);
-    if (attr != cudaSuccess) return attr;
+    const cudaError_t e = raise_smem_limit<contract_kernel<T, MODE, BM, BN, VEC>>(MOST - STATIC);
+    if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)((p.M + BM - 1) / BM), (unsigned)((p.N + BN - 1) / BN), (unsigned)p.splits);
     const long n = ((long)grid.x * grid.y * grid.z + 147) / 148;
     const int share = n <= 4 ? (int)(MOST / n) - 2048 - STATIC : 0;

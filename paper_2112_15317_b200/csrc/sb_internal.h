@@ -63,6 +63,20 @@ inline cudaError_t pdl_launch(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
     cfg.numAttrs = pdl_enabled() ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kern, KArgs(std::forward<Args>(args))...);
 }
+// Raises a kernel's dynamic shared-memory limit, once per device (the attribute belongs to the device's copy of the function).
+template <auto Kernel>
+inline cudaError_t raise_smem_limit(int bytes)
+{
+    static bool done[64] = {false};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (done[dev]) return cudaSuccess;
+    e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    done[dev] = e == cudaSuccess;
+    return e;
+}
 #define SB_LAUNCH(kern, grid, block, smem, st, ...) (void)::sb::pdl_launch((kern), dim3(grid), dim3(block), (size_t)(smem), (st), __VA_ARGS__)
 
 

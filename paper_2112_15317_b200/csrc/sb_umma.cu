@@ -2784,11 +2784,11 @@ sb_status umma_plan_layers(sb_model* m, int first_layer)
         LayerView lv = layer_view(m, i);
         UmmaLayer& um = *lv.um;
         const bool want_in_grad = i > 0;
-        if (lv.kind == SB_CONV3X3_RELU && !conv_umma_ok(mv, lv, i) && conv_in_umma_supported(lv.Cin, lv.Cout)) {
-            // input layer: the weight-gradient kernel fetches dy as [pixels][64] rows, 64 pixels per box
+        if (lv.kind == SB_CONV3X3_RELU && !conv_umma_ok(mv, lv, i) && conv_in_umma_supported(lv.H, lv.W, lv.Cin, lv.Cout)) {
+            // input layer: the weight-gradient kernel fetches dy as [pixels][64] rows, 128 pixels per box
             static const bool off = tune("SB_CONV_IN_UMMA", 1) == 0;
             if (!off) {
-                if (!mat_map(&um.wgrad.mapA, lv.dact, (long)B * lv.H * lv.W, lv.Cout, 64)) return fail_plan();
+                if (!mat_map(&um.wgrad.mapA, lv.dact, (long)B * lv.H * lv.W, lv.Cout, 128)) return fail_plan();
                 if (!mat_map(&um.fwd.mapA, lv.act, (long)B * lv.H * lv.W, lv.Cout, 128)) return fail_plan();
                 um.conv_in = true;
             }
