@@ -361,7 +361,7 @@ sb_status plan(const sb_layer* layers, int n, const sb_config* cfg, sb_model* m,
         if (l.kind == SB_CONV3X3_RELU) {
             l.thin_input = conv_in_supported(l.Cin, l.Cout);
             if (l.thin_input) {
-                const int nblk = std::max(conv_in_wgrad_blocks((int)B, l.H, l.W), conv_in_umma_wgrad_blocks((long)B * l.H * l.W));
+                const int nblk = std::max(conv_in_wgrad_blocks((int)B, l.H, l.W), conv_in_umma_supported(l.H, l.W, l.Cin, l.Cout) ? conv_in_umma_wgrad_blocks((int)B, l.H, l.W, l.Cin) : 0);
                 size_t nd = (size_t)nblk * (l.n_w + l.n_b);
                 if (nd > ws_floats) ws_floats = nd;
             }
@@ -708,7 +708,7 @@ sb_status backward_layer(sb_model* m, int i, cudaStream_t st, int part = SIDE_BO
             WgradSimtArgs a{};
             a.x = layer_input(m, i); a.tab = i == 0 ? &m->x_tab : nullptr; a.b_per_rep = b;
             a.dy = l.dact; a.part = ws_w; a.B = B; a.H = l.H; a.W = l.W; a.Cin = l.Cin; a.Cout = l.Cout;
-            const int nb = l.um.conv_in ? conv_in_umma_wgrad_blocks((long)B * l.H * l.W) : conv_in_wgrad_blocks(B, l.H, l.W);
+            const int nb = l.um.conv_in ? conv_in_umma_wgrad_blocks(B, l.H, l.W, l.Cin) : conv_in_wgrad_blocks(B, l.H, l.W);
             const size_t stride = l.n_w + l.n_b;
             if (l.um.conv_in)
                 L_TRY("conv_in_wgrad_umma", flops, pix * (l.Cin + l.Cout) * e + (double)l.n_w * 4.0, launch_conv_in_wgrad_umma(a, l.um.wgrad.mapA, m->status, st));

@@ -16,8 +16,8 @@
 //
 // Bound: the forward pass writes 2 * Cout bytes a pixel, the weight gradient reads them (HBM); below that, the latency chain of
 // a tile (window -> patch -> MMA -> epilogue), which the CTAs resident on an SM hide for one another.  Gathered as 27 two-byte
-// values a pixel with their bounds tests the two passes took 180 and 209 us at 64 x 224x224 images, and 17 and 23 us at
-// 128 x 32x32.  Every mbarrier wait is bounded and reports through the model's device status word.
+// values a pixel with their bounds tests the two passes took 180 and 209 us at 64 x 224x224 images (now 120 and 125; 3.4 TB/s), and
+// 17 and 23 us at 128 x 32x32 (15 and 17).  Every mbarrier wait is bounded and reports through the model's device status word.
 #include "sb_umma.h"
 #include "sb_tcgen05.cuh"
 
@@ -51,7 +51,7 @@ struct ConvInGeom {
     const __nv_bfloat16* x;        // [images][H][W][Cin], or tab: per-replica buffers of b_per_rep images
     PtrTab tab; int use_tab, b_per_rep;
     int H, W, npix, n_img, Cout;
-    uint32_t rcp_w, rcp_h, rcp_hp, rcp_rep, rcp_vpr;
+    uint32_t rcp_w, rcp_h, rcp_hp, rcp_rep;
     int pitch;                     // window: elements from row to row (a multiple of 8)
     int vpr, ve;                   // vectors per image row, elements per vector (8, 2; 1: plain copies)
     int win_bytes;                 // one window buffer
@@ -66,28 +66,25 @@ __device__ __forceinline__ void fetch_window(const ConvInGeom& g, __nv_bfloat16*
     const int last = min(p0 + CI_TILE, g.npix) - 1;
     const int f1 = div_rcp(last, g.rcp_w, g.W), n1 = div_rcp(f1, g.rcp_h, g.H);
     const int q0 = f0 + n0, rows = f1 + n1 - q0 + 3;         // (padded row of the image row above pixel p0's)
-    for (int v = threadIdx.x; v < rows * g.vpr; v += CI_THREADS) {
-        const int r = div_rcp(v, g.rcp_vpr, g.vpr), c = (v - r * g.vpr) * g.ve;
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    for (int r = warp; r < rows; r += CI_THREADS / 32) {
         const int q = q0 + r, n = div_rcp(q, g.rcp_hp, g.H + 1), h = q - n * (g.H + 1) - 1;
         const bool in = h >= 0 && n < g.n_img;
-        const __nv_bfloat16* src = g.x;
+        const __nv_bfloat16* src = g.use_tab ? (const __nv_bfloat16*)g.tab.p[0] : g.x;     // (an address that may be read, for the rows of zeros)
         if (in) {
-            if (g.use_tab) {
-                const int rep = div_rcp(n, g.rcp_rep, g.b_per_rep);
-                src = (const __nv_bfloat16*)g.tab.p[rep] + ((size_t)(n - rep * g.b_per_rep) * g.H + h) * g.W * CIN + c;
-            } else {
-                src = g.x + ((size_t)n * g.H + h) * g.W * CIN + c;
-            }
+            const int rep = g.use_tab ? div_rcp(n, g.rcp_rep, g.b_per_rep) : 0;
+            if (g.use_tab) src = (const __nv_bfloat16*)g.tab.p[rep];
+            src += ((size_t)(n - rep * g.b_per_rep) * g.H + h) * (size_t)(g.W * CIN);
         }
-        __nv_bfloat16* dst = win + r * g.pitch + CI_LEFT + c;
-        if (g.ve == 1) {
-            *dst = in ? *src : __nv_bfloat16();
+        __nv_bfloat16* dst = win + r * g.pitch + CI_LEFT;
+        if (g.ve == 8) {
+            const uint32_t d = smem_u32(dst), bytes = in ? 16u : 0u;
+            for (int c = lane; c < g.vpr; c += 32) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d + 16u * c), "l"(src + (in ? 8 * c : 0)), "r"(bytes) : "memory");
+        } else if (g.ve == 2) {
+            const uint32_t d = smem_u32(dst), bytes = in ? 4u : 0u;
+            for (int c = lane; c < g.vpr; c += 32) asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d + 4u * c), "l"(src + (in ? 2 * c : 0)), "r"(bytes) : "memory");
         } else {
-            const uint32_t d = smem_u32(dst);
-            // (nothing is read where the source size is zero; the address must still be a valid one)
-            const void* from = in ? (const void*)src : (g.use_tab ? g.tab.p[0] : (const void*)g.x);
-            if (g.ve == 8) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(from), "r"(in ? 16 : 0) : "memory");
-            else asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(from), "r"(in ? 4 : 0) : "memory");
+            for (int c = lane; c < g.vpr; c += 32) dst[c] = in ? src[c] : __nv_bfloat16();
         }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -197,6 +194,8 @@ conv_in_fwd_umma_kernel(const __grid_constant__ CUtensorMap mapY, const __grid_c
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     const uint32_t idesc = make_idesc(g.Cout, 0, 0);
+    const uint64_t dA = make_desc(smem_u32(sA), 16), dB = make_desc(smem_u32(sB), 16);
+    const uint32_t elected = warp == 0 && elect_one() ? 1u : 0u;
     uint32_t phase = 0;
     int wb = 0;
 
@@ -213,12 +212,13 @@ conv_in_fwd_umma_kernel(const __grid_constant__ CUtensorMap mapY, const __grid_c
         }
         fence_async_smem();          // the tensor core reads shared memory through the async proxy
         __syncthreads();
-        if (threadIdx.x == 0) {
+        if (warp == 0) {             // (the whole warp in lock-step, one elected lane issues)
             tc_fence_after();
 #pragma unroll
             for (int kk = 0; kk < P::KSTEPS; ++kk)
-                umma_bf16(tmem_base, make_desc(smem_u32(sA) + kk * 32, 16), make_desc(smem_u32(sB) + kk * 32, 16), idesc, kk > 0 ? 1u : 0u);
-            umma_commit(bar);
+                umma_bf16_lohi(tmem_base, (uint32_t)dA + 2u * kk, (uint32_t)(dA >> 32), (uint32_t)dB + 2u * kk, (uint32_t)(dB >> 32), idesc, kk > 0 ? 1u : 0u, elected);
+            if (elected) umma_commit(bar);
+            __syncwarp();
         }
         bool ok = true;
         if (lane == 0) ok = mbar_wait(bar, phase);
@@ -231,25 +231,26 @@ conv_in_fwd_umma_kernel(const __grid_constant__ CUtensorMap mapY, const __grid_c
             const uint32_t taddr = tmem_base + ((uint32_t)(warp * 32) << 16);
             // output row = up to 128 bytes, staged in the patch tile's buffer (the MMA has consumed it) in the 128-byte swizzle of
             // the output map, so that one TMA store writes the tile in full lines
-#pragma unroll 1
-            for (int c0 = 0; c0 < g.Cout; c0 += 16) {
-                uint32_t v[16];
-                tmem_ld16(taddr + c0, v);
-                float4 b[4];
+            const uint32_t row_s = smem_u32(sA) + (uint32_t)row * 128u, sw = (uint32_t)(row & 7), bias_s = smem_u32(s_bias);
 #pragma unroll
-                for (int j = 0; j < 4; ++j) b[j] = *(const float4*)(s_bias + c0 + 4 * j);
+            for (int c0 = 0; c0 < 64; c0 += 16) {
+                if (c0 >= g.Cout) break;
+                uint32_t v[16], pk[8];
+                tmem_ld16(taddr + c0, v);
+                float b[16];
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(b[4 * j]), "=f"(b[4 * j + 1]), "=f"(b[4 * j + 2]), "=f"(b[4 * j + 3]) : "r"(bias_s + (uint32_t)(c0 + 4 * j) * 4u));
                 tmem_ld_wait();
-                uint32_t pk[8];
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    float lo = __uint_as_float(v[2 * j]) + (j % 2 ? b[j / 2].z : b[j / 2].x), hi = __uint_as_float(v[2 * j + 1]) + (j % 2 ? b[j / 2].w : b[j / 2].y);
-                    if (relu) { lo = lo > 0.f ? lo : 0.f; hi = hi > 0.f ? hi : 0.f; }
-                    __nv_bfloat162 t = __floats2bfloat162_rn(lo, hi);
+                    __nv_bfloat162 t = __floats2bfloat162_rn(__uint_as_float(v[2 * j]) + b[2 * j], __uint_as_float(v[2 * j + 1]) + b[2 * j + 1]);
+                    if (relu) t = __hmax2(t, __nv_bfloat162(__nv_bfloat16(0.f), __nv_bfloat16(0.f)));      // (NaN -> 0, as the reference path)
                     pk[j] = *(uint32_t*)&t;
                 }
-                const int j0 = c0 >> 3;
-                *(uint4*)(sA + row * 128 + ((j0 ^ (row & 7)) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                *(uint4*)(sA + row * 128 + (((j0 + 1) ^ (row & 7)) << 4)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+                const uint32_t j0 = (uint32_t)c0 >> 3;
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(row_s + ((j0 ^ sw) << 4)), "r"(pk[0]), "r"(pk[1]), "r"(pk[2]), "r"(pk[3]) : "memory");
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(row_s + (((j0 + 1u) ^ sw) << 4)), "r"(pk[4]), "r"(pk[5]), "r"(pk[6]), "r"(pk[7]) : "memory");
             }
         }
         fence_async_smem();
@@ -324,6 +325,8 @@ conv_in_wgrad_umma_kernel(const __grid_constant__ CUtensorMap mapDy, const __gri
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     constexpr uint32_t idesc = make_idesc(P::COLS, 1, 1);
+    const uint64_t dDy = make_desc(smem_u32(sDy), 16384), dP = make_desc(smem_u32(sP), 8192);
+    const uint32_t elected = warp == 0 && elect_one() ? 1u : 0u;
 
     for (int it = 0; it < n_iters; ++it) {
         const int s = it & 1, p0 = (c_begin + it) * CI_TILE;
@@ -347,17 +350,18 @@ conv_in_wgrad_umma_kernel(const __grid_constant__ CUtensorMap mapDy, const __gri
         fence_async_smem();
         __syncthreads();
         if (*abort_flag) break;
-        if (threadIdx.x == 0) {
-            if (!mbar_wait(&full[s], (uint32_t)((it / 2) & 1))) {
-                *abort_flag = 1; atomicMax(status, (uint32_t)DEV_TIMEOUT_MMA);
+        if (warp == 0) {             // (the whole warp in lock-step, one elected lane issues)
+            if (!__all_sync(0xffffffffu, mbar_wait(&full[s], (uint32_t)((it / 2) & 1)) ? 1 : 0)) {
+                if (lane == 0) { *abort_flag = 1; atomicMax(status, (uint32_t)DEV_TIMEOUT_MMA); }
             } else {
                 tc_fence_after();
+                const uint32_t a_lo = (uint32_t)dDy + (uint32_t)s * (16384u >> 4);
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk)
-                    umma_bf16(tmem_base, make_desc(smem_u32(sDy + s * 16384) + kk * 2048, 16384), make_desc(smem_u32(sP) + kk * 2048, 8192), idesc,
-                              (it > 0 || kk > 0) ? 1u : 0u);
-                umma_commit(done);
+                    umma_bf16_lohi(tmem_base, a_lo + 128u * kk, (uint32_t)(dDy >> 32), (uint32_t)dP + 128u * kk, (uint32_t)(dP >> 32), idesc, (it > 0 || kk > 0) ? 1u : 0u, elected);
+                if (elected) umma_commit(done);
             }
+            __syncwarp();
         }
     }
     window_wait();
@@ -419,11 +423,12 @@ bool conv_in_umma_supported(int H, int W, int Cin, int Cout)
     return (Cin == 1 || Cin == 3 || Cin == 4) && Cout <= 64 && Cout % 16 == 0 && wgrad_smem(window_bytes(H, W, Cin)) <= 220 * 1024;
 }
 
-int conv_in_umma_wgrad_blocks(long npix)
+int conv_in_umma_wgrad_blocks(int B, int H, int W, int Cin)
 {
-    const long chunks = (npix + CI_TILE - 1) / CI_TILE;
+    const long chunks = ((long)B * H * W + CI_TILE - 1) / CI_TILE;
     long ctas = chunks / 2;                       // at least two chunks per CTA
-    if (ctas > 148 * 4) ctas = 148 * 4;           // four CTAs per SM hide one another's latency chains
+    const long resident = (227L * 1024) / (wgrad_smem(window_bytes(H, W, Cin)) + 1024);      // (three or four per SM hide one another's latency chains)
+    if (ctas > 148 * resident) ctas = 148 * resident;
     if (ctas < 1) ctas = 1;
     const long cpc = (chunks + ctas - 1) / ctas;
     return (int)((chunks + cpc - 1) / cpc);       // no empty trailing CTA
@@ -438,7 +443,7 @@ static ConvInGeom geom(const void* x, const PtrTab* tab, int b_per_rep, int B, i
     g.H = H; g.W = W; g.npix = B * H * W; g.n_img = B; g.Cout = Cout;
     g.ve = W * Cin % 8 == 0 ? 8 : W * Cin % 2 == 0 ? 2 : 1;
     g.vpr = W * Cin / g.ve;
-    g.rcp_w = rcp_of(W); g.rcp_h = rcp_of(H); g.rcp_hp = rcp_of(H + 1); g.rcp_rep = rcp_of(b_per_rep); g.rcp_vpr = rcp_of(g.vpr);
+    g.rcp_w = rcp_of(W); g.rcp_h = rcp_of(H); g.rcp_hp = rcp_of(H + 1); g.rcp_rep = rcp_of(b_per_rep);
     g.pitch = window_pitch(W, Cin);
     g.win_bytes = (int)window_bytes(H, W, Cin);
     return g;
@@ -478,7 +483,7 @@ static cudaError_t launch_wgrad_t(const WgradSimtArgs& a, const CUtensorMap& map
     const long npix = (long)a.B * a.H * a.W;
     if (npix + a.B + CI_TILE >= (1L << 31)) return cudaErrorInvalidValue;     // the kernel's pixel arithmetic is 32-bit
     const ConvInGeom g = geom(a.x, a.tab, a.b_per_rep, a.B, a.H, a.W, CIN, a.Cout);
-    const int chunks = (int)((npix + CI_TILE - 1) / CI_TILE), grid = conv_in_umma_wgrad_blocks(npix);
+    const int chunks = (int)((npix + CI_TILE - 1) / CI_TILE), grid = conv_in_umma_wgrad_blocks(a.B, a.H, a.W, CIN);
     const cudaError_t e = raise_smem_limit<conv_in_wgrad_umma_kernel<CIN>>(227 * 1024);
     if (e != cudaSuccess) return e;
     return pdl_launch(conv_in_wgrad_umma_kernel<CIN>, dim3(grid), dim3(CI_THREADS), (size_t)wgrad_smem(g.win_bytes), st, mapDy, g, a.part,

@@ -86,7 +86,7 @@ sb_status umma_fc_wgrad_update(sb_model* m, int layer, Hyper hy, cudaStream_t st
 // Input-layer convolution (1, 3 or 4 input channels, 16, 32, 48 or 64 output channels, bf16) on the tensor cores.
 bool conv_in_umma_supported(int H, int W, int Cin, int Cout);
 // Partial buffers the weight-gradient kernel writes ([blocks][Cout*9*Cin + Cout] floats, reduced in block order).
-int conv_in_umma_wgrad_blocks(long npix);
+int conv_in_umma_wgrad_blocks(int B, int H, int W, int Cin);
 // mapY, mapDy: tensor maps of the output and of its gradient as [pixels][Cout] with (64, 128) boxes
 cudaError_t launch_conv_in_fwd_umma(const ConvSimtArgs& a, const CUtensorMap& mapY, uint32_t* status, cudaStream_t st);
 cudaError_t launch_conv_in_wgrad_umma(const WgradSimtArgs& a, const CUtensorMap& mapDy, uint32_t* status, cudaStream_t st);
