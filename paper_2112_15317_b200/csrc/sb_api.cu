@@ -119,6 +119,7 @@ struct sb_model {
     int n_staged = 0, stage_next = 0;
     cudaStream_t cpstream = nullptr;
     cudaEvent_t ev_staged[2] = {nullptr, nullptr};
+    cudaEvent_t ev_side = nullptr;                   // fork and join of the copy stream around one step's inputs
     // Iterations in flight (sb_train_step_host_async): at most one per staging area; each writes its loss and the device
     // status word into its own pair of words of a small pinned host buffer and records ev_done[area].
     struct Flight { int slot; bool finished; float loss; sb_status status; char msg[160]; };
@@ -198,6 +199,7 @@ struct sb_model {
             if (ev_staged[k]) cudaEventDestroy(ev_staged[k]);
             if (ev_done[k]) cudaEventDestroy(ev_done[k]);
         }
+        if (ev_side) cudaEventDestroy(ev_side);
         if (host_res) cudaFreeHost(host_res);
         if (cpstream) cudaStreamDestroy(cpstream);
     }
@@ -1406,11 +1408,20 @@ static Hyper capture_hyper(sb_model* m, const sb_model::StepGraph& G, float lr, 
     if (G.exec && !G.fits(lr, momentum)) m->hyper_words = true;
     return Hyper{lr, momentum, m->hyper_words ? m->hyper : nullptr};
 }
-static sb_status launch_graph(sb_model* m, const sb_model::StepGraph& G, float lr, float momentum, cudaStream_t st)
+// The device words take new values behind what `st` holds so far.
+static sb_status set_hyper(sb_model* m, float lr, float momentum, cudaStream_t st)
 {
-    if (G.hy.dev && (m->hyper_lr != lr || m->hyper_mu != momentum)) {
+    if (m->hyper_words && (m->hyper_lr != lr || m->hyper_mu != momentum)) {
         CU_TRY(launch_hyper(m->hyper, lr, momentum, st));
         m->hyper_lr = lr; m->hyper_mu = momentum;
+    }
+    return SB_OK;
+}
+static sb_status launch_graph(sb_model* m, const sb_model::StepGraph& G, float lr, float momentum, cudaStream_t st)
+{
+    if (G.hy.dev) {
+        const sb_status s = set_hyper(m, lr, momentum, st);
+        if (s != SB_OK) return s;
     }
     CU_TRY(cudaGraphLaunch(G.exec, st));
     return SB_OK;
@@ -1472,6 +1483,7 @@ sb_status host_step_objects(sb_model* m)
     CU_TRY(cudaHostAlloc((void**)&m->host_res, 4 * sizeof(uint32_t), cudaHostAllocDefault));
     memset(m->host_res, 0, 4 * sizeof(uint32_t));
     CU_TRY(cudaStreamCreateWithFlags(&m->cpstream, cudaStreamNonBlocking));
+    CU_TRY(cudaEventCreateWithFlags(&m->ev_side, cudaEventDisableTiming));
     for (int k = 0; k < 2; ++k) {
         CU_TRY(cudaEventCreateWithFlags(&m->ev_staged[k], cudaEventDisableTiming));
         CU_TRY(cudaEventCreateWithFlags(&m->ev_done[k], cudaEventDisableTiming));
@@ -1549,8 +1561,15 @@ static sb_status host_step(sb_model* m, const void* host_x, const int32_t* host_
     bool finished = false;
     float loss = 0.f;
     if (!pre) {
+        // The images on the caller's stream; the labels (and the hyper-parameter words, below) beside them on the copy stream, which
+        // begins where the caller's stream is: one after the other each small operation adds 3 us to the step.
+        CU_TRY(cudaEventRecord(m->ev_side, st));
+        CU_TRY(cudaStreamWaitEvent(m->cpstream, m->ev_side, 0));
         CU_TRY(cudaMemcpyAsync(m->stage_x, host_x, xb, cudaMemcpyHostToDevice, st));
-        CU_TRY(cudaMemcpyAsync(m->stage_labels, host_labels, (size_t)m->B * 4, cudaMemcpyHostToDevice, st));
+        CU_TRY(cudaMemcpyAsync(m->stage_labels, host_labels, (size_t)m->B * 4, cudaMemcpyHostToDevice, m->cpstream));
+        if (!eager && (s = set_hyper(m, lr, momentum, m->cpstream)) != SB_OK) return s;
+        CU_TRY(cudaEventRecord(m->ev_side, m->cpstream));
+        CU_TRY(cudaStreamWaitEvent(st, m->ev_side, 0));
     }
     if (eager) {
         s = whole_step(m, xp, lp, Hyper{lr, momentum, nullptr}, stream);
@@ -1567,7 +1586,7 @@ static sb_status host_step(sb_model* m, const void* host_x, const int32_t* host_
             CU_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
             s = whole_step(m, xp, lp, hy, stream);
             if (s == SB_OK) {
-                const cudaError_t e = cudaMemcpyAsync(&m->host_res[2 * slot], m->loss, 8, cudaMemcpyDeviceToHost, st);      // loss and status word
+                const cudaError_t e = launch_report(m->loss, &m->host_res[2 * slot], st);      // loss and status word
                 if (e != cudaSuccess) s = fail(SB_ERR_CUDA, "capturing the read-back: %s", cudaGetErrorString(e));
             }
             if (s != SB_OK) { abandon_capture(st); return s; }

@@ -233,6 +233,8 @@ cudaError_t launch_dropout_state(uint32_t* state, int mode, uint64_t seed, uint3
 cudaError_t launch_sgd(float* w, float* v, const float* g, __nv_bfloat16* shadow, size_t n, Hyper hy, cudaStream_t st);
 // writes {lr, mu} to the two words a Hyper with `dev` set reads
 cudaError_t launch_hyper(float* dev, float lr, float mu, cudaStream_t st);
+// copies the loss and the status word behind it to pinned host memory (a memcpy node started 4 to 9 us after the last kernel)
+cudaError_t launch_report(const float* words, uint32_t* host, cudaStream_t st);
 cudaError_t launch_to_bf16(const float* w, __nv_bfloat16* shadow, size_t n, cudaStream_t st);
 
 enum { EPI_BIAS_ACT = 0, EPI_MASK = 1 };

@@ -697,6 +697,17 @@ __global__ void hyper_kernel(float* dev, float lr, float mu)
     pdl_prologue();
     if (threadIdx.x == 0) { dev[0] = lr; dev[1] = mu; }
 }
+// loss and status word (adjacent device words) into pinned host memory, as the last kernel of a replayed iteration
+__global__ void report_kernel(const uint32_t* words, volatile uint32_t* host)
+{
+    pdl_prologue();
+    if (threadIdx.x < 2) host[threadIdx.x] = words[threadIdx.x];
+}
+cudaError_t launch_report(const float* words, uint32_t* host, cudaStream_t st)
+{
+    SB_LAUNCH((report_kernel), 1, 32, 0, st, (const uint32_t*)words, (volatile uint32_t*)host);
+    return cudaGetLastError();
+}
 cudaError_t launch_hyper(float* dev, float lr, float mu, cudaStream_t st)
 {
     SB_LAUNCH((hyper_kernel), 1, 32, 0, st, dev, lr, mu);

@@ -67,6 +67,8 @@ struct UmmaParams {
     // epilogue
     int epi, relu, out_f32;
     int tma_out;          // FWD/DGRAD, bf16 output, no split: the tile is staged in shared memory and written by TMA stores (map C)
+    int a_skip;           // FC FWD/DGRAD on fewer than 128 rows: bytes of the A tile that its box leaves out (accumulator rows past the batch
+                          // then hold garbage that is never stored; MMA rows are independent)
     int w_first;          // FWD/DGRAD: the first ring of WEIGHT loads is issued before the wait for the predecessor kernel (the host sets it
                           // only when that kernel cannot have written the weights), the activation loads after it
     void* out;            // FWD/DGRAD: [pixels][ldc] bf16 (or float when out_f32); WGRAD: float partial sums
@@ -159,14 +161,14 @@ __device__ __forceinline__ void epi_bar_sync() { asm volatile("bar.sync 1, 128;"
 // is enough: whoever has passed the barrier of slab j has finished sweeping slab j - 1, whose buffer slab j + 1 reuses.
 template <int BN>
 __device__ __forceinline__ void wgrad_sweep_epilogue(const UmmaParams& p, uint32_t taddr, uint8_t* stage, int row, int m0, int m_hi,
-                                                      int n0, int n_hi, size_t tile_off, int slab_mult = 1, bool two_bufs = false)
+                                                      int n0, int n_hi, size_t tile_off, bool two_bufs, int slab_stride = 64, int slab_cols = 64)
 {
     const int t128 = threadIdx.x - 64, q = t128 >> 5, lane = t128 & 31;
     const int hl = lane & 15, sub = lane >> 4;
     const uint32_t stage_base = smem_u32(stage);
 #pragma unroll 1
     for (int c0 = 0; c0 < BN; c0 += 64) {
-        if (n0 + c0 >= n_hi) break;                       // (uniform)
+        if (BN != 192 && n0 + c0 >= n_hi) break;          // (uniform; 192 = three taps, a slab each)
         const uint32_t stage_s = stage_base + ((two_bufs && (c0 & 64)) ? 32768u : 0u);
 #pragma unroll
         for (int cc = 0; cc < 64; cc += 32) {
@@ -184,15 +186,14 @@ __device__ __forceinline__ void wgrad_sweep_epilogue(const UmmaParams& p, uint32
                 }
         }
         epi_bar_sync();
-        const int col = n0 + c0 + 4 * hl;
-        if (col < n_hi) {
+        if (4 * hl < slab_cols && (BN == 192 || n0 + c0 + 4 * hl < n_hi)) {
 #pragma unroll 2
             for (int rr = q * 2 + sub; rr < 128; rr += 8) {
                 if (m0 + rr >= m_hi) break;
                 float4 g;
                 asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(g.x), "=f"(g.y), "=f"(g.z), "=f"(g.w)
                              : "r"(stage_s + (uint32_t)rr * 256u + (((uint32_t)hl ^ (uint32_t)(rr & 7)) << 4)));
-                const size_t off = tile_off + (size_t)rr * p.ldc + (size_t)(c0 * slab_mult) + 4 * hl;   // (slab_mult: 64-column slabs three taps apart)
+                const size_t off = tile_off + (size_t)rr * p.ldc + (size_t)(c0 / 64 * slab_stride) + 4 * hl;
                 *(float4*)((float*)p.out + off) = g;
             }
         }
@@ -666,7 +667,7 @@ umma_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         const uint32_t sa = smem0 + ld_off, sb = sa + A_STAGE_BYTES, bar = full0 + 8u * (uint32_t)ld_s;
         if (part != 2)
         mbar_expect_tx_el(bar, (MODE == MODE_WGRAD && BN == 192 && p.hn_order ? (uint32_t)A_STAGE_BYTES + col_box_bytes : (uint32_t)C::STAGE_BYTES) -
-                                   (a_boxes == 2 ? 0u : 8192u), el);
+                                   (MODE == MODE_WGRAD ? (a_boxes == 2 ? 0u : 8192u) : (uint32_t)p.a_skip), el);
         if (MODE == MODE_WGRAD) {
             // pixel chunk -> box origin; A = dy (two 64-channel boxes), B = shifted activations
             const int cw = ld_a * p.bw, ch = ld_b * p.bh, cn = ld_c * p.bn;
@@ -956,13 +957,13 @@ umma_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                                                          (size_t)split * p.split_stride + (size_t)m0 * p.ldc + (size_t)tap_fixed * p.w_cols + n0, lr, mu) && lane == 0) {
                         *abort_flag = 1; atomicMax(p.status, (uint32_t)DEV_TIMEOUT_EPI);
                     }
-                } else if (BN == 192 && p.hn_order)      // slab j = tap row j of filter column tap_fixed / 3: gradient columns (3 j + column) * Cin ..
+                } else if (BN == 192)      // three taps, Cin gradient columns each: slab j = tap row j of filter column tap_fixed / 3 (hn_order), else tap tap_fixed + j
                     wgrad_sweep_epilogue<BN>(p, taddr, smem, row, m0, m_hi, n0, n_hi,
-                                             (size_t)split * p.split_stride + (size_t)m0 * p.ldc + (size_t)(tap_fixed / 3) * p.w_cols, 3,
-                                             STAGES * C::STAGE_BYTES >= 65536);
+                                             (size_t)split * p.split_stride + (size_t)m0 * p.ldc + (size_t)(p.hn_order ? tap_fixed / 3 : tap_fixed) * p.w_cols,
+                                             STAGES * C::STAGE_BYTES >= 65536, (p.hn_order ? 3 : 1) * p.w_cols, p.w_cols);
                 else
                     wgrad_sweep_epilogue<BN>(p, taddr, smem, row, m0, m_hi, n0, n_hi,
-                                             (size_t)split * p.split_stride + (size_t)m0 * p.ldc + (size_t)tap_fixed * p.w_cols + n0, 1,
+                                             (size_t)split * p.split_stride + (size_t)m0 * p.ldc + (size_t)tap_fixed * p.w_cols + n0,
                                              STAGES * C::STAGE_BYTES >= 65536);
             }
         } else if (ok) {
@@ -2635,8 +2636,7 @@ static ConvGeom conv_geom(const LayerView& lv, int B, bool force_pair, bool no_h
             // 20.3 -> 16.3 us, the 256-tile layers 7.3 -> 9.0 and 12.8 -> 13.5 us (one or two tiles per CTA do not repay the
             // second accumulator's set-up); ImageNet-size step -3.6 %, batch 256 -2 %, its 512-tile layers a further -1.5 %.
             static const long persist_min_tiles = (long)tune("SB_PERSIST_MIN_TILES", 3 * 148);
-            persist = persist_on && (tiles >= persist_min_tiles || force_persist) && lv.Cout <= persist_max_width && lv.Cin <= persist_max_width &&
-                      lv.Cout % 64 == 0 && lv.Cin % 64 == 0;
+            persist = persist_on && (tiles >= persist_min_tiles || force_persist) && lv.Cout <= persist_max_width && lv.Cin <= persist_max_width;
             if (!persist) halo = false;
         }
     }
@@ -2670,10 +2670,10 @@ static ConvGeom conv_geom(const LayerView& lv, int B, bool force_pair, bool no_h
     g.wg_bn = lv.Cin >= 256 ? 256 : (lv.Cin >= 128 ? 128 : 64);
     g.wg_n_tiles = cdiv_i(lv.Cin, g.wg_bn);
     g.wg_m_tiles = cdiv_i(lv.Cout, 128);
-    // 64 input channels: one CTA takes a whole filter row (three taps = 192 adjacent gradient columns), so the dy
+    // Up to 64 input channels: one CTA takes a whole filter row (three taps of Cin adjacent gradient columns), so the dy
     // tile is fetched once per three taps (SB_WGRAD_TAPS=1 restores one tap per CTA)
     static const bool taps1 = tune("SB_WGRAD_TAPS", 0) == 1;
-    g.wg_tap_group = (lv.Cin == 64 && !taps1) ? 3 : 1;
+    g.wg_tap_group = (lv.Cin <= 64 && !taps1) ? 3 : 1;
     if (g.wg_tap_group == 3) g.wg_bn = 192;
     // 128 input channels and at most 128 output channels (one M tile, so no CTA pair): two adjacent taps per CTA as one
     // 256-column tile (dy fetched once per two taps; five tap groups, the last with tap 8 alone).  SB_WGRAD_TAPS=1 turns it off.
@@ -2759,6 +2759,9 @@ static void apply_plan(OpBlock* b, const TilePlan& t, int k_iters, long m_tiles,
     if (t.persist) b->grid = dim3((unsigned)t.persist_ctas, 1, 1);
     b->rows = (long)rows;
 }
+
+// Rows of the activation box of an FC op: a batch of fewer than 128 rows fetches only its own (in eights, a swizzle group).
+static int fc_box_rows(int B) { return B >= 128 ? 128 : (B + 7) / 8 * 8; }
 
 // TMA-store epilogue of a FWD / DGRAD op: possible when the output is bf16, the reduction is not split, the columns
 // end on a 16-column chunk (the store clips the rest of a slab), and the idle operand ring can hold the staged tile.
@@ -2942,7 +2945,8 @@ sb_status umma_plan_layers(sb_model* m, int first_layer)
                 p.bias = mv.Wm + lv.p_b; p.status = mv.status;
                 apply_plan(b, g.fwd, p.kchunks, m_tiles, p.n_tiles, mv.ws, (size_t)B);
                 if (p.splits > 1 && (size_t)p.splits * (size_t)p.split_stride > mv.ws_floats) return SB_ERR_ARENA_TOO_SMALL;
-                if (!act_map(&um.fwd.mapA, lv.in_act, B, 1, 1, lv.in_f, 1, 1, 128)) return fail_plan();
+                if (!b->pair) p.a_skip = (128 - fc_box_rows(B)) * 128;
+                if (!act_map(&um.fwd.mapA, lv.in_act, B, 1, 1, lv.in_f, 1, 1, 128 - p.a_skip / 128)) return fail_plan();
                 if (!mat_map(&um.fwd.mapB, mv.Sm + lv.p_w, lv.out_f, lv.in_f, b->pair ? b->bn / 2 : b->bn)) return fail_plan();
                 if (tma_out_ok(b)) {
                     if (!act_map(&um.fwd.mapC, lv.act, B, 1, 1, lv.out_f, 1, 1, 128)) return fail_plan();
@@ -2964,7 +2968,8 @@ sb_status umma_plan_layers(sb_model* m, int first_layer)
                 p.status = mv.status;
                 apply_plan(b, g.dgrad, p.kchunks, m_tiles, p.n_tiles, mv.ws, (size_t)B);
                 if (p.splits > 1 && (size_t)p.splits * (size_t)p.split_stride > mv.ws_floats) return SB_ERR_ARENA_TOO_SMALL;
-                if (!act_map(&um.dgrad.mapA, lv.dact, B, 1, 1, lv.out_f, 1, 1, 128)) return fail_plan();
+                if (!b->pair) p.a_skip = (128 - fc_box_rows(B)) * 128;
+                if (!act_map(&um.dgrad.mapA, lv.dact, B, 1, 1, lv.out_f, 1, 1, 128 - p.a_skip / 128)) return fail_plan();
                 if (!mat_map(&um.dgrad.mapB, mv.Sm + lv.p_w, lv.out_f, lv.in_f, 64)) return fail_plan();
                 if (tma_out_ok(b)) {
                     if (!act_map(&um.dgrad.mapC, lv.d_below, B, 1, 1, lv.in_f, 1, 1, 128)) return fail_plan();
@@ -3012,7 +3017,7 @@ sb_status umma_bind_input(sb_model* m, const void* x)
     LayerView lv = layer_view(m, 0);
     UmmaLayer& um = *lv.um;
     if (um.bound_input == x) return SB_OK;
-    if (um.fwd.enabled && !act_map(&um.fwd.mapA, x, mv.B, 1, 1, lv.in_f, 1, 1, 128)) return SB_ERR_CUDA;
+    if (um.fwd.enabled && !act_map(&um.fwd.mapA, x, mv.B, 1, 1, lv.in_f, 1, 1, 128 - blk(um.fwd)->p.a_skip / 128)) return SB_ERR_CUDA;
     if (um.wgrad.enabled && !act_map(&um.wgrad.mapB, x, mv.B, 1, 1, lv.in_f, 1, 1, 64)) return SB_ERR_CUDA;
     um.bound_input = x;
     return SB_OK;
