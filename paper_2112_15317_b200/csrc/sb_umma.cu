@@ -634,9 +634,11 @@ umma_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
     }
     if (MODE != MODE_WGRAD) split = blockIdx.z;
     // k-iterations of this CTA: a contiguous range of the reduction
-    const int k_begin = split * p.chunks_per_split;
-    const int k_end = min(k_begin + p.chunks_per_split, p.total_chunks);
-    const int n_iters = k_end - k_begin;
+    // FC layers (one tap): the splits take turns (chunk split, split + splits, ...), so that the CTAs of one N tile read neighbouring
+    // 128-byte pieces of a weight row at the same time; other reductions are cut into contiguous ranges.
+    const bool in_turn = MODE != MODE_WGRAD && p.ntaps == 1;
+    const int k_begin = in_turn ? split : split * p.chunks_per_split, k_step = in_turn ? p.splits : 1;
+    const int n_iters = in_turn ? (p.total_chunks - split + p.splits - 1) / p.splits : min(p.chunks_per_split, p.total_chunks - k_begin);
     // (tap groups {3,4,5} and {4,5} both start with a tap every CTA grid has exactly once per M tile and split)
     const bool do_bias = MODE == MODE_WGRAD && p.bias_fused && n_idx == 0 && tap_fixed == (p.ntaps == 9 ? (p.tap_group == 3 ? 3 : 4) : 0);
 
@@ -711,7 +713,8 @@ umma_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
 #pragma unroll
                 for (int j = 0; j < BN / 64; ++j) tma_load_4d_el(&mapB, sb + j * 8192, bar, tap * p.w_cols + n0 + 64 * j, kc * 64, 0, 0, el);
             }
-            if (++ld_a == p.kchunks) { ld_a = 0; ++ld_b; }
+            ld_a += k_step;
+            if (ld_a >= p.kchunks) { ld_a = 0; ++ld_b; }
         }
         ++ld_s; ld_off += (uint32_t)C::STAGE_BYTES;
         if (ld_s == STAGES) { ld_s = 0; ld_off = 0; }
@@ -2185,10 +2188,10 @@ static cudaError_t launch_pair_mode(int bn, const UmmaOp& op, const UmmaParams& 
 template <int MODE>
 static cudaError_t launch_mode(int bn, const UmmaOp& op, const UmmaParams& p, dim3 grid, cudaStream_t st)
 {
-    if (MODE == MODE_WGRAD && bn == 192) return launch_one<MODE_WGRAD, 192>(op, p, grid, st);
     switch (bn) {
     case 64: return launch_one<MODE, 64>(op, p, grid, st);
     case 128: return launch_one<MODE, 128>(op, p, grid, st);
+    case 192: return launch_one<MODE, 192>(op, p, grid, st);
     case 256: return launch_one<MODE, 256>(op, p, grid, st);
     default: return cudaErrorInvalidValue;
     }
@@ -2349,7 +2352,7 @@ static double plan_cost(int bn, int s, int n_cols, long m_tiles, int k_iters)
     const long ctas = m_tiles * cdiv_i(n_cols, bn) * s;
     const double per_sm = (bn < 256 && ctas >= 296) ? 2.0 : 1.0;
     const double waves = (double)cdiv_i(ctas, (long)(148 * per_sm));
-    const double t_iter = bn >= 256 ? 0.38 : (bn >= 128 ? 0.315 : 0.245);
+    const double t_iter = bn >= 256 ? 0.38 : (bn >= 192 ? 0.35 : (bn >= 128 ? 0.315 : 0.245));
     const double partial_mb = (double)s * (double)m_tiles * 128.0 * (double)n_cols * 4.0 / 1.0e6;
     const double mb_us = 0.5;
     return waves * (cdiv_i(k_iters, s) * t_iter * (per_sm > 1.0 ? 1.6 : 1.0) + 3.0) + (s > 1 ? 4.0 + mb_us * partial_mb : 0.0);
@@ -2360,8 +2363,11 @@ static TilePlan plan_tiles(int n_cols, long m_tiles, int k_iters, bool backward,
     int best_bn = 64, best_s = 1;
     {
         double best = 1e300;
-        for (int bn = 64; bn <= 256; bn *= 2) {
+        for (int bn : {64, 128, 192, 256}) {
             if (bn > 64 && bn / 2 >= n_cols) break;      // never wider than the columns need
+            // 192 columns: one M tile whose weights stream from memory, where that gives almost every SM a CTA (25088 columns: 131 CTAs
+            // against 98 of 256 or 196 of 128, 55 -> 50 us at batch 128)
+            if (bn == 192 && (force_pair || m_tiles != 1 || (long)n_cols * k_iters < (1L << 19) || cdiv_i(n_cols, bn) <= 120 || cdiv_i(n_cols, bn) > 148)) continue;
             if (force_pair && bn < 256 && bn < n_cols) continue;   // forced pairs: the widest tile only
             for (int s = 1; s <= 32 && (s == 1 || k_iters / s >= 4); s *= 2) {
                 const double c = plan_cost(bn, s, n_cols, m_tiles, k_iters);
@@ -2373,7 +2379,7 @@ static TilePlan plan_tiles(int n_cols, long m_tiles, int k_iters, bool backward,
     const long tiles = m_tiles * cdiv_i(n_cols, t.bn);
     t.cps = cdiv_i(k_iters, best_s);
     t.splits = cdiv_i(k_iters, t.cps);
-    const int fit = t.bn >= 256 ? 4 : (t.bn >= 128 ? 6 : 8);
+    const int fit = t.bn >= 256 ? 4 : (t.bn >= 192 ? 5 : (t.bn >= 128 ? 6 : 8));
     int st = t.cps < fit ? t.cps : fit;
     if (tiles * t.splits >= 296) {               // >= 2 waves: prefer two resident CTAs per SM
         const int two = t.bn >= 256 ? 2 : (t.bn >= 128 ? 3 : 4);
@@ -2382,7 +2388,7 @@ static TilePlan plan_tiles(int n_cols, long m_tiles, int k_iters, bool backward,
     static const bool fwd_too = tune("SB_FWD_COHABIT", 0) != 0;
     // (a grid that leaves SMs idle need not share its SMs: the other stream's CTAs find free ones; SB_COHABIT_MIN_CTAS)
     static const long cohabit_min = (long)tune("SB_COHABIT_MIN_CTAS", 100);
-    if ((backward || fwd_too) && bwd_cohabit() && tiles * t.splits >= cohabit_min && st > cohabit_stages(t.bn)) st = cohabit_stages(t.bn);
+    if ((backward || fwd_too) && bwd_cohabit() && t.bn != 192 && tiles * t.splits >= cohabit_min && st > cohabit_stages(t.bn)) st = cohabit_stages(t.bn);
     // Grids of more than one CTA per SM: measured, the co-residency of CTAs (their set-up, first loads and
     // epilogues overlap one another's main loops) is worth more than ring depth -- the 1024-CTA 64-wide layer runs
     // 28 us with 2 stages (4 CTAs per SM) against 37 us with 4 and 60 us with 8; beyond 3 stages no layer gains.
@@ -2896,9 +2902,10 @@ sb_status umma_plan_layers(sb_model* m, int first_layer)
                     static const bool wg_pair = tune("SB_WG_PAIR", 1) != 0;
                     // (long reductions only: below 320 pixel chunks the pair's two cluster barriers and the separate column-sum
                     // kernel cost more than the halved activation fetch saves: from 64 chunks up CIFAR shape at batch 128 +0.7 % step,
-                    // from 160 up batch 256 +0.7 %; never at ImageNet shape +1.2 %)
+                    // from 160 up batch 256 +0.7 %; never at ImageNet shape +1.2 %.  512 x 512 channels, whose tiles fill the machine unsplit, from 160
+                    // chunks up: 107 -> 85 us alone at 14x14, batch 64)
                     static const int wg_pair_min_chunks = (int)tune("SB_WG_PAIR_MIN_CHUNKS", 320);
-                    if (wg_pair && (g.total_chunks >= wg_pair_min_chunks || (mv.cfg->flags & SB_FLAG_FORCE_PAIR)) && p.tap_group == 1 && (b->bn == 128 || b->bn == 256) && g.wg_m_tiles % 2 == 0 && lv.Cout % 128 == 0) {
+                    if (wg_pair && (g.total_chunks >= (lv.Cout >= 512 && lv.Cin >= 512 ? wg_pair_min_chunks / 2 : wg_pair_min_chunks) || (mv.cfg->flags & SB_FLAG_FORCE_PAIR)) && p.tap_group == 1 && (b->bn == 128 || b->bn == 256) && g.wg_m_tiles % 2 == 0 && lv.Cout % 128 == 0) {
                         b->pair = 1;
                         p.bias_fused = 0;
                         const int pfit = b->bn >= 256 ? 6 : 8, ptwo = b->bn >= 256 ? 3 : 4;
