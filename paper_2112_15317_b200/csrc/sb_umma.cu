@@ -94,6 +94,7 @@ struct UmmaParams {
     // (tile row = wi + bw * (ni + bn * hi)), one activation fetch of bh + 2 image rows serves the three taps of a filter column.
     int hn_order;         // 1: tile rows in (h, n, w) order; 0: (n, h, w)
     int a_stages;         // depth of the activation (halo) ring; `stages` is then the depth of the weight ring
+    int out_slots;        // halo kernel on CTA pairs: staging buffers of the epilogue (1 or 2)
     uint32_t rcp_bwbn;    // reciprocal of bw * bn (hn_order)
     uint32_t rcp_mtiles;  // reciprocal of tiles_w * tiles_h * tiles_n (persistent halo kernel: tile index -> N tile)
 #ifdef SB_CTA_TIMING
@@ -1962,6 +1963,277 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
 }
 
 // ------------------------------------------------------------------------------------------------
+// The persistent halo kernel on CTA pairs (3x3 FWD / DGRAD, layers of many tiles, 128 columns or more)
+// ------------------------------------------------------------------------------------------------
+// The operands of the halo kernel (one activation box per filter column, three taps read it), the pairs of umma_pair_kernel
+// (256 x BN per MMA, each CTA fetches its own pixels and half of the weights) and the tile walk of the persistent kernel
+// (rings that run on across tiles, two accumulators).  What bounds a single-CTA tile is its shared memory: per 64-channel
+// filter column of a 128-column tile the MMAs read 12 x 8 KB and the TMA writes 20 + 48 KB, 1330 cycles of the port for 768
+// of arithmetic; here 12 x 6 KB and 20 + 24 KB, 930 cycles, and with 256 columns 12 x 8 KB and 20 + 48 KB for 1536 of arithmetic.
+// The per-tap pairs write 64 KB per 1024 cycles of arithmetic and read as much again.
+//   * a_full / b_full live in the LEADER and count the bytes of both CTAs; a commit releases a slot, or hands over an accumulator, in both;
+//   * the epilogue of a tile is two groups of four warps, each with half of the columns, staging buffers (p.out_slots, in turn) and TMA stores
+//     of its own: an epilogue warp is a chain of latencies, and one group is slower than the MMAs of a short reduction;
+//   * acc_empty lives in the leader too and takes one arrival from each group of both CTAs.
+// With more than half of an SM's shared memory no other pair kernel fits beside it: two kernels that allocate tensor memory for pairs
+// must not wait for each other's columns, one on each SM.
+template <int BN> struct HaloPairCfg {
+    static constexpr int B_HALF_BYTES = BN * 64, GROUP_COLS = BN / 2, OUT_BYTES = BN * 128;      // (per group and slot)
+    static constexpr int THREADS = 64 + 256;
+    static constexpr int TMEM_COLS = 2 * BN;
+    static constexpr int MIN_SMEM = 136 * 1024;
+    static constexpr int smem_bytes(int a_stages, int a_slot_bytes, int b_stages, int out_slots)
+    {
+        const int need = a_stages * a_slot_bytes + b_stages * B_HALF_BYTES + 2 * out_slots * OUT_BYTES + 1024 + CTRL_BYTES;
+        return need < MIN_SMEM ? MIN_SMEM : need;
+    }
+};
+
+template <int MODE, int BN>
+__global__ void __launch_bounds__(HaloPairCfg<BN>::THREADS, 1)
+umma_halo_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapC,
+                      const UmmaParams p)
+{
+    static_assert(MODE == MODE_FWD || MODE == MODE_DGRAD, "forward and data gradient only");
+    static_assert(BN == 128 || BN == 256, "N tiles of 128 or 256");
+    using C = HaloPairCfg<BN>;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    const int SA = p.a_stages, SB = p.stages, SO = p.out_slots;
+    const uint32_t row_step = (uint32_t)(p.bw * p.bn) * 128u;
+    const uint32_t a_slot = (uint32_t)(p.bh + 2) * row_step;
+    uint8_t* b_ring = smem + (size_t)SA * a_slot;
+    uint8_t* stage_out = b_ring + (size_t)SB * C::B_HALF_BYTES;
+    uint8_t* ctrl = stage_out + (size_t)(2 * SO) * C::OUT_BYTES;
+    uint64_t* b_full = (uint64_t*)ctrl;               // [MAX_STAGES]
+    uint64_t* b_empty = b_full + MAX_STAGES;          // [MAX_STAGES]
+    uint64_t* a_full = b_empty + MAX_STAGES;          // [MAX_A_STAGES]
+    uint64_t* a_empty = a_full + MAX_A_STAGES;        // [MAX_A_STAGES]
+    uint64_t* acc_full = a_empty + MAX_A_STAGES;      // [2]
+    uint64_t* acc_empty = acc_full + 2;               // [2]
+    uint32_t* tmem_slot = (uint32_t*)(acc_empty + 2);
+    volatile uint32_t* abort_flag = tmem_slot + 1;
+    volatile uint32_t* epi_stop = tmem_slot + 2;      // [2]: written by the warps of one epilogue group only, so that all of them see the same value behind a barrier
+    float* s_bias = (float*)(ctrl + 512);             // [BN]
+
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const uint32_t rank = cluster_ctarank();
+    const bool leader = rank == 0;
+    const int m_tiles = p.tiles_w * p.tiles_h * p.tiles_n;
+    const int units = (m_tiles + 1) / 2 * p.n_tiles;             // pairs of M tiles x N tiles, N tiles of one pair next to each other
+    const int unit0 = blockIdx.x / 2, unit_step = gridDim.x / 2;
+    const int n_groups = p.total_chunks;                         // 3 * kchunks groups per tile
+    const uint32_t smem0 = smem_u32(smem), bring0 = smem_u32(b_ring);
+
+    // unit -> this CTA's pixel-box origin and the first output column (an M index past the last tile lies wholly out of bounds: zero
+    // loads, no stores)
+    auto tile_coords = [&](int u, int& pw0, int& ph0, int& pn0, int& n0) {
+        const int pair = u / p.n_tiles, m_idx = 2 * pair + (int)rank;
+        const int q1 = fast_div_exact(m_idx, p.rcp_tiles_w, p.tiles_w), q2 = fast_div_exact(m_idx, p.rcp_tiles_wh, p.tiles_w * p.tiles_h);
+        pw0 = (m_idx - q1 * p.tiles_w) * p.bw;
+        ph0 = (q1 - q2 * p.tiles_h) * p.bh;
+        pn0 = q2 * p.bn;
+        n0 = (u - pair * p.n_tiles) * BN;
+    };
+
+    // ---- one-time setup -----------------------------------------------------------------------
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < SB; ++s) { mbar_init(&b_full[s], 1); mbar_init(&b_empty[s], 1); }
+        for (int s = 0; s < SA; ++s) { mbar_init(&a_full[s], 1); mbar_init(&a_empty[s], 1); }
+        for (int s = 0; s < 2; ++s) { mbar_init(&acc_full[s], 1); mbar_init(&acc_empty[s], 4); epi_stop[s] = 0; }
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncwarp();
+    cluster_sync_all();    // both CTAs' barriers exist before any copy or commit can signal them
+    if (warp == 1) {
+        tmem_alloc_pair(tmem_slot, C::TMEM_COLS);
+        tmem_relinquish_pair();
+    }
+    pdl_wait();            // every thread that touches global memory waits for the predecessor kernel
+    if (warp == 0) pdl_trigger();
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();    // the peer's accumulator columns are allocated before the leader's first MMA writes them
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+
+    if (warp == 0) {
+        // =========================== TMA producer (both CTAs) ==================================
+        const uint32_t prod_el = elect_one() ? 1u : 0u;
+        const uint32_t afull0 = smem_u32(&a_full[0]), bfull0 = smem_u32(&b_full[0]);
+        const uint32_t afull_l = map_to_cta(afull0, 0), bfull_l = map_to_cta(bfull0, 0);
+        int la_s = 0, lb_s = 0;
+        uint32_t la_off = 0, lb_off = 0, pa_par = 1u, pb_par = 1u;
+        bool ok = true;
+        for (int u = unit0; u < units && ok; u += unit_step) {
+            int pw0, ph0, pn0, n0;
+            tile_coords(u, pw0, ph0, pn0, n0);
+            const int nb0 = n0 + (int)rank * (BN / 2);           // first B column this CTA fetches
+            int kc = 0, dsi = 0;
+            for (int g = 0; g < n_groups; ++g) {
+                const int s1 = lb_s, s2 = s1 + 1 == SB ? 0 : s1 + 1, s3 = s2 + 1 == SB ? 0 : s2 + 1;
+                const uint32_t p1 = pb_par, p2 = s2 == 0 ? p1 ^ 1u : p1, p3 = s3 == 0 ? p2 ^ 1u : p2;
+                const bool w0 = mbar_try_wait(&a_empty[la_s], pa_par), w1 = mbar_try_wait(&b_empty[s1], p1),
+                           w2 = mbar_try_wait(&b_empty[s2], p2), w3 = mbar_try_wait(&b_empty[s3], p3);
+                if (!__all_sync(0xffffffffu, (w0 && w1 && w2 && w3) ? 1 : 0)) {
+                    ok = __all_sync(0xffffffffu, (mbar_wait(&a_empty[la_s], pa_par) && mbar_wait(&b_empty[s1], p1) &&
+                                                  mbar_wait(&b_empty[s2], p2) && mbar_wait(&b_empty[s3], p3)) ? 1 : 0) != 0;
+                    if (!ok) break;
+                }
+                if (leader) mbar_expect_tx_el(afull0 + 8u * (uint32_t)la_s, 2u * a_slot, prod_el);
+                tma_load_4d_pair_el(&mapA, smem0 + la_off, afull_l + 8u * (uint32_t)la_s, kc * 64, pw0 + dsi - 1, pn0, ph0 - 1, prod_el);    // (c, w, n, h)
+                ++la_s; la_off += a_slot;
+                if (la_s == SA) { la_s = 0; la_off = 0; pa_par ^= 1u; }
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    const int tap = MODE == MODE_FWD ? 3 * j + dsi : 3 * (2 - j) + (2 - dsi);
+                    const uint32_t dst = bring0 + lb_off, bar = bfull_l + 8u * (uint32_t)lb_s;
+                    if (leader) mbar_expect_tx_el(bfull0 + 8u * (uint32_t)lb_s, 2u * (uint32_t)C::B_HALF_BYTES, prod_el);
+                    if (MODE == MODE_FWD) {
+                        tma_load_4d_pair_el(&mapB, dst, bar, tap * p.w_cols + kc * 64, nb0, 0, 0, prod_el);      // box of BN/2 rows
+                    } else {
+#pragma unroll
+                        for (int jj = 0; jj < BN / 128; ++jj)
+                            tma_load_4d_pair_el(&mapB, dst + jj * 8192, bar, tap * p.w_cols + nb0 + 64 * jj, kc * 64, 0, 0, prod_el);
+                    }
+                    ++lb_s; lb_off += (uint32_t)C::B_HALF_BYTES;
+                    if (lb_s == SB) { lb_s = 0; lb_off = 0; pb_par ^= 1u; }
+                }
+                if (++dsi == 3) { dsi = 0; ++kc; }
+            }
+        }
+        if (!ok && lane == 0) { *abort_flag = 1; atomicMax(p.status, (uint32_t)DEV_TIMEOUT_TMA); }
+        __syncwarp();
+    } else if (warp == 1) {
+        if (leader) {
+            // =========================== MMA issuer (leader) ====================================
+            constexpr uint32_t idesc = make_idesc(BN, 0, MODE != MODE_FWD, 256);
+            const uint32_t elected = elect_one() ? 1u : 0u;
+            // the MMA addresses both accumulators with one TMEM address: the pair must have been given the same columns
+            const bool tmem_ok = ld_cluster_u32(map_to_cta(smem_u32(tmem_slot), 1)) == tmem_base;
+            bool ok = tmem_ok;
+            if (!ok && lane == 0) { *abort_flag = 1; atomicMax(p.status, (uint32_t)DEV_PAIR_TMEM); }
+            const uint64_t dA0 = make_desc(smem0, 16);
+            const uint64_t dB0 = (MODE == MODE_FWD) ? make_desc(bring0, 16) : make_desc(bring0, 8192);
+            const uint32_t a_hi = (uint32_t)(dA0 >> 32), b_hi = (uint32_t)(dB0 >> 32);
+            const uint32_t a_lo0 = (uint32_t)dA0, b_lo0 = (uint32_t)dB0;
+            constexpr uint32_t A_STEP = 32u >> 4, B_STEP = ((MODE == MODE_FWD) ? 32u : 2048u) >> 4;
+            constexpr uint32_t BSTAGE16 = (uint32_t)C::B_HALF_BYTES >> 4;
+            const uint32_t aslot16 = a_slot >> 4, rowstep16 = row_step >> 4;
+            int sa = 0, sb_ = 0;
+            uint32_t pha = 0, phb = 0, aoff = 0, boff = 0;
+            int i = 0;                                  // tiles this pair has started
+            for (int u = unit0; u < units && ok; u += unit_step, ++i) {
+                const int buf = i & 1;
+                // both epilogues must have drained this accumulator's previous tile (a fresh barrier reports the phase before its first as complete)
+                ok = __all_sync(0xffffffffu, mbar_wait(&acc_empty[buf], (uint32_t)(((i >> 1) + 1) & 1)) ? 1 : 0) != 0;
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
+                for (int g = 0; g < n_groups; ++g) {
+                    ok = __all_sync(0xffffffffu, mbar_wait(&a_full[sa], pha) ? 1 : 0) != 0;
+                    if (!ok) break;
+#pragma unroll
+                    for (int j = 0; j < 3; ++j) {
+                        ok = __all_sync(0xffffffffu, mbar_wait(&b_full[sb_], phb) ? 1 : 0) != 0;
+                        if (!ok) break;
+                        tc_fence_after();
+                        const uint32_t alo = a_lo0 + aoff + (uint32_t)j * rowstep16, blo = b_lo0 + boff;
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk)
+                            umma_bf16_pair_lohi(d_tmem, alo + kk * A_STEP, a_hi, blo + kk * B_STEP, b_hi, idesc, (g > 0 || j > 0 || kk > 0) ? 1u : 0u, elected);
+                        if (elected) umma_commit_pair(&b_empty[sb_]);
+                        ++sb_; boff += BSTAGE16;
+                        if (sb_ == SB) { sb_ = 0; boff = 0; phb ^= 1u; }
+                    }
+                    if (!ok) break;
+                    if (elected) umma_commit_pair(&a_empty[sa]);
+                    __syncwarp();
+                    ++sa; aoff += aslot16;
+                    if (sa == SA) { sa = 0; aoff = 0; pha ^= 1u; }
+                }
+                if (!ok) break;
+                if (elected) umma_commit_pair(&acc_full[buf]);   // this tile's accumulators are complete once the MMAs above have run
+                __syncwarp();
+            }
+            if (tmem_ok && !ok && lane == 0) { *abort_flag = 1; atomicMax(p.status, (uint32_t)DEV_TIMEOUT_MMA); }
+            __syncwarp();
+        }
+    } else {
+        // =========================== epilogue (both CTAs, own pixels) ===========================
+        constexpr int GC = C::GROUP_COLS;
+        const int q = warp % 4, group = (warp - 2) / 4;               // TMEM lane quadrant of this warp; column half
+        const int row = q * 32 + lane;                                // accumulator row handled by this thread
+        const int t128 = (threadIdx.x - 64) % 128;
+        auto group_sync = [&]() { asm volatile("bar.sync %0, 128;" ::"r"(1 + group) : "memory"); };
+        // tile row = wi + bw * (ni + bn * hi): the same for every tile
+        const int r1 = fast_div(row, p.rcp_bw), hi_ = fast_div(row, p.rcp_bwbn);
+        const int wi = row - r1 * p.bw, ni = r1 - hi_ * p.bn;
+        const uint32_t acc_empty_l = map_to_cta(smem_u32(&acc_empty[0]), 0);
+        const int n_hi = p.n_total;
+        float* bias_g = s_bias + group * GC;
+        bool ok = true;
+        int i = 0, slot = 0;
+        for (int u = unit0; u < units; u += unit_step, ++i) {
+            const int buf = i & 1;
+            int pw0, ph0, pn0, n0;
+            tile_coords(u, pw0, ph0, pn0, n0);
+            const int nc = n0 + GC * group;
+            const int w = pw0 + wi, h = ph0 + hi_, n = pn0 + ni;
+            const bool row_ok = w < p.W && h < p.H && n < p.N;
+            const size_t row_off = (((size_t)n * p.H + h) * p.W + w) * p.ldc;
+            if (MODE == MODE_FWD && p.epi == UEPI_BIAS_ACT) {
+                // (the previous tile's epilogue has passed its last barrier: nobody still reads the old bias values)
+                if (t128 < GC) bias_g[t128] = (nc + t128 < n_hi) ? p.bias[nc + t128] : 0.f;
+            }
+            uint4 refq[MODE == MODE_DGRAD ? MaskRow<GC>::SLOTS : 1];
+            const bool have_refq = prefetch_mask_row<MODE, GC>(p, row_ok, row_off, nc, n_hi, refq);
+            if (lane == 0) ok = mbar_wait(&acc_full[buf], (uint32_t)((i >> 1) & 1));
+            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+            if (!ok && lane == 0) { epi_stop[group] = 1; *abort_flag = 1; atomicMax(p.status, (uint32_t)DEV_TIMEOUT_EPI); }
+            if (t128 == 0) {              // the staging buffer's previous tile has left it
+                if (SO > 1) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                else asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+            }
+            group_sync();                 // ... for everybody; bias staged; a timeout seen by one warp of the group is seen by all
+            if (epi_stop[group]) break;
+            tc_fence_after();
+            uint8_t* stage = stage_out + (2 * slot + group) * C::OUT_BYTES;
+            const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN + GC * group);
+            store_row<MODE, GC>(p, taddr, row_ok, row_off, nc, n_hi, 0, bias_g, stage, row, have_refq ? refq : nullptr);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            tc_fence_before();
+            group_sync();                 // the half tile is staged and every warp has finished reading the accumulator
+            if (t128 == 0) {
+                asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(acc_empty_l + 8u * (uint32_t)buf) : "memory");
+#pragma unroll
+                for (int j = 0; j < GC / 64; ++j)
+                    if (nc + 64 * j < n_hi) tma_store_4d(&mapC, smem_u32(stage) + j * 16384, nc + 64 * j, pw0, pn0, ph0);    // (c, w, n, h)
+                tma_store_commit();
+            }
+            if (MODE == MODE_FWD && p.pool_out != nullptr) pool_from_stage<GC>(p, stage, t128, nc, n_hi, pw0, ph0, pn0);
+            if (++slot == SO) slot = 0;
+        }
+        if (t128 == 0) tma_store_wait_read();
+    }
+
+    // ---- teardown: everyone meets here; TMEM is released on every path ----------------------------
+    tc_fence_before();
+    __syncthreads();
+    if (*abort_flag) {
+        const uint64_t t0 = globaltimer_ns();
+        while (globaltimer_ns() - t0 < 200000ull) { }
+        __syncthreads();
+    }
+    cluster_sync_all();    // neither CTA leaves (or frees TMEM) while its partner may still signal or read it
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc_pair(tmem_base, C::TMEM_COLS);
+    }
+}
+
+// ------------------------------------------------------------------------------------------------
 // Host side: tensor maps and launch planning
 // ------------------------------------------------------------------------------------------------
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -2145,6 +2417,40 @@ static cudaError_t launch_halo_persist_mode(int bn, const UmmaOp& op, const Umma
     }
 }
 
+template <int MODE, int BN>
+static cudaError_t launch_halo_pair_one(const UmmaOp& op, const UmmaParams& p, dim3 grid, cudaStream_t st)
+{
+    using C = HaloPairCfg<BN>;
+    const int smem = C::smem_bytes(p.a_stages, (p.bh + 2) * p.bw * p.bn * 128, p.stages, p.out_slots);
+    if (p.a_stages < 1 || p.a_stages > MAX_A_STAGES || p.stages < 3 || p.stages > MAX_STAGES || p.out_slots < 1 || p.out_slots > 2 || smem > 227 * 1024 ||
+        !p.tma_out || p.splits != 1 || (grid.x & 1u))
+        return cudaErrorInvalidValue;
+    cudaError_t e = raise_smem_limit<umma_halo_pair_kernel<MODE, BN>>(227 * 1024);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(C::THREADS);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = pdl_enabled() ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, umma_halo_pair_kernel<MODE, BN>, op.mapA, op.mapB, op.mapC, p);
+}
+template <int MODE>
+static cudaError_t launch_halo_pair_mode(int bn, const UmmaOp& op, const UmmaParams& p, dim3 grid, cudaStream_t st)
+{
+    switch (bn) {
+    case 128: return launch_halo_pair_one<MODE, 128>(op, p, grid, st);
+    case 256: return launch_halo_pair_one<MODE, 256>(op, p, grid, st);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
 // CTA-pair launch: clusters of two CTAs along x, programmatic dependent launch as everywhere else.
 template <int MODE, int BN>
 static cudaError_t launch_pair_one(const UmmaOp& op, const UmmaParams& p, dim3 grid, cudaStream_t st)
@@ -2269,7 +2575,9 @@ static sb_status launch_op(const UmmaOp& op, cudaStream_t st, int64_t* launches 
         pp.rcp_bwbn = fast_rcp((uint32_t)(pp.bw * pp.bn));
         pp.rcp_mtiles = fast_rcp((uint32_t)(pp.tiles_w * pp.tiles_h * pp.tiles_n));
     }
-    if (b->halo && b->persist && b->p.mode == MODE_FWD) e = launch_halo_persist_mode<MODE_FWD>(b->bn, op, pp, b->grid, st);
+    if (b->halo && b->pair && b->p.mode == MODE_FWD) e = launch_halo_pair_mode<MODE_FWD>(b->bn, op, pp, b->grid, st);
+    else if (b->halo && b->pair && b->p.mode == MODE_DGRAD) e = launch_halo_pair_mode<MODE_DGRAD>(b->bn, op, pp, b->grid, st);
+    else if (b->halo && b->persist && b->p.mode == MODE_FWD) e = launch_halo_persist_mode<MODE_FWD>(b->bn, op, pp, b->grid, st);
     else if (b->halo && b->persist && b->p.mode == MODE_DGRAD) e = launch_halo_persist_mode<MODE_DGRAD>(b->bn, op, pp, b->grid, st);
     else if (b->halo && b->p.mode == MODE_FWD) e = launch_halo_mode<MODE_FWD>(b->bn, op, pp, b->grid, st);
     else if (b->halo && b->p.mode == MODE_DGRAD) e = launch_halo_mode<MODE_DGRAD>(b->bn, op, pp, b->grid, st);
@@ -2328,7 +2636,7 @@ cudaError_t launch_wait_probe(uint32_t* status, unsigned long long limit_ns, cud
 //    reduced in split order by splitk_epilogue) while every CTA keeps at least 4 k-iterations,
 //  * ring depth = k-iterations per CTA, capped by what fits; for grids of several waves the ring is kept
 //    shallow enough that two CTAs share an SM, so one CTA's epilogue overlaps the other's main loop.
-struct TilePlan { int bn, splits, cps, stages, pair, halo, a_stages, persist, persist_ctas; };
+struct TilePlan { int bn, splits, cps, stages, pair, halo, a_stages, persist, persist_ctas, out_slots; double cost; };
 // Backward kernels of the two concurrent streams share SMs only if two CTAs fit side by side (shared
 // memory <= ~110 KB each, TMEM columns <= 256 each): SB_BWD_COHABIT=0 gives every kernel the full ring again.
 static bool bwd_cohabit()
@@ -2555,6 +2863,39 @@ static TilePlan plan_tiles_halo_persist(int n_cols, long m_tiles, int kchunks, i
     return t;
 }
 
+// Plan of the halo kernel on CTA pairs for one pixel box: N tile, ring depths, and the estimate (cycles) by which conv_geom chooses the
+// box.  A group of three taps costs its arithmetic (a 256 x N MMA takes N / 2 cycles) or what it moves through an SM's shared memory (the
+// TMA writes and the MMAs' reads, 128 bytes per cycle), whichever is longer; 74 pairs walk the tiles.
+static bool plan_tiles_halo_pair(int n_cols, long m_tiles, int kchunks, int a_slot_bytes, TilePlan* out)
+{
+    bool found = false;
+    for (int bn = 128; bn <= 256; bn *= 2) {
+        if (bn == 256 && n_cols <= 128) break;
+        TilePlan t{};
+        t.halo = 1; t.pair = 1; t.persist = 1; t.bn = bn; t.splits = 1; t.cps = 3 * kchunks;
+        const int b_half = bn * 64, room = 227 * 1024 - 1024 - CTRL_BYTES;
+        // rings: two groups of weight tiles and two activation boxes at least; then a second staging buffer, a third and fourth box, more weights
+        int sa = 2, sb = 6, so = 1;
+        auto need = [&]() { return sa * a_slot_bytes + sb * b_half + so * bn * 256; };
+        if (need() > room) continue;
+        so = 2; if (need() > room) so = 1;
+        sa = 3; if (need() > room) sa = 2;
+        sb = MAX_STAGES; while (need() > room) --sb;
+        if (sa == 3) { sa = 4; if (need() > room) sa = 3; }
+        if (sa > MAX_A_STAGES) sa = MAX_A_STAGES;
+        t.a_stages = sa; t.stages = sb; t.out_slots = so;
+        const long units = (m_tiles + 1) / 2 * cdiv_i(n_cols, bn);
+        t.persist_ctas = 2 * (int)(units < 74 ? units : 74);
+        const double math = 12.0 * bn / 2, port = (a_slot_bytes + 3.0 * b_half) / 128 + 12.0 * (32 + bn / 8);
+        const double unit = 3 * kchunks * (1.1 * (math > port ? math : port) + 60.0), epi = bn * 16.0;
+        t.cost = (double)cdiv_i(units, 74) * (unit > epi ? unit : epi) + epi + 3000.0;
+        if (!found || t.cost < out->cost) { *out = t; found = true; }
+    }
+    static const bool verbose = tune("SB_PLAN_VERBOSE", 0) != 0;
+    if (verbose && found) fprintf(stderr, "plan: halo pairs N=%d m_tiles=%ld kchunks=%d a_slot=%d -> bn=%d a_stages=%d b_stages=%d out_slots=%d ctas=%d (%.0f cycles)\n", n_cols, m_tiles, kchunks, a_slot_bytes, out->bn, out->a_stages, out->stages, out->out_slots, out->persist_ctas, out->cost);
+    return found;
+}
+
 // Conv weight-gradient split count. Splitting the pixel (K) dimension fills more SMs but every split
 // writes a float copy of the weight gradient and the ordered reduce reads them all back, so the choice is
 // a small cost model: waves x (chunks per CTA x per-chunk operand time + fixed CTA cost) for the GEMM
@@ -2646,6 +2987,34 @@ static ConvGeom conv_geom(const LayerView& lv, int B, bool force_pair, bool no_h
             if (!persist) halo = false;
         }
     }
+    // CTA pairs on halos: layers of more than one 128-column tile per SM with more than 64 columns in at least one direction.  The pixel
+    // box with the cheapest plans for the directions that take it.
+    bool hpair = false;
+    if (halo_on && !force_pair && !no_halo && (lv.Cout > 64 || lv.Cin > 64)) {
+        static const long hp_min_tiles = (long)tune("SB_HALO_PAIR_MIN_TILES", 160);
+        const int widest = lv.Cout < lv.Cin ? lv.Cout : lv.Cin;
+        double best = 1e300;
+        for (int w = 1; w <= 128; w *= 2)
+            for (int h = 2; w * h <= 128; h *= 2) {
+                const int n = 128 / (w * h);
+                if ((w * n) % 8 != 0) continue;
+                const long mt = (long)cdiv_i(lv.W, w) * cdiv_i(lv.H, h) * cdiv_i(B, n);
+                const int a_slot = (h + 2) * w * n * 128;
+                if (!force_persist && (double)lv.W * lv.H * B / 128 * cdiv_i(widest, widest >= 128 ? 128 : 64) <= hp_min_tiles) continue;
+                TilePlan f{}, d{};
+                if (lv.Cout > 64 && !plan_tiles_halo_pair(lv.Cout, mt, cdiv_i(lv.Cin, 64), a_slot, &f)) continue;
+                if (lv.Cin > 64 && !plan_tiles_halo_pair(lv.Cin, mt, cdiv_i(lv.Cout, 64), a_slot, &d)) continue;
+                const double c = f.cost + d.cost - 1e-3 * w;
+                if (c < best) {
+                    best = c;
+                    hpair = true; hbw = w; hbh = h; hbn = n;
+                }
+            }
+    }
+    if (hpair) {
+        halo = true;
+        persist = true;
+    }
     if (halo) {
         g.bw = hbw; g.bh = hbh; g.bn = hbn;
         g.halo = 1;
@@ -2655,9 +3024,11 @@ static ConvGeom conv_geom(const LayerView& lv, int B, bool force_pair, bool no_h
         if (persist) {
             g.fwd = plan_tiles_halo_persist(lv.Cout, g.m_tiles, cdiv_i(lv.Cin, 64), a_slot);
             g.dgrad = plan_tiles_halo_persist(lv.Cin, g.m_tiles, cdiv_i(lv.Cout, 64), a_slot);
+            if (hpair && lv.Cout > 64) plan_tiles_halo_pair(lv.Cout, g.m_tiles, cdiv_i(lv.Cin, 64), a_slot, &g.fwd);
+            if (hpair && lv.Cin > 64) plan_tiles_halo_pair(lv.Cin, g.m_tiles, cdiv_i(lv.Cout, 64), a_slot, &g.dgrad);
             if (force_persist) {      // (tests at small sizes: few CTAs, so that each walks several tiles and reuses both accumulators)
-                if (g.fwd.persist_ctas > 3) g.fwd.persist_ctas = 3;
-                if (g.dgrad.persist_ctas > 3) g.dgrad.persist_ctas = 3;
+                for (TilePlan* t : {&g.fwd, &g.dgrad})
+                    if (t->persist_ctas > 3) t->persist_ctas = t->pair ? 4 : 3;
             }
         } else {
             g.fwd = plan_tiles_halo(lv.Cout, g.m_tiles, cdiv_i(lv.Cin, 64), a_slot, false);
@@ -2755,6 +3126,7 @@ static void apply_plan(OpBlock* b, const TilePlan& t, int k_iters, long m_tiles,
     p.splits = t.splits;
     p.stages = t.stages;
     p.a_stages = t.a_stages;
+    p.out_slots = t.out_slots;
     p.hn_order = t.halo;
     b->halo = t.halo;
     b->persist = t.persist;
