@@ -94,6 +94,7 @@ struct UmmaParams {
     // (tile row = wi + bw * (ni + bn * hi)), one activation fetch of bh + 2 image rows serves the three taps of a filter column.
     int hn_order;         // 1: tile rows in (h, n, w) order; 0: (n, h, w)
     int a_stages;         // depth of the activation (halo) ring; `stages` is then the depth of the weight ring
+    int w_resident;       // persistent halo kernels: `stages` holds all weight tiles of the layer, fetched once per CTA
     int out_slots;        // halo kernel on CTA pairs: staging buffers of the epilogue (1 or 2)
     uint32_t rcp_bwbn;    // reciprocal of bw * bn (hn_order)
     uint32_t rcp_mtiles;  // reciprocal of tiles_w * tiles_h * tiles_n (persistent halo kernel: tile index -> N tile)
@@ -1025,6 +1026,7 @@ umma_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
 // weight tiles (stages slots, one per tap, as in umma_kernel).  Warp roles, bounded waits, epilogues, the pooled
 // output and programmatic dependent launch are those of umma_kernel; tile row = wi + bw * (ni + bn * hi).
 constexpr int MAX_A_STAGES = 4;
+constexpr int MAX_B_SLOTS = 12;        // weight tiles of the halo kernel on CTA pairs
 template <int BN> struct HaloCfg {
     static constexpr int B_STAGE_BYTES = BN * 128;
     static constexpr int TMEM_COLS = BN;
@@ -1333,53 +1335,55 @@ umma_halo_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
 // ------------------------------------------------------------------------------------------------
 // The persistent halo kernel: one CTA walks many output tiles
 // ------------------------------------------------------------------------------------------------
-// A layer of many tiles (several per SM) spends, one tile per CTA, more time in per-CTA fixed work -- barrier and TMEM
-// set-up (~1.3 us), the first operand round trip (~0.4 us), the accumulator drain and the epilogue (~1.5 us) -- than in
-// a short main loop (1 - 3 us at 64 - 128 input channels).  Here a CTA is launched once per SM slot and walks the tiles
-// t = blockIdx.x, blockIdx.x + gridDim.x, ... with
-//   * the operand rings running on across tile boundaries (the producer warp starts the next tile's first groups while
-//     the last ones of the current tile are still being multiplied), and
-//   * two TMEM accumulators: the MMA warp fills accumulator (i & 1) for the i-th tile while the four epilogue warps
-//     drain the other one (tcgen05.ld, bias + ReLU / mask, staging, TMA store, fused 2x2 pool), handing it back through
-//     acc_empty[].
-// The output tile is staged in its own shared-memory buffer (the rings are never idle here).  Unsplit reductions with
-// the TMA-store epilogue only (the planner checks); everything else as in umma_halo_kernel, every wait bounded.
-template <int BN> struct HaloPersistCfg {
-    static constexpr int B_STAGE_BYTES = BN * 128;
-    static constexpr int STAGE_OUT_BYTES = (BN / 64) * 16384;
-    static constexpr int TMEM_COLS = 2 * BN;                 // 128, 256 or 512: powers of two
-    static constexpr int smem_bytes(int a_stages, int a_slot_bytes, int b_stages)
+// Layers of several tiles per SM and at most 64 output columns.  A CTA per SM walks the tiles with two pipelines, every second tile each: a
+// producer warp, an MMA warp, rings that run on across tile boundaries, two TMEM accumulators, four epilogue warps and a staging buffer.  One
+// pipeline alone is a chain of latencies: its MMA warp issues a 64-column MMA every 70 cycles where the tensor core takes 48, and its
+// epilogue (tcgen05.ld, bias + ReLU / mask, staging, TMA store, fused 2x2 pool) is longer than the MMAs of a tile.
+//   * Up to 64 input channels, all weight tiles stay in shared memory, for both pipelines (p.w_resident): fetched per tile they are more
+//     bytes than the activations (72 against 60 KB of L2 reads and of shared-memory writes, beside 216 KB that the MMAs read).
+// Unsplit reductions with the TMA-store epilogue only (the planner checks); everything else as in umma_halo_kernel, every wait bounded.
+struct HaloPersistCfg {
+    static constexpr int BN = 64, B_STAGE_BYTES = BN * 128, OUT_BYTES = 16384, TMEM_COLS = 4 * BN;
+    static constexpr int THREADS = 384;               // warps 0, 1: TMA; 2, 3: MMA; 4..7, 8..11: epilogues
+    static constexpr int MAX_A = 4, MAX_B = 9;        // per pipeline (MAX_B resident tiles: for both)
+    static constexpr int smem_bytes(int a_stages, int a_slot_bytes, int b_stages, bool resident)
     {
-        return a_stages * a_slot_bytes + b_stages * B_STAGE_BYTES + STAGE_OUT_BYTES + 1024 /*alignment slack*/ + CTRL_BYTES;
+        return 2 * a_stages * a_slot_bytes + (resident ? 1 : 2) * b_stages * B_STAGE_BYTES + 2 * OUT_BYTES + 1024 /*alignment slack*/ + CTRL_BYTES;
     }
 };
 
-template <int MODE, int BN>
-__global__ void __launch_bounds__(UMMA_THREADS, 1)
+template <int MODE>
+__global__ void __launch_bounds__(HaloPersistCfg::THREADS, 1)
 umma_halo_persist_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapC,
                          const UmmaParams p)
 {
     static_assert(MODE == MODE_FWD || MODE == MODE_DGRAD, "halo kernel: forward and data gradient only");
-    using C = HaloPersistCfg<BN>;
+    using C = HaloPersistCfg;
+    constexpr int BN = C::BN;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int sub = warp < 4 ? warp & 1 : warp / 4 - 1;          // pipeline of this warp
     const int SA = p.a_stages, SB = p.stages;
+    const bool resident = p.w_resident != 0;                     // SB = all weight tiles of the layer, fetched once
     const uint32_t row_step = (uint32_t)(p.bw * p.bn) * 128u;
     const uint32_t a_slot = (uint32_t)(p.bh + 2) * row_step;
-    uint8_t* b_ring = smem + (size_t)SA * a_slot;
-    uint8_t* stage_out = b_ring + (size_t)SB * C::B_STAGE_BYTES;
-    uint8_t* ctrl = stage_out + C::STAGE_OUT_BYTES;
-    uint64_t* b_full = (uint64_t*)ctrl;               // [MAX_STAGES]
-    uint64_t* b_empty = b_full + MAX_STAGES;          // [MAX_STAGES]
-    uint64_t* a_full = b_empty + MAX_STAGES;          // [MAX_A_STAGES]
-    uint64_t* a_empty = a_full + MAX_A_STAGES;        // [MAX_A_STAGES]
-    uint64_t* acc_full = a_empty + MAX_A_STAGES;      // [2]
-    uint64_t* acc_empty = acc_full + 2;               // [2]
-    uint32_t* tmem_slot = (uint32_t*)(acc_empty + 2);
+    uint8_t* b_rings = smem + (size_t)(2 * SA) * a_slot;
+    uint8_t* stages_out = b_rings + (size_t)((resident ? 1 : 2) * SB) * C::B_STAGE_BYTES;
+    uint8_t* ctrl = stages_out + 2 * C::OUT_BYTES;
+    uint64_t* bars = (uint64_t*)ctrl;
+    uint64_t* b_full = bars + C::MAX_B * sub;                            // [MAX_B]
+    uint64_t* b_empty = bars + C::MAX_B * (2 + sub);                     // [MAX_B]
+    uint64_t* a_full = bars + 4 * C::MAX_B + C::MAX_A * sub;             // [MAX_A]
+    uint64_t* a_empty = bars + 4 * C::MAX_B + C::MAX_A * (2 + sub);      // [MAX_A]
+    uint64_t* acc_full = bars + 4 * (C::MAX_B + C::MAX_A) + 2 * sub;     // [2]
+    uint64_t* acc_empty = bars + 4 * (C::MAX_B + C::MAX_A) + 4 + 2 * sub;
+    uint64_t* w_full = bars + 4 * (C::MAX_B + C::MAX_A) + 8;             // resident weights
+    uint32_t* tmem_slot = (uint32_t*)(w_full + 1);
     volatile uint32_t* abort_flag = tmem_slot + 1;
-    float* s_bias = (float*)(ctrl + 512);             // [BN]
+    volatile uint32_t* epi_stop = tmem_slot + 2 + sub;                   // written by the epilogue warps of one pipeline only, so that all of them see the same value behind a barrier
+    float* s_bias = (float*)(ctrl + 512) + BN * sub;
 
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
 #ifdef SB_CTA_TIMING
     unsigned long long* tlog = (p.timing != nullptr && blockIdx.x < 1024) ? p.timing + 16ull * blockIdx.x : nullptr;
 #endif
@@ -1389,7 +1393,8 @@ umma_halo_persist_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_
     const int m_tiles = p.tiles_w * p.tiles_h * p.tiles_n;
     const int n_tiles_total = m_tiles * p.n_tiles;
     const int n_groups = p.total_chunks;                         // 3 * kchunks groups per tile
-    const uint32_t smem0 = smem_u32(smem), bring0 = smem_u32(b_ring);
+    const uint32_t smem0 = smem_u32(smem) + (uint32_t)(SA * sub) * a_slot, bring0 = smem_u32(b_rings) + (uint32_t)(resident ? 0 : SB * sub) * (uint32_t)C::B_STAGE_BYTES;
+    const int t0 = blockIdx.x + sub * gridDim.x, t_step = 2 * gridDim.x;       // tiles of this pipeline
 
     // tile index -> pixel-box origin and first output column
     auto tile_coords = [&](int t, int& pw0, int& ph0, int& pn0, int& n0) {
@@ -1403,17 +1408,14 @@ umma_halo_persist_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_
     };
 
     // ---- one-time setup -----------------------------------------------------------------------
-    if (warp == 0) {
-        if (lane == 0) {
-            for (int s = 0; s < SB; ++s) { mbar_init(&b_full[s], 1); mbar_init(&b_empty[s], 1); }
-            for (int s = 0; s < SA; ++s) { mbar_init(&a_full[s], 1); mbar_init(&a_empty[s], 1); }
-            for (int s = 0; s < 2; ++s) { mbar_init(&acc_full[s], 1); mbar_init(&acc_empty[s], 1); }
-            *abort_flag = 0;
-            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        }
-        __syncwarp();
+    if (threadIdx.x == 0) {
+        for (int e = 0; e < 4 * (C::MAX_B + C::MAX_A) + 9; ++e) mbar_init(bars + e, 1);
+        *abort_flag = 0;
+        tmem_slot[2] = tmem_slot[3] = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 1) {
+    __syncwarp();
+    if (warp == 2) {
         tmem_alloc(tmem_slot, C::TMEM_COLS);
         tmem_relinquish();
     }
@@ -1423,51 +1425,52 @@ umma_halo_persist_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = *tmem_slot + (uint32_t)(2 * BN * sub);
     SB_TLOG(threadIdx.x == 0, 1, clock64());   // set-up done
     SB_TRACE_STAMP(trace_b);
 
-    if (warp == 0) {
-        // =========================== TMA producer ===============================================
+    if (warp < 2) {
+        // =========================== TMA producers ===============================================
         // (whole warp in lock-step, elected issue, one group per round: see umma_halo_kernel; the rings never reset)
         const uint32_t prod_el = elect_one() ? 1u : 0u;
         const uint32_t afull0 = smem_u32(&a_full[0]), bfull0 = smem_u32(&b_full[0]);
         int la_s = 0, lb_s = 0;
         uint32_t la_off = 0, lb_off = 0, pa_par = 1u, pb_par = 1u;
         bool ok = true;
-        for (int t = blockIdx.x; t < n_tiles_total && ok; t += gridDim.x) {
+        if (resident && sub == 0) {          // (one 64-channel chunk, one N tile; slots in the order in which a tile's groups take them)
+            mbar_expect_tx_el(smem_u32(w_full), (uint32_t)(SB * C::B_STAGE_BYTES), prod_el);
+            for (int b = 0; b < SB; ++b) {
+                const int c = b / 3, j = b - 3 * c, tap = MODE == MODE_FWD ? 3 * j + c : 3 * (2 - j) + (2 - c);
+                tma_load_4d_el(&mapB, bring0 + (uint32_t)(b * C::B_STAGE_BYTES), smem_u32(w_full), tap * p.w_cols, 0, 0, 0, prod_el);
+            }
+        }
+        for (int t = t0; t < n_tiles_total && ok; t += t_step) {
             int pw0, ph0, pn0, n0;
             tile_coords(t, pw0, ph0, pn0, n0);
             int kc = 0, dsi = 0;
             for (int g = 0; g < n_groups; ++g) {
                 const int s1 = lb_s, s2 = s1 + 1 == SB ? 0 : s1 + 1, s3 = s2 + 1 == SB ? 0 : s2 + 1;
                 const uint32_t p1 = pb_par, p2 = s2 == 0 ? p1 ^ 1u : p1, p3 = s3 == 0 ? p2 ^ 1u : p2;
-                const bool w0 = mbar_try_wait(&a_empty[la_s], pa_par), w1 = mbar_try_wait(&b_empty[s1], p1),
-                           w2 = mbar_try_wait(&b_empty[s2], p2), w3 = mbar_try_wait(&b_empty[s3], p3);
+                const bool w0 = mbar_try_wait(&a_empty[la_s], pa_par), w1 = resident || mbar_try_wait(&b_empty[s1], p1),
+                           w2 = resident || mbar_try_wait(&b_empty[s2], p2), w3 = resident || mbar_try_wait(&b_empty[s3], p3);
                 if (!__all_sync(0xffffffffu, (w0 && w1 && w2 && w3) ? 1 : 0)) {
-                    ok = __all_sync(0xffffffffu, (mbar_wait(&a_empty[la_s], pa_par) && mbar_wait(&b_empty[s1], p1) &&
-                                                  mbar_wait(&b_empty[s2], p2) && mbar_wait(&b_empty[s3], p3)) ? 1 : 0) != 0;
+                    ok = __all_sync(0xffffffffu, (mbar_wait(&a_empty[la_s], pa_par) &&
+                                                  (resident || (mbar_wait(&b_empty[s1], p1) && mbar_wait(&b_empty[s2], p2) && mbar_wait(&b_empty[s3], p3)))) ? 1 : 0) != 0;
                     if (!ok) break;
                 }
+                const uint32_t a_bar = afull0 + 8u * (uint32_t)la_s;
                 {
-                    const uint32_t bar = afull0 + 8u * (uint32_t)la_s;
-                    mbar_expect_tx_el(bar, a_slot, prod_el);
-                    tma_load_4d_el(&mapA, smem0 + la_off, bar, kc * 64, pw0 + dsi - 1, pn0, ph0 - 1, prod_el);    // (c, w, n, h)
+                    mbar_expect_tx_el(a_bar, a_slot, prod_el);
+                    tma_load_4d_el(&mapA, smem0 + la_off, a_bar, kc * 64, pw0 + dsi - 1, pn0, ph0 - 1, prod_el);    // (c, w, n, h)
                     ++la_s; la_off += a_slot;
                     if (la_s == SA) { la_s = 0; la_off = 0; pa_par ^= 1u; }
                 }
 #pragma unroll
-                for (int j = 0; j < 3; ++j) {
+                for (int j = 0; j < 3 && !resident; ++j) {
                     const int tap = MODE == MODE_FWD ? 3 * j + dsi : 3 * (2 - j) + (2 - dsi);
                     const uint32_t dst = bring0 + lb_off, bar = bfull0 + 8u * (uint32_t)lb_s;
                     mbar_expect_tx_el(bar, (uint32_t)C::B_STAGE_BYTES, prod_el);
-                    if (MODE == MODE_FWD) {
-                        tma_load_4d_el(&mapB, dst, bar, tap * p.w_cols + kc * 64, n0, 0, 0, prod_el);
-                    } else {
-#pragma unroll
-                        for (int jj = 0; jj < BN / 64; ++jj)
-                            tma_load_4d_el(&mapB, dst + jj * 8192, bar, tap * p.w_cols + n0 + 64 * jj, kc * 64, 0, 0, prod_el);
-                    }
+                    tma_load_4d_el(&mapB, dst, bar, tap * p.w_cols + (MODE == MODE_FWD ? kc * 64 : n0), MODE == MODE_FWD ? n0 : kc * 64, 0, 0, prod_el);
                     ++lb_s; lb_off += (uint32_t)C::B_STAGE_BYTES;
                     if (lb_s == SB) { lb_s = 0; lb_off = 0; pb_par ^= 1u; }
                 }
@@ -1477,7 +1480,7 @@ umma_halo_persist_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_
         if (!ok && lane == 0) { *abort_flag = 1; atomicMax(p.status, (uint32_t)DEV_TIMEOUT_TMA); }
         SB_TRACE_STAMP(trace_c);
         __syncwarp();
-    } else if (warp == 1) {
+    } else if (warp < 4) {
         // =========================== MMA issuer =================================================
         constexpr uint32_t idesc = make_idesc(BN, 0, MODE != MODE_FWD);
         const uint32_t elected = elect_one() ? 1u : 0u;
@@ -1491,8 +1494,9 @@ umma_halo_persist_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_
         int sa = 0, sb_ = 0;
         uint32_t pha = 0, phb = 0, aoff = 0, boff = 0;
         bool ok = true;
-        int i = 0;                                  // tiles this CTA has started
-        for (int t = blockIdx.x; t < n_tiles_total && ok; t += gridDim.x, ++i) {
+        if (resident && t0 < n_tiles_total) ok = __all_sync(0xffffffffu, mbar_wait(w_full, 0u) ? 1 : 0) != 0;
+        int i = 0;                                  // tiles this pipeline has started
+        for (int t = t0; t < n_tiles_total && ok; t += t_step, ++i) {
             const int buf = i & 1;
             // the epilogue must have drained this accumulator's previous tile (use u of a buffer waits for release u - 1;
             // a fresh barrier reports the phase before its first as complete)
@@ -1501,13 +1505,14 @@ umma_halo_persist_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
             for (int g = 0; g < n_groups; ++g) {
+                // (one look at all barriers of the group: a wait per tap costs more than its four MMAs, 135 against 70 - 85 cycles per MMA)
                 const int s1 = sb_, s2 = s1 + 1 == SB ? 0 : s1 + 1, s3 = s2 + 1 == SB ? 0 : s2 + 1;
                 const uint32_t p1 = phb, p2 = s2 == 0 ? p1 ^ 1u : p1, p3 = s3 == 0 ? p2 ^ 1u : p2;
                 const uint32_t o1 = boff, o2 = s2 == 0 ? 0u : o1 + BSTAGE16, o3 = s3 == 0 ? 0u : o2 + BSTAGE16;
-                const bool w0 = mbar_try_wait(&a_full[sa], pha), w1 = mbar_try_wait(&b_full[s1], p1), w2 = mbar_try_wait(&b_full[s2], p2),
-                           w3 = mbar_try_wait(&b_full[s3], p3);
+                const bool w0 = mbar_try_wait(&a_full[sa], pha), w1 = resident || mbar_try_wait(&b_full[s1], p1),
+                           w2 = resident || mbar_try_wait(&b_full[s2], p2), w3 = resident || mbar_try_wait(&b_full[s3], p3);
                 if (!__all_sync(0xffffffffu, (w0 && w1) ? 1 : 0)) {
-                    ok = __all_sync(0xffffffffu, (mbar_wait(&a_full[sa], pha) && mbar_wait(&b_full[s1], p1)) ? 1 : 0) != 0;
+                    ok = __all_sync(0xffffffffu, (mbar_wait(&a_full[sa], pha) && (resident || mbar_wait(&b_full[s1], p1))) ? 1 : 0) != 0;
                     if (!ok) break;
                 }
                 tc_fence_after();
@@ -1515,7 +1520,7 @@ umma_halo_persist_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)
                     umma_bf16_lohi(d_tmem, alo + kk * A_STEP, a_hi, b_lo0 + o1 + kk * B_STEP, b_hi, idesc, (g > 0 || kk > 0) ? 1u : 0u, elected);
-                if (elected) umma_commit(&b_empty[s1]);
+                if (!resident && elected) umma_commit(&b_empty[s1]);
                 if (!__all_sync(0xffffffffu, w2 ? 1 : 0)) {
                     ok = __all_sync(0xffffffffu, mbar_wait(&b_full[s2], p2) ? 1 : 0) != 0;
                     if (!ok) break;
@@ -1524,7 +1529,7 @@ umma_halo_persist_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)
                     umma_bf16_lohi(d_tmem, alo + rowstep16 + kk * A_STEP, a_hi, b_lo0 + o2 + kk * B_STEP, b_hi, idesc, 1u, elected);
-                if (elected) umma_commit(&b_empty[s2]);
+                if (!resident && elected) umma_commit(&b_empty[s2]);
                 if (!__all_sync(0xffffffffu, w3 ? 1 : 0)) {
                     ok = __all_sync(0xffffffffu, mbar_wait(&b_full[s3], p3) ? 1 : 0) != 0;
                     if (!ok) break;
@@ -1534,7 +1539,7 @@ umma_halo_persist_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_
                 for (int kk = 0; kk < 4; ++kk)
                     umma_bf16_lohi(d_tmem, alo + 2 * rowstep16 + kk * A_STEP, a_hi, b_lo0 + o3 + kk * B_STEP, b_hi, idesc, 1u, elected);
                 if (elected) {
-                    umma_commit(&b_empty[s3]);
+                    if (!resident) umma_commit(&b_empty[s3]);
                     umma_commit(&a_empty[sa]);
                 }
                 __syncwarp();
@@ -1550,55 +1555,55 @@ umma_halo_persist_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_
         if (!ok && lane == 0) { *abort_flag = 1; atomicMax(p.status, (uint32_t)DEV_TIMEOUT_MMA); }
         __syncwarp();
     } else {
-        // =========================== epilogue ===================================================
+        // =========================== epilogues ==================================================
         const int q = warp % 4;               // TMEM lane quadrant of this warp
         const int row = q * 32 + lane;        // accumulator row handled by this thread
-        const int t128 = threadIdx.x - 64;
+        const int t128 = threadIdx.x % 128;
+        uint8_t* stage = stages_out + sub * C::OUT_BYTES;
+        auto group_sync = [&]() { asm volatile("bar.sync %0, 128;" ::"r"(1 + sub) : "memory"); };
         // tile row = wi + bw * (ni + bn * hi): the same for every tile
         const int r1 = fast_div(row, p.rcp_bw), hi_ = fast_div(row, p.rcp_bwbn);
         const int wi = row - r1 * p.bw, ni = r1 - hi_ * p.bn;
+        const int n_hi = p.n_total;
         bool ok = true;
         int i = 0;
-        for (int t = blockIdx.x; t < n_tiles_total; t += gridDim.x, ++i) {
+        for (int t = t0; t < n_tiles_total; t += t_step, ++i) {
             const int buf = i & 1;
             int pw0, ph0, pn0, n0;
             tile_coords(t, pw0, ph0, pn0, n0);
-            const int n_hi = p.n_total;
             const int w = pw0 + wi, h = ph0 + hi_, n = pn0 + ni;
             const bool row_ok = w < p.W && h < p.H && n < p.N;
             const size_t row_off = (((size_t)n * p.H + h) * p.W + w) * p.ldc;
             if (MODE == MODE_FWD && p.epi == UEPI_BIAS_ACT) {
                 // (the previous tile's epilogue has passed its last barrier: nobody still reads the old bias values)
-                for (int c = t128; c < BN; c += 128) s_bias[c] = (n0 + c < n_hi) ? p.bias[n0 + c] : 0.f;
+                if (t128 < BN) s_bias[t128] = (n0 + t128 < n_hi) ? p.bias[n0 + t128] : 0.f;
             }
             uint4 refq[MODE == MODE_DGRAD ? MaskRow<BN>::SLOTS : 1];
             const bool have_refq = prefetch_mask_row<MODE, BN>(p, row_ok, row_off, n0, n_hi, refq);
             if (lane == 0) ok = mbar_wait(&acc_full[buf], (uint32_t)((i >> 1) & 1));
             ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-            if (!ok) {
-                if (lane == 0) { *abort_flag = 1; atomicMax(p.status, (uint32_t)DEV_TIMEOUT_EPI); }
+            if (!ok && lane == 0) { *epi_stop = 1; *abort_flag = 1; atomicMax(p.status, (uint32_t)DEV_TIMEOUT_EPI); }
+            if (t128 == 0) {              // the staging buffer's previous tile has left it
+                asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
             }
-            epi_bar_sync();                       // bias staged; a timeout seen by any epilogue warp is seen by all below
-            if (*abort_flag) break;
-            SB_TLOG(t128 == 0 && i < 4, 8 + 2 * i, clock64());      // accumulator of tile i complete
+            group_sync();                 // ... for everybody; bias staged; a timeout seen by one warp of the group is seen by all
+            if (*epi_stop) break;
+            SB_TLOG(t128 == 0 && sub == 0 && i < 4, 8 + 2 * i, clock64());      // accumulator of tile i complete
             tc_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN);
-            store_row<MODE, BN>(p, taddr, row_ok, row_off, n0, n_hi, 0, s_bias, stage_out, row, have_refq ? refq : nullptr);
+            store_row<MODE, BN>(p, taddr, row_ok, row_off, n0, n_hi, 0, s_bias, stage, row, have_refq ? refq : nullptr);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             tc_fence_before();
-            epi_bar_sync();                       // the tile is staged and every warp has finished reading the accumulator
+            group_sync();                 // the tile is staged and every warp has finished reading the accumulator
             if (t128 == 0) {
                 asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_empty[buf])) : "memory");   // accumulator free
-#pragma unroll
-                for (int j = 0; j < BN / 64; ++j)
-                    if (n0 + 64 * j < n_hi) tma_store_4d(&mapC, smem_u32(stage_out) + j * 16384, n0 + 64 * j, pw0, pn0, ph0);    // (c, w, n, h)
+                if (n0 < n_hi) tma_store_4d(&mapC, smem_u32(stage), n0, pw0, pn0, ph0);    // (c, w, n, h)
                 tma_store_commit();
             }
-            if (MODE == MODE_FWD && p.pool_out != nullptr) pool_from_stage<BN>(p, stage_out, t128, n0, n_hi, pw0, ph0, pn0);
-            if (t128 == 0) tma_store_wait_read();
-            epi_bar_sync();                       // the stage may be overwritten by the next tile
-            SB_TLOG(t128 == 0 && i < 4, 9 + 2 * i, clock64());      // epilogue of tile i done
+            if (MODE == MODE_FWD && p.pool_out != nullptr) pool_from_stage<BN>(p, stage, t128, n0, n_hi, pw0, ph0, pn0);
+            SB_TLOG(t128 == 0 && sub == 0 && i < 4, 9 + 2 * i, clock64());      // epilogue of tile i done
         }
+        if (t128 == 0) tma_store_wait_read();
     }
 
     // ---- teardown: everyone meets here; TMEM is released on every path ----------------------------
@@ -1612,7 +1617,7 @@ umma_halo_persist_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_
         while (globaltimer_ns() - t0 < 200000ull) { }
         __syncthreads();
     }
-    if (warp == 1) {
+    if (warp == 2) {
         tc_fence_after();
         tmem_dealloc(tmem_base, C::TMEM_COLS);
     }
@@ -2000,14 +2005,15 @@ umma_halo_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_con
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const int SA = p.a_stages, SB = p.stages, SO = p.out_slots;
+    const bool resident = p.w_resident != 0;          // SB = all weight tiles of the layer: fetched with the first tile, then kept
     const uint32_t row_step = (uint32_t)(p.bw * p.bn) * 128u;
     const uint32_t a_slot = (uint32_t)(p.bh + 2) * row_step;
     uint8_t* b_ring = smem + (size_t)SA * a_slot;
     uint8_t* stage_out = b_ring + (size_t)SB * C::B_HALF_BYTES;
     uint8_t* ctrl = stage_out + (size_t)(2 * SO) * C::OUT_BYTES;
-    uint64_t* b_full = (uint64_t*)ctrl;               // [MAX_STAGES]
-    uint64_t* b_empty = b_full + MAX_STAGES;          // [MAX_STAGES]
-    uint64_t* a_full = b_empty + MAX_STAGES;          // [MAX_A_STAGES]
+    uint64_t* b_full = (uint64_t*)ctrl;               // [MAX_B_SLOTS]
+    uint64_t* b_empty = b_full + MAX_B_SLOTS;         // [MAX_B_SLOTS]
+    uint64_t* a_full = b_empty + MAX_B_SLOTS;         // [MAX_A_STAGES]
     uint64_t* a_empty = a_full + MAX_A_STAGES;        // [MAX_A_STAGES]
     uint64_t* acc_full = a_empty + MAX_A_STAGES;      // [2]
     uint64_t* acc_empty = acc_full + 2;               // [2]
@@ -2074,22 +2080,25 @@ umma_halo_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_con
             for (int g = 0; g < n_groups; ++g) {
                 const int s1 = lb_s, s2 = s1 + 1 == SB ? 0 : s1 + 1, s3 = s2 + 1 == SB ? 0 : s2 + 1;
                 const uint32_t p1 = pb_par, p2 = s2 == 0 ? p1 ^ 1u : p1, p3 = s3 == 0 ? p2 ^ 1u : p2;
-                const bool w0 = mbar_try_wait(&a_empty[la_s], pa_par), w1 = mbar_try_wait(&b_empty[s1], p1),
-                           w2 = mbar_try_wait(&b_empty[s2], p2), w3 = mbar_try_wait(&b_empty[s3], p3);
+                const bool with_b = !resident || u == unit0;
+                const bool w0 = mbar_try_wait(&a_empty[la_s], pa_par), w1 = resident || mbar_try_wait(&b_empty[s1], p1),
+                           w2 = resident || mbar_try_wait(&b_empty[s2], p2), w3 = resident || mbar_try_wait(&b_empty[s3], p3);
                 if (!__all_sync(0xffffffffu, (w0 && w1 && w2 && w3) ? 1 : 0)) {
-                    ok = __all_sync(0xffffffffu, (mbar_wait(&a_empty[la_s], pa_par) && mbar_wait(&b_empty[s1], p1) &&
-                                                  mbar_wait(&b_empty[s2], p2) && mbar_wait(&b_empty[s3], p3)) ? 1 : 0) != 0;
+                    ok = __all_sync(0xffffffffu, (mbar_wait(&a_empty[la_s], pa_par) &&
+                                                  (resident || (mbar_wait(&b_empty[s1], p1) && mbar_wait(&b_empty[s2], p2) && mbar_wait(&b_empty[s3], p3)))) ? 1 : 0) != 0;
                     if (!ok) break;
                 }
-                if (leader) mbar_expect_tx_el(afull0 + 8u * (uint32_t)la_s, 2u * a_slot, prod_el);
-                tma_load_4d_pair_el(&mapA, smem0 + la_off, afull_l + 8u * (uint32_t)la_s, kc * 64, pw0 + dsi - 1, pn0, ph0 - 1, prod_el);    // (c, w, n, h)
+                // (resident weights arrive on the barrier of the activation box that they come with)
+                const uint32_t a_bar = afull_l + 8u * (uint32_t)la_s;
+                if (leader) mbar_expect_tx_el(afull0 + 8u * (uint32_t)la_s, 2u * (a_slot + (resident && with_b ? 3u * (uint32_t)C::B_HALF_BYTES : 0u)), prod_el);
+                tma_load_4d_pair_el(&mapA, smem0 + la_off, a_bar, kc * 64, pw0 + dsi - 1, pn0, ph0 - 1, prod_el);    // (c, w, n, h)
                 ++la_s; la_off += a_slot;
                 if (la_s == SA) { la_s = 0; la_off = 0; pa_par ^= 1u; }
 #pragma unroll
-                for (int j = 0; j < 3; ++j) {
+                for (int j = 0; j < 3 && with_b; ++j) {
                     const int tap = MODE == MODE_FWD ? 3 * j + dsi : 3 * (2 - j) + (2 - dsi);
-                    const uint32_t dst = bring0 + lb_off, bar = bfull_l + 8u * (uint32_t)lb_s;
-                    if (leader) mbar_expect_tx_el(bfull0 + 8u * (uint32_t)lb_s, 2u * (uint32_t)C::B_HALF_BYTES, prod_el);
+                    const uint32_t dst = bring0 + lb_off, bar = resident ? a_bar : bfull_l + 8u * (uint32_t)lb_s;
+                    if (leader && !resident) mbar_expect_tx_el(bfull0 + 8u * (uint32_t)lb_s, 2u * (uint32_t)C::B_HALF_BYTES, prod_el);
                     if (MODE == MODE_FWD) {
                         tma_load_4d_pair_el(&mapB, dst, bar, tap * p.w_cols + kc * 64, nb0, 0, 0, prod_el);      // box of BN/2 rows
                     } else {
@@ -2132,24 +2141,46 @@ umma_halo_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_con
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
                 for (int g = 0; g < n_groups; ++g) {
-                    ok = __all_sync(0xffffffffu, mbar_wait(&a_full[sa], pha) ? 1 : 0) != 0;
-                    if (!ok) break;
+                    // (one look at all barriers of the group: a wait per tap costs more than its four MMAs, 135 against 70 - 85 cycles per MMA)
+                    const int s1 = sb_, s2 = s1 + 1 == SB ? 0 : s1 + 1, s3 = s2 + 1 == SB ? 0 : s2 + 1;
+                    const uint32_t p1 = phb, p2 = s2 == 0 ? p1 ^ 1u : p1, p3 = s3 == 0 ? p2 ^ 1u : p2;
+                    const uint32_t o1 = boff, o2 = s2 == 0 ? 0u : o1 + BSTAGE16, o3 = s3 == 0 ? 0u : o2 + BSTAGE16;
+                    const bool w0 = mbar_try_wait(&a_full[sa], pha), w1 = resident || mbar_try_wait(&b_full[s1], p1),
+                               w2 = resident || mbar_try_wait(&b_full[s2], p2), w3 = resident || mbar_try_wait(&b_full[s3], p3);
+                    if (!__all_sync(0xffffffffu, (w0 && w1) ? 1 : 0)) {
+                        ok = __all_sync(0xffffffffu, (mbar_wait(&a_full[sa], pha) && (resident || mbar_wait(&b_full[s1], p1))) ? 1 : 0) != 0;
+                        if (!ok) break;
+                    }
+                    tc_fence_after();
+                    const uint32_t alo = a_lo0 + aoff;
 #pragma unroll
-                    for (int j = 0; j < 3; ++j) {
-                        ok = __all_sync(0xffffffffu, mbar_wait(&b_full[sb_], phb) ? 1 : 0) != 0;
+                    for (int kk = 0; kk < 4; ++kk)
+                        umma_bf16_pair_lohi(d_tmem, alo + kk * A_STEP, a_hi, b_lo0 + o1 + kk * B_STEP, b_hi, idesc, (g > 0 || kk > 0) ? 1u : 0u, elected);
+                    if (!resident && elected) umma_commit_pair(&b_empty[s1]);
+                    if (!__all_sync(0xffffffffu, w2 ? 1 : 0)) {
+                        ok = __all_sync(0xffffffffu, mbar_wait(&b_full[s2], p2) ? 1 : 0) != 0;
                         if (!ok) break;
                         tc_fence_after();
-                        const uint32_t alo = a_lo0 + aoff + (uint32_t)j * rowstep16, blo = b_lo0 + boff;
-#pragma unroll
-                        for (int kk = 0; kk < 4; ++kk)
-                            umma_bf16_pair_lohi(d_tmem, alo + kk * A_STEP, a_hi, blo + kk * B_STEP, b_hi, idesc, (g > 0 || j > 0 || kk > 0) ? 1u : 0u, elected);
-                        if (elected) umma_commit_pair(&b_empty[sb_]);
-                        ++sb_; boff += BSTAGE16;
-                        if (sb_ == SB) { sb_ = 0; boff = 0; phb ^= 1u; }
                     }
-                    if (!ok) break;
-                    if (elected) umma_commit_pair(&a_empty[sa]);
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk)
+                        umma_bf16_pair_lohi(d_tmem, alo + rowstep16 + kk * A_STEP, a_hi, b_lo0 + o2 + kk * B_STEP, b_hi, idesc, 1u, elected);
+                    if (!resident && elected) umma_commit_pair(&b_empty[s2]);
+                    if (!__all_sync(0xffffffffu, w3 ? 1 : 0)) {
+                        ok = __all_sync(0xffffffffu, mbar_wait(&b_full[s3], p3) ? 1 : 0) != 0;
+                        if (!ok) break;
+                        tc_fence_after();
+                    }
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk)
+                        umma_bf16_pair_lohi(d_tmem, alo + 2 * rowstep16 + kk * A_STEP, a_hi, b_lo0 + o3 + kk * B_STEP, b_hi, idesc, 1u, elected);
+                    if (elected) {
+                        if (!resident) umma_commit_pair(&b_empty[s3]);
+                        umma_commit_pair(&a_empty[sa]);
+                    }
                     __syncwarp();
+                    sb_ = s3 + 1; boff = o3 + BSTAGE16; phb = p3;
+                    if (sb_ == SB) { sb_ = 0; boff = 0; phb ^= 1u; }
                     ++sa; aoff += aslot16;
                     if (sa == SA) { sa = 0; aoff = 0; pha ^= 1u; }
                 }
@@ -2387,34 +2418,15 @@ static cudaError_t launch_halo_mode(int bn, const UmmaOp& op, const UmmaParams& 
     }
 }
 
-template <int MODE, int BN>
-static cudaError_t launch_halo_persist_one(const UmmaOp& op, const UmmaParams& p, dim3 grid, cudaStream_t st)
-{
-    const int a_slot = (p.bh + 2) * p.bw * p.bn * 128;
-    const int smem = HaloPersistCfg<BN>::smem_bytes(p.a_stages, a_slot, p.stages);
-    if (p.a_stages < 1 || p.a_stages > MAX_A_STAGES || p.stages < 3 || p.stages > MAX_STAGES || smem > 227 * 1024 || !p.tma_out || p.splits != 1)
-        return cudaErrorInvalidValue;
-    static bool attr_set[64] = {false};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (!attr_set[dev]) {
-        e = cudaFuncSetAttribute(umma_halo_persist_kernel<MODE, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-        if (e != cudaSuccess) return e;
-        attr_set[dev] = true;
-    }
-    return pdl_launch(umma_halo_persist_kernel<MODE, BN>, grid, dim3(UMMA_THREADS), (size_t)smem, st, op.mapA, op.mapB, op.mapC, p);
-}
 template <int MODE>
-static cudaError_t launch_halo_persist_mode(int bn, const UmmaOp& op, const UmmaParams& p, dim3 grid, cudaStream_t st)
+static cudaError_t launch_halo_persist_mode(const UmmaOp& op, const UmmaParams& p, dim3 grid, cudaStream_t st)
 {
-    switch (bn) {
-    case 64: return launch_halo_persist_one<MODE, 64>(op, p, grid, st);
-    case 128: return launch_halo_persist_one<MODE, 128>(op, p, grid, st);
-    case 256: return launch_halo_persist_one<MODE, 256>(op, p, grid, st);
-    default: return cudaErrorInvalidValue;
-    }
+    const int smem = HaloPersistCfg::smem_bytes(p.a_stages, (p.bh + 2) * p.bw * p.bn * 128, p.stages, p.w_resident != 0);
+    if (p.a_stages < 1 || p.a_stages > HaloPersistCfg::MAX_A || p.stages < 3 || p.stages > HaloPersistCfg::MAX_B || smem > 227 * 1024 || !p.tma_out || p.splits != 1)
+        return cudaErrorInvalidValue;
+    const cudaError_t e = raise_smem_limit<umma_halo_persist_kernel<MODE>>(227 * 1024);
+    if (e != cudaSuccess) return e;
+    return pdl_launch(umma_halo_persist_kernel<MODE>, grid, dim3(HaloPersistCfg::THREADS), (size_t)smem, st, op.mapA, op.mapB, op.mapC, p);
 }
 
 template <int MODE, int BN>
@@ -2422,7 +2434,7 @@ static cudaError_t launch_halo_pair_one(const UmmaOp& op, const UmmaParams& p, d
 {
     using C = HaloPairCfg<BN>;
     const int smem = C::smem_bytes(p.a_stages, (p.bh + 2) * p.bw * p.bn * 128, p.stages, p.out_slots);
-    if (p.a_stages < 1 || p.a_stages > MAX_A_STAGES || p.stages < 3 || p.stages > MAX_STAGES || p.out_slots < 1 || p.out_slots > 2 || smem > 227 * 1024 ||
+    if (p.a_stages < 1 || p.a_stages > MAX_A_STAGES || p.stages < 3 || p.stages > MAX_B_SLOTS || p.out_slots < 1 || p.out_slots > 2 || smem > 227 * 1024 ||
         !p.tma_out || p.splits != 1 || (grid.x & 1u))
         return cudaErrorInvalidValue;
     cudaError_t e = raise_smem_limit<umma_halo_pair_kernel<MODE, BN>>(227 * 1024);
@@ -2577,8 +2589,8 @@ static sb_status launch_op(const UmmaOp& op, cudaStream_t st, int64_t* launches 
     }
     if (b->halo && b->pair && b->p.mode == MODE_FWD) e = launch_halo_pair_mode<MODE_FWD>(b->bn, op, pp, b->grid, st);
     else if (b->halo && b->pair && b->p.mode == MODE_DGRAD) e = launch_halo_pair_mode<MODE_DGRAD>(b->bn, op, pp, b->grid, st);
-    else if (b->halo && b->persist && b->p.mode == MODE_FWD) e = launch_halo_persist_mode<MODE_FWD>(b->bn, op, pp, b->grid, st);
-    else if (b->halo && b->persist && b->p.mode == MODE_DGRAD) e = launch_halo_persist_mode<MODE_DGRAD>(b->bn, op, pp, b->grid, st);
+    else if (b->halo && b->persist && b->p.mode == MODE_FWD) e = launch_halo_persist_mode<MODE_FWD>(op, pp, b->grid, st);
+    else if (b->halo && b->persist && b->p.mode == MODE_DGRAD) e = launch_halo_persist_mode<MODE_DGRAD>(op, pp, b->grid, st);
     else if (b->halo && b->p.mode == MODE_FWD) e = launch_halo_mode<MODE_FWD>(b->bn, op, pp, b->grid, st);
     else if (b->halo && b->p.mode == MODE_DGRAD) e = launch_halo_mode<MODE_DGRAD>(b->bn, op, pp, b->grid, st);
     else if (b->pair && b->p.mode == MODE_FWD) e = launch_pair_mode<MODE_FWD>(b->bn, op, pp, b->grid, st);
@@ -2636,7 +2648,7 @@ cudaError_t launch_wait_probe(uint32_t* status, unsigned long long limit_ns, cud
 //    reduced in split order by splitk_epilogue) while every CTA keeps at least 4 k-iterations,
 //  * ring depth = k-iterations per CTA, capped by what fits; for grids of several waves the ring is kept
 //    shallow enough that two CTAs share an SM, so one CTA's epilogue overlaps the other's main loop.
-struct TilePlan { int bn, splits, cps, stages, pair, halo, a_stages, persist, persist_ctas, out_slots; double cost; };
+struct TilePlan { int bn, splits, cps, stages, pair, halo, a_stages, persist, persist_ctas, out_slots, w_resident; double cost; };
 // Backward kernels of the two concurrent streams share SMs only if two CTAs fit side by side (shared
 // memory <= ~110 KB each, TMEM columns <= 256 each): SB_BWD_COHABIT=0 gives every kernel the full ring again.
 static bool bwd_cohabit()
@@ -2824,48 +2836,36 @@ static TilePlan plan_tiles_halo(int n_cols, long m_tiles, int kchunks, int a_slo
     return t;
 }
 
-// Plan of the persistent halo kernel (layers of several tiles per SM, unsplit): 128-wide tiles where the layer has the
-// columns (one CTA per SM with the deepest rings), 64-wide ones otherwise (two CTAs per SM with two-group rings).
+// Plan of the persistent halo kernel (64 columns per tile, one CTA per SM, unsplit): resident weights up to 64 input channels, else a ring of
+// two groups of weight tiles or more for each of the two pipelines; as many activation boxes as fit.
 static TilePlan plan_tiles_halo_persist(int n_cols, long m_tiles, int kchunks, int a_slot_bytes)
 {
     TilePlan t{};
     t.halo = 1;
     t.persist = 1;
-    static const int f_bn = (int)tune("SB_PERSIST_BN", 0);
-    t.bn = f_bn > 0 ? f_bn : (n_cols >= 128 ? 128 : 64);
+    t.bn = 64;
     t.splits = 1;
     t.cps = 3 * kchunks;
-    const int b_stage = t.bn * 128, stage_out = (t.bn / 64) * 16384;
-    int per_sm = 1, sa = 2, sb = 6;
-    if (2 * (2 * a_slot_bytes + 6 * b_stage + stage_out + 4 * 1024) <= 227 * 1024 && 2 * 2 * t.bn <= 512) {
-        per_sm = 2;
-        sb = ((227 * 1024 / 2) - 4 * 1024 - stage_out - 2 * a_slot_bytes) / b_stage;
-    } else {
-        sa = 3;
-        sb = (227 * 1024 - 4 * 1024 - stage_out - 3 * a_slot_bytes) / b_stage;
-        if (sb < 6) { sa = 2; sb = (227 * 1024 - 4 * 1024 - stage_out - 2 * a_slot_bytes) / b_stage; }
-    }
-    if (sb > MAX_STAGES) sb = MAX_STAGES;
-    if (sb < 3) sb = 3;
-    {
-        static const int f_sa = (int)tune("SB_PERSIST_SA", 0), f_sb = (int)tune("SB_PERSIST_SB", 0), f_per = (int)tune("SB_PERSIST_PER_SM", 0);
-        if (f_sa > 0) sa = f_sa;
-        if (f_sb > 0) sb = f_sb;
-        if (f_per > 0) per_sm = f_per;
-    }
+    t.w_resident = n_cols <= 64 && kchunks == 1;
+    int sa = 1, sb = t.w_resident ? 9 : 6;
+    const int room = 227 * 1024;
+    auto need = [&]() { return HaloPersistCfg::smem_bytes(sa, a_slot_bytes, sb, t.w_resident != 0); };
+    while (!t.w_resident && need() > room) --sb;
+    for (int more = 2; more <= HaloPersistCfg::MAX_A; ++more) { sa = more; if (need() > room) { --sa; break; } }
+    for (int more = sb + 1; more <= HaloPersistCfg::MAX_B && !t.w_resident; ++more) { sb = more; if (need() > room) { --sb; break; } }
     t.a_stages = sa;
     t.stages = sb;
     const long tiles = m_tiles * cdiv_i(n_cols, t.bn);
-    const long slots = 148L * per_sm;
-    t.persist_ctas = (int)(tiles < slots ? tiles : slots);
+    t.persist_ctas = (int)(tiles < 148 ? tiles : 148);
     static const bool verbose = tune("SB_PLAN_VERBOSE", 0) != 0;
-    if (verbose) fprintf(stderr, "plan: halo persistent N=%d m_tiles=%ld kchunks=%d -> bn=%d a_stages=%d b_stages=%d ctas=%d (%ld tiles)\n", n_cols, m_tiles, kchunks, t.bn, t.a_stages, t.stages, t.persist_ctas, tiles);
+    if (verbose) fprintf(stderr, "plan: halo persistent N=%d m_tiles=%ld kchunks=%d -> a_stages=%d b_stages=%d resident=%d ctas=%d (%ld tiles)\n", n_cols, m_tiles, kchunks, t.a_stages, t.stages, t.w_resident, t.persist_ctas, tiles);
     return t;
 }
 
 // Plan of the halo kernel on CTA pairs for one pixel box: N tile, ring depths, and the estimate (cycles) by which conv_geom chooses the
-// box.  A group of three taps costs its arithmetic (a 256 x N MMA takes N / 2 cycles) or what it moves through an SM's shared memory (the
-// TMA writes and the MMAs' reads, 128 bytes per cycle), whichever is longer; 74 pairs walk the tiles.
+// box.  A group of three taps costs its arithmetic (a 256 x N MMA takes N / 2 cycles), what it moves through an SM's shared memory (the
+// TMA writes and the MMAs' reads, 128 bytes per cycle) or its operands from L2 (32 bytes per cycle and SM with all of them fetching),
+// whichever is longest; 74 pairs walk the tiles.
 static bool plan_tiles_halo_pair(int n_cols, long m_tiles, int kchunks, int a_slot_bytes, TilePlan* out)
 {
     bool found = false;
@@ -2874,20 +2874,24 @@ static bool plan_tiles_halo_pair(int n_cols, long m_tiles, int kchunks, int a_sl
         TilePlan t{};
         t.halo = 1; t.pair = 1; t.persist = 1; t.bn = bn; t.splits = 1; t.cps = 3 * kchunks;
         const int b_half = bn * 64, room = 227 * 1024 - 1024 - CTRL_BYTES;
-        // rings: two groups of weight tiles and two activation boxes at least; then a second staging buffer, a third and fourth box, more weights
+        // rings: two groups of weight tiles and two activation boxes at least; for short groups (128 columns) up to four boxes and twelve
+        // weight tiles first: a group's boxes are under way for about 2400 cycles where its MMAs take 768 (128 -> 128 channels at 112x112, batch 64,
+        // forward: 237 us with two staging buffers and three boxes, 197 with one and four)
         int sa = 2, sb = 6, so = 1;
         auto need = [&]() { return sa * a_slot_bytes + sb * b_half + so * bn * 256; };
         if (need() > room) continue;
-        so = 2; if (need() > room) so = 1;
-        sa = 3; if (need() > room) sa = 2;
-        sb = MAX_STAGES; while (need() > room) --sb;
-        if (sa == 3) { sa = 4; if (need() > room) sa = 3; }
-        if (sa > MAX_A_STAGES) sa = MAX_A_STAGES;
+        // all weights resident (one N tile, 64 input channels): they cross L2 once per CTA instead of once per tile
+        t.w_resident = n_cols <= bn && kchunks == 1;
+        if (t.w_resident) { sb = 9; so = 2; if (need() > room) so = 1; }
+        for (int more = 3; more <= 4; ++more) { sa = more; if (need() > room) { --sa; break; } }
+        for (int more = sb + 1; more <= 12 && !t.w_resident; ++more) { sb = more; if (need() > room) { --sb; break; } }
         t.a_stages = sa; t.stages = sb; t.out_slots = so;
         const long units = (m_tiles + 1) / 2 * cdiv_i(n_cols, bn);
         t.persist_ctas = 2 * (int)(units < 74 ? units : 74);
-        const double math = 12.0 * bn / 2, port = (a_slot_bytes + 3.0 * b_half) / 128 + 12.0 * (32 + bn / 8);
-        const double unit = 3 * kchunks * (1.1 * (math > port ? math : port) + 60.0), epi = bn * 16.0;
+        const double bytes = a_slot_bytes + (t.w_resident ? 0.0 : 3.0 * b_half);
+        const double math = 12.0 * bn / 2, port = bytes / 128 + 12.0 * (32 + bn / 8), l2 = bytes / 32;
+        const double group = math > port ? (math > l2 ? math : l2) : (port > l2 ? port : l2);
+        const double unit = 3 * kchunks * (1.1 * group + 60.0), epi = bn * 16.0;
         t.cost = (double)cdiv_i(units, 74) * (unit > epi ? unit : epi) + epi + 3000.0;
         if (!found || t.cost < out->cost) { *out = t; found = true; }
     }
@@ -2970,46 +2974,33 @@ static ConvGeom conv_geom(const LayerView& lv, int B, bool force_pair, bool no_h
     static const long halo_max_tiles = (long)tune("SB_HALO_MAX_TILES", 160);
     int hbw = 0, hbh = 0, hbn = 0;
     bool halo = halo_on && !force_pair && !no_halo && choose_box_halo(lv.W, lv.H, B, &hbw, &hbh, &hbn);
-    static const bool persist_on = tune("SB_HALO_PERSIST", 1) != 0;
-    static const long persist_max_width = (long)tune("SB_PERSIST_MAX_WIDTH", 128);
-    bool persist = false;
+    bool persist = false, hpair = false;
     if (halo) {
         const long mt = (long)cdiv_i(lv.W, hbw) * cdiv_i(lv.H, hbh) * cdiv_i(B, hbn);
         const int widest = lv.Cout < lv.Cin ? lv.Cout : lv.Cin;
         const long tiles = mt * cdiv_i(widest, widest >= 128 ? 128 : 64);
         if (tiles > halo_max_tiles || force_persist) {
-            // Three or more tiles per SM: the persistent variant (layers up to 128 channels wide; wider ones do better on the
-            // per-tap kernel's CTA pairs with 256-column tiles).  Measured at CIFAR size, batch 128: the 1024-tile layer
-            // 20.3 -> 16.3 us, the 256-tile layers 7.3 -> 9.0 and 12.8 -> 13.5 us (one or two tiles per CTA do not repay the
-            // second accumulator's set-up); ImageNet-size step -3.6 %, batch 256 -2 %, its 512-tile layers a further -1.5 %.
+            // Layers of up to 64 channels and three or more tiles per SM: the persistent kernel (one or two tiles per CTA do not repay its
+            // set-up: measured at CIFAR size, batch 128, 7.3 -> 9.0 and 12.8 -> 13.5 us).
             static const long persist_min_tiles = (long)tune("SB_PERSIST_MIN_TILES", 3 * 148);
-            persist = persist_on && (tiles >= persist_min_tiles || force_persist) && lv.Cout <= persist_max_width && lv.Cin <= persist_max_width;
+            persist = (tiles >= persist_min_tiles || force_persist) && lv.Cout <= 64 && lv.Cin <= 64;
             if (!persist) halo = false;
-        }
-    }
-    // CTA pairs on halos: layers of more than one 128-column tile per SM with more than 64 columns in at least one direction.  The pixel
-    // box with the cheapest plans for the directions that take it.
-    bool hpair = false;
-    if (halo_on && !force_pair && !no_halo && (lv.Cout > 64 || lv.Cin > 64)) {
-        static const long hp_min_tiles = (long)tune("SB_HALO_PAIR_MIN_TILES", 160);
-        const int widest = lv.Cout < lv.Cin ? lv.Cout : lv.Cin;
-        double best = 1e300;
-        for (int w = 1; w <= 128; w *= 2)
-            for (int h = 2; w * h <= 128; h *= 2) {
-                const int n = 128 / (w * h);
-                if ((w * n) % 8 != 0) continue;
-                const long mt = (long)cdiv_i(lv.W, w) * cdiv_i(lv.H, h) * cdiv_i(B, n);
-                const int a_slot = (h + 2) * w * n * 128;
-                if (!force_persist && (double)lv.W * lv.H * B / 128 * cdiv_i(widest, widest >= 128 ? 128 : 64) <= hp_min_tiles) continue;
-                TilePlan f{}, d{};
-                if (lv.Cout > 64 && !plan_tiles_halo_pair(lv.Cout, mt, cdiv_i(lv.Cin, 64), a_slot, &f)) continue;
-                if (lv.Cin > 64 && !plan_tiles_halo_pair(lv.Cin, mt, cdiv_i(lv.Cout, 64), a_slot, &d)) continue;
-                const double c = f.cost + d.cost - 1e-3 * w;
-                if (c < best) {
-                    best = c;
-                    hpair = true; hbw = w; hbh = h; hbn = n;
+            // More than 64 channels in at least one direction: CTA pairs on halos there, with the pixel box whose plans are the cheapest.
+            static const long hp_min_tiles = (long)tune("SB_HALO_PAIR_MIN_TILES", 160);
+            double best = 1e300;
+            for (int w = 1; w <= 128 && (lv.Cout > 64 || lv.Cin > 64) && (tiles > hp_min_tiles || force_persist); w *= 2)
+                for (int h = 2; w * h <= 128; h *= 2) {
+                    const int n = 128 / (w * h);
+                    if ((w * n) % 8 != 0) continue;
+                    const long m = (long)cdiv_i(lv.W, w) * cdiv_i(lv.H, h) * cdiv_i(B, n);
+                    const int a_slot = (h + 2) * w * n * 128;
+                    TilePlan f{}, d{};
+                    if (lv.Cout > 64 && !plan_tiles_halo_pair(lv.Cout, m, cdiv_i(lv.Cin, 64), a_slot, &f)) continue;
+                    if (lv.Cin > 64 && !plan_tiles_halo_pair(lv.Cin, m, cdiv_i(lv.Cout, 64), a_slot, &d)) continue;
+                    const double c = f.cost + d.cost - 1e-3 * w;
+                    if (c < best) { best = c; hpair = true; hbw = w; hbh = h; hbn = n; }
                 }
-            }
+        }
     }
     if (hpair) {
         halo = true;
@@ -3127,6 +3118,7 @@ static void apply_plan(OpBlock* b, const TilePlan& t, int k_iters, long m_tiles,
     p.stages = t.stages;
     p.a_stages = t.a_stages;
     p.out_slots = t.out_slots;
+    p.w_resident = t.w_resident;
     p.hn_order = t.halo;
     b->halo = t.halo;
     b->persist = t.persist;
