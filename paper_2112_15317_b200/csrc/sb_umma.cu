@@ -2985,8 +2985,10 @@ static ConvGeom conv_geom(const LayerView& lv, int B, bool force_pair, bool no_h
             static const long persist_min_tiles = (long)tune("SB_PERSIST_MIN_TILES", 3 * 148);
             persist = (tiles >= persist_min_tiles || force_persist) && lv.Cout <= 64 && lv.Cin <= 64;
             if (!persist) halo = false;
-            // More than 64 channels in at least one direction: CTA pairs on halos there, with the pixel box whose plans are the cheapest.
-            static const long hp_min_tiles = (long)tune("SB_HALO_PAIR_MIN_TILES", 160);
+            // More than 64 channels in at least one direction and more than two tiles per SM: CTA pairs on halos there, with the pixel box
+            // whose plans are the cheapest.  (From one tile per SM up: CIFAR shape, batch 128, 536 -> 543 us -- the pairs' whole-SM rings keep
+            // the weight-gradient kernels out, and one tile per SM has no next tile to overlap; batch 256 +-0.)
+            static const long hp_min_tiles = (long)tune("SB_HALO_PAIR_MIN_TILES", 2 * 148);
             double best = 1e300;
             for (int w = 1; w <= 128 && (lv.Cout > 64 || lv.Cin > 64) && (tiles > hp_min_tiles || force_persist); w *= 2)
                 for (int h = 2; w * h <= 128; h *= 2) {
