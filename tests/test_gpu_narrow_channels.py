@@ -18,7 +18,7 @@ pytestmark = pytest.mark.gpu
     (32, 32, (48, 96), 9, 3),            # many tiles
     (4, 4, (16, 272), 17, 1),            # more than one 256-wide tile
 ])
-@pytest.mark.parametrize("flags", [0, 32])     # default / no halo kernel
+@pytest.mark.parametrize("flags", [0, 32, 64])     # default / no halo kernel / persistent kernels, several tiles per CTA
 def test_channel_counts_off_the_tiles(H, W, chans, b, R, flags):
     from paper_2112_15317_b200 import binding as sb
     layers = [(si.CONV3X3_RELU, c) for c in chans] + [(si.MAXPOOL2, 0), (si.FC_RELU, 40), (si.FC, 10), (si.SOFTMAX_XENT, 10)]
