@@ -2522,6 +2522,7 @@ struct OpBlock {
     int pair;      // FWD / DGRAD: run as CTA pairs (umma_pair_kernel); grid.x is then even
     int halo;      // 3x3 FWD / DGRAD: umma_halo_kernel (activation halos shared by the three taps of a filter column)
     int persist;   // ... its persistent variant: grid.x CTAs walk all tiles (umma_halo_persist_kernel)
+    int wg64;      // conv WGRAD: launch_conv64_wgrad
     int upd_maps;  // FC WGRAD: mapC / mapD are float maps over the layer's master weights and momentum
     dim3 grid;
     long rows;     // output rows (pixels / batch rows) of a FWD / DGRAD op
@@ -2598,6 +2599,11 @@ static sb_status launch_op(const UmmaOp& op, cudaStream_t st, int64_t* launches 
     else if (b->pair && b->p.mode == MODE_WGRAD) e = launch_pair_mode<MODE_WGRAD>(b->bn, op, pp, b->grid, st);
     else if (b->p.mode == MODE_FWD) e = launch_mode<MODE_FWD>(b->bn, op, pp, b->grid, st);
     else if (b->p.mode == MODE_DGRAD) e = launch_mode<MODE_DGRAD>(b->bn, op, pp, b->grid, st);
+    else if (b->wg64) {
+        const Conv64WgradArgs a{&op.mapA, &op.mapB, pp.bw, pp.bh, pp.bn, pp.tiles_w, pp.tiles_h, pp.total_chunks, pp.chunks_per_split, pp.w_cols, pp.m_total,
+                                (float*)pp.out, pp.split_stride, pp.bias_off, pp.status};
+        e = launch_conv64_wgrad(a, st);
+    }
     else e = launch_mode<MODE_WGRAD>(b->bn, op, pp, b->grid, st);
     if (e == cudaSuccess && b->p.mode != MODE_WGRAD && b->p.splits > 1) {
         // ordered sum of the split partial sums + the epilogue the tensor-core kernel skipped
@@ -2962,6 +2968,7 @@ struct ConvGeom {
     TilePlan fwd, dgrad;
     int cw, ch, cn, ctw, cth, ctn, total_chunks;   // 64-pixel boxes (WGRAD k-chunks)
     int wg_bn, wg_n_tiles, wg_m_tiles, wg_splits, wg_cps, wg_tap_group;
+    int wg64;                        // all nine taps in one CTA (launch_conv64_wgrad)
 };
 static ConvGeom conv_geom(const LayerView& lv, int B, bool force_pair, bool no_halo, bool force_persist)
 {
@@ -3051,6 +3058,37 @@ static ConvGeom conv_geom(const LayerView& lv, int B, bool force_pair, bool no_h
     // faster but the step is not (its 96 KB ring and 256 TMEM columns leave the data-gradient kernel less room beside it).
     static const int taps2_min_chunks = (int)tune("SB_WGRAD_TAPS2_MIN_CHUNKS", 2048);
     if (lv.Cin == 128 && lv.Cout <= 128 && !taps1 && g.total_chunks >= taps2_min_chunks) { g.wg_tap_group = 2; g.wg_bn = 256; g.wg_n_tiles = 1; }
+    // At most 64 channels on either side: all nine taps in one CTA, where the reduction is long enough for the partial gradients of its CTAs.
+    g.wg64 = 0;
+    static const int wg64_min_chunks = (int)tune("SB_WG64_MIN_CHUNKS", 8192);
+    if (lv.Cin <= 64 && lv.Cout <= 64 && !no_halo && !force_pair) {
+        int w64 = 0, h64 = 0, n64 = 0;
+        double best = 1e300;
+        for (int w = 1; w <= 64; w *= 2)
+            for (int h = 1; w * h <= 64; h *= 2) {
+                const int n = 64 / (w * h);
+                if ((w * n) % 8 != 0 || conv64_wgrad_stages(w, h, n) < 2) continue;
+                // (padded volume, weighted by the row of halo that a box fetches)
+                const double score = (double)cdiv_i(lv.W, w) * w * cdiv_i(lv.H, h) * h * cdiv_i(B, n) * n * (1.0 + 1.0 / h) * (1.0 - 1e-6 * w);
+                if (score < best) { best = score; w64 = w; h64 = h; n64 = n; }
+            }
+        const int chunks = w64 == 0 ? 0 : cdiv_i(lv.W, w64) * cdiv_i(lv.H, h64) * cdiv_i(B, n64);
+        if (chunks >= wg64_min_chunks || (force_persist && chunks > 0)) {
+            g.wg64 = 1;
+            g.cw = w64; g.ch = h64; g.cn = n64;
+            g.ctw = cdiv_i(lv.W, g.cw); g.cth = cdiv_i(lv.H, g.ch); g.ctn = cdiv_i(B, g.cn);
+            g.total_chunks = chunks;
+            // a CTA costs about 0.6 us per chunk and 6 us once; its partial gradient is written and read back at 3 TB/s
+            const double copy_us = ((double)lv.n_w + lv.n_b) * 4.0 / 3.0e6;
+            double best_us = 1e300;
+            for (int s = 1; s <= 148 && s <= chunks; ++s) {
+                const int cps = cdiv_i(chunks, s), real_s = cdiv_i(chunks, cps);
+                const double us = cps * 0.6 + (real_s > 1 ? 3.0 + (real_s + 1) * copy_us : 0.0);
+                if (us < best_us) { best_us = us; g.wg_cps = cps; g.wg_splits = real_s; }
+            }
+            return g;
+        }
+    }
     const int tap_groups = (9 + g.wg_tap_group - 1) / g.wg_tap_group;
     double cost = 0.0;
     int s = wgrad_splits((long)g.wg_m_tiles * g.wg_n_tiles * tap_groups, g.total_chunks, g.wg_bn, (size_t)lv.n_w + lv.n_b, &cost);
@@ -3283,13 +3321,17 @@ sb_status umma_plan_layers(sb_model* m, int first_layer)
                 }
                 p.out = p.splits > 1 ? (void*)mv.ws_wk[mv.n_wstreams > 0 ? i % mv.n_wstreams : 0] : (void*)(mv.Gm + lv.p_w);
                 p.status = mv.status;
+                b->wg64 = g.wg64 && (p.split_stride & 3) == 0 && (((uintptr_t)p.out) & 15) == 0;
                 b->grid = dim3((unsigned)g.wg_m_tiles, (unsigned)g.wg_n_tiles, (unsigned)((9 + p.tap_group - 1) / p.tap_group * p.splits));
                 if ((size_t)p.splits * (lv.n_w + lv.n_b) > mv.ws_floats && p.splits > 1) return SB_ERR_ARENA_TOO_SMALL;
                 // 64 input channels: one filter COLUMN per CTA instead of one filter row -- the three taps then share one
                 // activation box with a halo row above and below (the three N panels of the MMA are windows into it) instead
                 // of three boxes shifted in w.  Needs whole 8-row swizzle groups per image row of the box and the sweep epilogue.
                 static const bool col_on = tune("SB_WG_COLUMN", 1) != 0;
-                if (col_on && p.tap_group == 3 && !b->pair && (g.cw * g.cn) % 8 == 0 && (p.split_stride & 3) == 0 && (((uintptr_t)p.out) & 15) == 0 &&
+                if (b->wg64) {
+                    if (!act_map_hn(&um.wgrad.mapA, lv.dact, B, lv.H, lv.W, lv.Cout, g.cw, g.ch + 1, g.cn)) return fail_plan();
+                    if (!act_map_hn(&um.wgrad.mapB, lv.in_act, B, lv.H, lv.W, lv.Cin, g.cw, g.ch + 1, g.cn)) return fail_plan();
+                } else if (col_on && p.tap_group == 3 && !b->pair && (g.cw * g.cn) % 8 == 0 && (p.split_stride & 3) == 0 && (((uintptr_t)p.out) & 15) == 0 &&
                     !(mv.cfg->flags & SB_FLAG_NO_HALO)) {
                     p.hn_order = 1;
                     if (!act_map_hn(&um.wgrad.mapA, lv.dact, B, lv.H, lv.W, lv.Cout, g.cw, g.ch, g.cn)) return fail_plan();

@@ -91,6 +91,19 @@ int conv_in_umma_wgrad_blocks(int B, int H, int W, int Cin);
 cudaError_t launch_conv_in_fwd_umma(const ConvSimtArgs& a, const CUtensorMap& mapY, uint32_t* status, cudaStream_t st);
 cudaError_t launch_conv_in_wgrad_umma(const WgradSimtArgs& a, const CUtensorMap& mapDy, uint32_t* status, cudaStream_t st);
 
+// Weight gradient of a 3x3 layer with at most 64 channels on either side (sb_conv64_wgrad.cu).  The maps list the dimensions as
+// (c, w, n, h) with boxes of (64, bw, bn, bh + 1); the box of a chunk holds 64 pixels, bw * bn a multiple of 8.
+struct Conv64WgradArgs {
+    const CUtensorMap *mapDy, *mapX;
+    int bw, bh, bn, tiles_w, tiles_h, total_chunks, chunks_per_cta;
+    int Cin, Cout;
+    float* out;                      // one partial gradient per CTA, split_stride floats apart; 16-byte aligned, as is split_stride
+    long split_stride, bias_off;
+    uint32_t* status;
+};
+int conv64_wgrad_stages(int bw, int bh, int bn);      // ring depth that fits (at least 2 for the kernel to run)
+cudaError_t launch_conv64_wgrad(const Conv64WgradArgs& a, cudaStream_t st);
+
 const char* umma_last_error();
 // One CTA that waits (bounded by limit_ns) on a barrier nothing completes, then reports through the status word.
 cudaError_t launch_wait_probe(uint32_t* status, unsigned long long limit_ns, cudaStream_t st);
