@@ -2523,6 +2523,7 @@ struct OpBlock {
     int halo;      // 3x3 FWD / DGRAD: umma_halo_kernel (activation halos shared by the three taps of a filter column)
     int persist;   // ... its persistent variant: grid.x CTAs walk all tiles (umma_halo_persist_kernel)
     int wg64;      // conv WGRAD: launch_conv64_wgrad
+    int fc_persist;// FC WGRAD without the folded update: launch_fc_wgrad
     int upd_maps;  // FC WGRAD: mapC / mapD are float maps over the layer's master weights and momentum
     dim3 grid;
     long rows;     // output rows (pixels / batch rows) of a FWD / DGRAD op
@@ -2603,6 +2604,10 @@ static sb_status launch_op(const UmmaOp& op, cudaStream_t st, int64_t* launches 
         const Conv64WgradArgs a{&op.mapA, &op.mapB, pp.bw, pp.bh, pp.bn, pp.tiles_w, pp.tiles_h, pp.total_chunks, pp.chunks_per_split, pp.w_cols, pp.m_total,
                                 (float*)pp.out, pp.split_stride, pp.bias_off, pp.status};
         e = launch_conv64_wgrad(a, st);
+    }
+    else if (b->fc_persist && !fuse) {
+        const FcWgradArgs a{&op.mapA, &op.mapB, pp.N, pp.m_total, pp.n_total, (float*)pp.out, (float*)pp.out + pp.bias_off, pp.status};
+        e = launch_fc_wgrad(a, st);
     }
     else e = launch_mode<MODE_WGRAD>(b->bn, op, pp, b->grid, st);
     if (e == cudaSuccess && b->p.mode != MODE_WGRAD && b->p.splits > 1) {
@@ -3413,6 +3418,9 @@ sb_status umma_plan_layers(sb_model* m, int first_layer)
                 p.out = (void*)(mv.Gm + lv.p_w);
                 p.status = mv.status;
                 b->grid = dim3((unsigned)cdiv_i(lv.out_f, 128), (unsigned)n_tiles, 1);
+                // three or more tiles per SM: one CTA per SM walks them
+                static const long fc_min_tiles = (long)tune("SB_FC_WGRAD_MIN_TILES", 3 * 148);
+                b->fc_persist = b->bn == 256 && (long)b->grid.x * n_tiles >= fc_min_tiles && wgrad_sweep_ok(b);
                 if (!act_map(&um.wgrad.mapA, lv.dact, B, 1, 1, lv.out_f, 1, 1, 64)) return fail_plan();
                 if (!act_map(&um.wgrad.mapB, lv.in_act, B, 1, 1, lv.in_f, 1, 1, 64)) return fail_plan();
                 // float maps over the master weights and the momentum buffer, for the weight gradient with the update folded in

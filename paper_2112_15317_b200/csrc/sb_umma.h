@@ -104,6 +104,15 @@ struct Conv64WgradArgs {
 int conv64_wgrad_stages(int bw, int bh, int bn);      // ring depth that fits (at least 2 for the kernel to run)
 cudaError_t launch_conv64_wgrad(const Conv64WgradArgs& a, cudaStream_t st);
 
+// Stored weight gradient of a large FC layer (sb_fc_wgrad.cu); maps with boxes of 64 columns x 64 batch rows.
+struct FcWgradArgs {
+    const CUtensorMap *mapDy, *mapX;
+    int batch, out_f, in_f;
+    float *out, *bias;               // 16-byte aligned, in_f a multiple of 4
+    uint32_t* status;
+};
+cudaError_t launch_fc_wgrad(const FcWgradArgs& a, cudaStream_t st);
+
 const char* umma_last_error();
 // One CTA that waits (bounded by limit_ns) on a barrier nothing completes, then reports through the status word.
 cudaError_t launch_wait_probe(uint32_t* status, unsigned long long limit_ns, cudaStream_t st);
