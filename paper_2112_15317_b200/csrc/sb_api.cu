@@ -232,6 +232,8 @@ size_t contract_plan_layer(sb_model* m, int i, size_t max_part_floats)
     size_t need = 0;
     if (!has_weights(l) || l.narrow || umma_layer_ok(m, i)) return 0;
     for (int mode : {CMODE_FWD, CMODE_DGRAD, CMODE_WGRAD}) {
+        // (passes that run on the input-layer kernels, or not at all, take no scratch)
+        if (mode == CMODE_DGRAD ? i == 0 && !(m->cfg.flags & SB_FLAG_INPUT_GRAD) : l.thin_input) continue;
         const ContractArgs a = contract_args(m, i, mode);
         l.cplan[mode] = contract_plan(mode, a.B, a.H, a.W, a.taps, a.Cin, a.Cout, max_part_floats);
         const size_t result = mode == CMODE_WGRAD ? l.n_w + l.n_b : (size_t)a.B * a.H * a.W * (mode == CMODE_FWD ? a.Cout : a.Cin);
