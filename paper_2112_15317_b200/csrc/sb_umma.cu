@@ -22,9 +22,11 @@
 // normally (TMEM is always released), so a broken pipeline turns into SB_ERR_TIMEOUT on the
 // host instead of a stuck GPU.
 //
-// Large forward / data-gradient grids with 256-wide N tiles, and the weight gradients of layers with
+// Forward / data-gradient grids with 256-wide N tiles, and the weight gradients of layers with
 // 256+ output channels, run on CTA pairs (umma_pair_kernel, tcgen05.mma.cta_group::2): two
-// neighbouring M tiles share one fetch of the other operand, half of it per CTA.
+// neighbouring M tiles share one fetch of the other operand, half of it per CTA.  3x3 layers of about one tile per SM
+// run on umma_halo_kernel (an activation fetch per filter column), those of many tiles on persistent forms of it:
+// umma_halo_persist_kernel (up to 64 columns) and umma_halo_pair_kernel (CTA pairs).
 // No load uses multicast; the only multicast is the pair kernel's tcgen05.commit, which releases a
 // ring slot in both CTAs of the pair.
 //
@@ -1740,9 +1742,9 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
     const int m_idx = blockIdx.x, n_idx = blockIdx.y;
     int split = blockIdx.z, tap_fixed = 0, n0, n_hi, m0 = 0, m_hi = 0;
     if (MODE == MODE_WGRAD) {
-        tap_fixed = blockIdx.z / p.splits;
+        tap_fixed = blockIdx.z / p.splits * p.tap_group;
         split = blockIdx.z % p.splits;
-        n0 = n_idx * BN; n_hi = p.n_total;
+        n0 = n_idx * BN; n_hi = p.tap_group == 2 ? min(p.n_total, (9 - tap_fixed) * p.w_cols) : p.n_total;     // (the last pair of taps has one member)
         m0 = m_idx * 128; m_hi = p.m_total;
     } else {
         n0 = n_idx * BN;
@@ -1767,8 +1769,10 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
             ld_a = k_begin % p.kchunks; ld_b = k_begin / p.kchunks;
         }
     }
-    const int wg_dr = tap_fixed / 3 - 1, wg_ds = tap_fixed % 3 - 1;
-    const int nb0 = n0 + (int)rank * (BN / 2);                     // first B column this CTA fetches
+    // two taps (tap_group 2, 128 input channels): each CTA's half of B is one of them (past the last tap: any, its columns are not stored)
+    const int tap_b = p.tap_group == 2 ? min(tap_fixed + (int)rank, 8) : tap_fixed;
+    const int wg_dr = tap_b / 3 - 1, wg_ds = tap_b % 3 - 1;
+    const int nb0 = MODE == MODE_WGRAD && p.tap_group == 2 ? 0 : n0 + (int)rank * (BN / 2);      // first B column this CTA fetches
     const uint32_t full0_leader = map_to_cta(smem_u32(&full[0]), 0);
     // (whole producer warp in lock-step, elected issue: see the single-CTA kernel)
     int ld_s = 0;
@@ -3062,7 +3066,8 @@ static ConvGeom conv_geom(const LayerView& lv, int B, bool force_pair, bool no_h
     // Taken for long reductions only (ImageNet-size layers: 613 -> 290 us alone); at CIFAR size the kernel alone is 15 %
     // faster but the step is not (its 96 KB ring and 256 TMEM columns leave the data-gradient kernel less room beside it).
     static const int taps2_min_chunks = (int)tune("SB_WGRAD_TAPS2_MIN_CHUNKS", 2048);
-    if (lv.Cin == 128 && lv.Cout <= 128 && !taps1 && g.total_chunks >= taps2_min_chunks) { g.wg_tap_group = 2; g.wg_bn = 256; g.wg_n_tiles = 1; }
+    // On CTA pairs (256 output channels or more) each CTA fetches one of the two taps: 32 KB for twice the arithmetic of 24.
+    if (lv.Cin == 128 && (lv.Cout <= 128 || lv.Cout % 256 == 0) && !taps1 && (g.total_chunks >= taps2_min_chunks || (force_pair && lv.Cout > 128))) { g.wg_tap_group = 2; g.wg_bn = 256; g.wg_n_tiles = 1; }
     // At most 64 channels on either side: all nine taps in one CTA, where the reduction is long enough for the partial gradients of its CTAs.
     g.wg64 = 0;
     static const int wg64_min_chunks = (int)tune("SB_WG64_MIN_CHUNKS", 8192);
@@ -3314,7 +3319,7 @@ sb_status umma_plan_layers(sb_model* m, int first_layer)
                     // from 160 up batch 256 +0.7 %; never at ImageNet shape +1.2 %.  512 x 512 channels, whose tiles fill the machine unsplit, from 160
                     // chunks up: 107 -> 85 us alone at 14x14, batch 64)
                     static const int wg_pair_min_chunks = (int)tune("SB_WG_PAIR_MIN_CHUNKS", 320);
-                    if (wg_pair && (g.total_chunks >= (lv.Cout >= 512 && lv.Cin >= 512 ? wg_pair_min_chunks / 2 : wg_pair_min_chunks) || (mv.cfg->flags & SB_FLAG_FORCE_PAIR)) && p.tap_group == 1 && (b->bn == 128 || b->bn == 256) && g.wg_m_tiles % 2 == 0 && lv.Cout % 128 == 0) {
+                    if (wg_pair && (g.total_chunks >= (lv.Cout >= 512 && lv.Cin >= 512 ? wg_pair_min_chunks / 2 : wg_pair_min_chunks) || (mv.cfg->flags & SB_FLAG_FORCE_PAIR)) && (p.tap_group == 1 || p.tap_group == 2) && (b->bn == 128 || b->bn == 256) && g.wg_m_tiles % 2 == 0 && lv.Cout % 128 == 0) {
                         b->pair = 1;
                         p.bias_fused = 0;
                         const int pfit = b->bn >= 256 ? 6 : 8, ptwo = b->bn >= 256 ? 3 : 4;

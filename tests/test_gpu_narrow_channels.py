@@ -17,8 +17,9 @@ pytestmark = pytest.mark.gpu
     (16, 16, (64, 80, 144), 3, 1),       # a second, partly filled reduction chunk and column tile
     (32, 32, (48, 96), 9, 3),            # many tiles
     (4, 4, (16, 272), 17, 1),            # more than one 256-wide tile
+    (10, 8, (16, 128, 256), 3, 1),       # with pairs forced: two taps per CTA pair of the weight gradient
 ])
-@pytest.mark.parametrize("flags", [0, 32, 64])     # default / no halo kernel / persistent kernels, several tiles per CTA
+@pytest.mark.parametrize("flags", [0, 8, 32, 64])     # default / CTA pairs / no halo kernel / persistent kernels, several tiles per CTA
 def test_channel_counts_off_the_tiles(H, W, chans, b, R, flags):
     from paper_2112_15317_b200 import binding as sb
     layers = [(si.CONV3X3_RELU, c) for c in chans] + [(si.MAXPOOL2, 0), (si.FC_RELU, 40), (si.FC, 10), (si.SOFTMAX_XENT, 10)]
