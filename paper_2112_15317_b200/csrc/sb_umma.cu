@@ -1661,13 +1661,6 @@ __device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t caddr)
     return v;
 }
 // TMA load whose completion may signal a barrier in the peer CTA (`bar_caddr` is a shared::cluster address)
-__device__ __forceinline__ void tma_load_4d_pair(const CUtensorMap* map, void* dst, uint32_t bar_caddr, int c0, int c1, int c2, int c3)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-        ::"r"(smem_u32(dst)), "l"(map), "r"(bar_caddr), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
-        : "memory");
-}
 __device__ __forceinline__ void tma_load_4d_pair_el(const CUtensorMap* map, uint32_t dst_saddr, uint32_t bar_caddr, int c0, int c1, int c2, int c3,
                                                     uint32_t elected)
 {
@@ -1688,15 +1681,6 @@ __device__ __forceinline__ void tmem_relinquish_pair()
 __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols)
 {
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
-__device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
 }
 // arrives (once the MMAs issued so far have completed) on the barrier at this offset in both CTAs of the pair
 __device__ __forceinline__ void umma_commit_pair(uint64_t* bar)
@@ -2799,6 +2783,9 @@ static TilePlan plan_tiles_halo(int n_cols, long m_tiles, int kchunks, int a_slo
     int best_bn = 64, best_s = 1;
     static const double fixed_us = tune("SB_HALO_FIXED_US", 3.0), share_factor = tune("SB_HALO_SHARE", 1.6);
     static const double tap64 = tune("SB_HALO_TAP64", 0.16), tap128 = tune("SB_HALO_TAP128", 0.19), tap256 = tune("SB_HALO_TAP256", 0.33);
+    // (the second kernel of a split reduction: 3.5 us in a forward pass, where it starts under the first one -- one image at 224x224 186 -> 178 us,
+    // the 28x28 layers split two ways -- and 4 on the backward chain, beside the other streams: with 3 there CIFAR shape, batch 128, 537 -> 541 us)
+    const double reduce_us = backward ? 4.0 : 3.5;
     for (int bn = 64; bn <= 256; bn *= 2) {
         if (bn > 64 && bn / 2 >= n_cols) break;
         const double t_tap = bn >= 256 ? tap256 : (bn >= 128 ? tap128 : tap64);
@@ -2807,7 +2794,7 @@ static TilePlan plan_tiles_halo(int n_cols, long m_tiles, int kchunks, int a_slo
             const double per_sm = (bn < 256 && ctas >= 296) ? 2.0 : 1.0;
             const double waves = (double)cdiv_i(ctas, (long)(148 * per_sm));
             const double partial_mb = (double)s * (double)m_tiles * 128.0 * (double)n_cols * 4.0 / 1.0e6;
-            const double c = waves * (cdiv_i(groups, s) * 3.0 * t_tap * (per_sm > 1.0 ? share_factor : 1.0) + fixed_us) + (s > 1 ? 4.0 + 0.5 * partial_mb : 0.0);
+            const double c = waves * (cdiv_i(groups, s) * 3.0 * t_tap * (per_sm > 1.0 ? share_factor : 1.0) + fixed_us) + (s > 1 ? reduce_us + 0.5 * partial_mb : 0.0);
             if (c < best - 1e-9) { best = c; best_bn = bn; best_s = s; }
         }
     }
