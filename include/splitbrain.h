@@ -93,9 +93,9 @@ enum {
     SB_FLAG_NO_HALO = 32,    /* 3x3 forward / data-gradient GEMMs on the kernel that fetches an activation box per filter tap
                                 instead of the default one that shares a fetch of bh + 2 image rows between the three taps of
                                 a filter column (for tests: both kernels must give the same results) */
-    SB_FLAG_FORCE_PERSIST = 64 /* 3x3 forward / data-gradient GEMMs of layers up to 128 channels wide on the persistent kernel
-                                (a few CTAs walk all output tiles, two accumulators in turn), whatever the layer's size; by
-                                default only layers with several tiles per SM use it (for tests at small sizes) */
+    SB_FLAG_FORCE_PERSIST = 64 /* 3x3 forward / data-gradient GEMMs on the persistent kernels (a few CTAs walk all output tiles, accumulators
+                                in turn) and weight gradients of up to 64 channels with all taps in one CTA, whatever the layer's
+                                size; by default only layers of many tiles use them (for tests at small sizes) */
 };
 
 typedef struct {
