@@ -375,7 +375,7 @@ sb_status plan(const sb_layer* layers, int n, const sb_config* cfg, sb_model* m,
     for (int i = 0; i < n; ++i) ws_floats = std::max(ws_floats, contract_plan_layer(m, i, (size_t)16 << 20));
     size_t um_ws = 0;
     sb_status us = umma_plan_scratch(m, &um_ws);
-    if (us != SB_OK) return us;
+    if (us != SB_OK) return fail(us, "%s", umma_last_error());
     if (um_ws > ws_floats) ws_floats = um_ws;
     m->ws_floats = ws_floats;
     m->ws = (float*)take(ws_floats * 4);

@@ -144,12 +144,14 @@ constexpr int A_STAGE_BYTES = 16384;   // 128 rows x 128 B (K-major) or 2 boxes 
 
 constexpr int CTRL_BYTES = 2048;       // [0,512) barriers + flags, [512,1536) bias (FWD), [512,2048) partial bias gradients (WGRAD)
 constexpr int MAX_STAGES = 8;
+constexpr int SMEM_LIMIT = 227 * 1024; // shared memory a CTA can have
 template <int MODE, int BN> struct Cfg {
     static constexpr int B_STAGE_BYTES = BN * 128;
     static constexpr int STAGE_BYTES = A_STAGE_BYTES + B_STAGE_BYTES;
     static constexpr int MAX_STAGES_FIT = (BN >= 256) ? 4 : (BN >= 192 ? 5 : (BN >= 128 ? 6 : 8));   // what fits in 227 KB
     static constexpr int TMEM_COLS = BN == 192 ? 256 : BN;    // allocations are powers of two
     static constexpr int smem_bytes(int stages) { return stages * STAGE_BYTES + 1024 /*alignment slack*/ + CTRL_BYTES; }
+    static constexpr bool fits(int stages) { return stages >= 1 && stages <= MAX_STAGES_FIT && smem_bytes(stages) <= SMEM_LIMIT; }
 };
 
 __device__ __forceinline__ void epi_bar_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }   // the 128 epilogue threads (warps 2..5)
@@ -1036,6 +1038,10 @@ template <int BN> struct HaloCfg {
     {
         return a_stages * a_slot_bytes + b_stages * B_STAGE_BYTES + 1024 /*alignment slack*/ + CTRL_BYTES;
     }
+    static constexpr bool fits(int a_stages, int a_slot_bytes, int b_stages)
+    {
+        return a_stages >= 1 && a_stages <= MAX_A_STAGES && b_stages >= 1 && b_stages <= MAX_STAGES && smem_bytes(a_stages, a_slot_bytes, b_stages) <= SMEM_LIMIT;
+    }
 };
 
 template <int MODE, int BN>
@@ -1351,6 +1357,10 @@ struct HaloPersistCfg {
     static constexpr int smem_bytes(int a_stages, int a_slot_bytes, int b_stages, bool resident)
     {
         return 2 * a_stages * a_slot_bytes + (resident ? 1 : 2) * b_stages * B_STAGE_BYTES + 2 * OUT_BYTES + 1024 /*alignment slack*/ + CTRL_BYTES;
+    }
+    static constexpr bool fits(int a_stages, int a_slot_bytes, int b_stages, bool resident)
+    {
+        return a_stages >= 1 && a_stages <= MAX_A && b_stages >= 3 && b_stages <= MAX_B && smem_bytes(a_stages, a_slot_bytes, b_stages, resident) <= SMEM_LIMIT;
     }
 };
 
@@ -1696,6 +1706,7 @@ template <int BN> struct PairCfg {
     static constexpr int MAX_STAGES_FIT = (BN >= 256) ? 6 : 8;
     static constexpr int TMEM_COLS = BN;
     static constexpr int smem_bytes(int stages) { return stages * STAGE_BYTES + 1024 + CTRL_BYTES; }
+    static constexpr bool fits(int stages) { return stages >= 1 && stages <= MAX_STAGES_FIT && smem_bytes(stages) <= SMEM_LIMIT; }
 };
 
 template <int MODE, int BN>
@@ -1979,6 +1990,11 @@ template <int BN> struct HaloPairCfg {
     {
         const int need = a_stages * a_slot_bytes + b_stages * B_HALF_BYTES + 2 * out_slots * OUT_BYTES + 1024 + CTRL_BYTES;
         return need < MIN_SMEM ? MIN_SMEM : need;
+    }
+    static constexpr bool fits(int a_stages, int a_slot_bytes, int b_stages, int out_slots)
+    {
+        return a_stages >= 1 && a_stages <= MAX_A_STAGES && b_stages >= 3 && b_stages <= MAX_B_SLOTS && out_slots >= 1 && out_slots <= 2 &&
+               smem_bytes(a_stages, a_slot_bytes, b_stages, out_slots) <= SMEM_LIMIT;
     }
 };
 
@@ -2365,14 +2381,14 @@ static cudaError_t launch_one(const UmmaOp& op, const UmmaParams& p, dim3 grid, 
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!attr_set[dev]) {
         e = cudaFuncSetAttribute(umma_kernel<MODE, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 MODE == MODE_WGRAD ? 227 * 1024 : Cfg<MODE, BN>::smem_bytes(Cfg<MODE, BN>::MAX_STAGES_FIT));
+                                 MODE == MODE_WGRAD ? SMEM_LIMIT : Cfg<MODE, BN>::smem_bytes(Cfg<MODE, BN>::MAX_STAGES_FIT));
         if (e != cudaSuccess) return e;
         attr_set[dev] = true;
     }
-    if (p.stages < 1 || p.stages > Cfg<MODE, BN>::MAX_STAGES_FIT) return cudaErrorInvalidValue;
+    if (!Cfg<MODE, BN>::fits(p.stages)) return cudaErrorInvalidValue;
     // (a weight gradient with the update folded in carries two parameter slab buffers behind its control block)
     const size_t smem = (size_t)Cfg<MODE, BN>::smem_bytes(p.stages) + (MODE == MODE_WGRAD && p.sgd_w != nullptr ? (size_t)UPD_EXTRA_SMEM : 0);
-    if (smem > 227 * 1024) return cudaErrorInvalidValue;
+    if (smem > SMEM_LIMIT) return cudaErrorInvalidValue;
     return pdl_launch(umma_kernel<MODE, BN>, grid, dim3(UMMA_THREADS), smem, st, op.mapA, op.mapB, op.mapC, op.mapD, p);
 }
 
@@ -2381,7 +2397,7 @@ static cudaError_t launch_halo_one(const UmmaOp& op, const UmmaParams& p, dim3 g
 {
     const int a_slot = (p.bh + 2) * p.bw * p.bn * 128;
     const int smem = HaloCfg<BN>::smem_bytes(p.a_stages, a_slot, p.stages);
-    if (p.a_stages < 1 || p.a_stages > MAX_A_STAGES || p.stages < 1 || p.stages > MAX_STAGES || smem > 227 * 1024) return cudaErrorInvalidValue;
+    if (!HaloCfg<BN>::fits(p.a_stages, a_slot, p.stages)) return cudaErrorInvalidValue;
     // (the attribute belongs to the device's copy of the function: set it once per device)
     static bool attr_set[64] = {false};
     int dev = 0;
@@ -2389,7 +2405,7 @@ static cudaError_t launch_halo_one(const UmmaOp& op, const UmmaParams& p, dim3 g
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!attr_set[dev]) {
-        e = cudaFuncSetAttribute(umma_halo_kernel<MODE, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        e = cudaFuncSetAttribute(umma_halo_kernel<MODE, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
         if (e != cudaSuccess) return e;
         attr_set[dev] = true;
     }
@@ -2409,10 +2425,9 @@ static cudaError_t launch_halo_mode(int bn, const UmmaOp& op, const UmmaParams& 
 template <int MODE>
 static cudaError_t launch_halo_persist_mode(const UmmaOp& op, const UmmaParams& p, dim3 grid, cudaStream_t st)
 {
-    const int smem = HaloPersistCfg::smem_bytes(p.a_stages, (p.bh + 2) * p.bw * p.bn * 128, p.stages, p.w_resident != 0);
-    if (p.a_stages < 1 || p.a_stages > HaloPersistCfg::MAX_A || p.stages < 3 || p.stages > HaloPersistCfg::MAX_B || smem > 227 * 1024 || !p.tma_out || p.splits != 1)
-        return cudaErrorInvalidValue;
-    const cudaError_t e = raise_smem_limit<umma_halo_persist_kernel<MODE>>(227 * 1024);
+    const int a_slot = (p.bh + 2) * p.bw * p.bn * 128, smem = HaloPersistCfg::smem_bytes(p.a_stages, a_slot, p.stages, p.w_resident != 0);
+    if (!HaloPersistCfg::fits(p.a_stages, a_slot, p.stages, p.w_resident != 0) || !p.tma_out || p.splits != 1) return cudaErrorInvalidValue;
+    const cudaError_t e = raise_smem_limit<umma_halo_persist_kernel<MODE>>(SMEM_LIMIT);
     if (e != cudaSuccess) return e;
     return pdl_launch(umma_halo_persist_kernel<MODE>, grid, dim3(HaloPersistCfg::THREADS), (size_t)smem, st, op.mapA, op.mapB, op.mapC, p);
 }
@@ -2421,11 +2436,9 @@ template <int MODE, int BN>
 static cudaError_t launch_halo_pair_one(const UmmaOp& op, const UmmaParams& p, dim3 grid, cudaStream_t st)
 {
     using C = HaloPairCfg<BN>;
-    const int smem = C::smem_bytes(p.a_stages, (p.bh + 2) * p.bw * p.bn * 128, p.stages, p.out_slots);
-    if (p.a_stages < 1 || p.a_stages > MAX_A_STAGES || p.stages < 3 || p.stages > MAX_B_SLOTS || p.out_slots < 1 || p.out_slots > 2 || smem > 227 * 1024 ||
-        !p.tma_out || p.splits != 1 || (grid.x & 1u))
-        return cudaErrorInvalidValue;
-    cudaError_t e = raise_smem_limit<umma_halo_pair_kernel<MODE, BN>>(227 * 1024);
+    const int a_slot = (p.bh + 2) * p.bw * p.bn * 128, smem = C::smem_bytes(p.a_stages, a_slot, p.stages, p.out_slots);
+    if (!C::fits(p.a_stages, a_slot, p.stages, p.out_slots) || !p.tma_out || p.splits != 1 || (grid.x & 1u)) return cudaErrorInvalidValue;
+    cudaError_t e = raise_smem_limit<umma_halo_pair_kernel<MODE, BN>>(SMEM_LIMIT);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
@@ -2466,7 +2479,7 @@ static cudaError_t launch_pair_one(const UmmaOp& op, const UmmaParams& p, dim3 g
         if (e != cudaSuccess) return e;
         attr_set[dev] = true;
     }
-    if (p.stages < 1 || p.stages > PairCfg<BN>::MAX_STAGES_FIT || (grid.x & 1u)) return cudaErrorInvalidValue;
+    if (!PairCfg<BN>::fits(p.stages) || (grid.x & 1u)) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(UMMA_THREADS);
@@ -2648,6 +2661,29 @@ cudaError_t launch_wait_probe(uint32_t* status, unsigned long long limit_ns, cud
 //  * ring depth = k-iterations per CTA, capped by what fits; for grids of several waves the ring is kept
 //    shallow enough that two CTAs share an SM, so one CTA's epilogue overlaps the other's main loop.
 struct TilePlan { int bn, splits, cps, stages, pair, halo, a_stages, persist, persist_ctas, out_slots, w_resident; double cost; };
+// Whether the kernel that a FWD / DGRAD plan names can be launched with it: an N tile it exists for, rings within its barrier arrays and
+// within a CTA's shared memory.  The launchers hold the same limits; checked here, a plan that cannot run is an error of
+// sb_model_bytes instead of the first pass.
+static bool plan_fits(const TilePlan& t, int a_slot_bytes, int kchunks)
+{
+    if (t.halo && (t.persist || t.pair) && (t.splits != 1 || (t.w_resident && t.stages != 9 * kchunks))) return false;
+    if (t.halo && t.pair)
+        return t.bn == 128 ? HaloPairCfg<128>::fits(t.a_stages, a_slot_bytes, t.stages, t.out_slots)
+                           : t.bn == 256 && HaloPairCfg<256>::fits(t.a_stages, a_slot_bytes, t.stages, t.out_slots);
+    if (t.halo && t.persist) return t.bn == HaloPersistCfg::BN && HaloPersistCfg::fits(t.a_stages, a_slot_bytes, t.stages, t.w_resident != 0);
+    if (t.halo)
+        return t.bn == 64 ? HaloCfg<64>::fits(t.a_stages, a_slot_bytes, t.stages)
+                          : t.bn == 128 ? HaloCfg<128>::fits(t.a_stages, a_slot_bytes, t.stages)
+                                        : t.bn == 256 && HaloCfg<256>::fits(t.a_stages, a_slot_bytes, t.stages);
+    if (t.pair) return t.bn == 128 ? PairCfg<128>::fits(t.stages) : t.bn == 256 && PairCfg<256>::fits(t.stages);
+    switch (t.bn) {
+    case 64: return Cfg<MODE_FWD, 64>::fits(t.stages);
+    case 128: return Cfg<MODE_FWD, 128>::fits(t.stages);
+    case 192: return Cfg<MODE_FWD, 192>::fits(t.stages);
+    case 256: return Cfg<MODE_FWD, 256>::fits(t.stages);
+    default: return false;
+    }
+}
 // Backward kernels of the two concurrent streams share SMs only if two CTAs fit side by side (shared
 // memory <= ~110 KB each, TMEM columns <= 256 each): SB_BWD_COHABIT=0 gives every kernel the full ring again.
 static bool bwd_cohabit()
@@ -2817,13 +2853,13 @@ static TilePlan plan_tiles_halo(int n_cols, long m_tiles, int kchunks, int a_slo
     const int b_stage = t.bn * 128;
     int sa = 2, sb = 0;
     for (; want >= 1; --want) {
-        const int budget = (int)(227 * 1024 / want) - 4 * 1024;
+        const int budget = (int)(SMEM_LIMIT / want) - 4 * 1024;
         sb = (budget - 2 * a_slot_bytes) / b_stage;
         if (sb >= 6 || want == 1) break;
     }
     if (sb > MAX_STAGES) sb = MAX_STAGES;
     if (sb < 3) sb = 3;
-    if (want <= 1 && 227 * 1024 - 4 * 1024 - 3 * a_slot_bytes - sb * b_stage >= 0) sa = 3;
+    if (want <= 1 && SMEM_LIMIT - 4 * 1024 - 3 * a_slot_bytes - sb * b_stage >= 0) sa = 3;
     {
         static const int f_sa = (int)tune("SB_HALO_SA", 0), f_sb = (int)tune("SB_HALO_SB", 0);
         if (f_sa > 0) sa = f_sa;
@@ -2850,7 +2886,7 @@ static TilePlan plan_tiles_halo_persist(int n_cols, long m_tiles, int kchunks, i
     t.cps = 3 * kchunks;
     t.w_resident = n_cols <= 64 && kchunks == 1;
     int sa = 1, sb = t.w_resident ? 9 : 6;
-    const int room = 227 * 1024;
+    const int room = SMEM_LIMIT;
     auto need = [&]() { return HaloPersistCfg::smem_bytes(sa, a_slot_bytes, sb, t.w_resident != 0); };
     while (!t.w_resident && need() > room) --sb;
     for (int more = 2; more <= HaloPersistCfg::MAX_A; ++more) { sa = more; if (need() > room) { --sa; break; } }
@@ -2875,16 +2911,21 @@ static bool plan_tiles_halo_pair(int n_cols, long m_tiles, int kchunks, int a_sl
         if (bn == 256 && n_cols <= 128) break;
         TilePlan t{};
         t.halo = 1; t.pair = 1; t.persist = 1; t.bn = bn; t.splits = 1; t.cps = 3 * kchunks;
-        const int b_half = bn * 64, room = 227 * 1024 - 1024 - CTRL_BYTES;
+        const int b_half = bn * 64, room = SMEM_LIMIT - 1024 - CTRL_BYTES;
         // rings: two groups of weight tiles and two activation boxes at least; for short groups (128 columns) up to four boxes and twelve
         // weight tiles first: a group's boxes are under way for about 2400 cycles where its MMAs take 768 (128 -> 128 channels at 112x112, batch 64,
         // forward: 237 us with two staging buffers and three boxes, 197 with one and four)
         int sa = 2, sb = 6, so = 1;
         auto need = [&]() { return sa * a_slot_bytes + sb * b_half + so * bn * 256; };
         if (need() > room) continue;
-        // all weights resident (one N tile, 64 input channels): they cross L2 once per CTA instead of once per tile
+        // all weights resident (one N tile, 64 input channels): they cross L2 once per CTA instead of once per tile.  The nine tiles have to
+        // fit beside two activation boxes and a staging buffer, which those of 256 columns (144 KB beside 64) never do: rings there
         t.w_resident = n_cols <= bn && kchunks == 1;
-        if (t.w_resident) { sb = 9; so = 2; if (need() > room) so = 1; }
+        if (t.w_resident) {
+            sb = 9; so = 2;
+            if (need() > room) so = 1;
+            if (need() > room) { t.w_resident = 0; sb = 6; }
+        }
         for (int more = 3; more <= 4; ++more) { sa = more; if (need() > room) { --sa; break; } }
         for (int more = sb + 1; more <= 12 && !t.w_resident; ++more) { sb = more; if (need() > room) { --sb; break; } }
         t.a_stages = sa; t.stages = sb; t.out_slots = so;
@@ -3118,6 +3159,8 @@ static FcGeom fc_geom(const LayerView& lv, int B, bool force_pair)
     return g;
 }
 
+static sb_status fail_plan() { return SB_ERR_CUDA; }
+
 sb_status umma_plan_scratch(sb_model* m, size_t* floats)
 {
     ModelView mv = model_view(m);
@@ -3128,6 +3171,12 @@ sb_status umma_plan_scratch(sb_model* m, size_t* floats)
         if (lv.kind == SB_CONV3X3_RELU && conv_umma_ok(mv, lv, i)) {
             ConvGeom g = conv_geom(lv, mv.B, (mv.cfg->flags & SB_FLAG_FORCE_PAIR) != 0, (mv.cfg->flags & SB_FLAG_NO_HALO) != 0, (mv.cfg->flags & SB_FLAG_FORCE_PERSIST) != 0);
             const size_t pix = (size_t)mv.B * lv.H * lv.W;
+            const int a_slot = (g.bh + 2) * g.bw * g.bn * 128;
+            if (!plan_fits(g.fwd, a_slot, cdiv_i(lv.Cin, 64)) || !plan_fits(g.dgrad, a_slot, cdiv_i(lv.Cout, 64))) {
+                snprintf(g_umma_err, sizeof(g_umma_err), "layer %d: the tile plan of %d -> %d channels at %dx%d, %d images does not fit its kernel",
+                         i, lv.Cin, lv.Cout, lv.H, lv.W, mv.B);
+                return fail_plan();
+            }
             if (g.wg_splits > 1) upd((size_t)g.wg_splits * (lv.n_w + lv.n_b));
             if (g.fwd.splits > 1) upd((size_t)g.fwd.splits * pix * lv.Cout);
             if (g.dgrad.splits > 1) upd((size_t)g.dgrad.splits * pix * lv.Cin);
@@ -3140,8 +3189,6 @@ sb_status umma_plan_scratch(sb_model* m, size_t* floats)
     *floats = need;
     return SB_OK;
 }
-
-static sb_status fail_plan() { return SB_ERR_CUDA; }
 
 // Fills the split / ring fields of a FWD or DGRAD op from its tile plan.
 static void apply_plan(OpBlock* b, const TilePlan& t, int k_iters, long m_tiles, int n_tiles_total, float* ws, size_t rows)
@@ -3455,7 +3502,7 @@ bool umma_fc_wgrad_can_update(sb_model* m, int layer)
     // (512 CTAs) -3.4 %, 512 -> 4096 (64 CTAs) a further -1.4 %, a 1024 x 1024 layer (32 CTAs) +0.5 %)
     static const long min_ctas = (long)tune("SB_FC_UPDATE_MIN_CTAS", 64);
     return b->p.mode == MODE_WGRAD && b->upd_maps && !b->pair && b->p.ntaps == 1 && b->bn != 192 && b->p.splits == 1 && b->p.bias_fused && wgrad_sweep_ok(b) &&
-           (lv.p_w & 3) == 0 && (lv.in_f % 64) == 0 && smem <= 227 * 1024 && (long)b->grid.x * b->grid.y * b->grid.z >= min_ctas;
+           (lv.p_w & 3) == 0 && (lv.in_f % 64) == 0 && smem <= SMEM_LIMIT && (long)b->grid.x * b->grid.y * b->grid.z >= min_ctas;
 }
 sb_status umma_fc_wgrad_update(sb_model* m, int layer, Hyper hy, cudaStream_t st)
 {
