@@ -3181,9 +3181,12 @@ sb_status umma_plan_scratch(sb_model* m, size_t* floats)
             if (g.fwd.splits > 1) upd((size_t)g.fwd.splits * pix * lv.Cout);
             if (g.dgrad.splits > 1) upd((size_t)g.dgrad.splits * pix * lv.Cin);
         } else if ((lv.kind == SB_FC_RELU || lv.kind == SB_FC) && fc_umma_ok(mv, lv, i)) {
-            FcGeom g = fc_geom(lv, mv.B, (mv.cfg->flags & SB_FLAG_FORCE_PAIR) != 0);
-            if (g.fwd.splits > 1) upd((size_t)g.fwd.splits * mv.B * lv.out_f);
-            if (g.dgrad.splits > 1) upd((size_t)g.dgrad.splits * mv.B * lv.in_f);
+            // (fewer rows can mean more splits: the B / K rows of a sub-iteration are sized for too)
+            for (int rows : {mv.B, (mv.cfg->flags & SB_FLAG_MODULO_SCHEDULE) ? mv.B / mv.cfg->K : mv.B}) {
+                FcGeom g = fc_geom(lv, rows, (mv.cfg->flags & SB_FLAG_FORCE_PAIR) != 0);
+                if (g.fwd.splits > 1) upd((size_t)g.fwd.splits * rows * lv.out_f);
+                if (g.dgrad.splits > 1) upd((size_t)g.dgrad.splits * rows * lv.in_f);
+            }
         }
     }
     *floats = need;
@@ -3193,7 +3196,7 @@ sb_status umma_plan_scratch(sb_model* m, size_t* floats)
 // Fills the split / ring fields of a FWD or DGRAD op from its tile plan.
 static void apply_plan(OpBlock* b, const TilePlan& t, int k_iters, long m_tiles, int n_tiles_total, float* ws, size_t rows)
 {
-    // (the scratch for split partial sums was sized by umma_plan_scratch for the full batch; sub-batch plans are checked by the caller)
+    // (the scratch for split partial sums was sized by umma_plan_scratch, for the full batch and for the sub-batches)
     UmmaParams& p = b->p;
     b->bn = t.bn;
     p.total_chunks = k_iters;

@@ -20,6 +20,10 @@ CASES = {
     # K = 4: sub-batches of 32 rows) behind a one-layer conv front that also yields 512 features
     "cfg1_fc_stack": lambda: si.Workload("modulo_cfg1_fc", [(si.CONV3X3_RELU, 128), (si.MAXPOOL2, 0), (si.FC_RELU, 4096), (si.FC_RELU, 4096),
                                                            (si.FC, 10), (si.SOFTMAX_XENT, 10)], 4, 4, 3, 32, 4, 4),
+    # 192 rows in two tiles, sub-batches of 64 in one: the sub-batches split their reductions further than the full batch does,
+    # behind a conv front too small to need that much scratch
+    "split_sub_batches": lambda: si.Workload("modulo_split", [(si.CONV3X3_RELU, 16), (si.MAXPOOL2, 0), (si.FC_RELU, 2048), (si.FC, 1000),
+                                                              (si.SOFTMAX_XENT, 1000)], 4, 4, 4, 96, 2, 3),
     # K = 4 sub-iterations of a single replica
     "one_replica": lambda: si.Workload("modulo_r1", tensor_core_net(), 8, 8, 3, 8, 1, 4),
 }
