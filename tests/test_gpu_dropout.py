@@ -163,6 +163,41 @@ def test_graph_replays_advance_the_iteration_and_match_the_oracle():
     assert np.array_equal(fc_act(gm2, b.SB_T_ACT, 5) != 0, om2.fc_out[5] != 0)
 
 
+@pytest.mark.parametrize("name,bf16", [("tensor_core", True), ("tensor_core", False), ("ragged", True), ("ragged", False)])
+def test_replayed_passes_draw_a_new_mask_every_time(name, bf16):
+    """sb_forward / sb_backward on repeated buffers replay themselves as graphs; the iteration word then advances inside the
+    replayed pass.  Same masks, losses and gradients as a model that enqueues every pass kernel by kernel (default stream), also
+    when the seed is set again between two replays and when the word wraps."""
+    import torch
+    b = sb()
+    wl = WORKLOADS[name]()
+    params = si.make_params(wl, bias_std=0.2)
+    xs, ys = device_batch(wl, *si.make_batch(wl), bf16)
+    direct, replayed = (gpu_model(wl, params, b.SB_BF16 if bf16 else b.SB_FP32) for _ in range(2))
+    side = torch.cuda.Stream()
+    li = drop_layers(wl)[0]
+    masks = []
+    for step in range(9):
+        for m, stream in ((direct, torch.cuda.default_stream()), (replayed, side)):
+            with torch.cuda.stream(stream):
+                if step in (0, 7):
+                    m.dropout_seed(SEED + step, 0xFFFFFFFC)
+                m.forward(xs, ys)
+                m.backward()
+                m.sgd_step(0.01, 0.9)
+                stream.synchronize()
+        assert direct.loss() == replayed.loss(), step
+        acts = [fc_act(m, b.SB_T_ACT, li) for m in (direct, replayed)]
+        assert np.array_equal(*acts), step
+        masks.append(acts[0] != 0)
+        for p, q in zip(*(m.gather_params(b.SB_T_GRAD_W, b.SB_T_GRAD_B) for m in (direct, replayed))):
+            if p is not None:
+                assert np.array_equal(p["w"], q["w"]) and np.array_equal(p["b"], q["b"]), step
+    assert all(not np.array_equal(masks[i], masks[i + 1]) for i in range(8))
+    direct.close()
+    replayed.close()
+
+
 def test_full_size_vgg16_with_dropout_in_the_classifier():
     """The metric's network (VGG-16, CIFAR shape, batch 128, R = K = 4, bf16) with p = 0.5 dropout after both 4096-wide FC
     layers, in the launch configuration the benchmark times (sb_graph_step: multi-stream backward, update folded into the

@@ -20,6 +20,7 @@ pytestmark = pytest.mark.gpu
     (10, 8, (16, 128, 256), 3, 1),       # with pairs forced: two taps per CTA pair of the weight gradient
     (56, 56, (64, 256, 64), 13, 1),      # more than two tiles per SM: CTA pairs on halos by themselves, 256 columns of one reduction chunk
     (24, 40, (48, 144, 32), 41, 1),      # ... with partly filled tiles and chunks, in both directions
+    (136, 120, (32, 48), 33, 1),         # long enough for the nine-tap weight gradient by itself: every CTA's share of chunks, images ragged
 ])
 @pytest.mark.parametrize("flags", [0, 8, 32, 64])     # default / CTA pairs / no halo kernel / persistent kernels, several tiles per CTA
 def test_channel_counts_off_the_tiles(H, W, chans, b, R, flags):
