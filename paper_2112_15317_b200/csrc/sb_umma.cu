@@ -3353,10 +3353,11 @@ sb_status umma_plan_layers(sb_model* m, int first_layer)
                     static const bool wg_pair = tune("SB_WG_PAIR", 1) != 0;
                     // (long reductions only: below 320 pixel chunks the pair's two cluster barriers and the separate column-sum
                     // kernel cost more than the halved activation fetch saves: from 64 chunks up CIFAR shape at batch 128 +0.7 % step,
-                    // from 160 up batch 256 +0.7 %; never at ImageNet shape +1.2 %.  512 x 512 channels, whose tiles fill the machine unsplit, from 160
-                    // chunks up: 107 -> 85 us alone at 14x14, batch 64)
+                    // from 160 up batch 256 +0.7 %; never at ImageNet shape +1.2 %;
+                    // nor from 160 chunks up for 512 channels or more on both sides: the kernel alone falls from 92 to 78 us at 14x14, batch 64, with
+                    // the column sum and its reduce from 92 to 95, and the step is 5.88 against 5.85 ms; 512 -> 256 56 -> 64, 256 -> 256 39 -> 55)
                     static const int wg_pair_min_chunks = (int)tune("SB_WG_PAIR_MIN_CHUNKS", 320);
-                    if (wg_pair && (g.total_chunks >= (lv.Cout >= 512 && lv.Cin >= 512 ? wg_pair_min_chunks / 2 : wg_pair_min_chunks) || (mv.cfg->flags & SB_FLAG_FORCE_PAIR)) && (p.tap_group == 1 || p.tap_group == 2) && (b->bn == 128 || b->bn == 256) && g.wg_m_tiles % 2 == 0 && lv.Cout % 128 == 0) {
+                    if (wg_pair && (g.total_chunks >= wg_pair_min_chunks || (mv.cfg->flags & SB_FLAG_FORCE_PAIR)) && (p.tap_group == 1 || p.tap_group == 2) && (b->bn == 128 || b->bn == 256) && g.wg_m_tiles % 2 == 0 && lv.Cout % 128 == 0) {
                         b->pair = 1;
                         p.bias_fused = 0;
                         const int pfit = b->bn >= 256 ? 6 : 8, ptwo = b->bn >= 256 ? 3 : 4;
