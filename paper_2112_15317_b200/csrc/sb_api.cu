@@ -158,6 +158,7 @@ struct sb_model {
         int64_t launches = 0;
     };
     PassGraph g_fwd, g_bwd;
+    cudaStream_t capstream = nullptr;      // what they are captured on
     // Debug aids that stand in for a memory checker: every arena region is followed by a 256-byte guard holding a fixed
     // pattern (sb_debug_check_guards), and the regions a step overwrites are listed so that they can be filled with NaN
     // bit patterns before a step (sb_debug_poison).
@@ -202,6 +203,7 @@ struct sb_model {
         if (ev_side) cudaEventDestroy(ev_side);
         if (host_res) cudaFreeHost(host_res);
         if (cpstream) cudaStreamDestroy(cpstream);
+        if (capstream) cudaStreamDestroy(capstream);
     }
 };
 
@@ -1089,15 +1091,18 @@ static sb_status end_capture(sb_model::StepGraph& G, cudaStream_t st)
 // One pass on the model's current inputs, replayed as a CUDA graph where that pays: enqueued kernel by kernel a pass costs the host 2
 // to 3.5 us a launch (more than the kernels of a small network take), the graph 2.5 us in all.  It is captured once the
 // same buffers have come several times in a row (each capture that later buffers make useless doubles that number), so a
-// caller whose buffers change from call to call never pays for one.
+// caller whose buffers change from call to call never pays for one.  It is captured on a stream of the model's own: while a blocking
+// stream of the caller's were under capture, other threads could not use the legacy default stream.  Where no graph can be had
+// (instantiating one takes device memory), the pass runs kernel by kernel.
 }  // extern "C"
 template <typename Pass>
 static sb_status pass_replay(sb_model* m, sb_model::PassGraph& G, cudaStream_t st, Pass pass)
 {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     // (a network that begins with an FC layer binds its input into tensor maps: kernel by kernel)
-    if (m->profiling || m->debug_sync || st == nullptr || m->first_fc == 0 || cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
-        return pass();
+    if (m->profiling || m->debug_sync || st == nullptr || st == cudaStreamLegacy || m->first_fc == 0 || cudaStreamIsCapturing(st, &cap) != cudaSuccess ||
+        cap != cudaStreamCaptureStatusNone)
+        return pass(st);
     const int R = m->cfg.R;
     if (G.same > 0 && same_ptrs(G.last_x, m->x_tab, R) && same_ptrs(G.last_labels, m->label_tab, R)) {
         if (G.same < G.need) ++G.same;
@@ -1105,17 +1110,21 @@ static sb_status pass_replay(sb_model* m, sb_model::PassGraph& G, cudaStream_t s
         G.last_x = m->x_tab; G.last_labels = m->label_tab; G.same = 1;
     }
     if (!(G.exec && same_ptrs(G.x, m->x_tab, R) && same_ptrs(G.labels, m->label_tab, R))) {
-        if (G.same < G.need) return pass();
-        CU_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+        if (G.same < G.need) return pass(st);
+        if (G.need < (1 << 20)) G.need *= 2;
+        if (!m->capstream) CU_TRY(cudaStreamCreateWithFlags(&m->capstream, cudaStreamNonBlocking));
+        CU_TRY(cudaStreamBeginCapture(m->capstream, cudaStreamCaptureModeThreadLocal));
         const int64_t l0 = m->launches;
-        sb_status s = pass();
-        if (s != SB_OK) { abandon_capture(st); return s; }
+        const sb_status s = pass(m->capstream);
+        if (s != SB_OK) { abandon_capture(m->capstream); return s; }
         G.launches = m->launches - l0;
         m->launches = l0;
-        s = end_capture(G, st);
-        if (s != SB_OK) return s;
+        if (end_capture(G, m->capstream) != SB_OK) {
+            cudaGetLastError();
+            G.same = 0;
+            return pass(st);
+        }
         G.x = m->x_tab; G.labels = m->label_tab;
-        if (G.need < (1 << 20)) G.need *= 2;
     }
     m->launches += G.launches;
     CU_TRY(cudaGraphLaunch(G.exec, st));
@@ -1144,7 +1153,7 @@ static sb_status forward_on(sb_model* m, const void* const* x, const int32_t* co
     sb_status s = set_inputs(m, x, labels);
     if (s != SB_OK) return s;
     m->launches = 0;
-    s = by_itself ? pass_replay(m, m->g_fwd, st, [&] { return forward_pass(m, st); }) : forward_pass(m, st);
+    s = by_itself ? pass_replay(m, m->g_fwd, st, [&](cudaStream_t on) { return forward_pass(m, on); }) : forward_pass(m, st);
     if (s == SB_OK) m->have_fwd = true;
     return s;
 }
@@ -1268,7 +1277,7 @@ sb_status sb_backward(sb_model* m, void* stream)
     if (!m) return fail(SB_ERR_INVALID_ARG, "null model");
     if (!m->have_fwd) return fail(SB_ERR_STATE, "sb_backward needs a preceding sb_forward");
     cudaStream_t st = (cudaStream_t)stream;
-    return pass_replay(m, m->g_bwd, st, [&] { return backward_pass(m, st, false, Hyper{}, nullptr); });
+    return pass_replay(m, m->g_bwd, st, [&](cudaStream_t on) { return backward_pass(m, on, false, Hyper{}, nullptr); });
 }
 
 // forward + backward + update of one iteration, with the update folded into the backward pass when possible

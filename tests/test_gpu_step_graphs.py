@@ -67,3 +67,32 @@ def test_passes_replayed_on_repeated_buffers():
                 assert np.array_equal(p["w"], q["w"]) and np.array_equal(p["b"], q["b"])
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("handle", [1, 2])     # cudaStreamLegacy (cannot be captured), cudaStreamPerThread
+def test_repeated_passes_on_the_default_streams_by_handle(handle):
+    import ctypes
+
+    import torch
+
+    from paper_2112_15317_b200 import binding as sb
+    wl = si.config(0)
+    params = si.make_params(wl, bias_std=0.1)
+    a, b = tu.gpu_model(wl, params, sb.SB_BF16), tu.gpu_model(wl, params, sb.SB_BF16)
+    xs, ys = tu.device_batch(wl, *si.make_batch(wl), True)
+    ptrs = b._ptr_arrays(xs, ys)
+    st = ctypes.c_void_p(handle)
+    torch.cuda.synchronize()
+    for _ in range(6):
+        a.forward(xs, ys)
+        a.backward()
+        a.sgd_step(0.01, 0.9)
+        for call in (lambda: sb.sb_forward(b.h, *ptrs, st), lambda: sb.sb_backward(b.h, st), lambda: sb.sb_sgd_step(b.h, 0.01, 0.9, st)):
+            assert call() == 0, sb.sb_last_error()
+        torch.cuda.synchronize()
+        assert a.loss() == b.loss()
+    for p, q in zip(a.gather_params(sb.SB_T_WEIGHT, sb.SB_T_BIAS), b.gather_params(sb.SB_T_WEIGHT, sb.SB_T_BIAS)):
+        if p is not None:
+            assert np.array_equal(p["w"], q["w"]) and np.array_equal(p["b"], q["b"])
+    a.close()
+    b.close()
