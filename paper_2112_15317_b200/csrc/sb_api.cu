@@ -56,7 +56,7 @@ struct Layer {
     bool narrow = false;                        // FC with out <= 16: dedicated narrow kernels
     int K = 1;                                  // FC: column shards of this layer (the model's K, or 1 for a layer kept whole)
     int act_dt = SB_DT_F32;
-    ContractPlan cplan[3];                      // forward / data gradient / weight gradient on CUDA cores, where these run there
+    ContractPlan cplan[3];                      // forward / data gradient / weight gradient as contractions on CUDA cores (float: or tensor cores), where these run there
     UmmaLayer um;                               // tensor-core plan of this layer (tcgen05 path)
     // Sub-batch copies of the first FC layer (modulo schedule): where its input comes from and where its input
     // gradient goes, instead of the layer below's buffers
@@ -222,12 +222,13 @@ ContractArgs contract_args(sb_model* m, int i, int mode)
     a.H = conv ? l.H : 1; a.W = conv ? l.W : 1;
     a.Cin = conv ? l.Cin : l.in_f; a.Cout = conv ? l.Cout : l.out_f;
     a.plan = l.cplan[mode];
+    a.status = m->status;
     a.act = l.in_override ? l.in_override : (i > 0 ? m->L[i - 1].act : nullptr);
     if (i == 0) { a.tab = &m->x_tab; a.tab_imgs = m->cfg.batch_per_replica; }
     return a;
 }
 
-// Plans the CUDA-core passes of layer i for the model's current batch; returns the scratch floats they need.
+// Plans the contractions of layer i for the model's current batch; returns the scratch floats they need.
 size_t contract_plan_layer(sb_model* m, int i, size_t max_part_floats)
 {
     Layer& l = m->L[i];
@@ -237,7 +238,7 @@ size_t contract_plan_layer(sb_model* m, int i, size_t max_part_floats)
         // (passes that run on the input-layer kernels, or not at all, take no scratch)
         if (mode == CMODE_DGRAD ? i == 0 && !(m->cfg.flags & SB_FLAG_INPUT_GRAD) : l.thin_input) continue;
         const ContractArgs a = contract_args(m, i, mode);
-        l.cplan[mode] = contract_plan(mode, a.B, a.H, a.W, a.taps, a.Cin, a.Cout, max_part_floats);
+        l.cplan[mode] = contract_plan(mode, a.B, a.H, a.W, a.taps, a.Cin, a.Cout, max_part_floats, !m->bf16 && i > 0 && !(m->cfg.flags & SB_FLAG_FORCE_SIMT));
         const size_t result = mode == CMODE_WGRAD ? l.n_w + l.n_b : (size_t)a.B * a.H * a.W * (mode == CMODE_FWD ? a.Cout : a.Cin);
         if (l.cplan[mode].splits > 1) need = std::max(need, l.cplan[mode].splits * result);
     }
@@ -447,7 +448,7 @@ inline const char* layer_input(const sb_model* m, int i) { return m->L[i].in_ove
 
 const void* weights_of(const sb_model* m, const Layer& l) { return m->bf16 ? (const void*)(m->Sm + l.p_w) : (const void*)(m->Wm + l.p_w); }
 
-// CUDA-core passes of one layer
+// Contractions of one layer on CUDA cores, or in float on tensor cores (launch class "..._f32_umma")
 sb_status contract_forward(sb_model* m, int i, const char* tag, double flops, double bytes, cudaStream_t st)
 {
     const Layer& l = m->L[i];
@@ -455,7 +456,7 @@ sb_status contract_forward(sb_model* m, int i, const char* tag, double flops, do
     a.wt = weights_of(m, l); a.bias = m->Wm + l.p_b; a.relu = l.relu;
     if (l.act_dt == SB_DT_F32) a.out32 = (float*)l.act; else a.out = l.act;
     a.part = m->ws; a.split_stride = (long)a.B * a.H * a.W * a.Cout;
-    L_TRY(tag, flops, bytes, launch_contract(a, m->bf16, st));
+    L_TRY(!a.plan.umma ? tag : a.taps == 9 ? "conv_fwd_f32_umma" : "fc_fwd_f32_umma", flops, bytes, launch_contract(a, m->bf16, st));
     if (a.plan.splits > 1) ++m->launches;
     return SB_OK;
 }
@@ -465,7 +466,7 @@ sb_status contract_dgrad(sb_model* m, int i, const char* tag, double flops, doub
     ContractArgs a = contract_args(m, i, CMODE_DGRAD);
     a.wt = weights_of(m, l); a.dy = l.dact; a.out = dx; a.ref = ref;
     a.part = m->ws; a.split_stride = (long)a.B * a.H * a.W * a.Cin;
-    L_TRY(tag, flops, bytes, launch_contract(a, m->bf16, st));
+    L_TRY(!a.plan.umma ? tag : a.taps == 9 ? "conv_dgrad_f32_umma" : "fc_dgrad_f32_umma", flops, bytes, launch_contract(a, m->bf16, st));
     if (a.plan.splits > 1) ++m->launches;
     return SB_OK;
 }
@@ -635,7 +636,7 @@ sb_status backward_layer(sb_model* m, int i, cudaStream_t st, int part = SIDE_BO
         a.part = *S > 1 ? ws_w : m->Gm + l.p_w;
         a.split_stride = (long)(l.n_w + l.n_b);
         a.bias_off = *S > 1 ? (long)l.n_w : (long)(l.p_b - l.p_w);
-        L_TRY(tag, flops, bytes, launch_contract(a, bf, st));
+        L_TRY(!a.plan.umma ? tag : a.taps == 9 ? "conv_wgrad_f32_umma" : "fc_wgrad_f32_umma", flops, bytes, launch_contract(a, bf, st));
         return SB_OK;
     };
     sb_status fs = SB_OK;

@@ -1,4 +1,4 @@
-// CUDA-core contractions of the float mode (and of layers whose widths the tensor-core tiles do not take): 3x3 convolution and
+// CUDA-core contractions of the float mode's small and odd layers (and of layers whose widths the tensor-core tiles do not take): 3x3 convolution and
 // fully-connected forward, data gradient and weight gradient as one tiled kernel.
 //
 //   FWD   : y[pixel, o]  = sum_{tap, c} x[pixel + tap, c]  * W[o, tap, c]      rows = pixels, columns = output channels
@@ -6,6 +6,10 @@
 //   WGRAD : dW[o, n]     = sum_{pixel}  dy[pixel, o] * x[pixel + tap, c]       rows = output channels, columns n = (tap, c)
 //
 // A fully-connected layer is the same thing with one tap and 1x1 images (pixel = batch row).
+//
+// Large enough float layers whose channel counts are multiples of eight run on the tensor cores instead (sb_contract_umma.cu): the plan
+// takes whichever the two cost models below say is faster.  3x3 over 64 channels at 32x32, batch 96: 181 us here, 102 there; 256
+// channels at 8x8: 157 and 57; 16 -> 32 channels at 16x16, batch 8, forward: 8.0 and 8.0.
 //
 // What bounds it: the FFMA pipe (measured 70 TFLOP/s of packed fma.rn.f32x2 on registers, 68 of scalar FFMA).  A block of
 // BM x BN outputs gives every thread an 8 x 8 square, so that 16 shared-memory words feed 64 multiply-adds; the packed form
@@ -360,6 +364,11 @@ struct TileShape { int bm, bn, resident; double lone, more; };
 static const TileShape shapes[] = {{128, 128, 2, 0.45, 1.25}, {128, 64, 4, 0.75, 0.65}, {64, 128, 4, 0.75, 0.63},
                                    {64, 64, 6, 0.62, 0.30},   {128, 32, 6, 0.85, 0.30}, {32, 128, 6, 0.85, 0.30}};
 
+// The tensor-core form (one CTA per SM): microseconds per 64 reduction steps, per tile and per launch, by tile width and mode,
+// from a sweep of both widths and 1 to 64 splits over 25 layers (residual 6 to 10 %).
+struct UmmaCost { double step, tile, launch; };
+static const UmmaCost umma_cost[2][3] = {{{1.41, 3.7, 3.3}, {1.48, 3.3, 3.3}, {1.72, 7.8, -2.2}}, {{1.04, 2.6, 3.3}, {1.18, 2.4, 3.0}, {1.34, 4.6, -0.8}}};
+
 static bool vec_ok(int Cin, int Cout) { return Cin % 4 == 0 && Cout % 4 == 0; }
 static long contract_iters(int mode, int B, int H, int W, int taps, int Cin, int Cout)
 {
@@ -367,7 +376,7 @@ static long contract_iters(int mode, int B, int H, int W, int taps, int Cin, int
     return mode == CMODE_WGRAD ? ((long)B * H * W + BK - 1) / BK : (long)taps * ((cred + BK - 1) / BK);
 }
 
-ContractPlan contract_plan(int mode, int B, int H, int W, int taps, int Cin, int Cout, size_t max_part_floats)
+ContractPlan contract_plan(int mode, int B, int H, int W, int taps, int Cin, int Cout, size_t max_part_floats, bool umma)
 {
     const long pix = (long)B * H * W, M = mode == CMODE_WGRAD ? Cout : pix;
     const long N = mode == CMODE_FWD ? Cout : mode == CMODE_DGRAD ? Cin : (long)taps * Cin;
@@ -385,7 +394,22 @@ ContractPlan contract_plan(int mode, int B, int H, int W, int taps, int Cin, int
             const double step = (double)(n / s.resident) * (s.lone + s.more * s.resident) + (rest ? s.lone + s.more * rest : 0.0);
             double t = per * step * (mode == CMODE_WGRAD ? 1.08 : 1.0) + 3.0;
             if (real > 1) t += 3.0 + (double)real * M * N * 8.0 / 7.0e6;
-            if (t < best_t) { best_t = t; best = ContractPlan{s.bm, s.bn, (int)per, real}; }
+            if (t < best_t) { best_t = t; best = ContractPlan{s.bm, s.bn, (int)per, real, false}; }
+        }
+    }
+    if (umma && contract_umma_ok(taps, Cin, Cout)) {
+        const long K = mode == CMODE_WGRAD ? pix : (long)taps * (mode == CMODE_DGRAD ? Cout : Cin), chunks = (K + 63) / 64;
+        for (int bn : {128, 64}) {
+            const UmmaCost& u = umma_cost[bn == 64][mode];
+            const long tiles = ((M + 127) / 128) * ((N + bn - 1) / bn);
+            for (int split = 1; split <= 256 && split <= chunks; split = split < 8 ? split + 1 : split + split / 4) {
+                const long per = (chunks + split - 1) / split;
+                const int real = (int)((chunks + per - 1) / per);
+                if (real > 1 && (size_t)real * M * (N + (mode == CMODE_WGRAD ? 1 : 0)) > max_part_floats) break;
+                double t = (double)((tiles * real + 147) / 148) * (per * u.step + u.tile) + u.launch;
+                if (real > 1) t += mode == CMODE_WGRAD ? 3.0 + (double)real * M * N * 8.0 / 7.0e6 : (double)real * M * N * 13.0 / 7.0e6;
+                if (t < best_t) { best_t = t; best = ContractPlan{128, bn, (int)per, real, true}; }
+            }
         }
     }
     return best;
@@ -445,7 +469,8 @@ cudaError_t launch_contract(const ContractArgs& a, bool bf16, cudaStream_t st)
     p.part = a.part; p.split_stride = a.split_stride; p.bias_off = a.bias_off;
     p.out = a.out; p.out32 = a.out32; p.bias = a.bias; p.relu = a.relu; p.ref = a.ref;
     cudaError_t e;
-    if (a.mode == CMODE_FWD) e = bf16 ? launch_vec<__nv_bfloat16, CMODE_FWD>(a.plan, p, st) : launch_vec<float, CMODE_FWD>(a.plan, p, st);
+    if (a.plan.umma) e = launch_contract_umma(a, st);
+    else if (a.mode == CMODE_FWD) e = bf16 ? launch_vec<__nv_bfloat16, CMODE_FWD>(a.plan, p, st) : launch_vec<float, CMODE_FWD>(a.plan, p, st);
     else if (a.mode == CMODE_DGRAD) e = bf16 ? launch_vec<__nv_bfloat16, CMODE_DGRAD>(a.plan, p, st) : launch_vec<float, CMODE_DGRAD>(a.plan, p, st);
     else e = bf16 ? launch_vec<__nv_bfloat16, CMODE_WGRAD>(a.plan, p, st) : launch_vec<float, CMODE_WGRAD>(a.plan, p, st);
     if (e != cudaSuccess || a.mode == CMODE_WGRAD || p.splits == 1) return e;

@@ -126,11 +126,13 @@ struct WgradSimtArgs {
     int B, H, W, Cin, Cout;
 };
 
-// 3x3 convolution (taps = 9) or fully-connected layer (taps = 1, H = W = 1) on CUDA cores: sb_contract_simt.cu.
+// 3x3 convolution (taps = 9) or fully-connected layer (taps = 1, H = W = 1) on CUDA cores (sb_contract_simt.cu) or, for float
+// operands, on tensor cores with every float as three bf16 terms (sb_contract_umma.cu).
 enum { CMODE_FWD = 0, CMODE_DGRAD = 1, CMODE_WGRAD = 2 };
-struct ContractPlan { int bm = 64, bn = 64, iters = 0, splits = 1; };     // block tile, reduction steps per split, splits
+struct ContractPlan { int bm = 64, bn = 64, iters = 0, splits = 1; bool umma = false; };     // block tile, reduction steps (16 or, umma, 64) per split, splits
 // max_part_floats: room for split partial sums ([splits][result], for WGRAD with the bias gradient behind each)
-ContractPlan contract_plan(int mode, int B, int H, int W, int taps, int Cin, int Cout, size_t max_part_floats);
+// umma: the tensor-core form may be chosen (float operands; the layer input is one buffer)
+ContractPlan contract_plan(int mode, int B, int H, int W, int taps, int Cin, int Cout, size_t max_part_floats, bool umma);
 struct ContractArgs {
     int mode, taps, B, H, W, Cin, Cout;
     const void *act, *wt, *dy;             // layer input (or tab), weights [Cout][taps][Cin], output gradient, in the activation dtype
@@ -141,8 +143,11 @@ struct ContractArgs {
     void* out; float* out32;               // FWD / DGRAD result (out32: float instead of the activation dtype)
     const float* bias; int relu;           // FWD
     const void* ref;                       // DGRAD: zero where ref <= 0
+    uint32_t* status;                      // device status word of the bounded waits
 };
 cudaError_t launch_contract(const ContractArgs& a, bool bf16, cudaStream_t st);
+bool contract_umma_ok(int taps, int Cin, int Cout);
+cudaError_t launch_contract_umma(const ContractArgs& a, cudaStream_t st);      // (without the second kernel of a split FWD / DGRAD)
 
 // Input-layer convolution (Cin of 1, 3 or 4; Cout a multiple of 8): dedicated forward and weight+bias
 // gradient kernels.  The gradient kernel writes conv_in_wgrad_blocks() partial buffers of

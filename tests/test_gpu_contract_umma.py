@@ -1,0 +1,100 @@
+"""Float contractions on the tensor cores (every float as three bf16 terms) at the edges of their tiles, chunks and splits: one conv and
+one FC layer's three passes against double-precision torch on the layer's own stored inputs, and non-finite operands against the
+CUDA-core kernels."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import sb_inputs as si
+import sb_testutil as tu
+
+pytestmark = pytest.mark.gpu
+
+# Bound on the 2-norm: products left out 2^-26, truncation of the leading products over 64 steps 4 x 2^-25, the rounded running sum
+# 2^-25 sqrt(chunks) of up to 60 chunks: below 4e-7 in all; the largest measured over a sweep of 25 layers is 2.1e-7.
+BOUND = 5e-7
+
+
+def _net(H, W, c0, c1, width, b, R):
+    wl = si.Workload("contract_umma", [(si.CONV3X3_RELU, c0), (si.CONV3X3_RELU, c1), (si.FC_RELU, width), (si.FC, 10), (si.SOFTMAX_XENT, 10)], H, W, 4, b, R, 1)
+    return wl, si.make_params(wl, bias_std=0.2), si.make_batch(wl)
+
+
+@pytest.mark.parametrize("H,W,c0,c1,width,b,R,on", [
+    (9, 7, 24, 72, 40, 17, 2, 5),        # chunks that cross taps, ragged rows, columns and chunks
+    (6, 6, 8, 136, 72, 29, 2, 5),        # one run of eight channels a tap; more columns than a 128-wide tile
+    (8, 8, 64, 128, 128, 24, 2, 6),      # whole tiles, split reductions
+    (16, 12, 64, 64, 64, 16, 2, 4),      # one column tile, long weight-gradient reduction
+    (4, 4, 264, 248, 520, 3, 1, 5),      # less than a row tile, long forward and data-gradient reductions
+])
+def test_passes_against_double(H, W, c0, c1, width, b, R, on):
+    import torch
+    import torch.nn.functional as F
+
+    from paper_2112_15317_b200 import binding as sb
+    wl, params, batch = _net(H, W, c0, c1, width, b, R)
+    m = tu.gpu_model(wl, params, sb.SB_FP32, sb.SB_FLAG_PROFILE_LAYERS)
+    xs, ys = tu.device_batch(wl, *batch, False)
+    m.profile_begin()
+    m.forward(xs, ys)
+    m.backward()
+    names = [e["name"] for e in m.profile_end()]
+    ran = {n for n in names if "f32_umma" in n}
+    assert len(ran) >= on, names
+    t = lambda what, li: torch.from_numpy(np.concatenate([m.read(what, li, r, squeeze=False) for r in range(R if li < 2 else 1)])).double()  # noqa: E731
+    wt = lambda what, li: torch.from_numpy(m.read(what, li, 0, squeeze=False)).double()  # noqa: E731
+    checks = tu.Checks()
+
+    x = t(sb.SB_T_ACT, 0).permute(0, 3, 1, 2).requires_grad_()
+    w = wt(sb.SB_T_WEIGHT, 1).permute(0, 3, 1, 2).requires_grad_()
+    bias = wt(sb.SB_T_BIAS, 1).reshape(-1).requires_grad_()
+    y = F.conv2d(x, w, bias, padding=1)
+    y.backward(t(sb.SB_T_DACT, 1).permute(0, 3, 1, 2))
+    checks.le("conv forward", tu.frob(t(sb.SB_T_ACT, 1), y.relu().permute(0, 2, 3, 1).detach()), BOUND)
+    checks.le("conv input gradient", tu.frob(t(sb.SB_T_DACT, 0), (x.grad * (x > 0)).permute(0, 2, 3, 1).detach()), BOUND)
+    checks.le("conv weight gradient", tu.frob(wt(sb.SB_T_GRAD_W, 1), w.grad.permute(0, 2, 3, 1)), BOUND)
+    checks.le("conv bias gradient", tu.frob(wt(sb.SB_T_GRAD_B, 1).reshape(-1), bias.grad), BOUND)
+
+    x = t(sb.SB_T_ACT, 1).reshape(wl.B, -1).requires_grad_()
+    w = wt(sb.SB_T_WEIGHT, 2)[:, :, 0, 0].requires_grad_()
+    bias = wt(sb.SB_T_BIAS, 2).reshape(-1).requires_grad_()
+    y = F.linear(x, w, bias)
+    y.backward(t(sb.SB_T_DACT, 2)[:, :, 0, 0])
+    checks.le("fc forward", tu.frob(t(sb.SB_T_ACT, 2)[:, :, 0, 0], y.relu().detach()), BOUND)
+    checks.le("fc input gradient", tu.frob(t(sb.SB_T_DACT, 1).reshape(wl.B, -1), (x.grad * (x > 0)).detach()), BOUND)
+    checks.le("fc weight gradient", tu.frob(wt(sb.SB_T_GRAD_W, 2)[:, :, 0, 0], w.grad), BOUND)
+    checks.le("fc bias gradient", tu.frob(wt(sb.SB_T_GRAD_B, 2).reshape(-1), bias.grad), BOUND)
+    assert m.debug_check_guards()[0] == 0
+    m.loss()       # raises if a bounded wait ran out
+    m.close()
+    checks.finish()
+
+
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan, 3.4e38])
+def test_non_finite_operands_as_on_cuda_cores(bad):
+    """Infinities and values that round to one in bf16 give the infinities, NaNs and numbers of plain multiply-adds."""
+    from paper_2112_15317_b200 import binding as sb
+    wl, params, batch = _net(8, 8, 64, 128, 128, 24, 2)
+    xs, ys = tu.device_batch(wl, *batch, False)
+    a, ref = tu.gpu_model(wl, params, sb.SB_FP32), tu.gpu_model(wl, params, sb.SB_FP32, sb.SB_FLAG_FORCE_SIMT)
+    dy = 0.01 * np.cos(np.arange(24 * 8 * 8 * 128, dtype=np.float32)).reshape(24, 8, 8, 128)
+    got = []
+    for m in (a, ref):
+        m.forward(xs, ys)
+        act = m.read(sb.SB_T_ACT, 0, 0, squeeze=False)
+        act[1, 3, 4, 5] = bad
+        m.write(sb.SB_T_ACT, 0, 0, act)
+        m.forward_layers(1, 1)
+        y = [m.read(sb.SB_T_ACT, 1, r) for r in range(2)]
+        for r in range(2):
+            m.write(sb.SB_T_DACT, 1, r, dy)
+        m.backward_layers(1, 1)
+        got.append(y + [m.read(sb.SB_T_GRAD_W, 1), m.read(sb.SB_T_DACT, 0, 0)])
+    for u, v in zip(*got):
+        assert np.array_equal(np.isnan(u), np.isnan(v)) and np.array_equal(np.isinf(u), np.isinf(v))
+        fin = np.isfinite(v)
+        assert np.array_equal(np.sign(u[~fin & ~np.isnan(v)]), np.sign(v[~fin & ~np.isnan(v)]))
+        assert tu.maxrel(u[fin], v[fin]) < 1e-5
+    a.close()
+    ref.close()
