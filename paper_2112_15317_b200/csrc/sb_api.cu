@@ -103,6 +103,11 @@ struct sb_model {
     bool hyper_words = false;         // they have changed from one captured iteration to the next: captures read the words
     int last_dropout = -1;            // index of the network's last dropout layer: its forward kernel is followed by the iteration bump
     bool st_clean = false;     // the chain stream's last kernel belongs to the current forward / backward pass (it cannot have written weights)
+    // Head of a whole pass: the logits layer's narrow kernel computes the loss layer as well (head_ok while such a pass is enqueued;
+    // xent_by_fc is the loss layer it has covered).  The mean of the row losses is a kernel of its own: behind it on the same
+    // stream, or (mean_aside) left to the backward pass, which enqueues it beside the chain.
+    bool head_ok = false, mean_aside = false, mean_pending = false;
+    int xent_by_fc = -1;
     int pooled_by_conv = -1;   // index of the pool layer whose output the conv kernel just before it has already written (same forward call)
     // Set by the multi-stream backward pass while it enqueues the weight side of one conv layer: the layer's split
     // reduces then apply the update themselves (launch_reduce_sgd) once `ev` (the layer's input-gradient kernel, which
@@ -471,6 +476,26 @@ sb_status contract_dgrad(sb_model* m, int i, const char* tag, double flops, doub
     return SB_OK;
 }
 
+// The loss layer (index i) on the model's current rows
+XentArgs xent_args(sb_model* m, int i)
+{
+    const Layer& fc = m->L[i - 1];
+    XentArgs a{};
+    a.logits = (const float*)fc.act; a.labels = m->label_tab; a.b_per_rep = m->cfg.batch_per_replica;
+    a.row_loss = m->row_loss; a.loss = m->loss; a.dZ = fc.dact; a.counter = m->counter;
+    a.B = m->B; a.C = m->L[i].out;
+    if (m->sub_active) {
+        // rows [sub_row0, sub_row0 + B) of the full batch, labels already in sub-iteration order; every row's
+        // gradient carries 1/full_B and the mean loss is taken over all rows written so far and before
+        a.labels = PtrTab{};
+        a.labels.p[0] = m->mod_labels + m->sub_row0;
+        a.b_per_rep = m->B;
+        a.row_loss = m->row_loss + m->sub_row0;
+        a.scale_B = m->full_B; a.loss_base = m->row_loss; a.loss_rows = m->full_B;
+    }
+    return a;
+}
+
 sb_status forward_layer(sb_model* m, int i, cudaStream_t st)
 {
     Layer& l = m->L[i];
@@ -542,6 +567,13 @@ sb_status forward_layer(sb_model* m, int i, cudaStream_t st)
             a.pass = 0; a.X = layer_input(m, i); a.tab = i == 0 ? &m->x_tab : nullptr; a.tab_b = b; a.W = wts;
             a.bias = m->Wm + l.p_b; a.relu = l.relu; a.B = B; a.in_f = l.in_f; a.out_f = l.out_f;
             if (l.kind == SB_FC) a.Y32 = (float*)l.act; else a.Y = l.act;
+            if (m->head_ok && m->have_labels && l.kind == SB_FC) {
+                const XentArgs x = xent_args(m, i + 1);
+                a.xent = &x;
+                L_TRY("fc_narrow_xent", flops, bytes + (double)B * (l.out_f * e + 8.0), launch_fc_narrow(a, bf, st));
+                m->xent_by_fc = i + 1;
+                break;
+            }
             L_TRY("fc_narrow_fwd", flops, bytes, launch_fc_narrow(a, bf, st));
             break;
         }
@@ -561,19 +593,12 @@ sb_status forward_layer(sb_model* m, int i, cudaStream_t st)
     }
     case SB_SOFTMAX_XENT: {
         if (!m->have_labels) return fail(SB_ERR_STATE, "the loss layer needs label pointers");
-        Layer& fc = m->L[i - 1];
-        XentArgs a{};
-        a.logits = (const float*)fc.act; a.labels = m->label_tab; a.b_per_rep = b;
-        a.row_loss = m->row_loss; a.loss = m->loss; a.dZ = fc.dact; a.counter = m->counter;
-        a.B = B; a.C = l.out;
-        if (m->sub_active) {
-            // rows [sub_row0, sub_row0 + B) of the full batch, labels already in sub-iteration order; every row's
-            // gradient carries 1/full_B and the mean loss is taken over all rows written so far and before
-            a.labels = PtrTab{};
-            a.labels.p[0] = m->mod_labels + m->sub_row0;
-            a.b_per_rep = B;
-            a.row_loss = m->row_loss + m->sub_row0;
-            a.scale_B = m->full_B; a.loss_base = m->row_loss; a.loss_rows = m->full_B;
+        const XentArgs a = xent_args(m, i);
+        if (m->xent_by_fc == i) {      // (the logits layer's kernel has computed the row losses and dZ)
+            m->xent_by_fc = -1;
+            if (m->mean_aside) m->mean_pending = true;
+            else L_TRY("loss_mean", 0.0, 4.0 * a.B, launch_loss_mean(a, st));
+            break;
         }
         L_TRY("softmax_xent", 0.0, (double)B * l.out * (4.0 + e) + 8.0 * B, launch_softmax_xent(a, bf, st));
         break;
@@ -1136,14 +1161,15 @@ extern "C" {
 static sb_status forward_pass(sb_model* m, cudaStream_t st)
 {
     m->pooled_by_conv = -1;
+    m->xent_by_fc = -1;
     m->st_clean = false;
-    for (int i = 0; i < m->n_layers; ++i) {
-        const sb_status s = chain_fwd(m, i, st);
-        if (s != SB_OK) return s;
-    }
+    m->head_ok = true;
+    sb_status s = SB_OK;
+    for (int i = 0; i < m->n_layers && s == SB_OK; ++i) s = chain_fwd(m, i, st);
+    m->head_ok = false;
     m->st_clean = false;
     m->pooled_by_conv = -1;
-    return SB_OK;
+    return s;
 }
 
 // sb_forward / whole iterations: inputs, then the pass (by itself: replayed where that pays)
@@ -1170,6 +1196,9 @@ static sb_status weight_side(sb_model* m, int i, cudaStream_t wst, bool classic)
     return s;
 }
 
+// Whether a pass may use streams beside the caller's
+static bool side_streams(const sb_model* m) { return m->n_wstreams > 0 && !m->profiling && !m->debug_sync; }
+
 // Backward pass; with `fuse_update` the SGD update of each layer's parameters is enqueued on the weight-side
 // stream as soon as that layer's gradients are complete and its input gradient (which reads the weights) has
 // been computed, so the bandwidth-bound update overlaps the rest of the backward pass.  Element for element the
@@ -1182,7 +1211,7 @@ static sb_status backward_pass(sb_model* m, cudaStream_t st, bool fuse_update, H
     // while the input-gradient chain is the critical path: the former runs on the model's second stream,
     // ordered by one event per layer ("the gradient w.r.t. this layer's output is ready") and joined at the
     // end.  Profiling and debug-sync modes keep everything on one stream.
-    const bool two_streams = m->n_wstreams > 0 && !m->profiling && !m->debug_sync;
+    const bool two_streams = side_streams(m);
     const bool fuse = fuse_update && two_streams;
     if (updated) *updated = fuse;
     m->st_clean = false;
@@ -1205,6 +1234,11 @@ static sb_status backward_pass(sb_model* m, cudaStream_t st, bool fuse_update, H
             used_streams |= 1u << (i % m->n_wstreams);
             CU_TRY(cudaEventRecord(m->ev_ready[i], st));
             CU_TRY(cudaStreamWaitEvent(wst, m->ev_ready[i], 0));
+            if (m->mean_pending) {
+                cudaStream_t st = wst;   // the launch bracket below records on the stream it launches on
+                m->mean_pending = false;
+                L_TRY("loss_mean", 0.0, 4.0 * m->B, launch_loss_mean(xent_args(m, m->n_layers - 1), st));
+            }
             // Conv layers in a fused pass: the input-gradient kernel is enqueued first and its event recorded, so that the
             // layer's split reduces on the weight stream can wait for it and apply the update themselves.
             static const bool reduce_updates = tune("SB_REDUCE_SGD", 1) != 0;
@@ -1291,7 +1325,9 @@ static sb_status update_all(sb_model* m, Hyper hy, cudaStream_t st)
 }
 static sb_status whole_step(sb_model* m, const void* const* x, const int32_t* const* labels, Hyper hy, void* stream)
 {
+    m->mean_aside = side_streams(m);
     sb_status s = forward_on(m, x, labels, (cudaStream_t)stream, false);
+    m->mean_aside = false;
     if (s != SB_OK) return s;
     bool updated = false;
     s = backward_pass(m, (cudaStream_t)stream, true, hy, &updated);
@@ -1338,6 +1374,8 @@ static sb_status modulo_step_direct(sb_model* m, const void* const* x, const int
         // The FC updates of a sub-iteration run on the weight streams -- folded into the weight-gradient kernels of the large layers,
         // as in the synchronous step -- while the chain goes on; a layer's next forward pass waits for its own update only.
         // (VGG-16 at 32x32, batch 128, K = 4: 138 us a sub-iteration with one update of all FC parameters behind the backward pass.)
+        m->xent_by_fc = -1;
+        m->head_ok = true; m->mean_aside = side_streams(m);
         for (int i = ff; i < m->n_layers && s == SB_OK; ++i) {
             if (k > 0 && updated && has_weights(m->L[i])) {
                 m->st_clean = false;
@@ -1345,6 +1383,8 @@ static sb_status modulo_step_direct(sb_model* m, const void* const* x, const int
             }
             if (s == SB_OK) s = chain_fwd(m, i, st);
         }
+        m->head_ok = m->mean_aside = false;
+        if (k + 1 < K) m->mean_pending = false;     // (the mean over all rows is complete with the last sub-iteration's)
         if (s == SB_OK) s = backward_pass(m, st, true, hy, &updated, m->n_layers - 1, ff, false);
         m->st_clean = false;
         m->B = m->full_B; m->sub_active = false; m->sub_row0 = 0;

@@ -157,6 +157,7 @@ cudaError_t launch_conv_in_fwd(const ConvSimtArgs& a, bool bf16, cudaStream_t st
 int conv_in_wgrad_blocks(int B, int H, int W);
 cudaError_t launch_conv_in_wgrad(const WgradSimtArgs& a, bool bf16, cudaStream_t st);
 
+struct XentArgs;
 // Narrow FC layer (out <= 16): pass 0 forward, 1 weight+bias gradient, 2 input gradient.
 struct FcNarrowArgs {
     int pass;
@@ -166,6 +167,8 @@ struct FcNarrowArgs {
     const void* dY; float* dW; float* db;          // gradient inputs/outputs
     const void* ref; void* dX;                     // dgrad: optional ReLU mask source and output [B,in]
     int B, in_f, out_f;
+    const XentArgs* xent;                          // forward of the logits layer: the loss layer's row losses and dZ in the same kernel
+                                                   // (launch_softmax_xent's bits; the mean loss is left to launch_loss_mean)
 };
 bool fc_narrow_supported(int out_f, int B);
 cudaError_t launch_fc_narrow(const FcNarrowArgs& a, bool bf16, cudaStream_t st);
@@ -210,6 +213,7 @@ struct XentArgs {
     int loss_rows = 0;
 };
 cudaError_t launch_softmax_xent(const XentArgs& a, bool bf16, cudaStream_t st);
+cudaError_t launch_loss_mean(const XentArgs& a, cudaStream_t st);
 
 // Modulo layer as an explicit copy (sub-iteration schedule): R replicas of b rows, K slices of b/K rows each.
 // gather : dst[k*(R*b/K) + r*(b/K) + i] = src[r*b + k*(b/K) + i]   (rows of `row_bytes` bytes, a multiple of 16)

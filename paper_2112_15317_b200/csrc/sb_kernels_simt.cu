@@ -396,6 +396,31 @@ cudaError_t launch_pool_bwd(const PoolBwdArgs& a, bool bf16, cudaStream_t st)
 // Softmax cross-entropy: one warp per row (shuffle max / sum), dZ = (softmax - onehot)/B.
 // The last block to finish adds the row losses in row order, so the mean is deterministic.
 // =============================================================================================
+// mean of the row losses by one warp, in a fixed order: chunks of 32 rows, tree inside
+__device__ __forceinline__ float mean_loss(const float* row_loss, int rows)
+{
+    const int lane = threadIdx.x % 32;
+    float t = 0.f;
+    for (int i0 = 0; i0 < rows; i0 += 32) {
+        float v = (i0 + lane < rows) ? ((volatile const float*)row_loss)[i0 + lane] : 0.f;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        t += v;
+    }
+    return t / (float)rows;
+}
+__global__ void __launch_bounds__(32)
+loss_mean_kernel(const float* __restrict__ row_loss, int rows, float* __restrict__ loss)
+{
+    pdl_prologue();
+    const float t = mean_loss(row_loss, rows);
+    if (threadIdx.x == 0) *loss = t;
+}
+cudaError_t launch_loss_mean(const XentArgs& a, cudaStream_t st)
+{
+    SB_LAUNCH((loss_mean_kernel), 1, 32, 0, st, a.loss_rows > 0 ? a.loss_base : a.row_loss, a.loss_rows > 0 ? a.loss_rows : a.B, a.loss);
+    return cudaGetLastError();
+}
 template <typename T>
 __global__ void __launch_bounds__(256)
 softmax_xent_kernel(const float* __restrict__ logits, PtrTab labels, int b_per_rep, float* __restrict__ row_loss,
@@ -431,14 +456,8 @@ softmax_xent_kernel(const float* __restrict__ logits, PtrTab labels, int b_per_r
     __syncthreads();
     if (last && warp == 0) {
         __threadfence();
-        float t = 0.f;
-        for (int i0 = 0; i0 < loss_rows; i0 += 32) {   // fixed order: chunks of 32 rows, tree inside
-            float v = (i0 + lane < loss_rows) ? ((volatile const float*)loss_base)[i0 + lane] : 0.f;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            t += v;
-        }
-        if (lane == 0) { *loss = t / (float)loss_rows; *counter = 0u; }
+        const float t = mean_loss(loss_base, loss_rows);
+        if (lane == 0) { *loss = t; *counter = 0u; }
     }
 }
 cudaError_t launch_softmax_xent(const XentArgs& a, bool bf16, cudaStream_t st)
@@ -1028,84 +1047,80 @@ cudaError_t launch_conv_in_wgrad(const WgradSimtArgs& a, bool bf16, cudaStream_t
 
 // =============================================================================================
 // Narrow FC layers (out <= 16, e.g. the 10-class logits layer): too narrow for any GEMM tile.
-//   forward : one block per batch row, threads split the reduction, block-wide shuffle reduce
+//   forward : one block per batch row, a warp per output
 //   wgrad   : one thread per input column, dY staged in shared memory
-//   dgrad   : one thread per (row, input column)
+//   dgrad   : one thread per 16 bytes of an input row and two batch rows
 // =============================================================================================
 constexpr int NARROW_MAX = 16;
 
-// Forward: one warp per batch row, 8 rows per block; a lane walks the reduction in steps of 8 values
-// (one 16-byte load of X and of each weight row for bf16), then the warp shuffle-reduces its out_f sums.
 template <typename T> struct Vec8;
 template <> struct Vec8<float> { static constexpr int N = 4; typedef float4 V; };
 template <> struct Vec8<__nv_bfloat16> { static constexpr int N = 8; typedef uint4 V; };
 
-// Block = 2 batch rows x 4 reduction quarters (one warp each).  A lane issues all its 16-byte loads of X and
-// of the out_f weight rows for its slice up front (many loads in flight: the kernel is pure latency), the warp
-// shuffle-reduces, and the 4 quarters of a row are added in order through shared memory.
-template <typename T, bool TAB, int KS, bool VEC>
-__global__ void __launch_bounds__(64 * KS)
+// Forward.  Block = one batch row, a warp per output: the kernel is pure latency, so every lane has eight 16-byte loads in flight and
+// the code is one short loop.  (Two rows a block, the reduction in four slices and all outputs in a lane's registers: 6.5 us for
+// 4096 -> 10 at batch 128 in the replayed VGG-16 iteration; here 4.9 with the softmax.)
+// XENT: softmax cross-entropy of the row by warp 0, with the operations of softmax_xent_kernel in its order, without that kernel's
+// 4.3 us on the chain (most of them the last block's wait for every row loss).
+struct HeadArgs { PtrTab labels; int b_per_rep; float* row_loss; void* dZ; int scale_B; };
+template <typename T, bool TAB, bool VEC, bool XENT>
+__global__ void __launch_bounds__(32 * NARROW_MAX)
 fc_narrow_fwd_kernel(const T* __restrict__ X, PtrTab tab, int tab_b, const T* __restrict__ Wt, const float* __restrict__ bias,
-                     T* __restrict__ Y, float* __restrict__ Y32, int B, int in_f, int out_f, int relu)
+                     T* __restrict__ Y, float* __restrict__ Y32, int in_f, int out_f, int relu, const __grid_constant__ HeadArgs head)
 {
     pdl_prologue();
     constexpr int VN = Vec8<T>::N;
     typedef typename Vec8<T>::V V;
-    __shared__ float s_part[2][KS][NARROW_MAX];
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    const int rl = warp / KS, ks = warp % KS;
-    const int g = blockIdx.x * 2 + rl;
-    const int kq = in_f / KS;                 // reduction elements of this warp (multiple of 32*VN or handled by the tail loop)
-    float acc[NARROW_MAX];
+    __shared__ float s_z[NARROW_MAX];
+    const int j = threadIdx.x / 32, lane = threadIdx.x % 32, g = blockIdx.x;
+    const T* xr = TAB ? (const T*)tab.p[g / tab_b] + (size_t)(g % tab_b) * in_f : X + (size_t)g * in_f;
+    const T* wr = Wt + (size_t)j * in_f;
+    int label = 0;
+    if (XENT && j == 0) label = ((const int32_t*)head.labels.p[g / head.b_per_rep])[g % head.b_per_rep];
+    float acc = 0.f;
+    if (VEC) {
+        // (the host only selects this variant when every row starts 16-byte aligned)
+#pragma unroll 1
+        for (int k0 = lane * VN; k0 < in_f; k0 += 128 * VN) {
+            V xv[4], wv[4];
 #pragma unroll
-    for (int j = 0; j < NARROW_MAX; ++j) acc[j] = 0.f;
-    if (g < B) {
-        const T* xr = (TAB ? (const T*)tab.p[g / tab_b] + (size_t)(g % tab_b) * in_f : X + (size_t)g * in_f) + (size_t)ks * kq;
-        const T* wr = Wt + (size_t)ks * kq;
-        if (VEC) {
-            // 16-byte loads: the host only selects this variant when every row and every slice starts 16-byte aligned
-            for (int k = lane * VN; k + VN <= kq; k += 32 * VN) {
-                const V xv = *(const V*)(xr + k);
-                V wv[NARROW_MAX];
-#pragma unroll
-                for (int j = 0; j < NARROW_MAX; ++j)
-                    if (j < out_f) wv[j] = *(const V*)(wr + (size_t)j * in_f + k);
-#pragma unroll
-                for (int j = 0; j < NARROW_MAX; ++j)
-                    if (j < out_f) {
-#pragma unroll
-                        for (int i = 0; i < VN; ++i) acc[j] = fmaf(ldf((const T*)&xv + i), ldf((const T*)&wv[j] + i), acc[j]);
-                    }
+            for (int u = 0; u < 4; ++u) {
+                const int k = k0 + u * 32 * VN;
+                const V zero = V();
+                xv[u] = k < in_f ? *(const V*)(xr + k) : zero;
+                wv[u] = k < in_f ? *(const V*)(wr + k) : zero;
             }
-        } else {
-            for (int k = lane; k < kq; k += 32) {
-                const float xv = ldf(xr + k);
 #pragma unroll
-                for (int j = 0; j < NARROW_MAX; ++j)
-                    if (j < out_f) acc[j] = fmaf(xv, ldf(wr + (size_t)j * in_f + k), acc[j]);
-            }
+            for (int u = 0; u < 4; ++u)
+                if (k0 + u * 32 * VN < in_f)
+#pragma unroll
+                    for (int i = 0; i < VN; ++i) acc = fmaf(ldf((const T*)&xv[u] + i), ldf((const T*)&wv[u] + i), acc);
         }
+    } else {
+        for (int k = lane; k < in_f; k += 32) acc = fmaf(ldf(xr + k), ldf(wr + k), acc);
     }
 #pragma unroll
-    for (int j = 0; j < NARROW_MAX; ++j) {
-        float v = acc[j];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) s_part[rl][ks][j] = v;
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) {
+        float v = bias[j] + acc;
+        if (relu && !(v > 0.f)) v = 0.f;
+        if (Y32) Y32[(size_t)g * out_f + j] = v;
+        if (Y) stf(Y + (size_t)g * out_f + j, v);
+        s_z[j] = v;
     }
+    if (!XENT) return;
     __syncthreads();
-    if (threadIdx.x < 2 * NARROW_MAX) {
-        const int r2 = threadIdx.x / NARROW_MAX, j = threadIdx.x % NARROW_MAX;
-        const int g2 = blockIdx.x * 2 + r2;
-        if (g2 < B && j < out_f) {
-            float v = bias[j];
+    if (j != 0) return;
+    const float z = lane < out_f ? s_z[lane] : -INFINITY;
+    float m = fmaxf(-INFINITY, z);
 #pragma unroll
-            for (int q = 0; q < KS; ++q) v += s_part[r2][q][j];
-            if (relu && !(v > 0.f)) v = 0.f;
-            if (Y32) Y32[(size_t)g2 * out_f + j] = v;
-            if (Y) stf(Y + (size_t)g2 * out_f + j, v);
-        }
-    }
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    float s = lane < out_f ? expf(z - m) : 0.f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    const float lse = m + logf(s), invB = 1.0f / (float)head.scale_B;
+    if (lane < out_f) stf((T*)head.dZ + (size_t)g * out_f + lane, (expf(z - lse) - (lane == label ? 1.f : 0.f)) * invB);
+    if (lane == 0) head.row_loss[g] = (label >= 0 && label < out_f) ? lse - s_z[label] : 0.f;
 }
 
 // Weight + bias gradient: block = 32 input columns x 8 row lanes; lane l sums batch rows l, l+8, ... for its
@@ -1174,6 +1189,48 @@ fc_narrow_dgrad_kernel(const T* __restrict__ dY, const T* __restrict__ Wt, const
     stf(dX + (size_t)g * in_f + i, acc);
 }
 
+// By 16-byte accesses: a thread takes VN columns of ROWS batch rows (same products in the same order as the kernel above; 4096 columns at
+// batch 128, a column and a row per thread: 6.5 us in the replayed iteration, here 3.6).
+template <typename T, int ROWS>
+__global__ void __launch_bounds__(64)
+fc_narrow_dgrad_vec_kernel(const T* __restrict__ dY, const T* __restrict__ Wt, const T* __restrict__ ref, T* __restrict__ dX, int B, int in_f, int out_f)
+{
+    pdl_prologue();
+    constexpr int VN = Vec8<T>::N;
+    typedef typename Vec8<T>::V V;
+    const int i = (blockIdx.x * 64 + threadIdx.x) * VN, g0 = blockIdx.y * ROWS;
+    if (i >= in_f) return;
+    V r[ROWS];
+    float acc[ROWS][VN];
+#pragma unroll
+    for (int u = 0; u < ROWS; ++u) {
+        if (ref != nullptr && g0 + u < B) r[u] = *(const V*)(ref + (size_t)(g0 + u) * in_f + i);
+#pragma unroll
+        for (int k = 0; k < VN; ++k) acc[u][k] = 0.f;
+    }
+#pragma unroll 4
+    for (int j = 0; j < out_f; ++j) {
+        const V w = *(const V*)(Wt + (size_t)j * in_f + i);
+#pragma unroll
+        for (int u = 0; u < ROWS; ++u) {
+            const float d = ldf(dY + (size_t)min(g0 + u, B - 1) * out_f + j);
+#pragma unroll
+            for (int k = 0; k < VN; ++k) acc[u][k] = fmaf(d, ldf((const T*)&w + k), acc[u][k]);
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < ROWS; ++u) {
+        if (g0 + u >= B) break;
+        V o;
+#pragma unroll
+        for (int k = 0; k < VN; ++k) {
+            if (ref != nullptr && !(ldf((const T*)&r[u] + k) > 0.f)) acc[u][k] = 0.f;
+            stf((T*)&o + k, acc[u][k]);
+        }
+        *(V*)(dX + (size_t)(g0 + u) * in_f + i) = o;
+    }
+}
+
 bool fc_narrow_supported(int out_f, int B) { return out_f <= NARROW_MAX && (size_t)B * out_f * 4 <= 24 * 1024; }
 
 template <typename T>
@@ -1183,23 +1240,26 @@ static cudaError_t launch_fc_narrow_t(const FcNarrowArgs& a, cudaStream_t st)
     if (a.tab) tab = *a.tab;
     const int tb = a.tab_b > 0 ? a.tab_b : 1;
     if (a.pass == 0) {
-        const int blocks = (a.B + 1) / 2;
-        // 16-byte loads need every row (and every quarter of a row) to start on a 16-byte boundary
-        const bool aligned_ptrs = (((uintptr_t)a.W | (uintptr_t)a.X) & 15) == 0 && !a.tab;
-        const bool vec = aligned_ptrs && a.in_f % Vec8<T>::N == 0;
-        const bool quarters = vec && a.in_f % (4 * Vec8<T>::N) == 0;
-#define SB_NF(TABF, KS, VECF) SB_LAUNCH((fc_narrow_fwd_kernel<T, TABF, KS, VECF>), blocks, 64 * KS, 0, st,  \
-            (const T*)a.X, tab, tb, (const T*)a.W, a.bias, (T*)a.Y, a.Y32, a.B, a.in_f, a.out_f, a.relu)
-        if (quarters) SB_NF(false, 4, true);
-        else if (vec) SB_NF(false, 1, true);
-        else if (a.tab) SB_NF(true, 1, false);
-        else SB_NF(false, 1, false);
+        const bool vec = (((uintptr_t)a.W | (uintptr_t)a.X) & 15) == 0 && !a.tab && a.in_f % Vec8<T>::N == 0;
+        HeadArgs head{};
+        if (a.xent) head = HeadArgs{a.xent->labels, a.xent->b_per_rep, a.xent->row_loss, a.xent->dZ, a.xent->scale_B > 0 ? a.xent->scale_B : a.xent->B};
+#define SB_NFX(TABF, VECF, XENTF) SB_LAUNCH((fc_narrow_fwd_kernel<T, TABF, VECF, XENTF>), a.B, 32 * a.out_f, 0, st,  \
+            (const T*)a.X, tab, tb, (const T*)a.W, a.bias, (T*)a.Y, a.Y32, a.in_f, a.out_f, a.relu, head)
+#define SB_NF(TABF, VECF) do { if (a.xent) SB_NFX(TABF, VECF, true); else SB_NFX(TABF, VECF, false); } while (0)
+        if (vec) SB_NF(false, true);
+        else if (a.tab) SB_NF(true, false);
+        else SB_NF(false, false);
 #undef SB_NF
+#undef SB_NFX
     } else if (a.pass == 1) {
         const size_t smem = (size_t)a.B * a.out_f * 4 + 8 * 32 * NARROW_MAX * 4;
         const int blocks = (a.in_f + 31) / 32;
         if (a.tab) SB_LAUNCH((fc_narrow_wgrad_kernel<T, true>), blocks, 256, smem, st, nullptr, tab, tb, (const T*)a.dY, a.dW, a.db, a.B, a.in_f, a.out_f);
         else SB_LAUNCH((fc_narrow_wgrad_kernel<T, false>), blocks, 256, smem, st, (const T*)a.X, tab, tb, (const T*)a.dY, a.dW, a.db, a.B, a.in_f, a.out_f);
+    } else if (a.in_f % Vec8<T>::N == 0 && (((uintptr_t)a.W | (uintptr_t)a.ref | (uintptr_t)a.dX) & 15) == 0) {
+        const int bx = (a.in_f / Vec8<T>::N + 63) / 64;
+        if (a.B > 64) SB_LAUNCH((fc_narrow_dgrad_vec_kernel<T, 2>), dim3(bx, (a.B + 1) / 2), 64, 0, st, (const T*)a.dY, (const T*)a.W, (const T*)a.ref, (T*)a.dX, a.B, a.in_f, a.out_f);
+        else SB_LAUNCH((fc_narrow_dgrad_vec_kernel<T, 1>), dim3(bx, a.B), 64, 0, st, (const T*)a.dY, (const T*)a.W, (const T*)a.ref, (T*)a.dX, a.B, a.in_f, a.out_f);
     } else {
         dim3 grid((a.in_f + 255) / 256, a.B);
         SB_LAUNCH((fc_narrow_dgrad_kernel<T>), grid, 256, 0, st, (const T*)a.dY, (const T*)a.W, (const T*)a.ref, (T*)a.dX, a.in_f, a.out_f);
