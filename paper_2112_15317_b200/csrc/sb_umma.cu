@@ -2712,7 +2712,7 @@ static double plan_cost(int bn, int s, int n_cols, long m_tiles, int k_iters)
     const double mb_us = 0.5;
     return waves * (cdiv_i(k_iters, s) * t_iter * (per_sm > 1.0 ? 1.6 : 1.0) + 3.0) + (s > 1 ? 4.0 + mb_us * partial_mb : 0.0);
 }
-static TilePlan plan_tiles(int n_cols, long m_tiles, int k_iters, bool backward, bool force_pair)
+static TilePlan plan_tiles(int n_cols, long m_tiles, int k_iters, bool backward, bool force_pair, bool fc = false)
 {
     TilePlan t;
     int best_bn = 64, best_s = 1;
@@ -2743,7 +2743,11 @@ static TilePlan plan_tiles(int n_cols, long m_tiles, int k_iters, bool backward,
     static const bool fwd_too = tune("SB_FWD_COHABIT", 0) != 0;
     // (a grid that leaves SMs idle need not share its SMs: the other stream's CTAs find free ones; SB_COHABIT_MIN_CTAS)
     static const long cohabit_min = (long)tune("SB_COHABIT_MIN_CTAS", 100);
-    if ((backward || fwd_too) && bwd_cohabit() && t.bn != 192 && tiles * t.splits >= cohabit_min && st > cohabit_stages(t.bn)) st = cohabit_stages(t.bn);
+    // (the data gradient of an FC layer in one wave keeps its ring and with it one CTA per SM: two of 128 CTAs on some SMs and none on
+    // others made 4096 -> 4096 at batch 32 take 15 us where 9 do, depending on which SMs the kernel before it left free; only the narrow
+    // layer's small blocks run beside it)
+    const bool one_wave = fc && tiles * t.splits <= 148;
+    if ((backward || fwd_too) && !one_wave && bwd_cohabit() && t.bn != 192 && tiles * t.splits >= cohabit_min && st > cohabit_stages(t.bn)) st = cohabit_stages(t.bn);
     // Grids of more than one CTA per SM: measured, the co-residency of CTAs (their set-up, first loads and
     // epilogues overlap one another's main loops) is worth more than ring depth -- the 1024-CTA 64-wide layer runs
     // 28 us with 2 stages (4 CTAs per SM) against 37 us with 4 and 60 us with 8; beyond 3 stages no layer gains.
@@ -3155,7 +3159,7 @@ static FcGeom fc_geom(const LayerView& lv, int B, bool force_pair)
     FcGeom g;
     g.m_tiles = cdiv_i(B, 128);
     g.fwd = plan_tiles(lv.out_f, g.m_tiles, cdiv_i(lv.in_f, 64), false, force_pair);
-    g.dgrad = plan_tiles(lv.in_f, g.m_tiles, cdiv_i(lv.out_f, 64), true, force_pair);
+    g.dgrad = plan_tiles(lv.in_f, g.m_tiles, cdiv_i(lv.out_f, 64), true, force_pair, true);
     return g;
 }
 
