@@ -57,6 +57,16 @@ __device__ __forceinline__ void tma_load_4d(const CUtensorMap* map, void* dst, u
         ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
         : "memory");
 }
+// the same for data that is read once: the first to leave L2
+__device__ __forceinline__ void tma_load_4d_stream(const CUtensorMap* map, void* dst, uint64_t* bar, int c0, int c1, int c2, int c3)
+{
+    asm volatile(
+        "{\n\t.reg .b64 pol;\n\t"
+        "createpolicy.fractional.L2::evict_first.b64 pol, 1.0;\n\t"
+        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4, %5, %6}], [%2], pol;\n\t}"
+        ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+        : "memory");
+}
 // Predicated forms for a converged producer warp: every lane executes the slot, the lane with `elected` != 0 issues.
 __device__ __forceinline__ void mbar_expect_tx_el(uint32_t bar_saddr, uint32_t bytes, uint32_t elected)
 {

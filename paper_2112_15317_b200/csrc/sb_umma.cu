@@ -221,8 +221,8 @@ __device__ __forceinline__ void upd_request_slab(const CUtensorMap* mapW, const 
 {
     // one thread: a 64-column x 128-row box of w and one of v (rows past the matrix read as zeros and are never stored)
     mbar_expect_tx(bar, (uint32_t)UPD_SLAB_BYTES);
-    tma_load_4d(mapW, buf, bar, col, m0, 0, 0);
-    tma_load_4d(mapV, buf + 32768, bar, col, m0, 0, 0);
+    tma_load_4d_stream(mapW, buf, bar, col, m0, 0, 0);
+    tma_load_4d_stream(mapV, buf + 32768, bar, col, m0, 0, 0);
 }
 template <int BN>
 __device__ __forceinline__ bool wgrad_sweep_update_epilogue(const UmmaParams& p, const CUtensorMap* mapW, const CUtensorMap* mapV, uint32_t taddr,
