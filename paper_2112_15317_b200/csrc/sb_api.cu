@@ -151,6 +151,7 @@ struct sb_model {
         PtrTab x{}, labels{};
         Hyper hy{};            // captured with these values, or with the device words
         bool warmed = false;
+        bool priorities = false;   // its launches carry priorities
         bool fits(float lr, float mu) const { return hy.dev || (hy.lr == lr && hy.mu == mu); }
     };
     StepGraph g_dev, g_mod;
@@ -1032,8 +1033,10 @@ sb_status sb_model_destroy(sb_model* m)
 static sb_status chain_fwd(sb_model* m, int i, cudaStream_t st)
 {
     weights_first() = m->st_clean ? 1 : 0;
+    launch_priority() = m->sub_active ? -2 : 0;
     const int64_t l0 = m->launches;
     const sb_status s = forward_layer(m, i, st);
+    launch_priority() = 0;
     weights_first() = 0;
     if (m->launches > l0) m->st_clean = true;
     return s;
@@ -1041,8 +1044,10 @@ static sb_status chain_fwd(sb_model* m, int i, cudaStream_t st)
 static sb_status chain_bwd(sb_model* m, int i, cudaStream_t st, int part)
 {
     weights_first() = m->st_clean ? 1 : 0;
+    launch_priority() = m->sub_active ? -2 : 0;
     const int64_t l0 = m->launches;
     const sb_status s = backward_layer(m, i, st, part);
+    launch_priority() = 0;
     weights_first() = 0;
     if (m->launches > l0) m->st_clean = true;
     return s;
@@ -1108,7 +1113,7 @@ static sb_status end_capture(sb_model::StepGraph& G, cudaStream_t st)
         e = cudaGraphExecUpdate(G.exec, graph, &info);
         if (e != cudaSuccess) { cudaGetLastError(); cudaGraphExecDestroy(G.exec); G.exec = nullptr; }
     }
-    if (e != cudaSuccess) e = cudaGraphInstantiate(&G.exec, graph, 0);
+    if (e != cudaSuccess) e = cudaGraphInstantiate(&G.exec, graph, G.priorities ? cudaGraphInstantiateFlagUseNodePriority : 0);
     cudaGraphDestroy(graph);
     if (e != cudaSuccess) { G.exec = nullptr; return fail(SB_ERR_CUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(e)); }
     return SB_OK;
@@ -1191,7 +1196,10 @@ sb_status sb_forward(sb_model* m, const void* const* x, const int32_t* const* la
 static sb_status weight_side(sb_model* m, int i, cudaStream_t wst, bool classic)
 {
     pdl_classic() = classic ? 1 : 0;
+    // (sub-iterations: the first FC layer's update goes before those of the large layers above it, see modulo_step_direct)
+    if (m->sub_active && i == m->first_fc) launch_priority() = -1;
     const sb_status s = backward_layer(m, i, wst, SIDE_W);
+    launch_priority() = 0;
     pdl_classic() = 0;
     return s;
 }
@@ -1522,6 +1530,7 @@ sb_status sb_modulo_step(sb_model* m, const void* const* x, const int32_t* const
 {
     if (!m) return fail(SB_ERR_INVALID_ARG, "null model");
     if (!(m->cfg.flags & SB_FLAG_MODULO_SCHEDULE)) return fail(SB_ERR_STATE, "the model was created without SB_FLAG_MODULO_SCHEDULE");
+    m->g_mod.priorities = true;
     sb_status s = graph_replay(m, m->g_mod, modulo_step_direct, x, labels, lr, momentum, stream);
     if (s == SB_OK) m->have_fwd = false;
     return s;

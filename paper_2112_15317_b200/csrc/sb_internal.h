@@ -48,6 +48,9 @@ inline bool pdl_enabled()
     static const bool on = [] { const char* e = getenv("SB_PDL"); return !(e && e[0] == '0'); }();
     return on && !pdl_classic();
 }
+// Scheduling priority of the calling thread's next launches (0 = least, negative before it): which of the kernels that are ready gets
+// the SMs another one's finished blocks leave.  In a graph it counts where the graph is instantiated with its nodes' priorities.
+inline int& launch_priority() { static thread_local int p = 0; return p; }
 template <typename... KArgs, typename... Args>
 inline cudaError_t pdl_launch(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args)
 {
@@ -56,11 +59,18 @@ inline cudaError_t pdl_launch(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute at[2];
+    int n = 0;
+    if (pdl_enabled()) {
+        at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (launch_priority() != 0) {
+        at[n].id = cudaLaunchAttributePriority;
+        at[n++].val.priority = launch_priority();
+    }
     cfg.attrs = at;
-    cfg.numAttrs = pdl_enabled() ? 1 : 0;
+    cfg.numAttrs = n;
     return cudaLaunchKernelEx(&cfg, kern, KArgs(std::forward<Args>(args))...);
 }
 // Raises a kernel's dynamic shared-memory limit, once per device (the attribute belongs to the device's copy of the function).
