@@ -108,6 +108,8 @@ struct sb_model {
     // stream, or (mean_aside) left to the backward pass, which enqueues it beside the chain.
     bool head_ok = false, mean_aside = false, mean_pending = false;
     int xent_by_fc = -1;
+    int bwd_lo = 1 << 30;      // lowest layer of the backward call that is being enqueued
+    int unpooled = -1;         // index of the pool layer whose input gradient the layer above has already written (same backward call)
     int pooled_by_conv = -1;   // index of the pool layer whose output the conv kernel just before it has already written (same forward call)
     // Set by the multi-stream backward pass while it enqueues the weight side of one conv layer: the layer's split
     // reduces then apply the update themselves (launch_reduce_sgd) once `ev` (the layer's input-gradient kernel, which
@@ -497,6 +499,28 @@ XentArgs xent_args(sb_model* m, int i)
     return a;
 }
 
+// The pool layer above conv layer i (its split reduction may pool in the same pass), or below layer i (whose split data gradient may
+// lead on through it: only where the pool layer belongs to the same backward call); p / dx == nullptr: there is none.
+SplitPool pool_above(sb_model* m, int i)
+{
+    SplitPool o{};
+    if (i + 1 < m->n_layers && m->L[i + 1].kind == SB_MAXPOOL2) {
+        const Layer& pl = m->L[i + 1];
+        o.H = pl.H; o.W = pl.W; o.C = pl.Cin; o.p = pl.act; o.idx = pl.idx;
+    }
+    return o;
+}
+SplitPool pool_below(sb_model* m, int i)
+{
+    SplitPool o{};
+    if (i >= 2 && i - 1 >= m->bwd_lo && !m->L[i].dbelow_override && m->L[i - 1].kind == SB_MAXPOOL2) {
+        const Layer &pl = m->L[i - 1], &cl = m->L[i - 2];
+        o.H = pl.H; o.W = pl.W; o.C = pl.Cin; o.idx = pl.idx; o.dx = cl.dact;
+        o.mask = cl.kind == SB_CONV3X3_RELU ? pl.act : nullptr;
+    }
+    return o;
+}
+
 sb_status forward_layer(sb_model* m, int i, cudaStream_t st)
 {
     Layer& l = m->L[i];
@@ -513,9 +537,13 @@ sb_status forward_layer(sb_model* m, int i, cudaStream_t st)
         const double bytes = pix * l.Cin * e + (double)l.n_w * e + pix * l.Cout * e;
         if (l.um.fwd.enabled) {
             const double pool_bytes = l.um.pool_fused ? pix / 4.0 * l.Cout * (e + 1.0) : 0.0;
-            U_TRY("conv_fwd_umma", flops, bytes + pool_bytes, umma_conv_fwd(m, i, st));
+            SplitPool offer = pool_above(m, i);
+            split_pool() = offer.p ? &offer : nullptr;
+            const sb_status us = [&]() -> sb_status { U_TRY("conv_fwd_umma", flops, bytes + pool_bytes, umma_conv_fwd(m, i, st)); return SB_OK; }();
+            split_pool() = nullptr;
+            if (us != SB_OK) return us;
             ++m->launches;
-            if (l.um.pool_fused) m->pooled_by_conv = i + 1;
+            if (l.um.pool_fused || offer.done) m->pooled_by_conv = i + 1;
             break;
         }
         sb_status fs = SB_OK;
@@ -525,7 +553,14 @@ sb_status forward_layer(sb_model* m, int i, cudaStream_t st)
         a.B = B; a.H = l.H; a.W = l.W; a.Cin = l.Cin; a.Cout = l.Cout; a.relu = 1;
         if (l.thin_input && l.um.conv_in) L_TRY("conv_in_fwd_umma", flops, bytes, launch_conv_in_fwd_umma(a, l.um.fwd.mapA, m->status, st));
         else if (l.thin_input) L_TRY("conv_in_fwd", flops, bytes, launch_conv_in_fwd(a, bf, st));
-        else if ((fs = contract_forward(m, i, "conv_fwd_simt", flops, bytes, st)) != SB_OK) return fs;
+        else {
+            SplitPool offer = pool_above(m, i);
+            split_pool() = offer.p ? &offer : nullptr;
+            fs = contract_forward(m, i, "conv_fwd_simt", flops, bytes, st);
+            split_pool() = nullptr;
+            if (fs != SB_OK) return fs;
+            if (offer.done) m->pooled_by_conv = i + 1;
+        }
         break;
     }
     case SB_MAXPOOL2: {
@@ -705,12 +740,17 @@ sb_status backward_layer(sb_model* m, int i, cudaStream_t st, int part = SIDE_BO
         if (want_in_grad && (part & SIDE_D)) {
             // shard-layer / modulo-layer backward: dX = sum_j dY_j W_j, rows stay with their replica
             const double bytes = act_bytes + (double)l.n_w * e + (below_relu ? (double)B * l.in_f * e : 0.0);
+            SplitPool offer = pool_below(m, i);
+            split_pool() = offer.dx ? &offer : nullptr;
             if (l.um.dgrad.enabled) {
-                U_TRY("fc_dgrad_umma", flops, bytes, umma_fc_dgrad(m, i, st));
+                fs = [&]() -> sb_status { U_TRY("fc_dgrad_umma", flops, bytes, umma_fc_dgrad(m, i, st)); return SB_OK; }();
                 ++m->launches;
             } else {
-                if ((fs = contract_dgrad(m, i, "fc_dgrad_simt", flops, bytes, d_below, below_relu ? layer_input(m, i) : nullptr, st)) != SB_OK) return fs;
+                fs = contract_dgrad(m, i, "fc_dgrad_simt", flops, bytes, d_below, below_relu ? layer_input(m, i) : nullptr, st);
             }
+            split_pool() = nullptr;
+            if (fs != SB_OK) return fs;
+            if (offer.done) m->unpooled = i - 1;
         }
         break;
     }
@@ -725,6 +765,7 @@ sb_status backward_layer(sb_model* m, int i, cudaStream_t st, int part = SIDE_BO
     }
     case SB_MAXPOOL2: {
         if (!(part & SIDE_D)) break;
+        if (m->unpooled == i) { m->unpooled = -1; break; }      // the layer above's split reduce has written it
         PoolBwdArgs a{l.dact, l.idx, below_relu ? l.act : nullptr, d_below, B, l.H, l.W, l.Cin};
         const double pooled = (double)B * l.out_per_img;
         L_TRY("pool_bwd", 0.0, pooled * (e + 1 + (below_relu ? e : 0.0) + 4 * e), launch_pool_bwd(a, bf, st));
@@ -787,12 +828,17 @@ sb_status backward_layer(sb_model* m, int i, cudaStream_t st, int part = SIDE_BO
         }
         if (want_in_grad && (part & SIDE_D)) {
             const double bytes = pix * (l.Cin + l.Cout) * e + (double)l.n_w * e + (below_relu ? pix * l.Cin * e : 0.0);
+            SplitPool offer = pool_below(m, i);
+            split_pool() = offer.dx ? &offer : nullptr;
             if (l.um.dgrad.enabled) {
-                U_TRY("conv_dgrad_umma", flops, bytes, umma_conv_dgrad(m, i, st));
+                fs = [&]() -> sb_status { U_TRY("conv_dgrad_umma", flops, bytes, umma_conv_dgrad(m, i, st)); return SB_OK; }();
                 ++m->launches;
             } else {
-                if ((fs = contract_dgrad(m, i, "conv_dgrad_simt", flops, bytes, d_below, below_relu ? m->L[i - 1].act : nullptr, st)) != SB_OK) return fs;
+                fs = contract_dgrad(m, i, "conv_dgrad_simt", flops, bytes, d_below, below_relu ? m->L[i - 1].act : nullptr, st);
             }
+            split_pool() = nullptr;
+            if (fs != SB_OK) return fs;
+            if (offer.done) m->unpooled = i - 1;
         }
         break;
     }
@@ -1077,12 +1123,12 @@ sb_status sb_backward_layers(sb_model* m, int32_t last, int32_t first, void* str
     if (!m) return fail(SB_ERR_INVALID_ARG, "null model");
     if (first < 0 || last >= m->n_layers || first > last) return fail(SB_ERR_INVALID_ARG, "bad layer range %d..%d", last, first);
     m->st_clean = false;
-    for (int i = last; i >= first; --i) {
-        sb_status s = chain_bwd(m, i, (cudaStream_t)stream, SIDE_BOTH);
-        if (s != SB_OK) return s;
-    }
+    m->bwd_lo = first; m->unpooled = -1;
+    sb_status s = SB_OK;
+    for (int i = last; i >= first && s == SB_OK; --i) s = chain_bwd(m, i, (cudaStream_t)stream, SIDE_BOTH);
+    m->bwd_lo = 1 << 30;
     m->st_clean = false;
-    return SB_OK;
+    return s;
 }
 
 static bool same_ptrs(const PtrTab& a, const PtrTab& b, int n)
@@ -1215,6 +1261,11 @@ static bool side_streams(const sb_model* m) { return m->n_wstreams > 0 && !m->pr
 static sb_status backward_pass(sb_model* m, cudaStream_t st, bool fuse_update, Hyper hy, bool* updated, int hi = -1, int lo = 0, bool join = true)
 {
     if (hi < 0) hi = m->n_layers - 1;     // layers hi .. lo, top down
+    struct Range {                        // (this call's layers, see pool_below)
+        sb_model* m;
+        Range(sb_model* m_, int lo_) : m(m_) { m->bwd_lo = lo_; m->unpooled = -1; }
+        ~Range() { m->bwd_lo = 1 << 30; }
+    } range(m, lo);
     // The weight-gradient work of a layer (and its split reduce) only has to be finished before the update,
     // while the input-gradient chain is the critical path: the former runs on the model's second stream,
     // ordered by one event per layer ("the gradient w.r.t. this layer's output is ready") and joined at the

@@ -267,4 +267,11 @@ struct SplitKEpiArgs {
 };
 cudaError_t launch_splitk_epilogue(const SplitKEpiArgs& a, bool bf16, cudaStream_t st);
 
+// Pooling next to a contraction, offered by the calling thread around its launch: where the reduction is split, the epilogue kernel of the
+// split sums does it in the same pass and sets `done`; elsewhere the offer is left untouched.  H, W, C are the pool layer's input.
+//   forward (dx == nullptr): the result is that input; p and idx are the pool layer's output
+//   backward: the result is the gradient of the pool layer's output; idx and mask (its output, or nullptr) lead it on to dx
+struct SplitPool { int H, W, C; void* p; uint8_t* idx; const void* mask; void* dx; bool done; };
+inline SplitPool*& split_pool() { static thread_local SplitPool* offer = nullptr; return offer; }
+
 }  // namespace sb
