@@ -667,26 +667,27 @@ sb_status backward_layer(sb_model* m, int i, cudaStream_t st, int part = SIDE_BO
     const bool fuse = m->fuse.on && (part & SIDE_W) && !(part & SIDE_D) && l.n_w % 4 == 0 && l.n_b % 4 == 0 && l.p_w % 4 == 0 && l.p_b % 4 == 0;
     // (in_place: with S = 1 the kernel wrote the gradient into the arena itself; the input-layer kernels always write
     // partial buffers, so a single one still has to be carried over)
-    auto finish = [&](const float* src, size_t stride, size_t goff, size_t n, int S, bool in_place = true) -> sb_status {
+    auto finish = [&](const float* src, size_t stride, size_t goff, size_t n, int S, bool in_place = true, Gap gap = Gap{}) -> sb_status {
         const bool reduce = S > 1 || !in_place;
         if (!fuse) {
-            if (reduce) L_TRY("split_reduce", 0.0, (double)n * 4.0 * (S + 1), launch_reduce_partials(src, stride, m->Gm + goff, n, S, st));
+            if (reduce) L_TRY("split_reduce", 0.0, (double)n * 4.0 * (S + 1), launch_reduce_partials(src, stride, m->Gm + goff, n, S, st, gap));
             return SB_OK;
         }
         if (!m->fuse.waited) { CU_TRY(cudaStreamWaitEvent(st, m->fuse.ev, 0)); m->fuse.waited = true; }
         __nv_bfloat16* sh = m->Sm ? m->Sm + goff : nullptr;
         if (reduce)
             L_TRY("split_reduce_sgd", 0.0, (double)n * (4.0 * S + (m->bf16 ? 18.0 : 16.0)),
-                  launch_reduce_sgd(src, stride, n, S, m->Wm + goff, m->Vm + goff, sh, m->fuse.hy, st));
+                  launch_reduce_sgd(src, stride, n, S, m->Wm + goff, m->Vm + goff, sh, m->fuse.hy, st, gap));
         else
             L_TRY("sgd", 0.0, (double)n * (m->bf16 ? 22.0 : 20.0), launch_sgd(m->Wm + goff, m->Vm + goff, m->Gm + goff, sh, n, m->fuse.hy, st));
         m->fuse.covered += n;
         return SB_OK;
     };
-    // weights and bias gradient of a CUDA-core contraction: S > 1 copies of [n_w][n_b] at `src`
-    auto finish_both = [&](const float* src, int S) -> sb_status {
+    // weights and bias gradient together: S copies of [n_w][n_b] at `src` (in the arenas the bias may lie behind some padding)
+    auto finish_both = [&](const float* src, int S, bool in_place = true) -> sb_status {
         const size_t stride = l.n_w + l.n_b;
-        if (l.p_b == l.p_w + l.n_w) return finish(src, stride, l.p_w, stride, S);
+        if (l.p_b == l.p_w + l.n_w) return finish(src, stride, l.p_w, stride, S, in_place);
+        if (S > 1 || !in_place) return finish(src, stride, l.p_w, stride, S, in_place, Gap{l.n_w, l.p_b - l.p_w - l.n_w});
         const sb_status s = finish(src, stride, l.p_w, l.n_w, S);
         return s != SB_OK ? s : finish(src + l.n_w, stride, l.p_b, l.n_b, S);
     };
@@ -783,18 +784,11 @@ sb_status backward_layer(sb_model* m, int i, cudaStream_t st, int part = SIDE_BO
             a.x = layer_input(m, i); a.tab = i == 0 ? &m->x_tab : nullptr; a.b_per_rep = b;
             a.dy = l.dact; a.part = ws_w; a.B = B; a.H = l.H; a.W = l.W; a.Cin = l.Cin; a.Cout = l.Cout;
             const int nb = l.um.conv_in ? conv_in_umma_wgrad_blocks(B, l.H, l.W, l.Cin) : conv_in_wgrad_blocks(B, l.H, l.W);
-            const size_t stride = l.n_w + l.n_b;
             if (l.um.conv_in)
                 L_TRY("conv_in_wgrad_umma", flops, pix * (l.Cin + l.Cout) * e + (double)l.n_w * 4.0, launch_conv_in_wgrad_umma(a, l.um.wgrad.mapA, m->status, st));
             else
                 L_TRY("conv_in_wgrad", flops, pix * (l.Cin + l.Cout) * e + (double)l.n_w * 4.0, launch_conv_in_wgrad(a, bf, st));
-            if (l.p_b == l.p_w + l.n_w) {
-                // the bias vector directly follows the weights in the gradient arena, as it does in a partial buffer
-                if ((fs = finish(ws_w, stride, l.p_w, stride, nb, false)) != SB_OK) return fs;
-            } else {
-                if ((fs = finish(ws_w, stride, l.p_w, l.n_w, nb, false)) != SB_OK) return fs;
-                if ((fs = finish(ws_w + l.n_w, stride, l.p_b, l.n_b, nb, false)) != SB_OK) return fs;
-            }
+            if ((fs = finish_both(ws_w, nb, false)) != SB_OK) return fs;
         } else if (l.um.wgrad.enabled) {
             int S = 1;
             float* part = nullptr;

@@ -185,11 +185,17 @@ cudaError_t launch_fc_narrow(const FcNarrowArgs& a, bool bf16, cudaStream_t st);
 
 // part[s][n] = sum over the rows of split s of in[row][n] (bf16, N a multiple of 8).
 cudaError_t launch_colsum(const void* in, float* part, int M, int N, int splits, cudaStream_t st);
+// Elements from `at` on lie `by` further on where a reduce writes (or updates) them: a layer's bias vector behind the padding of its weights.
+struct Gap {
+    size_t at = 0, by = 0;
+    __host__ __device__ size_t over(size_t i) const { return i < at ? i : i + by; }
+    bool by4() const { return at % 4 == 0 && by % 4 == 0; }
+};
 // out[i] = sum_{s<splits} part[s*stride + i], s ascending.
-cudaError_t launch_reduce_partials(const float* part, size_t stride, float* out, size_t n, int splits, cudaStream_t st);
+cudaError_t launch_reduce_partials(const float* part, size_t stride, float* out, size_t n, int splits, cudaStream_t st, Gap gap = Gap{});
 // the same ordered sum, consumed at once by the SGD step of the n parameters at w / v (shadow: their bf16 copies or nullptr)
 cudaError_t launch_reduce_sgd(const float* part, size_t stride, size_t n, int splits, float* w, float* v, __nv_bfloat16* shadow,
-                              Hyper hy, cudaStream_t st);
+                              Hyper hy, cudaStream_t st, Gap gap = Gap{});
 
 struct PoolArgs {
     const void* x;  // [B,H,W,C]

@@ -93,17 +93,17 @@ cudaError_t launch_colsum(const void* in, float* part, int M, int N, int splits,
 }
 
 __global__ void __launch_bounds__(256)
-reduce_partials_kernel(const float* __restrict__ part, size_t stride, float* __restrict__ out, size_t n, int splits)
+reduce_partials_kernel(const float* __restrict__ part, size_t stride, float* __restrict__ out, size_t n, int splits, Gap gap)
 {
     pdl_prologue();
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         float t = 0.f;
         for (int s = 0; s < splits; ++s) t += part[(size_t)s * stride + i];
-        out[i] = t;
+        out[gap.over(i)] = t;
     }
 }
 __global__ void __launch_bounds__(256)
-reduce_partials4_kernel(const float4* __restrict__ part, size_t stride4, float4* __restrict__ out, size_t n4, int splits)
+reduce_partials4_kernel(const float4* __restrict__ part, size_t stride4, float4* __restrict__ out, size_t n4, int splits, Gap gap4)
 {
     pdl_prologue();
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
@@ -117,7 +117,7 @@ reduce_partials4_kernel(const float4* __restrict__ part, size_t stride4, float4*
 #pragma unroll
             for (int u = 0; u < 8; ++u) { t.x += v[u].x; t.y += v[u].y; t.z += v[u].z; t.w += v[u].w; }
         }
-        out[i] = t;
+        out[gap4.over(i)] = t;
     }
 }
 // Many splits, few elements: 32 elements per block, LANES lanes share the splits of each element (lane l takes
@@ -138,7 +138,7 @@ __device__ __forceinline__ float many_lane_sum(const float* __restrict__ part, s
 }
 template <int LANES>
 __global__ void __launch_bounds__(32 * LANES)
-reduce_partials_many_kernel(const float* __restrict__ part, size_t stride, float* __restrict__ out, size_t n, int splits)
+reduce_partials_many_kernel(const float* __restrict__ part, size_t stride, float* __restrict__ out, size_t n, int splits, Gap gap)
 {
     pdl_prologue();
     __shared__ float s[LANES][33];
@@ -150,23 +150,23 @@ reduce_partials_many_kernel(const float* __restrict__ part, size_t stride, float
         float r = 0.f;
 #pragma unroll
         for (int j = 0; j < LANES; ++j) r += s[j][e];
-        out[i] = r;
+        out[gap.over(i)] = r;
     }
 }
-cudaError_t launch_reduce_partials(const float* part, size_t stride, float* out, size_t n, int splits, cudaStream_t st)
+cudaError_t launch_reduce_partials(const float* part, size_t stride, float* out, size_t n, int splits, cudaStream_t st, Gap gap)
 {
     if (splits >= 128 && n <= (1u << 20)) {
-        SB_LAUNCH((reduce_partials_many_kernel<32>), cdiv((long)n, 32), 1024, 0, st, part, stride, out, n, splits);
+        SB_LAUNCH((reduce_partials_many_kernel<32>), cdiv((long)n, 32), 1024, 0, st, part, stride, out, n, splits, gap);
     } else if (splits >= 32 && n <= (1u << 20)) {
-        SB_LAUNCH((reduce_partials_many_kernel<8>), cdiv((long)n, 32), 256, 0, st, part, stride, out, n, splits);
-    } else if (n % 4 == 0 && stride % 4 == 0 && (((uintptr_t)part | (uintptr_t)out) & 15) == 0) {
+        SB_LAUNCH((reduce_partials_many_kernel<8>), cdiv((long)n, 32), 256, 0, st, part, stride, out, n, splits, gap);
+    } else if (n % 4 == 0 && stride % 4 == 0 && gap.by4() && (((uintptr_t)part | (uintptr_t)out) & 15) == 0) {
         int blocks = cdiv((long)(n / 4), 256);
         if (blocks > 148 * 8) blocks = 148 * 8;
-        SB_LAUNCH((reduce_partials4_kernel), blocks, 256, 0, st, (const float4*)part, stride / 4, (float4*)out, n / 4, splits);
+        SB_LAUNCH((reduce_partials4_kernel), blocks, 256, 0, st, (const float4*)part, stride / 4, (float4*)out, n / 4, splits, Gap{gap.at / 4, gap.by / 4});
     } else {
         int blocks = cdiv((long)n, 256);
         if (blocks > 148 * 8) blocks = 148 * 8;
-        SB_LAUNCH((reduce_partials_kernel), blocks, 256, 0, st, part, stride, out, n, splits);
+        SB_LAUNCH((reduce_partials_kernel), blocks, 256, 0, st, part, stride, out, n, splits, gap);
     }
     return cudaGetLastError();
 }
@@ -734,12 +734,13 @@ sgd_kernel(float4* __restrict__ w, float4* __restrict__ v, const float4* __restr
 template <bool SHADOW>
 __global__ void __launch_bounds__(256)
 reduce_sgd4_kernel(const float4* __restrict__ part, size_t stride4, int splits, float4* __restrict__ w, float4* __restrict__ v,
-                   uint2* __restrict__ shadow, size_t n4, Hyper hy)
+                   uint2* __restrict__ shadow, size_t n4, Hyper hy, Gap gap4)
 {
     pdl_prologue();
     const float lr = hy.rate(), mu = hy.decay();
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
-        float4 ww = w[i], vv = v[i];
+        const size_t o = gap4.over(i);
+        float4 ww = w[o], vv = v[o];
         float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
         for (int s0 = 0; s0 < splits; s0 += 8) {
             float4 pv[8];
@@ -749,9 +750,9 @@ reduce_sgd4_kernel(const float4* __restrict__ part, size_t stride4, int splits, 
 #pragma unroll
             for (int u = 0; u < 8; ++u) { t.x += pv[u].x; t.y += pv[u].y; t.z += pv[u].z; t.w += pv[u].w; }
         }
-        sgd_apply<SHADOW>(ww, vv, t, lr, mu, SHADOW ? shadow + i : nullptr);
-        v[i] = vv;
-        w[i] = ww;
+        sgd_apply<SHADOW>(ww, vv, t, lr, mu, SHADOW ? shadow + o : nullptr);
+        v[o] = vv;
+        w[o] = ww;
     }
 }
 __device__ __forceinline__ void sgd_apply_scalar(float* w, float* v, float g, __nv_bfloat16* shadow, size_t i, float lr, float mu)
@@ -764,7 +765,7 @@ __device__ __forceinline__ void sgd_apply_scalar(float* w, float* v, float g, __
 template <int LANES>
 __global__ void __launch_bounds__(32 * LANES)
 reduce_sgd_many_kernel(const float* __restrict__ part, size_t stride, int splits, float* __restrict__ w, float* __restrict__ v,
-                       __nv_bfloat16* __restrict__ shadow, size_t n, Hyper hy)
+                       __nv_bfloat16* __restrict__ shadow, size_t n, Hyper hy, Gap gap)
 {
     pdl_prologue();
     const float lr = hy.rate(), mu = hy.decay();
@@ -777,38 +778,38 @@ reduce_sgd_many_kernel(const float* __restrict__ part, size_t stride, int splits
         float r = 0.f;
 #pragma unroll
         for (int j = 0; j < LANES; ++j) r += s[j][e];
-        sgd_apply_scalar(w, v, r, shadow, i, lr, mu);
+        sgd_apply_scalar(w, v, r, shadow, gap.over(i), lr, mu);
     }
 }
 __global__ void __launch_bounds__(256)
 reduce_sgd_kernel(const float* __restrict__ part, size_t stride, int splits, float* __restrict__ w, float* __restrict__ v,
-                  __nv_bfloat16* __restrict__ shadow, size_t n, Hyper hy)
+                  __nv_bfloat16* __restrict__ shadow, size_t n, Hyper hy, Gap gap)
 {
     pdl_prologue();
     const float lr = hy.rate(), mu = hy.decay();
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         float t = 0.f;
         for (int sp = 0; sp < splits; ++sp) t += part[(size_t)sp * stride + i];
-        sgd_apply_scalar(w, v, t, shadow, i, lr, mu);
+        sgd_apply_scalar(w, v, t, shadow, gap.over(i), lr, mu);
     }
 }
 cudaError_t launch_reduce_sgd(const float* part, size_t stride, size_t n, int splits, float* w, float* v, __nv_bfloat16* shadow,
-                              Hyper hy, cudaStream_t st)
+                              Hyper hy, cudaStream_t st, Gap gap)
 {
     // (the same case split as launch_reduce_partials: each case sums in the same order there and here)
     if (splits >= 128 && n <= (1u << 20)) {
-        SB_LAUNCH((reduce_sgd_many_kernel<32>), cdiv((long)n, 32), 1024, 0, st, part, stride, splits, w, v, shadow, n, hy);
+        SB_LAUNCH((reduce_sgd_many_kernel<32>), cdiv((long)n, 32), 1024, 0, st, part, stride, splits, w, v, shadow, n, hy, gap);
     } else if (splits >= 32 && n <= (1u << 20)) {
-        SB_LAUNCH((reduce_sgd_many_kernel<8>), cdiv((long)n, 32), 256, 0, st, part, stride, splits, w, v, shadow, n, hy);
-    } else if (n % 4 == 0 && stride % 4 == 0 && (((uintptr_t)part | (uintptr_t)w | (uintptr_t)v) & 15) == 0 && (((uintptr_t)shadow) & 7) == 0) {
+        SB_LAUNCH((reduce_sgd_many_kernel<8>), cdiv((long)n, 32), 256, 0, st, part, stride, splits, w, v, shadow, n, hy, gap);
+    } else if (n % 4 == 0 && stride % 4 == 0 && gap.by4() && (((uintptr_t)part | (uintptr_t)w | (uintptr_t)v) & 15) == 0 && (((uintptr_t)shadow) & 7) == 0) {
         int blocks = cdiv((long)(n / 4), 256);
         if (blocks > 148 * 8) blocks = 148 * 8;
-        if (shadow) SB_LAUNCH((reduce_sgd4_kernel<true>), blocks, 256, 0, st, (const float4*)part, stride / 4, splits, (float4*)w, (float4*)v, (uint2*)shadow, n / 4, hy);
-        else SB_LAUNCH((reduce_sgd4_kernel<false>), blocks, 256, 0, st, (const float4*)part, stride / 4, splits, (float4*)w, (float4*)v, nullptr, n / 4, hy);
+        if (shadow) SB_LAUNCH((reduce_sgd4_kernel<true>), blocks, 256, 0, st, (const float4*)part, stride / 4, splits, (float4*)w, (float4*)v, (uint2*)shadow, n / 4, hy, Gap{gap.at / 4, gap.by / 4});
+        else SB_LAUNCH((reduce_sgd4_kernel<false>), blocks, 256, 0, st, (const float4*)part, stride / 4, splits, (float4*)w, (float4*)v, nullptr, n / 4, hy, Gap{gap.at / 4, gap.by / 4});
     } else {
         int blocks = cdiv((long)n, 256);
         if (blocks > 148 * 8) blocks = 148 * 8;
-        SB_LAUNCH((reduce_sgd_kernel), blocks, 256, 0, st, part, stride, splits, w, v, shadow, n, hy);
+        SB_LAUNCH((reduce_sgd_kernel), blocks, 256, 0, st, part, stride, splits, w, v, shadow, n, hy, gap);
     }
     return cudaGetLastError();
 }
