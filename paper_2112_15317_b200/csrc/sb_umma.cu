@@ -3341,7 +3341,7 @@ sb_status umma_plan_layers(sb_model* m, int first_layer)
                 {
                     // (the filter-row kernel keeps its whole five-stage ring: with two slots per round the deeper ring is worth more
                     // than a neighbour on the SM -- steps -0.2 to -1.6 % against a ring cut to two or three 40 KB stages)
-                    const int cap = b->bn == 192 ? 5 : cohabit_stages(b->bn);
+                    const int cap = b->bn == 192 ? 4 : cohabit_stages(b->bn);
                     // (grids that leave SMs idle too: whole rings for those of fewer than 100 CTAs cost the step 1.2 % at CIFAR size, batch 128)
                     if (bwd_cohabit() && p.stages > cap) p.stages = cap;
                 }
