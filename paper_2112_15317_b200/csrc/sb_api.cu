@@ -79,6 +79,8 @@ struct sb_model {
     size_t P = 0;  // padded parameter element count
     float *Wm = nullptr, *Vm = nullptr, *Gm = nullptr;
     __nv_bfloat16* Sm = nullptr;
+    __nv_bfloat16* Tm = nullptr;      // float mode: the conv weights as three planes of bf16 terms (launch_split_weights), t_n elements a plane
+    size_t t_n = 0;                   // (the conv layers' parameters lie first in the parameter regions)
     float* ws = nullptr;    // scratch of the data-side kernels (split partial sums of forward / data gradient)
     float* ws_wk[8] = {};   // one weight-side scratch region per weight stream
     float* ws_w = nullptr;  // scratch of the weight-side kernels (split partial sums of weight / bias gradients), so that
@@ -219,6 +221,13 @@ namespace {
 
 inline bool has_weights(const Layer& l) { return l.kind == SB_CONV3X3_RELU || l.kind == SB_FC_RELU || l.kind == SB_FC; }
 
+// Whether a conv layer's forward / data gradient reads its weights as bf16 terms that a kernel of their own has split: those of the float
+// contractions on tensor cores whose row tiles would else take the same weights apart again and again.
+bool wants_terms(const Layer& l, int mode)
+{
+    return l.kind == SB_CONV3X3_RELU && l.cplan[mode].umma && contract_umma_whole_taps(mode, l.Cin, l.Cout);
+}
+
 // Shape, plan and layer input of layer i as a CUDA-core contraction (the FC layers' K column shards lie one after another in the
 // weight matrix and in the output rows, so they are one contraction over the whole width).
 ContractArgs contract_args(sb_model* m, int i, int mode)
@@ -231,6 +240,7 @@ ContractArgs contract_args(sb_model* m, int i, int mode)
     a.Cin = conv ? l.Cin : l.in_f; a.Cout = conv ? l.Cout : l.out_f;
     a.plan = l.cplan[mode];
     a.status = m->status;
+    if (mode != CMODE_WGRAD && wants_terms(l, mode)) { a.wterms = m->Tm + l.p_w; a.wterms_stride = m->t_n; }
     a.act = l.in_override ? l.in_override : (i > 0 ? m->L[i - 1].act : nullptr);
     if (i == 0) { a.tab = &m->x_tab; a.tab_imgs = m->cfg.batch_per_replica; }
     return a;
@@ -384,6 +394,10 @@ sb_status plan(const sb_layer* layers, int n, const sb_config* cfg, sb_model* m,
     }
     // CUDA-core layers: partial sums of split reductions, 64 MB at most
     for (int i = 0; i < n; ++i) ws_floats = std::max(ws_floats, contract_plan_layer(m, i, (size_t)16 << 20));
+    m->t_n = 0;
+    for (int i = 0; i < n; ++i)
+        if (wants_terms(m->L[i], CMODE_FWD) || wants_terms(m->L[i], CMODE_DGRAD)) m->t_n = m->L[i].p_w + align_up(m->L[i].n_w, 64);
+    m->Tm = m->t_n ? (__nv_bfloat16*)take(m->t_n * 3 * sizeof(__nv_bfloat16)) : nullptr;
     size_t um_ws = 0;
     sb_status us = umma_plan_scratch(m, &um_ws);
     if (us != SB_OK) return fail(us, "%s", umma_last_error());
@@ -1093,6 +1107,18 @@ static sb_status chain_bwd(sb_model* m, int i, cudaStream_t st, int part)
     return s;
 }
 
+// The conv weights as bf16 terms, at the beginning of every call that reads them so (layers first .. last): the weights may have changed
+// since the last one.  4 us for the 7-conv net's 1.7 M parameters.
+static sb_status split_weights(sb_model* m, int first, int last, bool fwd, bool dgrad, cudaStream_t st)
+{
+    bool any = false;
+    for (int i = first; i <= last; ++i) any = any || (fwd && wants_terms(m->L[i], CMODE_FWD)) || (dgrad && wants_terms(m->L[i], CMODE_DGRAD));
+    if (!any) return SB_OK;
+    m->cur_layer = -1;
+    L_TRY("split_weights", 0.0, 10.0 * m->t_n, launch_split_weights(m->Wm, m->Tm, m->t_n, m->t_n, st));
+    return SB_OK;
+}
+
 sb_status sb_forward_layers(sb_model* m, int32_t first, int32_t last, const void* const* x, const int32_t* const* labels, void* stream)
 {
     if (!m) return fail(SB_ERR_INVALID_ARG, "null model");
@@ -1103,6 +1129,8 @@ sb_status sb_forward_layers(sb_model* m, int32_t first, int32_t last, const void
     }
     m->pooled_by_conv = -1;     // a pool layer run on its own (or first in the range) computes its output itself
     m->st_clean = false;
+    const sb_status ss = split_weights(m, first, last, true, false, (cudaStream_t)stream);
+    if (ss != SB_OK) return ss;
     for (int i = first; i <= last; ++i) {
         sb_status s = chain_fwd(m, i, (cudaStream_t)stream);
         if (s != SB_OK) return s;
@@ -1118,7 +1146,7 @@ sb_status sb_backward_layers(sb_model* m, int32_t last, int32_t first, void* str
     if (first < 0 || last >= m->n_layers || first > last) return fail(SB_ERR_INVALID_ARG, "bad layer range %d..%d", last, first);
     m->st_clean = false;
     m->bwd_lo = first; m->unpooled = -1;
-    sb_status s = SB_OK;
+    sb_status s = split_weights(m, first, last, false, true, (cudaStream_t)stream);
     for (int i = last; i >= first && s == SB_OK; --i) s = chain_bwd(m, i, (cudaStream_t)stream, SIDE_BOTH);
     m->bwd_lo = 1 << 30;
     m->st_clean = false;
@@ -1203,13 +1231,14 @@ static sb_status pass_replay(sb_model* m, sb_model::PassGraph& G, cudaStream_t s
 }
 
 extern "C" {
-static sb_status forward_pass(sb_model* m, cudaStream_t st)
+// (by_itself: no backward pass of the same call follows, which would read the same weights)
+static sb_status forward_pass(sb_model* m, cudaStream_t st, bool by_itself)
 {
     m->pooled_by_conv = -1;
     m->xent_by_fc = -1;
     m->st_clean = false;
     m->head_ok = true;
-    sb_status s = SB_OK;
+    sb_status s = split_weights(m, 0, m->n_layers - 1, true, !by_itself, st);
     for (int i = 0; i < m->n_layers && s == SB_OK; ++i) s = chain_fwd(m, i, st);
     m->head_ok = false;
     m->st_clean = false;
@@ -1225,7 +1254,7 @@ static sb_status forward_on(sb_model* m, const void* const* x, const int32_t* co
     sb_status s = set_inputs(m, x, labels);
     if (s != SB_OK) return s;
     m->launches = 0;
-    s = by_itself ? pass_replay(m, m->g_fwd, st, [&](cudaStream_t on) { return forward_pass(m, on); }) : forward_pass(m, st);
+    s = by_itself ? pass_replay(m, m->g_fwd, st, [&](cudaStream_t on) { return forward_pass(m, on, true); }) : forward_pass(m, st, false);
     if (s == SB_OK) m->have_fwd = true;
     return s;
 }
@@ -1365,7 +1394,10 @@ sb_status sb_backward(sb_model* m, void* stream)
     if (!m) return fail(SB_ERR_INVALID_ARG, "null model");
     if (!m->have_fwd) return fail(SB_ERR_STATE, "sb_backward needs a preceding sb_forward");
     cudaStream_t st = (cudaStream_t)stream;
-    return pass_replay(m, m->g_bwd, st, [&](cudaStream_t on) { return backward_pass(m, on, false, Hyper{}, nullptr); });
+    return pass_replay(m, m->g_bwd, st, [&](cudaStream_t on) {
+        const sb_status s = split_weights(m, 0, m->n_layers - 1, false, true, on);
+        return s != SB_OK ? s : backward_pass(m, on, false, Hyper{}, nullptr);
+    });
 }
 
 // forward + backward + update of one iteration, with the update folded into the backward pass when possible
@@ -1408,6 +1440,7 @@ static sb_status modulo_step_direct(sb_model* m, const void* const* x, const int
     const int ff = m->first_fc, K = m->cfg.K, R = m->cfg.R, b = m->cfg.batch_per_replica, Bk = m->B / K;
     const size_t D = (size_t)m->L[ff].in_f;
     m->st_clean = false;
+    if ((s = split_weights(m, 0, ff - 1, true, true, st)) != SB_OK) return s;
     for (int i = 0; i < ff; ++i) {
         s = chain_fwd(m, i, st);
         if (s != SB_OK) return s;

@@ -8,8 +8,8 @@
 // A fully-connected layer is the same thing with one tap and 1x1 images (pixel = batch row).
 //
 // Large enough float layers whose channel counts are multiples of eight run on the tensor cores instead (sb_contract_umma.cu): the plan
-// takes whichever the two cost models below say is faster.  3x3 over 64 channels at 32x32, batch 96: 181 us here, 102 there; 256
-// channels at 8x8: 157 and 57; 16 -> 32 channels at 16x16, batch 8, forward: 8.0 and 8.0.
+// takes whichever the two cost models below say is faster.  3x3 over 64 channels at 32x32, batch 96: 180 us here, 66 there; 256
+// channels at 8x8: 157 and 50; 16 -> 32 channels at 16x16, batch 8, forward: 8.0 and 7.3; 4096 -> 1024 weight gradient at batch 8: 6.8 and 14.
 //
 // What bounds it: the FFMA pipe (measured 70 TFLOP/s of packed fma.rn.f32x2 on registers, 68 of scalar FFMA).  A block of
 // BM x BN outputs gives every thread an 8 x 8 square, so that 16 shared-memory words feed 64 multiply-adds; the packed form
@@ -367,7 +367,7 @@ static const TileShape shapes[] = {{128, 128, 2, 0.45, 1.25}, {128, 64, 4, 0.75,
 // The tensor-core form (one CTA per SM): microseconds per 64 reduction steps, per tile and per launch, by tile width and mode,
 // from a sweep of both widths and 1 to 64 splits over 25 layers (residual 6 to 10 %).
 struct UmmaCost { double step, tile, launch; };
-static const UmmaCost umma_cost[2][3] = {{{1.41, 3.7, 3.3}, {1.48, 3.3, 3.3}, {1.72, 7.8, -2.2}}, {{1.04, 2.6, 3.3}, {1.18, 2.4, 3.0}, {1.34, 4.6, -0.8}}};
+static const UmmaCost umma_cost[2][3] = {{{1.36, 0.7, 6.5}, {1.40, 0.4, 7.4}, {1.47, 5.9, 0.6}}, {{0.99, 0.9, 5.2}, {0.99, 0.9, 5.8}, {1.12, 1.8, 2.5}}};
 
 static bool vec_ok(int Cin, int Cout) { return Cin % 4 == 0 && Cout % 4 == 0; }
 static long contract_iters(int mode, int B, int H, int W, int taps, int Cin, int Cout)
@@ -393,6 +393,7 @@ ContractPlan contract_plan(int mode, int B, int H, int W, int taps, int Cin, int
             const long n = (tiles * real + 147) / 148, rest = n % s.resident;        // blocks of the fullest SM
             const double step = (double)(n / s.resident) * (s.lone + s.more * s.resident) + (rest ? s.lone + s.more * rest : 0.0);
             double t = per * step * (mode == CMODE_WGRAD ? 1.08 : 1.0) + 3.0;
+            if (mode == CMODE_DGRAD && real == 1) t += 3.5;      // (a thread's sixteen mask loads, one behind the other)
             if (real > 1) t += 3.0 + (double)real * M * N * 8.0 / 7.0e6;
             if (t < best_t) { best_t = t; best = ContractPlan{s.bm, s.bn, (int)per, real, false}; }
         }

@@ -17,24 +17,31 @@
 //   4096 -> 1024, batch 96                         1.8e-7 -> 1.0e-7                  2.1e-7 -> 0.9e-7                   1.3e-7 -> 0.5e-7
 //   3x3, 8 -> 40 channels at 5x7, batch 3          0.8e-7 -> 0.6e-7                  1.2e-7 -> 0.8e-7                   1.2e-7 -> 0.5e-7
 //
-// Roles (24 warps; registers are moved between them): warp 0 allocates TMEM and issues the MMAs; warps 4-7 keep the running sums and
-// write the results; warps 8-23 fetch floats to registers, take them apart and store the terms, A into tensor memory (a lane per
-// row) and B as 128-byte swizzled rows of shared memory, the next chunk's loads in flight behind the conversion of the present one.
-// A in tensor memory keeps its terms off the shared-memory port, which would else carry 40 KB per 16 steps of a 128 x 128 tile.
+// One CTA per SM walks (tile, split) units; the results of a unit are written while the next one is under way.  Roles (24 warps; registers
+// are moved between them): warp 0 allocates TMEM and issues the MMAs; warp 1 fetches A as raw floats and warp 2 the weights' terms by TMA;
+// warps 4-7 keep the running sums and write the results; warps 8-23 take the floats apart and store the terms, A into tensor memory (a
+// lane per row; WGRAD: transposed on the way) and B as 128-byte swizzled rows of shared memory, the next chunk of B in flight behind the
+// conversion of the present one.  A in tensor memory keeps its terms off the shared-memory port, which would else carry 40 KB per 16 steps of
+// a 128 x 128 tile.  The weights of a convolution are read by every row tile, so a kernel of their own takes them apart once a call.
 //
-// What bounds it: the converters' loads.  A 128 x 128 x 64 chunk takes 2850 cycles where its 24 MMAs take 1536 (tensor pipe 49 %
-// busy): a row per lane makes each 32-byte load of A 32 wavefronts of the L1 port (1280 cycles a chunk with those of B, 1150 for
-// the stores and the MMAs' reads), and the 16 converter warps fill half of the issue slots.  64 -> 64 channels at 32x32, batch 96:
-// 181 -> 102 us forward; 256 -> 256 at 8x8: 157 -> 57 us (7-conv / 3-FC net, batch 96: 2.54 -> 1.12 ms an iteration).
+// What bounds it: issue slots.  A chunk of 128 x 128 x 64 takes 2500 - 2700 cycles where its 24 MMAs take 1536, one of 128 x 64 x 64 2000
+// (768): 16 converter warps of some 200 instructions a chunk (350 where they convert B as well), the summing warps' 128 additions and the
+// MMA warp share the four schedulers, and the single buffer of leading products of the wide tile makes MMA and sums wait for each other.
+// Without TMA and with a CTA per unit the same layers took a third longer (a row per lane made each load of A 32 wavefronts of the L1
+// port).  Float CUDA cores -> here, us at batch 96: 3x3 over 64 channels at 32x32 forward 180 -> 66, input gradient 175 -> 75, weight gradient
+// 177 -> 91; 128 channels at 16x16 155 / 164 / 156 -> 65 / 59 / 50; 256 channels at 8x8 157 / 170 / 159 -> 50 / 50 / 47; 4096 -> 1024 30 / 27
+// / 23 -> 18 / 18 / 18.  The 7-conv / 3-FC net: 2.54 -> 0.98 ms an iteration.
 //
 // Non-finite operands: infinity - infinity in the splitting makes the terms NaN where a float multiply-add would give an infinity, so
 // a row with a NaN in it is computed again with plain multiply-adds by the thread that owns it.
-#include "sb_internal.h"
+#include "sb_umma.h"
 #include "sb_tcgen05.cuh"
 
 namespace sb {
 
 namespace {
+
+uint32_t rcp_of(int d) { return d <= 1 ? 0u : (uint32_t)(0x100000000ull / (uint32_t)d) + 1u; }
 
 struct SplitParams {
     const float *act, *wt, *dy;
@@ -42,6 +49,8 @@ struct SplitParams {
     uint32_t rcp_w, rcp_hw;
     int M, N, K;                   // rows, columns, reduction length (WGRAD: pixels)
     int chunks, cps, splits;       // 64-step chunks, per split
+    int m_tiles, n_tiles, units;   // (tile, split) pairs, walked by the CTAs in turn
+    uint32_t rcp_m, rcp_n;
     float* part; long split_stride;
     long bias_off;
     float* out; const float* bias; int relu;
@@ -51,11 +60,18 @@ struct SplitParams {
 
 // 24 warps: 4 for the MMAs (one works), 4 running sums, 16 converters.  Registers of the 80 a thread at launch: 32 + 160 + 4 * 72 = 6 * 80.
 constexpr int THREADS = 768, CONV0 = 256, REGS_ISSUE = 32, REGS_SUMS = 160, REGS_CONV = 72;
-constexpr int STAGES = 2, CTRL = 8192;
-// one term of the B tile: BN rows of 128 bytes (FWD), or 64-column boxes of 64 rows
-template <int BN> struct SplitCfg { static constexpr int PLANE = BN * 128, STAGE = 3 * PLANE, SMEM = STAGES * STAGE + 1024 + CTRL; };
-// tensor memory columns: leading products, the other products, then the terms of A (2 stages x 3 x 32)
-constexpr uint32_t COL_A = 256, A_TERM = 32, A_STAGE = 3 * A_TERM, TMEM_COLS = 512;
+constexpr int STAGES = 2, RAWS = 2, RAW = 32768, CTRL = 8192;
+// PLANE: one term of the B tile, BN rows of 128 bytes (FWD) or 64-column boxes of 64 rows.  RAW: a chunk of A as floats, 32-column
+// boxes of 128-byte swizzled rows.  Tensor memory columns: buffers of leading products, buffers of the other products, then the
+// terms of A (2 stages x 3 x 32).
+template <int BN> struct SplitCfg {
+    static constexpr int PLANE = BN * 128, STAGE = 3 * PLANE;
+    static constexpr int smem(bool tma) { return STAGES * STAGE + (tma ? RAWS * RAW : 0) + 1024 + CTRL; }
+    static constexpr int LEADS = BN == 64 ? 3 : 1, RESTS = BN == 64 ? 2 : 1;
+    static constexpr uint32_t COL_REST = LEADS * BN, COL_A = COL_REST + RESTS * BN;
+};
+constexpr uint32_t A_TERM = 32, A_STAGE = 3 * A_TERM, TMEM_COLS = 512;
+static_assert(SplitCfg<64>::COL_A + STAGES * A_STAGE <= TMEM_COLS && SplitCfg<128>::COL_A + STAGES * A_STAGE <= TMEM_COLS, "tensor memory");
 
 __device__ __forceinline__ int div_rcp(int n, uint32_t mul, int d)
 {
@@ -120,12 +136,6 @@ __device__ __forceinline__ void umma_ta(uint32_t d_tmem, uint32_t a_tmem, uint32
         ::"r"(d_tmem), "r"(a_tmem), "r"(blo), "r"(bhi), "r"(idesc), "r"(accumulate), "r"(elected)
         : "memory");
 }
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8])
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "r"(taddr) : "memory");
-}
-
 // Element (m, n) over reduction steps [k0, k1) with plain multiply-adds (rows with a non-finite operand).
 template <int MODE>
 __device__ __noinline__ float plain_sum(const SplitParams& p, int m, int n, int k0, int k1)
@@ -170,36 +180,62 @@ __device__ __forceinline__ void finish8(const SplitParams& p, float (&f)[8], siz
     }
 }
 
-// K64: the channels of the reduction are a multiple of 64, so that a chunk lies in one tap (FWD, DGRAD)
-template <int MODE, int BN, bool K64>
+template <bool TMA> struct Maps { CUtensorMap a, b; };      // raw floats of A, terms of the weights
+template <> struct Maps<false> { };
+// One (tile, split) pair
+struct Unit { int m0, n0, split, chunk0, n_iters; };
+template <int BN>
+__device__ __forceinline__ Unit unit_at(const SplitParams& p, int u)
+{
+    const int r = div_rcp(u, p.rcp_m, p.m_tiles), z = div_rcp(r, p.rcp_n, p.n_tiles);
+    Unit t;
+    t.m0 = (u - r * p.m_tiles) * 128;
+    t.n0 = (r - z * p.n_tiles) * BN;
+    t.split = z;
+    t.chunk0 = z * p.cps;
+    t.n_iters = min(p.cps, p.chunks - t.chunk0);
+    return t;
+}
+// slot of a ring and the parity of its current use
+struct Ring {
+    int i = 0;
+    uint32_t ph = 0;
+    __device__ __forceinline__ void next(int n) { if (++i == n) { i = 0; ph ^= 1u; } }
+};
+
+// TMA: A arrives as raw floats by TMA (FWD, DGRAD: the channels of the reduction are a multiple of 64, so that a chunk lies in one
+// tap and its rows are those of the tile, shifted; WGRAD: always); otherwise the converters load it themselves.
+// WT: B arrives as terms by TMA (FWD, DGRAD of convolutions, whose weights every row tile reads: launch_split_weights).
+template <int MODE, int BN, bool TMA, bool WT>
 __global__ void __launch_bounds__(THREADS, 1)
-contract_umma_kernel(const __grid_constant__ SplitParams p)
+contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_constant__ SplitParams p)
 {
     using C = SplitCfg<BN>;
     constexpr int NB = BN / 64;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t* ctrl = smem + STAGES * C::STAGE;
-    uint64_t* full = (uint64_t*)ctrl;               // [STAGES] terms stored: one arrival per converter warp
+    uint8_t* raw = smem + STAGES * C::STAGE;
+    uint8_t* ctrl = raw + (TMA ? RAWS * RAW : 0);
+    uint64_t* full = (uint64_t*)ctrl;               // [STAGES] terms stored: one arrival per converter warp (WT: and the weights' bytes)
     uint64_t* empty = full + STAGES;                // [STAGES] read by their MMAs
-    uint64_t* lead_full = empty + STAGES;           // leading products of a chunk complete
-    uint64_t* lead_empty = lead_full + 1;           // ... and taken over: one arrival per summing warp
-    uint64_t* done = lead_empty + 1;                // everything complete
-    uint32_t* tmem_slot = (uint32_t*)(done + 1);
+    uint64_t* raw_full = empty + STAGES;            // [RAWS] a chunk of A has landed
+    uint64_t* raw_empty = raw_full + RAWS;          // [RAWS] ... and is in registers: one arrival per converter warp
+    uint64_t* lead_full = raw_empty + RAWS;         // [LEADS] leading products of a chunk complete
+    uint64_t* lead_empty = lead_full + C::LEADS;    // [LEADS] ... and taken over: one arrival per summing warp
+    uint64_t* rest_full = lead_empty + C::LEADS;    // [RESTS] everything of a unit complete
+    uint64_t* rest_empty = rest_full + C::RESTS;    // [RESTS] ... and taken over
+    uint32_t* tmem_slot = (uint32_t*)(rest_empty + C::RESTS);
     volatile uint32_t* abort_flag = tmem_slot + 1;
     float* s_bias = (float*)(ctrl + 1024);          // [3][128]: WGRAD, sums of dy over the later quarters of the chunks
 
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    const int m0 = blockIdx.x * 128, n0 = blockIdx.y * BN;
-    const int chunk0 = blockIdx.z * p.cps, n_iters = min(p.cps, p.chunks - chunk0);
-
     if (warp == 0) {
-        if (lane == 0) {
-            for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 16); mbar_init(&empty[s], 1); }
-            mbar_init(lead_full, 1);
-            mbar_init(lead_empty, 4);
-            mbar_init(done, 1);
-            *abort_flag = 0;
+        // (the barriers lie one after another: a lane each)
+        constexpr int B0 = STAGES, B1 = B0 + STAGES, B2 = B1 + RAWS, B3 = B2 + RAWS, B4 = B3 + C::LEADS, B5 = B4 + C::LEADS, B6 = B5 + C::RESTS, B7 = B6 + C::RESTS;
+        if (lane < B7) {
+            const uint32_t n = lane < B0 ? (WT ? 17u : 16u) : lane < B2 ? 1u : lane < B3 ? 16u : lane < B4 ? 1u : lane < B5 ? 4u : lane < B6 ? 1u : 4u;
+            mbar_init(&full[lane], n);
+            if (lane == 0) *abort_flag = 0;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
         __syncwarp();
@@ -212,281 +248,385 @@ contract_umma_kernel(const __grid_constant__ SplitParams p)
     const uint32_t tmem = *tmem_slot;
     pdl_wait();
     pdl_trigger();
+    const int Cred = MODE == CMODE_DGRAD ? p.Cout : p.Cin;
 
     if (warp < 4) {
-        // =========================== MMA issuer (warp 0 in lock-step, one elected lane issues) ===================================
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_ISSUE));
         if (warp == 0) {
+            // =========================== MMA issuer (the warp in lock-step, one elected lane issues) =============================
             constexpr bool B_MN = MODE != CMODE_FWD;
             constexpr uint32_t idesc = make_idesc(BN, 0, B_MN);
             constexpr uint32_t A_STEP = 8, B_STEP = (B_MN ? 2048u : 32u) >> 4, BP = C::PLANE >> 4;     // per 16 reduction steps: columns, 16-byte units
             const uint32_t elected = elect_one() ? 1u : 0u;
             const uint64_t dB = make_desc(smem_u32(smem), B_MN ? 8192u : 16u);
-            const uint32_t b_hi = (uint32_t)(dB >> 32), rest = tmem + BN;
-            int s = 0;
-            uint32_t ph = 0;
+            const uint32_t b_hi = (uint32_t)(dB >> 32);
+            Ring st, lead, rest;
+            int chunk = 0, unit = 0;      // (a buffer's first use needs no wait)
             bool ok = true;
-            for (int it = 0; it < n_iters; ++it) {
-                bool w = mbar_wait(&full[s], ph);
-                if (it >= 1) w = w && mbar_wait(lead_empty, (uint32_t)((it & 1) ^ 1));
-                ok = __all_sync(0xffffffffu, w ? 1 : 0) != 0;
-                if (!ok) break;
-                tc_fence_after();
-                const uint32_t a = tmem + COL_A + (uint32_t)s * A_STAGE, b = (uint32_t)dB + (uint32_t)s * (C::STAGE >> 4);
+            for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x, ++unit) {
+                const int n_iters = unit_at<BN>(p, u).n_iters;
+                for (int it = 0; it < n_iters; ++it, ++chunk) {
+                    bool w = mbar_wait(&full[st.i], st.ph);
+                    if (chunk >= C::LEADS) w = w && mbar_wait(&lead_empty[lead.i], lead.ph ^ 1u);
+                    if (it == 0 && unit >= C::RESTS) w = w && mbar_wait(&rest_empty[rest.i], rest.ph ^ 1u);
+                    ok = __all_sync(0xffffffffu, w ? 1 : 0) != 0;
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t a = tmem + C::COL_A + (uint32_t)st.i * A_STAGE, b = (uint32_t)dB + (uint32_t)st.i * (C::STAGE >> 4);
+                    const uint32_t d0 = tmem + (uint32_t)lead.i * BN, d1 = tmem + C::COL_REST + (uint32_t)rest.i * BN;
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) umma_ta(tmem, a + kk * A_STEP, b + kk * B_STEP, b_hi, idesc, kk > 0 ? 1u : 0u, elected);
-                if (elected) umma_commit(lead_full);
+                    for (int kk = 0; kk < 4; ++kk) umma_ta(d0, a + kk * A_STEP, b + kk * B_STEP, b_hi, idesc, kk > 0 ? 1u : 0u, elected);
+                    if (elected) umma_commit(&lead_full[lead.i]);
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    const uint32_t ak = a + kk * A_STEP, bk = b + kk * B_STEP;
-                    umma_ta(rest, ak + 2 * A_TERM, bk, b_hi, idesc, (it > 0 || kk > 0) ? 1u : 0u, elected);     // a2 b0
-                    umma_ta(rest, ak, bk + 2 * BP, b_hi, idesc, 1u, elected);                                   // a0 b2
-                    umma_ta(rest, ak + A_TERM, bk + BP, b_hi, idesc, 1u, elected);                              // a1 b1
-                    umma_ta(rest, ak + A_TERM, bk, b_hi, idesc, 1u, elected);                                   // a1 b0
-                    umma_ta(rest, ak, bk + BP, b_hi, idesc, 1u, elected);                                       // a0 b1
+                    for (int kk = 0; kk < 4; ++kk) {
+                        const uint32_t ak = a + kk * A_STEP, bk = b + kk * B_STEP;
+                        umma_ta(d1, ak + 2 * A_TERM, bk, b_hi, idesc, (it > 0 || kk > 0) ? 1u : 0u, elected);     // a2 b0
+                        umma_ta(d1, ak, bk + 2 * BP, b_hi, idesc, 1u, elected);                                   // a0 b2
+                        umma_ta(d1, ak + A_TERM, bk + BP, b_hi, idesc, 1u, elected);                              // a1 b1
+                        umma_ta(d1, ak + A_TERM, bk, b_hi, idesc, 1u, elected);                                   // a1 b0
+                        umma_ta(d1, ak, bk + BP, b_hi, idesc, 1u, elected);                                       // a0 b1
+                    }
+                    if (elected) umma_commit(&empty[st.i]);
+                    if (elected && it + 1 == n_iters) umma_commit(&rest_full[rest.i]);
+                    __syncwarp();
+                    st.next(STAGES);
+                    lead.next(C::LEADS);
                 }
-                if (elected) umma_commit(&empty[s]);
-                __syncwarp();
-                if (++s == STAGES) { s = 0; ph ^= 1u; }
+                rest.next(C::RESTS);
             }
             if (!ok && lane == 0) { *abort_flag = 1; atomicMax(p.status, (uint32_t)DEV_TIMEOUT_MMA); }
-            if (ok && elected) umma_commit(done);
+            __syncwarp();
+        } else if (TMA && warp == 1) {
+            // =========================== raw floats of A =========================================================================
+            if constexpr (TMA) if (lane == 0) {
+                Ring r;
+                int n = 0;
+                bool ok = true;
+                for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
+                    const Unit t = unit_at<BN>(p, u);
+                    int tap = MODE == CMODE_WGRAD ? 0 : t.chunk0 * 64 / Cred, c = MODE == CMODE_WGRAD ? 0 : t.chunk0 * 64 - tap * Cred;
+                    for (int it = 0; it < t.n_iters; ++it, ++n) {
+                        if (n >= RAWS && !(ok = mbar_wait(&raw_empty[r.i], r.ph ^ 1u))) break;
+                        uint8_t* dst = raw + r.i * RAW;
+                        mbar_expect_tx(&raw_full[r.i], (uint32_t)RAW);
+                        if (MODE == CMODE_WGRAD) {
+#pragma unroll
+                            for (int b = 0; b < 4; ++b) tma_load_4d(&maps.a, dst + b * 8192, &raw_full[r.i], t.m0 + 32 * b, (t.chunk0 + it) * 64, 0, 0);
+                        } else {
+                            int shift = 0;      // in rows; rows of other images or of none are left out when the terms are taken
+                            if (p.taps == 9) {
+                                const int tr = tap / 3, ts = tap - 3 * tr;
+                                shift = MODE == CMODE_FWD ? (tr - 1) * p.W + ts - 1 : (1 - tr) * p.W + 1 - ts;
+                            }
+#pragma unroll
+                            for (int b = 0; b < 2; ++b) tma_load_4d(&maps.a, dst + b * 16384, &raw_full[r.i], c + 32 * b, t.m0 + shift, 0, 0);
+                            c += 64;
+                            if (c >= Cred) { c -= Cred; ++tap; }
+                        }
+                        r.next(RAWS);
+                    }
+                }
+                if (!ok) { *abort_flag = 1; atomicMax(p.status, (uint32_t)DEV_TIMEOUT_TMA); }
+            }
+            __syncwarp();
+        } else if (WT && warp == 2) {
+            // =========================== terms of the weights ====================================================================
+            if constexpr (WT) if (lane == 0) {
+                Ring r;
+                int n = 0;
+                bool ok = true;
+                for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
+                    const Unit t = unit_at<BN>(p, u);
+                    int tap = t.chunk0 * 64 / Cred, c = t.chunk0 * 64 - tap * Cred;
+                    for (int it = 0; it < t.n_iters; ++it, ++n) {
+                        if (n >= STAGES && !(ok = mbar_wait(&empty[r.i], r.ph ^ 1u))) break;
+                        uint8_t* dst = smem + r.i * C::STAGE;
+                        mbar_expect_tx(&full[r.i], (uint32_t)C::STAGE);
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) {
+                            if (MODE == CMODE_FWD) tma_load_4d(&maps.b, dst + k * C::PLANE, &full[r.i], (t.chunk0 + it) * 64, t.n0, k, 0);
+                            else
+#pragma unroll
+                                for (int j = 0; j < NB; ++j) tma_load_4d(&maps.b, dst + k * C::PLANE + j * 8192, &full[r.i], tap * p.Cin + t.n0 + 64 * j, c, k, 0);
+                        }
+                        c += 64;
+                        if (c >= Cred) { c -= Cred; ++tap; }
+                        r.next(STAGES);
+                    }
+                }
+                if (!ok) { *abort_flag = 1; atomicMax(p.status, (uint32_t)DEV_TIMEOUT_TMA); }
+            }
             __syncwarp();
         }
     } else if (warp < 8) {
         // =========================== running sums and results ====================================================================
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_SUMS));
-        const int q = warp % 4, m = m0 + q * 32 + lane;
+        const int q = warp % 4;
         const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16);
-        float acc[BN];
-#pragma unroll
-        for (int j = 0; j < BN; ++j) acc[j] = 0.f;
+        const bool raw_sums = MODE == CMODE_WGRAD || p.splits > 1;
+        Ring lead, rest;
         bool ok = true;
-        for (int it = 0; it < n_iters; ++it) {
-            ok = __all_sync(0xffffffffu, mbar_wait(lead_full, (uint32_t)(it & 1)) ? 1 : 0) != 0;
-            if (!ok) break;
-            tc_fence_after();
+        for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
+            const Unit t = unit_at<BN>(p, u);
+            float acc[BN];
 #pragma unroll
-            for (int c = 0; c < BN; c += 16) {
-                uint32_t v[16];
-                tmem_ld16(taddr + c, v);
-                tmem_ld_wait();
+            for (int j = 0; j < BN; ++j) acc[j] = 0.f;
+            for (int it = 0; it <= t.n_iters; ++it) {
+                // the leading products chunk by chunk, then the others
+                const bool last = it == t.n_iters;
+                uint64_t* in = last ? &rest_full[rest.i] : &lead_full[lead.i];
+                ok = __all_sync(0xffffffffu, mbar_wait(in, last ? rest.ph : lead.ph) ? 1 : 0) != 0;
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t from = taddr + (last ? C::COL_REST + (uint32_t)rest.i * BN : (uint32_t)lead.i * BN);
 #pragma unroll
-                for (int j = 0; j < 16; ++j) acc[c + j] += __uint_as_float(v[j]);
+                for (int c = 0; c < BN; c += 16) {
+                    uint32_t v[16];
+                    tmem_ld16(from + c, v);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) acc[c + j] += __uint_as_float(v[j]);
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(last ? &rest_empty[rest.i] : &lead_empty[lead.i]));
+                if (last) rest.next(C::RESTS);
+                else lead.next(C::LEADS);
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(lead_empty));
-        }
-        if (ok) ok = __all_sync(0xffffffffu, mbar_wait(done, 0) ? 1 : 0) != 0;
-        if (!ok && lane == 0) { *abort_flag = 1; atomicMax(p.status, (uint32_t)DEV_TIMEOUT_EPI); }
-        if (ok) {
-            tc_fence_after();
-            const bool raw = MODE == CMODE_WGRAD || p.splits > 1;
+            const int m = t.m0 + q * 32 + lane;
+            if (!ok || m >= p.M) continue;
             const size_t row = (size_t)m * p.N;
-            float* dst = (raw ? p.part + (size_t)blockIdx.z * p.split_stride : p.out) + row;
-            const bool row_ok = m < p.M;
+            float* dst = (raw_sums ? p.part + (size_t)t.split * p.split_stride : p.out) + row;
             bool bad = false;
 #pragma unroll
             for (int c = 0; c < BN; c += 8) {
-                uint32_t v[8];
-                tmem_ld8(taddr + BN + c, v);
-                tmem_ld_wait();
+                if (t.n0 + c >= p.N) continue;
                 float f[8];
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    f[j] = acc[c + j] + __uint_as_float(v[j]);
+                    f[j] = acc[c + j];
                     bad = bad || f[j] != f[j];
                 }
-                if (row_ok && n0 + c < p.N) {
-                    if (!raw) finish8<MODE>(p, f, row + n0 + c, n0 + c);
-                    float4* d = (float4*)(dst + n0 + c);
-                    d[0] = make_float4(f[0], f[1], f[2], f[3]);
-                    d[1] = make_float4(f[4], f[5], f[6], f[7]);
-                }
+                if (!raw_sums) finish8<MODE>(p, f, row + t.n0 + c, t.n0 + c);
+                float4* d = (float4*)(dst + t.n0 + c);
+                d[0] = make_float4(f[0], f[1], f[2], f[3]);
+                d[1] = make_float4(f[4], f[5], f[6], f[7]);
             }
-            if (row_ok && bad) {
-                const int k0 = chunk0 * 64, k1 = min(p.K, (chunk0 + n_iters) * 64);
-                for (int n = n0; n < min(n0 + BN, p.N); n += 8) {
+            if (bad) {
+                const int k0 = t.chunk0 * 64, k1 = min(p.K, (t.chunk0 + t.n_iters) * 64);
+                for (int n = t.n0; n < min(t.n0 + BN, p.N); n += 8) {
                     float f[8];
                     for (int j = 0; j < 8; ++j) f[j] = plain_sum<MODE>(p, m, n + j, k0, k1);
-                    if (!raw) finish8<MODE>(p, f, row + n, n);
+                    if (!raw_sums) finish8<MODE>(p, f, row + n, n);
                     for (int j = 0; j < 8; ++j) dst[n + j] = f[j];
                 }
             }
         }
+        if (!ok && lane == 0) { *abort_flag = 1; atomicMax(p.status, (uint32_t)DEV_TIMEOUT_EPI); }
     } else {
         // =========================== converters ==================================================================================
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_CONV));
         const int t = threadIdx.x - CONV0, HW = p.H * p.W;
-        const int Cred = MODE == CMODE_DGRAD ? p.Cout : p.Cin;
         F8 ra[2], rb[NB];
-        int kpos = chunk0 * 64;           // first reduction step of the chunk
 
         // A: this thread's row is the TMEM lane of its warp's quadrant, its reduction steps a quarter of the chunk
-        const int row = (warp & 3) * 32 + lane, quarter = (warp - 8) >> 2, m = m0 + row;
-        const uint32_t a_at = tmem + COL_A + ((uint32_t)((warp & 3) * 32) << 16) + 8u * quarter;
-        const float* a_px = nullptr;      // FWD / DGRAD: the pixel, and which taps fall inside the image; WGRAD: the column of dy
-        uint32_t a_in = 0u;
-        int a_tap = 0, a_c = 0;           // FWD / DGRAD: place of the thread's quarter along the reduction
-        // B: row r and the q-th run of eight floats of each 64-float row piece (FWD: rows r, r + 64; DGRAD, WGRAD: row r along the
-        // reduction, NB boxes of columns)
+        const int row = (warp & 3) * 32 + lane, quarter = (warp - 8) >> 2;
+        const uint32_t a_at = tmem + C::COL_A + ((uint32_t)((warp & 3) * 32) << 16) + 8u * quarter;
+        // its place in the raw chunk: FWD, DGRAD: four 16-byte runs of its row; WGRAD: its column of 16 rows
+        const uint32_t raw_at = smem_u32(raw) + (MODE == CMODE_WGRAD ? (uint32_t)(row >> 5) * 8192u + (uint32_t)quarter * 2048u + (uint32_t)(row & 3) * 4u
+                                                                     : (uint32_t)(quarter >> 1) * 16384u + (uint32_t)row * 128u);
+        uint32_t a_in = 0u;               // FWD, DGRAD: which taps of the unit's row fall inside the image
+        int a_tap = 0, a_c = 0;           // place of the chunk (TMA) or of the thread's quarter (otherwise) along the reduction
+        const float* a_px = nullptr;      // without TMA: the pixel, of the unit whose chunk is loaded next
+        uint32_t a_px_in = 0u;
+        // B, of the chunk loaded next: row r and the q-th run of eight floats of each 64-float row piece (FWD: rows r, r + 64; DGRAD,
+        // WGRAD: row r along the reduction, NB boxes of columns)
         const int q = t & 7, r = t >> 3;
         const uint32_t b_at = smem_u32(smem) + (uint32_t)r * 128u + (uint32_t)((q ^ (r & 7)) << 4);
+        int kpos = 0;                     // its first reduction step
         const float* b_px = nullptr;      // FWD: weight row; DGRAD: column run of the weights
         bool b_in[NB];
         int b_tap = 0, b_o = 0;                     // DGRAD: the weight row's tap and output channel
         int b_h = 0, b_w = 0, dr[NB], ds[NB];       // WGRAD: the pixel row's place; per run its tap shift and
         int b_shift[NB];                            // the float it starts at relative to the pixel's first
-        if (MODE != CMODE_WGRAD) {
-            const int k = kpos + 16 * quarter;
-            a_tap = k / Cred; a_c = k - a_tap * Cred;
-            if (m < p.M) {
-                const int n = div_rcp(m, p.rcp_hw, HW), w = m - n * HW, h = div_rcp(w, p.rcp_w, p.W), x = w - h * p.W;
-                a_px = (MODE == CMODE_FWD ? p.act : p.dy) + (size_t)m * Cred;
-                if (p.taps == 1) a_in = 1u;
-                else
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) {
-                        const int er = MODE == CMODE_FWD ? i / 3 - 1 : 1 - i / 3, es = MODE == CMODE_FWD ? i % 3 - 1 : 1 - i % 3;
-                        if ((unsigned)(h + er) < (unsigned)p.H && (unsigned)(x + es) < (unsigned)p.W) a_in |= 1u << i;
-                    }
-            }
-        } else {
-            a_px = p.dy + m;
-        }
-        if (MODE == CMODE_FWD) {
-            b_px = p.wt + (size_t)(n0 + r) * p.K + 8 * q;
-#pragma unroll
-            for (int j = 0; j < NB; ++j) b_in[j] = n0 + r + 64 * j < p.N;
-        } else {
-#pragma unroll
-            for (int j = 0; j < NB; ++j) b_in[j] = n0 + 64 * j + 8 * q < p.N;
-            if (MODE == CMODE_DGRAD) {
-                b_px = p.wt + n0 + 8 * q;
-                b_tap = (kpos + r) / Cred; b_o = kpos + r - b_tap * Cred;
-            } else {
-                const int w = kpos + r - div_rcp(kpos + r, p.rcp_hw, HW) * HW;
-                b_h = div_rcp(w, p.rcp_w, p.W); b_w = w - b_h * p.W;
-#pragma unroll
-                for (int j = 0; j < NB; ++j) {
-                    const int n = n0 + 64 * j + 8 * q, tap = b_in[j] ? n / p.Cin : 0;
-                    dr[j] = p.taps == 9 ? tap / 3 - 1 : 0; ds[j] = p.taps == 9 ? tap % 3 - 1 : 0;
-                    b_shift[j] = (dr[j] * p.W + ds[j]) * p.Cin + (n - tap * p.Cin);
-                }
-            }
-        }
         const int step_h = (64 / p.W) % p.H, step_w = 64 % p.W;       // WGRAD: one chunk on, in rows and columns
 
-        auto tap_shift = [&](int tap) {
-            if (p.taps == 1) return 0;
-            const int tr = tap >= 6 ? 2 : (tap >= 3 ? 1 : 0), ts = tap - 3 * tr;
-            return (MODE == CMODE_FWD ? (tr - 1) * p.W + ts - 1 : (1 - tr) * p.W + 1 - ts) * Cred;
+        auto taps_inside = [&](int m) {
+            uint32_t in = 0u;
+            if (m >= p.M) return in;
+            if (p.taps == 1) return 1u;
+            const int n = div_rcp(m, p.rcp_hw, HW), w = m - n * HW, h = div_rcp(w, p.rcp_w, p.W), x = w - h * p.W;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                const int er = MODE == CMODE_FWD ? i / 3 - 1 : 1 - i / 3, es = MODE == CMODE_FWD ? i % 3 - 1 : 1 - i % 3;
+                if ((unsigned)(h + er) < (unsigned)p.H && (unsigned)(x + es) < (unsigned)p.W) in |= 1u << i;
+            }
+            return in;
         };
-        auto load_a = [&] {
-            if (MODE == CMODE_WGRAD) {
-                const int k = kpos + 16 * quarter, left = m < p.M ? p.K - k : 0;
-                const float* d = a_px + (size_t)k * p.Cout;
+        // the first chunk of a unit
+        auto first_chunk = [&](const Unit& un) {
+            kpos = un.chunk0 * 64;
+            if (MODE == CMODE_FWD) {
+                b_px = p.wt + (size_t)(un.n0 + r) * p.K + 8 * q;
 #pragma unroll
-                for (int j = 0; j < 16; ++j) ra[j / 8].v[j % 8] = j < left ? __ldg(d + (size_t)j * p.Cout) : 0.f;
-            } else if (K64) {
-                const float* d = a_px + (long)tap_shift(a_tap) + a_c;
-                const bool in = (a_in >> a_tap) & 1u;
-                load8(ra[0], d, in);
-                load8(ra[1], d + 8, in);
+                for (int j = 0; j < NB; ++j) b_in[j] = un.n0 + r + 64 * j < p.N;
             } else {
-                int tap = a_tap, c = a_c;
 #pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    load8(ra[i], a_px + (long)tap_shift(tap) + c, (a_in >> tap) & 1u);
-                    c += 8;
-                    if (c == Cred) { c = 0; ++tap; }
+                for (int j = 0; j < NB; ++j) b_in[j] = un.n0 + 64 * j + 8 * q < p.N;
+                if (MODE == CMODE_DGRAD) {
+                    b_px = p.wt + un.n0 + 8 * q;
+                    b_tap = (kpos + r) / Cred; b_o = kpos + r - b_tap * Cred;
+                } else {
+                    const int w = kpos + r - div_rcp(kpos + r, p.rcp_hw, HW) * HW;
+                    b_h = div_rcp(w, p.rcp_w, p.W); b_w = w - b_h * p.W;
+#pragma unroll
+                    for (int j = 0; j < NB; ++j) {
+                        const int n = un.n0 + 64 * j + 8 * q, tap = b_in[j] ? n / p.Cin : 0;
+                        dr[j] = p.taps == 9 ? tap / 3 - 1 : 0; ds[j] = p.taps == 9 ? tap % 3 - 1 : 0;
+                        b_shift[j] = (dr[j] * p.W + ds[j]) * p.Cin + (n - tap * p.Cin);
+                    }
                 }
             }
+            if (!TMA) {
+                const int k = kpos + 16 * quarter, m = un.m0 + row;
+                a_tap = k / Cred; a_c = k - a_tap * Cred;
+                a_px = (MODE == CMODE_FWD ? p.act : p.dy) + (size_t)m * Cred;
+                a_px_in = taps_inside(m);
+            }
         };
-        auto load_b = [&](int j) {
-            if (MODE == CMODE_FWD) load8(rb[j], b_px + (size_t)(64 * j) * p.K + kpos, b_in[j] && (K64 || kpos + 8 * q < p.K));
-            else if (MODE == CMODE_DGRAD) load8(rb[j], b_px + ((size_t)b_o * p.taps + b_tap) * p.Cin + 64 * j, b_in[j] && b_tap < p.taps);
-            else load8(rb[j], p.act + (long)(kpos + r) * p.Cin + b_shift[j],
-                       b_in[j] && kpos + r < p.K && (unsigned)(b_h + dr[j]) < (unsigned)p.H && (unsigned)(b_w + ds[j]) < (unsigned)p.W);
-        };
-        auto advance = [&] {
+        auto next_chunk = [&] {
             kpos += 64;
             if (MODE == CMODE_WGRAD) {
                 b_w += step_w; b_h += step_h;
                 if (b_w >= p.W) { b_w -= p.W; ++b_h; }
                 if (b_h >= p.H) b_h -= p.H;
-            } else if (K64) {
-                a_c += 64;
-                if (a_c >= Cred) { a_c -= Cred; ++a_tap; }
-            } else {
-                for (a_c += 64; a_c >= Cred; a_c -= Cred) ++a_tap;
             }
             if (MODE == CMODE_DGRAD)
                 for (b_o += 64; b_o >= Cred; b_o -= Cred) ++b_tap;
+            if (!TMA)
+                for (a_c += 64; a_c >= Cred; a_c -= Cred) ++a_tap;
         };
-        const bool do_bias = MODE == CMODE_WGRAD && blockIdx.y == 0;
-        float bsum = 0.f;
-
-        load_a();
+        auto load_a = [&] {               // (without TMA)
+            int tap = a_tap, c = a_c;
 #pragma unroll
-        for (int j = 0; j < NB; ++j) load_b(j);
-        int s = 0;
-        uint32_t ph = 1;      // (a stage's first use needs no wait)
+            for (int i = 0; i < 2; ++i) {
+                int shift = 0;
+                if (p.taps == 9) {
+                    const int tr = tap >= 6 ? 2 : (tap >= 3 ? 1 : 0), ts = tap - 3 * tr;
+                    shift = (MODE == CMODE_FWD ? (tr - 1) * p.W + ts - 1 : (1 - tr) * p.W + 1 - ts) * Cred;
+                }
+                load8(ra[i], a_px + (long)shift + c, (a_px_in >> tap) & 1u);
+                c += 8;
+                if (c == Cred) { c = 0; ++tap; }
+            }
+        };
+        auto load_b = [&](int j) {
+            if (MODE == CMODE_FWD) load8(rb[j], b_px + (size_t)(64 * j) * p.K + kpos, b_in[j] && (TMA || kpos + 8 * q < p.K));
+            else if (MODE == CMODE_DGRAD) load8(rb[j], b_px + ((size_t)b_o * p.taps + b_tap) * p.Cin + 64 * j, b_in[j] && b_tap < p.taps);
+            else load8(rb[j], p.act + (long)(kpos + r) * p.Cin + b_shift[j],
+                       b_in[j] && kpos + r < p.K && (unsigned)(b_h + dr[j]) < (unsigned)p.H && (unsigned)(b_w + ds[j]) < (unsigned)p.W);
+        };
+
+        if (!WT) {
+            first_chunk(unit_at<BN>(p, blockIdx.x));
+            if (!TMA) load_a();
+#pragma unroll
+            for (int j = 0; j < NB; ++j) load_b(j);
+        }
+        Ring st, rw;
+        int chunk = 0;
         bool ok = true;
-        for (int it = 0; it < n_iters; ++it) {
-            if (it >= STAGES) {
-                ok = __all_sync(0xffffffffu, mbar_wait(&empty[s], ph) ? 1 : 0) != 0;
+        for (int u = blockIdx.x; u < p.units; u += gridDim.x) {      // (to the end also after a wait that gave up: the barriers below want every warp)
+            const Unit un = unit_at<BN>(p, u);
+            const bool do_bias = MODE == CMODE_WGRAD && un.n0 == 0;
+            float bsum = 0.f;
+            if (TMA && MODE != CMODE_WGRAD) {
+                a_in = taps_inside(un.m0 + row);
+                a_tap = un.chunk0 * 64 / Cred; a_c = un.chunk0 * 64 - a_tap * Cred;
+            }
+            for (int it = 0; it < un.n_iters && ok; ++it, ++chunk) {
+                bool w = true;
+                if (TMA) w = mbar_wait(&raw_full[rw.i], rw.ph);
+                if (TMA) {
+                    const uint32_t at = raw_at + (uint32_t)rw.i * RAW;
+                    if (MODE == CMODE_WGRAD) {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j)
+                            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(ra[j / 8].v[j % 8]) : "r"(at + 128u * j + (((uint32_t)(row >> 2) & 7u) ^ (uint32_t)(j & 7)) * 16u));
+                    } else {
+                        const bool in = (a_in >> a_tap) & 1u;
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            float* f = &ra[i / 2].v[4 * (i % 2)];
+                            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(f[0]), "=f"(f[1]), "=f"(f[2]), "=f"(f[3])
+                                         : "r"(at + ((((uint32_t)(quarter & 1) * 4u + i) ^ (uint32_t)(row & 7)) << 4)));
+                        }
+                        if (!in)
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) ra[j / 8].v[j % 8] = 0.f;
+                        a_c += 64;
+                        if (a_c >= Cred) { a_c -= Cred; ++a_tap; }
+                    }
+                }
+                if (chunk >= STAGES) w = w && mbar_wait(&empty[st.i], st.ph ^ 1u);
+                ok = __all_sync(0xffffffffu, w ? 1 : 0) != 0;
                 if (!ok) break;
                 tc_fence_after();
-            }
-            const bool more = it + 1 < n_iters;
-            if (more) advance();
-            {
-                uint32_t t0[8], t1[8], t2[8];
-                take_terms(ra[0], t0, t1, t2);
-                take_terms(ra[1], t0 + 4, t1 + 4, t2 + 4);
-                if (do_bias)
+                const bool more = it + 1 < un.n_iters || u + (int)gridDim.x < p.units;
+                if (WT) {
+                } else if (it + 1 < un.n_iters) next_chunk();
+                else if (more) first_chunk(unit_at<BN>(p, u + gridDim.x));
+                {
+                    uint32_t t0[8], t1[8], t2[8];
+                    take_terms(ra[0], t0, t1, t2);
+                    take_terms(ra[1], t0 + 4, t1 + 4, t2 + 4);
+                    if (do_bias)
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) bsum += ra[j / 8].v[j % 8];
+                        for (int j = 0; j < 16; ++j) bsum += ra[j / 8].v[j % 8];
+                    __syncwarp();
+                    if (TMA) {
+                        if (lane == 0) mbar_arrive(smem_u32(&raw_empty[rw.i]));
+                        rw.next(RAWS);
+                    }
+                    const uint32_t at = a_at + (uint32_t)st.i * A_STAGE;
+                    tmem_st8(at, t0);
+                    tmem_st8(at + A_TERM, t1);
+                    tmem_st8(at + 2 * A_TERM, t2);
+                    if (!TMA && more) load_a();
+                }
+#pragma unroll
+                for (int j = 0; j < (WT ? 0 : NB); ++j) {
+                    uint32_t t0[4], t1[4], t2[4];
+                    take_terms(rb[j], t0, t1, t2);
+                    const uint32_t at = b_at + (uint32_t)st.i * C::STAGE + 8192u * j;
+                    st_shared16(at, t0);
+                    st_shared16(at + C::PLANE, t1);
+                    st_shared16(at + 2 * C::PLANE, t2);
+                    if (more) load_b(j);
+                }
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                if (!WT) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                tc_fence_before();
                 __syncwarp();
-                const uint32_t at = a_at + (uint32_t)s * A_STAGE;
-                tmem_st8(at, t0);
-                tmem_st8(at + A_TERM, t1);
-                tmem_st8(at + 2 * A_TERM, t2);
-                if (more) load_a();
+                if (lane == 0) mbar_arrive(smem_u32(&full[st.i]));
+                st.next(STAGES);
             }
-#pragma unroll
-            for (int j = 0; j < NB; ++j) {
-                uint32_t t0[4], t1[4], t2[4];
-                take_terms(rb[j], t0, t1, t2);
-                const uint32_t at = b_at + (uint32_t)s * C::STAGE + 8192u * j;
-                st_shared16(at, t0);
-                st_shared16(at + C::PLANE, t1);
-                st_shared16(at + 2 * C::PLANE, t2);
-                if (more) load_b(j);
+            if (MODE == CMODE_WGRAD && do_bias) {
+                if (quarter > 0) s_bias[(quarter - 1) * 128 + row] = bsum;
+                asm volatile("bar.sync 2, 512;" ::: "memory");
+                if (quarter == 0 && un.m0 + row < p.M)
+                    p.part[(size_t)un.split * p.split_stride + p.bias_off + un.m0 + row] = ((bsum + s_bias[row]) + s_bias[128 + row]) + s_bias[256 + row];
+                asm volatile("bar.sync 2, 512;" ::: "memory");
             }
-            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&full[s]));
-            if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
         if (!ok && lane == 0) { *abort_flag = 1; atomicMax(p.status, (uint32_t)DEV_TIMEOUT_TMA); }
-        if (do_bias) {
-            if (quarter > 0) s_bias[(quarter - 1) * 128 + row] = bsum;
-            asm volatile("bar.sync 2, 512;" ::: "memory");
-            if (quarter == 0 && m < p.M)
-                p.part[(size_t)blockIdx.z * p.split_stride + p.bias_off + m] = ((bsum + s_bias[row]) + s_bias[128 + row]) + s_bias[256 + row];
-        }
     }
 
     // ---- teardown: TMEM is released on every path ----------------------------------------------------------------------------
     tc_fence_before();
     __syncthreads();
     if (*abort_flag) {
-        const uint64_t t0 = globaltimer_ns();          // MMAs that may still be in flight read shared memory
+        const uint64_t t0 = globaltimer_ns();          // copies and MMAs that may still be in flight use shared memory
         while (globaltimer_ns() - t0 < 200000ull) { }
         __syncthreads();
     }
@@ -496,27 +636,68 @@ contract_umma_kernel(const __grid_constant__ SplitParams p)
     }
 }
 
-uint32_t rcp_of(int d) { return d <= 1 ? 0u : (uint32_t)(0x100000000ull / (uint32_t)d) + 1u; }
 
-template <int MODE, int BN, bool K64>
-cudaError_t launch_one(const SplitParams& p, cudaStream_t st)
+template <int MODE, int BN, bool TMA, bool WT>
+cudaError_t launch_one(const ContractArgs& a, SplitParams p, cudaStream_t st)
 {
-    constexpr int SMEM = SplitCfg<BN>::SMEM;
-    const cudaError_t e = raise_smem_limit<contract_umma_kernel<MODE, BN, K64>>(SMEM);
+    constexpr int SMEM = SplitCfg<BN>::smem(TMA);
+    const cudaError_t e = raise_smem_limit<contract_umma_kernel<MODE, BN, TMA, WT>>(SMEM);
     if (e != cudaSuccess) return e;
-    return pdl_launch(contract_umma_kernel<MODE, BN, K64>, dim3((unsigned)((p.M + 127) / 128), (unsigned)((p.N + BN - 1) / BN), (unsigned)p.splits), dim3(THREADS),
-                      (size_t)SMEM, st, p);
+    Maps<TMA> maps{};
+    if constexpr (TMA) {
+        if (!(MODE == CMODE_WGRAD ? umma_map_f32_rows(&maps.a, p.dy, p.npix, p.Cout, 64)
+                                  : umma_map_f32_rows(&maps.a, MODE == CMODE_FWD ? p.act : p.dy, p.npix, MODE == CMODE_FWD ? p.Cin : p.Cout, 128)))
+            return cudaErrorInvalidValue;
+        if (WT && !umma_map_terms(&maps.b, a.wterms, p.Cout, (long)p.taps * p.Cin, a.wterms_stride, MODE == CMODE_FWD ? BN : 64)) return cudaErrorInvalidValue;
+    }
+    p.m_tiles = (p.M + 127) / 128; p.n_tiles = (p.N + BN - 1) / BN;
+    const long units = (long)p.m_tiles * p.n_tiles * p.splits;
+    if (units >= (1L << 30)) return cudaErrorInvalidValue;
+    p.units = (int)units;
+    p.rcp_m = rcp_of(p.m_tiles); p.rcp_n = rcp_of(p.n_tiles);
+    return pdl_launch(contract_umma_kernel<MODE, BN, TMA, WT>, dim3((unsigned)(units < 148 ? units : 148)), dim3(THREADS), (size_t)SMEM, st, maps, p);
+}
+template <int MODE, int BN>
+cudaError_t launch_form(const ContractArgs& a, const SplitParams& p, cudaStream_t st)
+{
+    if constexpr (MODE == CMODE_WGRAD) return launch_one<MODE, BN, true, false>(a, p, st);
+    else {
+        return a.wterms != nullptr ? launch_one<MODE, BN, true, true>(a, p, st) : launch_one<MODE, BN, false, false>(a, p, st);
+    }
 }
 template <int MODE>
-cudaError_t launch_mode(int bn, const SplitParams& p, cudaStream_t st)
+cudaError_t launch_mode(const ContractArgs& a, const SplitParams& p, cudaStream_t st)
 {
-    if (MODE == CMODE_WGRAD || (MODE == CMODE_DGRAD ? p.Cout : p.Cin) % 64 == 0)
-        return bn == 128 ? launch_one<MODE, 128, true>(p, st) : launch_one<MODE, 64, true>(p, st);
-    return bn == 128 ? launch_one<MODE, 128, MODE == CMODE_WGRAD>(p, st) : launch_one<MODE, 64, MODE == CMODE_WGRAD>(p, st);
+    return a.plan.bn == 128 ? launch_form<MODE, 128>(a, p, st) : launch_form<MODE, 64>(a, p, st);
+}
+
+// n floats as three planes of bf16 terms, `stride` elements apart
+__global__ void __launch_bounds__(256)
+split_weights_kernel(const float4* __restrict__ w, uint2* __restrict__ terms, size_t n4, size_t stride4)
+{
+    pdl_prologue();
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
+        float4 v = __ldg(w + i);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            uint2 t;
+            t.x = take_term(v.x, v.y);
+            t.y = take_term(v.z, v.w);
+            terms[k * stride4 + i] = t;
+        }
+    }
 }
 
 }  // namespace
 
+cudaError_t launch_split_weights(const float* w, __nv_bfloat16* terms, size_t n, size_t stride, cudaStream_t st)
+{
+    const size_t n4 = n / 4;
+    const long blocks = (long)((n4 + 255) / 256);
+    SB_LAUNCH((split_weights_kernel), (int)(blocks < 148 * 8 ? blocks : 148 * 8), 256, 0, st, (const float4*)w, (uint2*)terms, n4, stride / 4);
+    return cudaGetLastError();
+}
+bool contract_umma_whole_taps(int mode, int Cin, int Cout) { return (mode == CMODE_DGRAD ? Cout : Cin) % 64 == 0; }
 bool contract_umma_ok(int taps, int Cin, int Cout) { return Cin % 8 == 0 && Cout % 8 == 0 && (taps == 1 || taps == 9); }
 
 cudaError_t launch_contract_umma(const ContractArgs& a, cudaStream_t st)
@@ -533,8 +714,8 @@ cudaError_t launch_contract_umma(const ContractArgs& a, cudaStream_t st)
     p.part = a.part; p.split_stride = a.split_stride; p.bias_off = a.bias_off;
     p.out = a.out32 ? a.out32 : (float*)a.out; p.bias = a.bias; p.relu = a.relu; p.ref = (const float*)a.ref;
     p.status = a.status;
-    if (a.mode == CMODE_FWD) return launch_mode<CMODE_FWD>(a.plan.bn, p, st);
-    return a.mode == CMODE_DGRAD ? launch_mode<CMODE_DGRAD>(a.plan.bn, p, st) : launch_mode<CMODE_WGRAD>(a.plan.bn, p, st);
+    if (a.mode == CMODE_FWD) return launch_mode<CMODE_FWD>(a, p, st);
+    return a.mode == CMODE_DGRAD ? launch_mode<CMODE_DGRAD>(a, p, st) : launch_mode<CMODE_WGRAD>(a, p, st);
 }
 
 }  // namespace sb

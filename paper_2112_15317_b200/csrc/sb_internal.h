@@ -154,9 +154,13 @@ struct ContractArgs {
     const float* bias; int relu;           // FWD
     const void* ref;                       // DGRAD: zero where ref <= 0
     uint32_t* status;                      // device status word of the bounded waits
+    const __nv_bfloat16* wterms;           // umma, FWD / DGRAD: the weights as three planes of bf16 terms, wterms_stride elements apart (or nullptr)
+    size_t wterms_stride;
 };
 cudaError_t launch_contract(const ContractArgs& a, bool bf16, cudaStream_t st);
 bool contract_umma_ok(int taps, int Cin, int Cout);
+bool contract_umma_whole_taps(int mode, int Cin, int Cout);      // a reduction chunk never crosses taps: the forms that fetch by TMA
+cudaError_t launch_split_weights(const float* w, __nv_bfloat16* terms, size_t n, size_t stride, cudaStream_t st);     // n, stride: multiples of 4
 cudaError_t launch_contract_umma(const ContractArgs& a, cudaStream_t st);      // (without the second kernel of a split FWD / DGRAD)
 
 // Input-layer convolution (Cin of 1, 3 or 4; Cout a multiple of 8): dedicated forward and weight+bias

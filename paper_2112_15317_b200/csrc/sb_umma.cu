@@ -2336,21 +2336,33 @@ static bool mat_map(CUtensorMap* map, const void* ptr, long rows, long cols, int
     return encode_map(map, ptr, d, s, b);
 }
 
-// Row-major float matrix [rows][cols] -> map (cols, rows, 1, 1) with a (64, 128, 1, 1) box, no swizzle: 128 rows of 256 bytes.
-static bool mat_map_f32(CUtensorMap* map, const void* ptr, long rows, long cols)
+// Row-major float matrix [rows][cols] -> map (cols, rows, 1, 1) with a (box_cols, box_rows, 1, 1) box.
+static bool encode_f32(CUtensorMap* map, const void* ptr, long rows, long cols, int box_cols, int box_rows, CUtensorMapSwizzle swizzle)
 {
     if (!get_encode()) return false;
     cuuint64_t gd[4] = {(cuuint64_t)cols, (cuuint64_t)rows, 1, 1};
     cuuint64_t gs[3] = {(cuuint64_t)cols * 4, (cuuint64_t)rows * cols * 4, (cuuint64_t)rows * cols * 4};
-    cuuint32_t bx[4] = {64, 128, 1, 1};
+    cuuint32_t bx[4] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows, 1, 1};
     cuuint32_t es[4] = {1, 1, 1, 1};
     CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<void*>(ptr), gd, gs, bx, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                          CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                          swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
         snprintf(g_umma_err, sizeof(g_umma_err), "cuTensorMapEncodeTiled (float matrix %ld x %ld) failed (%d)", rows, cols, (int)r);
         return false;
     }
     return true;
+}
+
+// 128 rows of 256 bytes, no swizzle
+static bool mat_map_f32(CUtensorMap* map, const void* ptr, long rows, long cols) { return encode_f32(map, ptr, rows, cols, 64, 128, CU_TENSOR_MAP_SWIZZLE_NONE); }
+bool umma_map_f32_rows(CUtensorMap* map, const void* ptr, long rows, long cols, int box_rows) { return encode_f32(map, ptr, rows, cols, 32, box_rows, CU_TENSOR_MAP_SWIZZLE_128B); }
+
+bool umma_map_terms(CUtensorMap* map, const void* ptr, long rows, long cols, size_t plane_stride, int box_rows)
+{
+    uint64_t d[4] = {(uint64_t)cols, (uint64_t)rows, 3, 1};
+    uint64_t s[3] = {(uint64_t)cols * 2, (uint64_t)plane_stride * 2, (uint64_t)plane_stride * 6};
+    uint32_t b[4] = {64, (uint32_t)box_rows, 1, 1};
+    return encode_map(map, ptr, d, s, b);
 }
 
 static int cdiv_i(long a, long b) { return (int)((a + b - 1) / b); }

@@ -113,6 +113,11 @@ struct FcWgradArgs {
 };
 cudaError_t launch_fc_wgrad(const FcWgradArgs& a, cudaStream_t st);
 
+// Tensor map of a row-major float matrix with boxes of 32 columns x box_rows rows: rows of 128 bytes in the 128-byte swizzle.
+bool umma_map_f32_rows(CUtensorMap* map, const void* ptr, long rows, long cols, int box_rows);
+// Tensor map of three row-major bf16 matrices, plane_stride elements apart, with boxes of 64 columns x box_rows rows of one plane.
+bool umma_map_terms(CUtensorMap* map, const void* ptr, long rows, long cols, size_t plane_stride, int box_rows);
+
 const char* umma_last_error();
 // One CTA that waits (bounded by limit_ns) on a barrier nothing completes, then reports through the status word.
 cudaError_t launch_wait_probe(uint32_t* status, unsigned long long limit_ns, cudaStream_t st);

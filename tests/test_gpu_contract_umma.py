@@ -65,6 +65,18 @@ def test_passes_against_double(H, W, c0, c1, width, b, R, on):
     checks.le("fc input gradient", tu.frob(t(sb.SB_T_DACT, 1).reshape(wl.B, -1), (x.grad * (x > 0)).detach()), BOUND)
     checks.le("fc weight gradient", tu.frob(wt(sb.SB_T_GRAD_W, 2)[:, :, 0, 0], w.grad), BOUND)
     checks.le("fc bias gradient", tu.frob(wt(sb.SB_T_GRAD_B, 2).reshape(-1), bias.grad), BOUND)
+
+    # weights changed between the calls: each call reads them as they are
+    x = t(sb.SB_T_ACT, 0).permute(0, 3, 1, 2).requires_grad_()
+    new = -0.5 * m.read(sb.SB_T_WEIGHT, 1, 0, squeeze=False) + 0.01
+    m.write(sb.SB_T_WEIGHT, 1, 0, new)
+    m.forward_layers(1, 1)
+    m.write(sb.SB_T_WEIGHT, 1, 0, 2.0 * new)
+    m.backward_layers(1, 1)
+    y = F.conv2d(x, torch.from_numpy(new).double().permute(0, 3, 1, 2), bias=wt(sb.SB_T_BIAS, 1).reshape(-1), padding=1)
+    (2.0 * y).backward(t(sb.SB_T_DACT, 1).permute(0, 3, 1, 2))
+    checks.le("conv forward, new weights", tu.frob(t(sb.SB_T_ACT, 1), y.relu().permute(0, 2, 3, 1).detach()), BOUND)
+    checks.le("conv input gradient, new weights", tu.frob(t(sb.SB_T_DACT, 0), (x.grad * (x > 0)).permute(0, 2, 3, 1).detach()), BOUND)
     assert m.debug_check_guards()[0] == 0
     m.loss()       # raises if a bounded wait ran out
     m.close()
