@@ -177,7 +177,7 @@ fc_wgrad_kernel(const __grid_constant__ CUtensorMap mapDy, const __grid_constant
                 if (col < p.in_f)
 #pragma unroll
                     for (int r = 0; r < 32; ++r)
-                        if (row0 + r0 + r < p.out_f) dst[(size_t)r * p.in_f] = __uint_as_float(v[r / 16][r % 16]);
+                        if (row0 + r0 + r < p.out_f) __stcs(dst + (size_t)r * p.in_f, __uint_as_float(v[r / 16][r % 16]));
                 dst += (size_t)32 * p.in_f;
             }
             tc_fence_before();
