@@ -1267,8 +1267,9 @@ sb_status sb_forward(sb_model* m, const void* const* x, const int32_t* const* la
 static sb_status weight_side(sb_model* m, int i, cudaStream_t wst, bool classic)
 {
     pdl_classic() = classic ? 1 : 0;
-    // (sub-iterations: the first FC layer's update goes before those of the large layers above it, see modulo_step_direct)
-    if (m->sub_active && i == m->first_fc) launch_priority() = -1;
+    // (sub-iterations: the small layers' updates -- the first FC layer's, which the next sub-iteration reads first, and the narrow
+    // logits layer's -- go before those of the large layers between them)
+    if (m->sub_active && (i == m->first_fc || m->L[i].narrow)) launch_priority() = -1;
     const sb_status s = backward_layer(m, i, wst, SIDE_W);
     launch_priority() = 0;
     pdl_classic() = 0;
@@ -1301,6 +1302,39 @@ static sb_status backward_pass(sb_model* m, cudaStream_t st, bool fuse_update, H
     m->st_clean = false;
     unsigned used_streams = 0;   // weight streams that received work in this pass (only those are joined)
     bool used_ustream = false;   // likewise the update stream
+    // The update of layer i runs on a third stream: after the layer's gradients are complete (weight stream) and after its
+    // input-gradient kernel, which reads the weights the update rewrites (main stream).
+    auto update_aside = [&](int i, cudaStream_t wst) -> sb_status {
+        const Layer& l = m->L[i];
+        CU_TRY(cudaEventRecord(m->ev_wdone[i], wst));
+        CU_TRY(cudaStreamWaitEvent(m->ustream, m->ev_dgrad[i], 0));
+        CU_TRY(cudaStreamWaitEvent(m->ustream, m->ev_wdone[i], 0));
+        used_ustream = true;
+        const size_t off = l.p_w, cnt = (l.p_b - l.p_w) + align_up(l.n_b, 64);
+        cudaStream_t st = m->ustream;   // the launch bracket below records on the stream it launches on
+        m->cur_layer = i;
+        launch_priority() = m->sub_active && l.narrow ? -1 : 0;
+        const cudaError_t e = launch_sgd(m->Wm + off, m->Vm + off, m->Gm + off, m->Sm ? m->Sm + off : nullptr, cnt, hy, st);
+        launch_priority() = 0;
+        L_TRY("sgd", 0.0, (double)cnt * (m->bf16 ? 22.0 : 20.0), e);
+        if (!join) CU_TRY(cudaEventRecord(m->ev_wdone[i], st));
+        return SB_OK;
+    };
+    // The narrow layer's weight side is left until the data gradient of the layer below has run: its blocks keep that kernel's 200 KB CTAs
+    // from starting on their SMs (4096 -> 4096 at batch 32 took 15 - 18 us beside it, 9.5 without), and nothing waits for its result.
+    int held = -1;
+    bool held_classic = false;
+    auto held_weight_side = [&]() -> sb_status {
+        const int i = held;
+        held = -1;
+        if (i < 0) return SB_OK;
+        cudaStream_t wst = m->wstreams[i % m->n_wstreams];
+        CU_TRY(cudaEventRecord(m->ev_join, st));
+        CU_TRY(cudaStreamWaitEvent(wst, m->ev_join, 0));
+        const sb_status s = weight_side(m, i, wst, held_classic);
+        if (s != SB_OK) return s;
+        return fuse ? update_aside(i, wst) : SB_OK;
+    };
     for (int i = hi; i >= lo; --i) {
         Layer& l = m->L[i];
         const bool has_params = l.kind == SB_CONV3X3_RELU || l.kind == SB_FC_RELU || l.kind == SB_FC;
@@ -1331,6 +1365,13 @@ static sb_status backward_pass(sb_model* m, cudaStream_t st, bool fuse_update, H
             const bool in_reduce = fuse && ((reduce_updates && (l.kind == SB_CONV3X3_RELU || (!l.narrow && !l.um.wgrad.enabled))) ||
                                             (fc_wgrad_update && l.kind != SB_CONV3X3_RELU && !l.narrow && umma_fc_wgrad_can_update(m, i)));
             sb_status s = SB_OK;
+            if (l.narrow && i > lo && held < 0) {
+                s = chain_bwd(m, i, st, SIDE_D);
+                if (s != SB_OK) return s;
+                if (fuse) CU_TRY(cudaEventRecord(m->ev_dgrad[i], st));
+                held = i; held_classic = classic;
+                continue;
+            }
             if (in_reduce) {
                 s = chain_bwd(m, i, st, SIDE_D);
                 if (s != SB_OK) return s;
@@ -1341,6 +1382,8 @@ static sb_status backward_pass(sb_model* m, cudaStream_t st, bool fuse_update, H
                 if (s != SB_OK) return s;
                 if (m->fuse.covered == l.n_w + l.n_b) {     // every parameter of the layer has taken its update
                     if (!join) CU_TRY(cudaEventRecord(m->ev_wdone[i], wst));
+                    s = held_weight_side();
+                    if (s != SB_OK) return s;
                     continue;
                 }
                 if (m->fuse.covered != 0) return fail(SB_ERR_STATE, "layer %d: update folded into part of its reduces only", i);
@@ -1351,26 +1394,20 @@ static sb_status backward_pass(sb_model* m, cudaStream_t st, bool fuse_update, H
                 if (s != SB_OK) return s;
             }
             if (fuse) {
-                // The update of this layer runs on a third stream: after the layer's gradients are complete (weight
-                // stream) and after its input-gradient kernel, which reads the weights the update rewrites (main stream).
                 if (!in_reduce) CU_TRY(cudaEventRecord(m->ev_dgrad[i], st));
-                CU_TRY(cudaEventRecord(m->ev_wdone[i], wst));
-                CU_TRY(cudaStreamWaitEvent(m->ustream, m->ev_dgrad[i], 0));
-                CU_TRY(cudaStreamWaitEvent(m->ustream, m->ev_wdone[i], 0));
-                used_ustream = true;
-                const size_t off = l.p_w, cnt = (l.p_b - l.p_w) + align_up(l.n_b, 64);
-                {
-                    cudaStream_t st = m->ustream;   // the launch bracket below records on the stream it launches on
-                    m->cur_layer = i;
-                    L_TRY("sgd", 0.0, (double)cnt * (m->bf16 ? 22.0 : 20.0),
-                          launch_sgd(m->Wm + off, m->Vm + off, m->Gm + off, m->Sm ? m->Sm + off : nullptr, cnt, hy, st));
-                    if (!join) CU_TRY(cudaEventRecord(m->ev_wdone[i], st));
-                }
+                s = update_aside(i, wst);
+                if (s != SB_OK) return s;
             }
+            s = held_weight_side();
+            if (s != SB_OK) return s;
         } else {
             sb_status s = chain_bwd(m, i, st, SIDE_BOTH);
             if (s != SB_OK) return s;
         }
+    }
+    {
+        const sb_status s = held_weight_side();
+        if (s != SB_OK) return s;
     }
     m->st_clean = false;
     if (fuse && !join) return SB_OK;
