@@ -17,20 +17,22 @@
 //   4096 -> 1024, batch 96                         1.8e-7 -> 1.0e-7                  2.1e-7 -> 0.9e-7                   1.3e-7 -> 0.5e-7
 //   3x3, 8 -> 40 channels at 5x7, batch 3          0.8e-7 -> 0.6e-7                  1.2e-7 -> 0.8e-7                   1.2e-7 -> 0.5e-7
 //
-// One CTA per SM walks (tile, split) units; the results of a unit are written while the next one is under way.  Roles (24 warps; registers
-// are moved between them): warp 0 allocates TMEM and issues the MMAs; warp 1 fetches A as raw floats and warp 2 the weights' terms by TMA;
-// warps 4-7 keep the running sums and write the results; warps 8-23 take the floats apart and store the terms, A into tensor memory (a
-// lane per row; WGRAD: transposed on the way) and B as 128-byte swizzled rows of shared memory, the next chunk of B in flight behind the
-// conversion of the present one.  A in tensor memory keeps its terms off the shared-memory port, which would else carry 40 KB per 16 steps of
-// a 128 x 128 tile.  The weights of a convolution are read by every row tile, so a kernel of their own takes them apart once a call.
+// One CTA per SM walks (tile, split) units; the results of a unit are written while the next one is under way.  Roles (24 warps, 16
+// where the weights arrive as terms; registers are moved between them): warp 0 allocates TMEM and issues the MMAs; warp 1 fetches A as
+// raw floats and warp 2 the weights' terms by TMA; warps 4-7 keep the running sums and write the results; warps 8 and up take the
+// floats apart and store the terms, A into tensor memory (a lane per row; WGRAD: transposed on the way) and B as 128-byte swizzled
+// rows of shared memory, the next chunk of B in flight behind the conversion of the present one.  A in tensor memory keeps its terms
+// off the shared-memory port, which would else carry 40 KB per 16 steps of a 128 x 128 tile.  The weights of a convolution are read by
+// every row tile, so a kernel of their own takes them apart once a call.
 //
-// What bounds it: issue slots.  A chunk of 128 x 128 x 64 takes 2500 - 2700 cycles where its 24 MMAs take 1536, one of 128 x 64 x 64 2000
-// (768): 16 converter warps of some 200 instructions a chunk (350 where they convert B as well), the summing warps' 128 additions and the
-// MMA warp share the four schedulers, and the single buffer of leading products of the wide tile makes MMA and sums wait for each other.
+// What bounds it: issue slots.  A chunk of 128 x 128 x 64 takes 2500 - 2700 cycles where its 24 MMAs take 1536, one of 128 x 64 x 64
+// 2000 (768): the converters' instructions (16 warps of 350 a chunk, or, without B to convert, eight of twice a row's elements: a wait
+// and an arrival per 32 elements, not per 16, forward of 64 channels 66 -> 62), the summing warps' 128 additions and the MMA warp
+// share the four schedulers, and the single buffer of leading products of the wide tile makes MMA and sums wait for each other.
 // Without TMA and with a CTA per unit the same layers took a third longer (a row per lane made each load of A 32 wavefronts of the L1
-// port).  Float CUDA cores -> here, us at batch 96: 3x3 over 64 channels at 32x32 forward 180 -> 66, input gradient 175 -> 75, weight gradient
-// 177 -> 91; 128 channels at 16x16 155 / 164 / 156 -> 65 / 59 / 50; 256 channels at 8x8 157 / 170 / 159 -> 50 / 50 / 47; 4096 -> 1024 30 / 27
-// / 23 -> 18 / 18 / 18.  The 7-conv / 3-FC net: 2.54 -> 0.98 ms an iteration.
+// port).  Float CUDA cores -> here, us at batch 96: 3x3 over 64 channels at 32x32 forward 180 -> 62, input gradient 175 -> 72, weight
+// gradient 177 -> 91; 128 channels at 16x16 155 / 164 / 156 -> 65 / 59 / 50; 256 channels at 8x8 157 / 170 / 159 -> 47 / 48 / 47; 4096
+// -> 1024 30 / 27 / 23 -> 18 / 18 / 18.  The 7-conv / 3-FC net: 2.54 -> 0.96 ms an iteration.
 //
 // Non-finite operands: infinity - infinity in the splitting makes the terms NaN where a float multiply-add would give an infinity, so
 // a row with a NaN in it is computed again with plain multiply-adds by the thread that owns it.
@@ -58,8 +60,15 @@ struct SplitParams {
     uint32_t* status;
 };
 
-// 24 warps: 4 for the MMAs (one works), 4 running sums, 16 converters.  Registers of the 80 a thread at launch: 32 + 160 + 4 * 72 = 6 * 80.
-constexpr int THREADS = 768, CONV0 = 256, REGS_ISSUE = 32, REGS_SUMS = 160, REGS_CONV = 72;
+// Warps: 4 issue, 4 keep sums, CW convert: 16, or 8 where they convert A only.  Registers are a share of those at launch:
+// 80 a thread: 32 + 160 + 4 * 72 = 6 * 80; 128 a thread: 40 + 200 + 2 * 136 = 4 * 128.
+template <bool WT> struct Roles {
+    static constexpr int CW = WT ? 8 : 16, THREADS = 256 + 32 * CW, PARTS = 16 / CW;      // PARTS: quarters of a chunk's row a converter takes
+    static constexpr int REGS_ISSUE = WT ? 40 : 32, REGS_SUMS = WT ? 200 : 160, REGS_CONV = WT ? 136 : 72;
+};
+static_assert(Roles<true>::REGS_ISSUE < 128 && Roles<true>::REGS_CONV > 128 && Roles<true>::REGS_ISSUE + Roles<true>::REGS_SUMS + 2 * Roles<true>::REGS_CONV <= 4 * 128, "dec lowers, inc raises, within the launch's");
+static_assert(Roles<false>::REGS_ISSUE < 80 && Roles<false>::REGS_CONV < 80 && Roles<false>::REGS_ISSUE + Roles<false>::REGS_SUMS + 4 * Roles<false>::REGS_CONV <= 6 * 80, "");
+constexpr int CONV0 = 256;
 constexpr int STAGES = 2, RAWS = 2, RAW = 32768, CTRL = 8192;
 // PLANE: one term of the B tile, BN rows of 128 bytes (FWD) or 64-column boxes of 64 rows.  RAW: a chunk of A as floats, 32-column
 // boxes of 128-byte swizzled rows.  Tensor memory columns: buffers of leading products, buffers of the other products, then the
@@ -207,10 +216,11 @@ struct Ring {
 // tap and its rows are those of the tile, shifted; WGRAD: always); otherwise the converters load it themselves.
 // WT: B arrives as terms by TMA (FWD, DGRAD of convolutions, whose weights every row tile reads: launch_split_weights).
 template <int MODE, int BN, bool TMA, bool WT>
-__global__ void __launch_bounds__(THREADS, 1)
+__global__ void __launch_bounds__(Roles<WT>::THREADS, 1)
 contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_constant__ SplitParams p)
 {
     using C = SplitCfg<BN>;
+    using R = Roles<WT>;
     constexpr int NB = BN / 64;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -233,7 +243,7 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
         // (the barriers lie one after another: a lane each)
         constexpr int B0 = STAGES, B1 = B0 + STAGES, B2 = B1 + RAWS, B3 = B2 + RAWS, B4 = B3 + C::LEADS, B5 = B4 + C::LEADS, B6 = B5 + C::RESTS, B7 = B6 + C::RESTS;
         if (lane < B7) {
-            const uint32_t n = lane < B0 ? (WT ? 17u : 16u) : lane < B2 ? 1u : lane < B3 ? 16u : lane < B4 ? 1u : lane < B5 ? 4u : lane < B6 ? 1u : 4u;
+            const uint32_t n = lane < B0 ? (uint32_t)(R::CW + (WT ? 1 : 0)) : lane < B2 ? 1u : lane < B3 ? (uint32_t)R::CW : lane < B4 ? 1u : lane < B5 ? 4u : lane < B6 ? 1u : 4u;
             mbar_init(&full[lane], n);
             if (lane == 0) *abort_flag = 0;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -251,7 +261,7 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
     const int Cred = MODE == CMODE_DGRAD ? p.Cout : p.Cin;
 
     if (warp < 4) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_ISSUE));
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R::REGS_ISSUE));
         if (warp == 0) {
             // =========================== MMA issuer (the warp in lock-step, one elected lane issues) =============================
             constexpr bool B_MN = MODE != CMODE_FWD;
@@ -360,10 +370,11 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
         }
     } else if (warp < 8) {
         // =========================== running sums and results ====================================================================
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_SUMS));
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(R::REGS_SUMS));
         const int q = warp % 4;
         const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16);
         const bool raw_sums = MODE == CMODE_WGRAD || p.splits > 1;
+        constexpr int LD = WT ? 2 : 1;      // loads per wait: what the registers allow
         Ring lead, rest;
         bool ok = true;
         for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
@@ -380,12 +391,15 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
                 tc_fence_after();
                 const uint32_t from = taddr + (last ? C::COL_REST + (uint32_t)rest.i * BN : (uint32_t)lead.i * BN);
 #pragma unroll
-                for (int c = 0; c < BN; c += 16) {
-                    uint32_t v[16];
-                    tmem_ld16(from + c, v);
+                for (int c = 0; c < BN; c += 16 * LD) {
+                    uint32_t v[LD][16];
+#pragma unroll
+                    for (int l = 0; l < LD; ++l) tmem_ld16(from + c + 16 * l, v[l]);
                     tmem_ld_wait();
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) acc[c + j] += __uint_as_float(v[j]);
+                    for (int l = 0; l < LD; ++l)
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) acc[c + 16 * l + j] += __uint_as_float(v[l][j]);
                 }
                 tc_fence_before();
                 __syncwarp();
@@ -425,12 +439,13 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
         if (!ok && lane == 0) { *abort_flag = 1; atomicMax(p.status, (uint32_t)DEV_TIMEOUT_EPI); }
     } else {
         // =========================== converters ==================================================================================
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_CONV));
+        if constexpr (WT) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(R::REGS_CONV));     // (above those at launch)
+        else asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R::REGS_CONV));
         const int t = threadIdx.x - CONV0, HW = p.H * p.W;
-        F8 ra[2], rb[NB];
+        F8 ra[2 * R::PARTS], rb[NB];
 
-        // A: this thread's row is the TMEM lane of its warp's quadrant, its reduction steps a quarter of the chunk
-        const int row = (warp & 3) * 32 + lane, quarter = (warp - 8) >> 2;
+        // A: this thread's row is the TMEM lane of its warp's quadrant, its reduction steps PARTS quarters of the chunk
+        const int row = (warp & 3) * 32 + lane, quarter = ((warp - 8) >> 2) * R::PARTS;
         const uint32_t a_at = tmem + C::COL_A + ((uint32_t)((warp & 3) * 32) << 16) + 8u * quarter;
         // its place in the raw chunk: FWD, DGRAD: four 16-byte runs of its row; WGRAD: its column of 16 rows
         const uint32_t raw_at = smem_u32(raw) + (MODE == CMODE_WGRAD ? (uint32_t)(row >> 5) * 8192u + (uint32_t)quarter * 2048u + (uint32_t)(row & 3) * 4u
@@ -556,14 +571,14 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
                     } else {
                         const bool in = (a_in >> a_tap) & 1u;
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
+                        for (int i = 0; i < 4 * R::PARTS; ++i) {
                             float* f = &ra[i / 2].v[4 * (i % 2)];
                             asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(f[0]), "=f"(f[1]), "=f"(f[2]), "=f"(f[3])
                                          : "r"(at + ((((uint32_t)(quarter & 1) * 4u + i) ^ (uint32_t)(row & 7)) << 4)));
                         }
                         if (!in)
 #pragma unroll
-                            for (int j = 0; j < 16; ++j) ra[j / 8].v[j % 8] = 0.f;
+                            for (int j = 0; j < 16 * R::PARTS; ++j) ra[j / 8].v[j % 8] = 0.f;
                         a_c += 64;
                         if (a_c >= Cred) { a_c -= Cred; ++a_tap; }
                     }
@@ -576,19 +591,20 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
                 if (WT) {
                 } else if (it + 1 < un.n_iters) next_chunk();
                 else if (more) first_chunk(unit_at<BN>(p, u + gridDim.x));
-                {
+#pragma unroll
+                for (int h = 0; h < R::PARTS; ++h) {
                     uint32_t t0[8], t1[8], t2[8];
-                    take_terms(ra[0], t0, t1, t2);
-                    take_terms(ra[1], t0 + 4, t1 + 4, t2 + 4);
+                    take_terms(ra[2 * h], t0, t1, t2);
+                    take_terms(ra[2 * h + 1], t0 + 4, t1 + 4, t2 + 4);
                     if (do_bias)
 #pragma unroll
                         for (int j = 0; j < 16; ++j) bsum += ra[j / 8].v[j % 8];
                     __syncwarp();
-                    if (TMA) {
+                    if (TMA && h + 1 == R::PARTS) {
                         if (lane == 0) mbar_arrive(smem_u32(&raw_empty[rw.i]));
                         rw.next(RAWS);
                     }
-                    const uint32_t at = a_at + (uint32_t)st.i * A_STAGE;
+                    const uint32_t at = a_at + (uint32_t)st.i * A_STAGE + 8u * h;
                     tmem_st8(at, t0);
                     tmem_st8(at + A_TERM, t1);
                     tmem_st8(at + 2 * A_TERM, t2);
@@ -655,7 +671,7 @@ cudaError_t launch_one(const ContractArgs& a, SplitParams p, cudaStream_t st)
     if (units >= (1L << 30)) return cudaErrorInvalidValue;
     p.units = (int)units;
     p.rcp_m = rcp_of(p.m_tiles); p.rcp_n = rcp_of(p.n_tiles);
-    return pdl_launch(contract_umma_kernel<MODE, BN, TMA, WT>, dim3((unsigned)(units < 148 ? units : 148)), dim3(THREADS), (size_t)SMEM, st, maps, p);
+    return pdl_launch(contract_umma_kernel<MODE, BN, TMA, WT>, dim3((unsigned)(units < 148 ? units : 148)), dim3(Roles<WT>::THREADS), (size_t)SMEM, st, maps, p);
 }
 template <int MODE, int BN>
 cudaError_t launch_form(const ContractArgs& a, const SplitParams& p, cudaStream_t st)
