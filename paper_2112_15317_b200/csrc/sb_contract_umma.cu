@@ -12,7 +12,7 @@
 // rounded multiply-adds of the CUDA cores.  The leading products a0 b0 are therefore accumulated over 64 reduction steps only (four
 // instructions) and then added to a rounded running sum in registers; the remaining products, 2^-9 times smaller, stay in an
 // accumulator of their own until the end.  Error against 64-bit sums (2-norm; half-normal x, normal w and dy), CUDA cores -> here:
-//   3x3, 64 channels at 32x32, batch 96    forward 3.0e-7 -> 0.8e-7   input gradient 4.2e-7 -> 0.9e-7   weight gradient 4.6e-7 -> 1.9e-7
+//   3x3, 64 channels at 32x32, batch 96    forward 3.0e-7 -> 0.9e-7   input gradient 4.2e-7 -> 0.9e-7   weight gradient 4.6e-7 -> 1.9e-7
 //   3x3, 256 channels at 8x8, batch 96             3.4e-7 -> 0.9e-7                  4.8e-7 -> 1.0e-7                   3.3e-7 -> 1.1e-7
 //   4096 -> 1024, batch 96                         1.8e-7 -> 1.0e-7                  2.1e-7 -> 0.9e-7                   1.3e-7 -> 0.5e-7
 //   3x3, 8 -> 40 channels at 5x7, batch 3          0.8e-7 -> 0.6e-7                  1.2e-7 -> 0.8e-7                   1.2e-7 -> 0.5e-7
@@ -25,14 +25,18 @@
 // off the shared-memory port, which would else carry 40 KB per 16 steps of a 128 x 128 tile.  The weights of a convolution are read by
 // every row tile, so a kernel of their own takes them apart once a call.
 //
-// What bounds it: issue slots.  A chunk of 128 x 128 x 64 takes 2500 - 2700 cycles where its 24 MMAs take 1536, one of 128 x 64 x 64
-// 2000 (768): the converters' instructions (16 warps of 350 a chunk, or, without B to convert, eight of twice a row's elements: a wait
-// and an arrival per 32 elements, not per 16, forward of 64 channels 66 -> 62), the summing warps' 128 additions and the MMA warp
-// share the four schedulers, and the single buffer of leading products of the wide tile makes MMA and sums wait for each other.
-// Without TMA and with a CTA per unit the same layers took a third longer (a row per lane made each load of A 32 wavefronts of the L1
-// port).  Float CUDA cores -> here, us at batch 96: 3x3 over 64 channels at 32x32 forward 180 -> 62, input gradient 175 -> 72, weight
-// gradient 177 -> 91; 128 channels at 16x16 155 / 164 / 156 -> 65 / 59 / 50; 256 channels at 8x8 157 / 170 / 159 -> 47 / 48 / 47; 4096
-// -> 1024 30 / 27 / 23 -> 18 / 18 / 18.  The 7-conv / 3-FC net: 2.54 -> 0.96 ms an iteration.
+// What bounds it: forward and input gradient, the chain through the issuing warp: a chunk of 128 x 128 x 64 takes 2350 cycles where
+// its 24 MMAs take 1536, one of 128 x 64 x 64 1750 (768). Measured with clocks in the kernel: of 1890 cycles of the narrow chunk 1290
+// went into getting 24 instructions out (54 each) and 600 into waits, most of them for barriers that had long flipped. Hence 16
+// instructions of twice the width there, and the next chunk's barriers tested behind the last queued instructions: 66 -> 58 us forward
+// over 64 channels, 7-conv / 3-FC net 957 -> 925 an iteration. (A's rows fetched once for the three taps of a filter row and a deeper
+// ring for the weights' terms gave 1 - 6 us alone and took 17 in the iteration: fetches don't bound it, and 226 KB kept the next
+// kernel out.) WGRAD: issue slots, 2.9 of 4 a cycle: 16 converter warps of 350 instructions a chunk, the summing warps' 128 additions
+// and the MMA warp. Without TMA and with a CTA per unit the same layers took a third longer (a row per lane made each load of A 32
+// wavefronts of the L1 port). Where the weights arrive as terms eight warps of 32 elements convert, not 16 of 16 (half the waits and
+// arrivals: 66 -> 62). Float CUDA cores -> here, us at batch 96: 3x3 over 64 channels at 32x32 forward 180 -> 58, input gradient 175
+// -> 66, weight gradient 177 -> 90; 128 channels at 16x16 155 / 164 / 156 -> 57 / 53 / 49; 256 channels at 8x8 157 / 170 / 159 -> 44 /
+// 45 / 47; 4096 -> 1024 30 / 27 / 23 -> 17 / 18 / 18. The 7-conv / 3-FC net: 2.54 -> 0.92 ms an iteration.
 //
 // Non-finite operands: infinity - infinity in the splitting makes the terms NaN where a float multiply-add would give an infinity, so
 // a row with a NaN in it is computed again with plain multiply-adds by the thread that owns it.
@@ -72,12 +76,16 @@ constexpr int CONV0 = 256;
 constexpr int STAGES = 2, RAWS = 2, RAW = 32768, CTRL = 8192;
 // PLANE: one term of the B tile, BN rows of 128 bytes (FWD) or 64-column boxes of 64 rows.  RAW: a chunk of A as floats, 32-column
 // boxes of 128-byte swizzled rows.  Tensor memory columns: buffers of leading products, buffers of the other products, then the
-// terms of A (2 stages x 3 x 32).
+// terms of A (2 stages x 3 x 32).  PAIRED (64 wide): the other products lie side by side, a0 b1 + a1 b0 and a0 b2 + a1 b1 + a2 b0, so
+// that one instruction multiplies a term of A with two terms of B, neighbours in shared memory: 16 instructions a chunk, not 24, of
+// which the issuing warp gets one out in 54 cycles (a 64-wide one takes the tensor pipe 32).
 template <int BN> struct SplitCfg {
     static constexpr int PLANE = BN * 128, STAGE = 3 * PLANE;
     static constexpr int smem(bool tma) { return STAGES * STAGE + (tma ? RAWS * RAW : 0) + 1024 + CTRL; }
-    static constexpr int LEADS = BN == 64 ? 3 : 1, RESTS = BN == 64 ? 2 : 1;
-    static constexpr uint32_t COL_REST = LEADS * BN, COL_A = COL_REST + RESTS * BN;
+    static constexpr int LEADS = BN == 64 ? 3 : 1, RESTS = 1;
+    static constexpr bool PAIRED = BN == 64;
+    static constexpr int REST = PAIRED ? 2 * BN : BN;      // columns
+    static constexpr uint32_t COL_REST = LEADS * BN, COL_A = COL_REST + RESTS * REST;
 };
 constexpr uint32_t A_TERM = 32, A_STAGE = 3 * A_TERM, TMEM_COLS = 512;
 static_assert(SplitCfg<64>::COL_A + STAGES * A_STAGE <= TMEM_COLS && SplitCfg<128>::COL_A + STAGES * A_STAGE <= TMEM_COLS, "tensor memory");
@@ -88,6 +96,14 @@ __device__ __forceinline__ int div_rcp(int n, uint32_t mul, int d)
     uint32_t q = __umulhi((uint32_t)n, mul);
     if (q * (uint32_t)d > (uint32_t)n) --q;
     return (int)q;
+}
+// whether a phase of a barrier has ended (does not wait)
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity)
+{
+    uint32_t done;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(done) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+    return done != 0;
 }
 struct F8 { float v[8]; };
 // eight floats at a 32-byte boundary (zeros where the place is outside the operand)
@@ -265,42 +281,60 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
         if (warp == 0) {
             // =========================== MMA issuer (the warp in lock-step, one elected lane issues) =============================
             constexpr bool B_MN = MODE != CMODE_FWD;
-            constexpr uint32_t idesc = make_idesc(BN, 0, B_MN);
+            constexpr uint32_t idesc = make_idesc(BN, 0, B_MN), idesc2 = make_idesc(2 * BN, 0, B_MN);
             constexpr uint32_t A_STEP = 8, B_STEP = (B_MN ? 2048u : 32u) >> 4, BP = C::PLANE >> 4;     // per 16 reduction steps: columns, 16-byte units
             const uint32_t elected = elect_one() ? 1u : 0u;
             const uint64_t dB = make_desc(smem_u32(smem), B_MN ? 8192u : 16u);
             const uint32_t b_hi = (uint32_t)(dB >> 32);
             Ring st, lead, rest;
             int chunk = 0, unit = 0;      // (a buffer's first use needs no wait)
-            bool ok = true;
+            bool ok = true, ready = false;      // ready: the next chunk's terms and its buffer of leading products were seen to be
             for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x, ++unit) {
                 const int n_iters = unit_at<BN>(p, u).n_iters;
                 for (int it = 0; it < n_iters; ++it, ++chunk) {
-                    bool w = mbar_wait(&full[st.i], st.ph);
-                    if (chunk >= C::LEADS) w = w && mbar_wait(&lead_empty[lead.i], lead.ph ^ 1u);
-                    if (it == 0 && unit >= C::RESTS) w = w && mbar_wait(&rest_empty[rest.i], rest.ph ^ 1u);
-                    ok = __all_sync(0xffffffffu, w ? 1 : 0) != 0;
-                    if (!ok) break;
+                    if (!ready) {
+                        bool w = mbar_wait(&full[st.i], st.ph);
+                        if (chunk >= C::LEADS) w = w && mbar_wait(&lead_empty[lead.i], lead.ph ^ 1u);
+                        ok = __all_sync(0xffffffffu, w ? 1 : 0) != 0;
+                        if (!ok) break;
+                    }
                     tc_fence_after();
                     const uint32_t a = tmem + C::COL_A + (uint32_t)st.i * A_STAGE, b = (uint32_t)dB + (uint32_t)st.i * (C::STAGE >> 4);
-                    const uint32_t d0 = tmem + (uint32_t)lead.i * BN, d1 = tmem + C::COL_REST + (uint32_t)rest.i * BN;
+                    const uint32_t d0 = tmem + (uint32_t)lead.i * BN, d1 = tmem + C::COL_REST + (uint32_t)rest.i * C::REST;
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk) umma_ta(d0, a + kk * A_STEP, b + kk * B_STEP, b_hi, idesc, kk > 0 ? 1u : 0u, elected);
                     if (elected) umma_commit(&lead_full[lead.i]);
-#pragma unroll
-                    for (int kk = 0; kk < 4; ++kk) {
-                        const uint32_t ak = a + kk * A_STEP, bk = b + kk * B_STEP;
-                        umma_ta(d1, ak + 2 * A_TERM, bk, b_hi, idesc, (it > 0 || kk > 0) ? 1u : 0u, elected);     // a2 b0
-                        umma_ta(d1, ak, bk + 2 * BP, b_hi, idesc, 1u, elected);                                   // a0 b2
-                        umma_ta(d1, ak + A_TERM, bk + BP, b_hi, idesc, 1u, elected);                              // a1 b1
-                        umma_ta(d1, ak + A_TERM, bk, b_hi, idesc, 1u, elected);                                   // a1 b0
-                        umma_ta(d1, ak, bk + BP, b_hi, idesc, 1u, elected);                                       // a0 b1
+                    if (it == 0 && unit >= C::RESTS) {
+                        ok = __all_sync(0xffffffffu, mbar_wait(&rest_empty[rest.i], rest.ph ^ 1u) ? 1 : 0) != 0;
+                        if (!ok) break;
+                        tc_fence_after();
                     }
-                    if (elected) umma_commit(&empty[st.i]);
-                    if (elected && it + 1 == n_iters) umma_commit(&rest_full[rest.i]);
-                    __syncwarp();
+                    const int st_now = st.i;
                     st.next(STAGES);
                     lead.next(C::LEADS);
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk) {
+                        const uint32_t ak = a + kk * A_STEP, bk = b + kk * B_STEP, acc = (it > 0 || kk > 0) ? 1u : 0u;
+                        if (kk == 3) {      // behind the instructions still queued, not after them
+                            bool w = mbar_test(&full[st.i], st.ph);
+                            if (chunk + 1 >= C::LEADS) w = w && mbar_test(&lead_empty[lead.i], lead.ph ^ 1u);
+                            ready = __all_sync(0xffffffffu, w ? 1 : 0) != 0;
+                        }
+                        if (C::PAIRED) {
+                            umma_ta(d1, ak, bk + BP, b_hi, idesc2, acc, elected);                                     // a0 b1 | a0 b2
+                            umma_ta(d1 + BN, ak + 2 * A_TERM, bk, b_hi, idesc, 1u, elected);                          //         a2 b0
+                            umma_ta(d1, ak + A_TERM, bk, b_hi, idesc2, 1u, elected);                                  // a1 b0 | a1 b1
+                        } else {
+                            umma_ta(d1, ak + 2 * A_TERM, bk, b_hi, idesc, acc, elected);                              // a2 b0
+                            umma_ta(d1, ak, bk + 2 * BP, b_hi, idesc, 1u, elected);                                   // a0 b2
+                            umma_ta(d1, ak + A_TERM, bk + BP, b_hi, idesc, 1u, elected);                              // a1 b1
+                            umma_ta(d1, ak + A_TERM, bk, b_hi, idesc, 1u, elected);                                   // a1 b0
+                            umma_ta(d1, ak, bk + BP, b_hi, idesc, 1u, elected);                                       // a0 b1
+                        }
+                    }
+                    if (elected) umma_commit(&empty[st_now]);
+                    if (elected && it + 1 == n_iters) umma_commit(&rest_full[rest.i]);
+                    __syncwarp();
                 }
                 rest.next(C::RESTS);
             }
@@ -389,18 +423,22 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
                 ok = __all_sync(0xffffffffu, mbar_wait(in, last ? rest.ph : lead.ph) ? 1 : 0) != 0;
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t from = taddr + (last ? C::COL_REST + (uint32_t)rest.i * BN : (uint32_t)lead.i * BN);
+                const uint32_t from = taddr + (last ? C::COL_REST + (uint32_t)rest.i * C::REST : (uint32_t)lead.i * BN);
+                auto add = [&](uint32_t at) {
 #pragma unroll
-                for (int c = 0; c < BN; c += 16 * LD) {
-                    uint32_t v[LD][16];
+                    for (int c = 0; c < BN; c += 16 * LD) {
+                        uint32_t v[LD][16];
 #pragma unroll
-                    for (int l = 0; l < LD; ++l) tmem_ld16(from + c + 16 * l, v[l]);
-                    tmem_ld_wait();
+                        for (int l = 0; l < LD; ++l) tmem_ld16(at + c + 16 * l, v[l]);
+                        tmem_ld_wait();
 #pragma unroll
-                    for (int l = 0; l < LD; ++l)
+                        for (int l = 0; l < LD; ++l)
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) acc[c + 16 * l + j] += __uint_as_float(v[l][j]);
-                }
+                            for (int j = 0; j < 16; ++j) acc[c + 16 * l + j] += __uint_as_float(v[l][j]);
+                    }
+                };
+                add(from);
+                if (C::PAIRED && last) add(from + BN);
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(last ? &rest_empty[rest.i] : &lead_empty[lead.i]));
