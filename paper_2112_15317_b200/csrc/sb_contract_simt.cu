@@ -364,10 +364,16 @@ struct TileShape { int bm, bn, resident; double lone, more; };
 static const TileShape shapes[] = {{128, 128, 2, 0.45, 1.25}, {128, 64, 4, 0.75, 0.65}, {64, 128, 4, 0.75, 0.63},
                                    {64, 64, 6, 0.62, 0.30},   {128, 32, 6, 0.85, 0.30}, {32, 128, 6, 0.85, 0.30}};
 
-// The tensor-core form (one CTA per SM): microseconds per 64 reduction steps, per tile and per launch, by tile width and mode,
-// from a sweep of both widths and 1 to 64 splits over 25 layers (residual 6 to 10 %).
-struct UmmaCost { double step, tile, launch; };
-static const UmmaCost umma_cost[2][3] = {{{1.36, 0.7, 6.5}, {1.40, 0.4, 7.4}, {1.47, 5.9, 0.6}}, {{0.99, 0.9, 5.2}, {0.99, 0.9, 5.8}, {1.12, 1.8, 2.5}}};
+// The tensor-core form (one CTA per SM): microseconds per 64 reduction steps, per tile and per launch, and, where the sums of splits are
+// added up by a kernel of their own, per call and per million of them, by what converts B (the kernel itself, or the split weights of a
+// convolution), tile width and mode.  From a sweep of both widths and 1 to 64 splits over 25 layers (residual 5 to 10 %); the plan it
+// chooses takes on average 0.6 % longer than the fastest of the sweep.
+struct UmmaCost { double step, tile, launch, sums, sum; };
+static const UmmaCost umma_cost[2][2][3] = {
+    {{{1.26, 0.7, 5.9, 1.0, 2.45}, {1.21, 0.7, 7.5, -1.1, 2.43}, {1.47, 5.9, 0.2, 3.0, 1.14}},
+     {{0.97, 1.0, 4.8, 1.0, 1.55}, {1.06, 0.5, 5.6, -0.1, 2.20}, {1.06, 2.0, 2.4, 3.0, 1.14}}},
+    {{{1.18, 0.4, 9.0, -2.2, 1.66}, {1.26, 0.7, 8.5, -2.1, 1.49}, {1.47, 5.9, 0.2, 3.0, 1.14}},
+     {{0.81, 0.1, 8.0, -0.9, 1.09}, {0.82, 0.5, 8.0, -1.3, 0.75}, {1.06, 2.0, 2.4, 3.0, 1.14}}}};
 
 static bool vec_ok(int Cin, int Cout) { return Cin % 4 == 0 && Cout % 4 == 0; }
 static long contract_iters(int mode, int B, int H, int W, int taps, int Cin, int Cout)
@@ -400,15 +406,16 @@ ContractPlan contract_plan(int mode, int B, int H, int W, int taps, int Cin, int
     }
     if (umma && contract_umma_ok(taps, Cin, Cout)) {
         const long K = mode == CMODE_WGRAD ? pix : (long)taps * (mode == CMODE_DGRAD ? Cout : Cin), chunks = (K + 63) / 64;
+        const bool terms = taps == 9 && contract_umma_whole_taps(mode, Cin, Cout);
         for (int bn : {128, 64}) {
-            const UmmaCost& u = umma_cost[bn == 64][mode];
+            const UmmaCost& u = umma_cost[terms][bn == 64][mode];
             const long tiles = ((M + 127) / 128) * ((N + bn - 1) / bn);
-            for (int split = 1; split <= 256 && split <= chunks; split = split < 8 ? split + 1 : split + split / 4) {
+            for (int split = 1; split <= 256 && split <= chunks; split = split < 16 ? split + 1 : split + split / 8) {
                 const long per = (chunks + split - 1) / split;
                 const int real = (int)((chunks + per - 1) / per);
                 if (real > 1 && (size_t)real * M * (N + (mode == CMODE_WGRAD ? 1 : 0)) > max_part_floats) break;
                 double t = (double)((tiles * real + 147) / 148) * (per * u.step + u.tile) + u.launch;
-                if (real > 1) t += mode == CMODE_WGRAD ? 3.0 + (double)real * M * N * 8.0 / 7.0e6 : (double)real * M * N * 13.0 / 7.0e6;
+                if (real > 1) t += u.sums + (double)real * M * N * 1e-6 * u.sum;
                 if (t < best_t) { best_t = t; best = ContractPlan{128, bn, (int)per, real, true}; }
             }
         }

@@ -35,8 +35,8 @@
 // and the MMA warp. Without TMA and with a CTA per unit the same layers took a third longer (a row per lane made each load of A 32
 // wavefronts of the L1 port). Where the weights arrive as terms eight warps of 32 elements convert, not 16 of 16 (half the waits and
 // arrivals: 66 -> 62). Float CUDA cores -> here, us at batch 96: 3x3 over 64 channels at 32x32 forward 180 -> 58, input gradient 175
-// -> 66, weight gradient 177 -> 90; 128 channels at 16x16 155 / 164 / 156 -> 57 / 53 / 49; 256 channels at 8x8 157 / 170 / 159 -> 44 /
-// 45 / 47; 4096 -> 1024 30 / 27 / 23 -> 17 / 18 / 18. The 7-conv / 3-FC net: 2.54 -> 0.92 ms an iteration.
+// -> 66, weight gradient 177 -> 90; 128 channels at 16x16 155 / 164 / 156 -> 52 / 53 / 47; 256 channels at 8x8 157 / 170 / 159 -> 44 /
+// 45 / 47; 4096 -> 1024 30 / 27 / 23 -> 17 / 16 / 18. The 7-conv / 3-FC net: 2.54 -> 0.91 ms an iteration.
 //
 // Non-finite operands: infinity - infinity in the splitting makes the terms NaN where a float multiply-add would give an infinity, so
 // a row with a NaN in it is computed again with plain multiply-adds by the thread that owns it.
