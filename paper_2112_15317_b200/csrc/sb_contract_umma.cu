@@ -39,7 +39,7 @@
 // 45 / 47; 4096 -> 1024 30 / 27 / 23 -> 17 / 16 / 18. The 7-conv / 3-FC net: 2.54 -> 0.91 ms an iteration.
 //
 // Non-finite operands: infinity - infinity in the splitting makes the terms NaN where a float multiply-add would give an infinity, so
-// a row with a NaN in it is computed again with plain multiply-adds by the thread that owns it.
+// elements that come out as NaN are computed again with plain multiply-adds.
 #include "sb_umma.h"
 #include "sb_tcgen05.cuh"
 
@@ -161,29 +161,29 @@ __device__ __forceinline__ void umma_ta(uint32_t d_tmem, uint32_t a_tmem, uint32
         ::"r"(d_tmem), "r"(a_tmem), "r"(blo), "r"(bhi), "r"(idesc), "r"(accumulate), "r"(elected)
         : "memory");
 }
-// Element (m, n) over reduction steps [k0, k1) with plain multiply-adds (rows with a non-finite operand).
+// Element (m, n) with plain multiply-adds over reduction steps k, k + step, ... below k1, up to `most` of them or the first NaN.
+// (Places outside the image are zeros that are multiplied, as in contract_kernel: 0 x infinity is NaN.)
 template <int MODE>
-__device__ __noinline__ float plain_sum(const SplitParams& p, int m, int n, int k0, int k1)
+__device__ __noinline__ float plain_sum(const SplitParams& p, int m, int n, int k, int k1, int step, int most)
 {
     const int HW = p.H * p.W;
     float s = 0.f;
     if (MODE == CMODE_WGRAD) {
         const int t = n / p.Cin, c = n - t * p.Cin, dr = p.taps == 9 ? t / 3 - 1 : 0, ds = p.taps == 9 ? t % 3 - 1 : 0;
-        for (int k = k0; k < k1; ++k) {
+        for (; k < k1 && most > 0 && s == s; k += step, --most) {
             const int r = k % HW, h = r / p.W + dr, w = r % p.W + ds;
-            if ((unsigned)h >= (unsigned)p.H || (unsigned)w >= (unsigned)p.W) continue;
-            s = fmaf(p.dy[(size_t)k * p.Cout + m], p.act[((long)k + (long)dr * p.W + ds) * p.Cin + n - t * p.Cin], s);
+            const bool in = (unsigned)h < (unsigned)p.H && (unsigned)w < (unsigned)p.W;
+            s = fmaf(p.dy[(size_t)k * p.Cout + m], in ? p.act[((long)k + (long)dr * p.W + ds) * p.Cin + c] : 0.f, s);
         }
-        (void)c;
         return s;
     }
     const int Cred = MODE == CMODE_DGRAD ? p.Cout : p.Cin, r = m % HW, h0 = r / p.W, w0 = r % p.W;
-    for (int k = k0; k < k1; ++k) {
+    for (; k < k1 && most > 0 && s == s; k += step, --most) {
         const int t = k / Cred, c = k - t * Cred;
         int dr = p.taps == 9 ? t / 3 - 1 : 0, ds = p.taps == 9 ? t % 3 - 1 : 0;
         if (MODE == CMODE_DGRAD) { dr = -dr; ds = -ds; }
-        if ((unsigned)(h0 + dr) >= (unsigned)p.H || (unsigned)(w0 + ds) >= (unsigned)p.W) continue;
-        const float a = (MODE == CMODE_FWD ? p.act : p.dy)[((long)m + (long)dr * p.W + ds) * Cred + c];
+        const bool in = (unsigned)(h0 + dr) < (unsigned)p.H && (unsigned)(w0 + ds) < (unsigned)p.W;
+        const float a = in ? (MODE == CMODE_FWD ? p.act : p.dy)[((long)m + (long)dr * p.W + ds) * Cred + c] : 0.f;
         s = fmaf(a, MODE == CMODE_FWD ? p.wt[(size_t)n * p.K + k] : p.wt[((size_t)c * p.taps + t) * p.Cin + n], s);
     }
     return s;
@@ -203,6 +203,16 @@ __device__ __forceinline__ void finish8(const SplitParams& p, float (&f)[8], siz
             if (p.relu && !(f[j] > 0.f)) f[j] = 0.f;
         } else if (!(e[j] > 0.f)) f[j] = 0.f;
     }
+}
+
+template <int MODE>
+__device__ __forceinline__ float finish1(const SplitParams& p, float f, size_t at, int n)
+{
+    if (MODE == CMODE_FWD) {
+        f += p.bias[n];
+        return p.relu && !(f > 0.f) ? 0.f : f;
+    }
+    return p.ref != nullptr && !(p.ref[at] > 0.f) ? 0.f : f;
 }
 
 template <bool TMA> struct Maps { CUtensorMap a, b; };      // raw floats of A, terms of the weights
@@ -445,32 +455,57 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
                 if (last) rest.next(C::RESTS);
                 else lead.next(C::LEADS);
             }
+            if (!ok) break;
             const int m = t.m0 + q * 32 + lane;
-            if (!ok || m >= p.M) continue;
-            const size_t row = (size_t)m * p.N;
-            float* dst = (raw_sums ? p.part + (size_t)t.split * p.split_stride : p.out) + row;
+            float* const base = raw_sums ? p.part + (size_t)t.split * p.split_stride : p.out;
             bool bad = false;
+            if (m < p.M) {
+                const size_t row = (size_t)m * p.N;
 #pragma unroll
-            for (int c = 0; c < BN; c += 8) {
-                if (t.n0 + c >= p.N) continue;
-                float f[8];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    f[j] = acc[c + j];
-                    bad = bad || f[j] != f[j];
-                }
-                if (!raw_sums) finish8<MODE>(p, f, row + t.n0 + c, t.n0 + c);
-                float4* d = (float4*)(dst + t.n0 + c);
-                d[0] = make_float4(f[0], f[1], f[2], f[3]);
-                d[1] = make_float4(f[4], f[5], f[6], f[7]);
-            }
-            if (bad) {
-                const int k0 = t.chunk0 * 64, k1 = min(p.K, (t.chunk0 + t.n_iters) * 64);
-                for (int n = t.n0; n < min(t.n0 + BN, p.N); n += 8) {
+                for (int c = 0; c < BN; c += 8) {
+                    if (t.n0 + c >= p.N) continue;
                     float f[8];
-                    for (int j = 0; j < 8; ++j) f[j] = plain_sum<MODE>(p, m, n + j, k0, k1);
-                    if (!raw_sums) finish8<MODE>(p, f, row + n, n);
-                    for (int j = 0; j < 8; ++j) dst[n + j] = f[j];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        f[j] = acc[c + j];
+                        bad = bad || f[j] != f[j];
+                    }
+                    if (!raw_sums) finish8<MODE>(p, f, row + t.n0 + c, t.n0 + c);
+                    float4* d = (float4*)(base + row + t.n0 + c);
+                    d[0] = make_float4(f[0], f[1], f[2], f[3]);
+                    d[1] = make_float4(f[4], f[5], f[6], f[7]);
+                }
+            }
+            if (__any_sync(0xffffffffu, bad)) {
+                // What is NaN in plain arithmetic too has been stored as such.  Each lane sorts out of its row what 32 multiply-adds show
+                // to be (all of it where a whole operand is NaN); the warp then shares the reduction of every element that is left, so
+                // that one long row does not outlast the other warps' bounded waits.
+                const int k0 = t.chunk0 * 64, k1 = min(p.K, (t.chunk0 + t.n_iters) * 64);
+#pragma unroll
+                for (int c = 0; c < BN; c += 32) {
+                    uint32_t nan = 0u;
+#pragma unroll
+                    for (int j = 0; j < 32; ++j)
+                        if (acc[c + j] != acc[c + j] && m < p.M && t.n0 + c + j < p.N) nan |= 1u << j;
+                    uint32_t left = 0u;
+                    for (; nan != 0u; nan &= nan - 1u) {
+                        const int j = __ffs(nan) - 1;
+                        const float s = plain_sum<MODE>(p, m, t.n0 + c + j, k0, k1, 1, 32);
+                        if (s == s) left |= 1u << j;
+                    }
+                    __syncwarp();
+                    for (uint32_t rows = __ballot_sync(0xffffffffu, left != 0u); rows != 0u; rows &= rows - 1u) {
+                        const int src = __ffs(rows) - 1, mr = t.m0 + q * 32 + src;
+                        for (uint32_t b = __shfl_sync(0xffffffffu, left, src); b != 0u; b &= b - 1u) {
+                            const int n = t.n0 + c + __ffs(b) - 1;
+                            float s = plain_sum<MODE>(p, mr, n, k0 + lane, k1, 32, 1 << 30);
+                            __syncwarp();
+#pragma unroll
+                            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                            const size_t at = (size_t)mr * p.N + n;
+                            if (lane == src) base[at] = raw_sums ? s : finish1<MODE>(p, s, at, n);
+                        }
+                    }
                 }
             }
         }

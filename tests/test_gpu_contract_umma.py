@@ -110,3 +110,43 @@ def test_non_finite_operands_as_on_cuda_cores(bad):
         assert tu.maxrel(u[fin], v[fin]) < 1e-5
     a.close()
     ref.close()
+
+
+@pytest.mark.parametrize("where", ["all weights NaN", "one gradient pixel inf", "one gradient value inf", "one weight -inf", "inputs of one image NaN"])
+def test_non_finite_operands_over_long_reductions(where):
+    """Whole operands and single values, 16384 pixels: the results of plain multiply-adds, and no wait that runs out meanwhile."""
+    from paper_2112_15317_b200 import binding as sb
+    wl, params, batch = _net(32, 32, 64, 64, 64, 16, 1)
+    xs, ys = tu.device_batch(wl, *batch, False)
+    a, ref = tu.gpu_model(wl, params, sb.SB_FP32), tu.gpu_model(wl, params, sb.SB_FP32, sb.SB_FLAG_FORCE_SIMT)
+    dy = 0.01 * np.cos(np.arange(16 * 32 * 32 * 64, dtype=np.float32)).reshape(16, 32, 32, 64)
+    if where == "one gradient pixel inf":
+        dy[9, 30, 17, :] = np.inf
+    elif where == "one gradient value inf":
+        dy[15, 31, 31, 63] = np.inf
+    got = []
+    for m in (a, ref):
+        m.forward(xs, ys)
+        w = m.read(sb.SB_T_WEIGHT, 1, 0, squeeze=False)
+        act = m.read(sb.SB_T_ACT, 0, 0, squeeze=False)
+        if where == "all weights NaN":
+            w[:] = np.nan
+        elif where == "one weight -inf":
+            w[33, 2, 1, 40] = -np.inf
+        elif where == "inputs of one image NaN":
+            act[3] = np.nan
+        m.write(sb.SB_T_WEIGHT, 1, 0, w)
+        m.write(sb.SB_T_ACT, 0, 0, act)
+        m.forward_layers(1, 1)
+        y = m.read(sb.SB_T_ACT, 1, 0)
+        m.write(sb.SB_T_DACT, 1, 0, dy)
+        m.backward_layers(1, 1)
+        m.loss()       # raises if a bounded wait ran out
+        got.append([y, m.read(sb.SB_T_GRAD_W, 1), m.read(sb.SB_T_DACT, 0, 0)])
+    for u, v in zip(*got):
+        assert np.array_equal(np.isnan(u), np.isnan(v)) and np.array_equal(np.isinf(u), np.isinf(v))
+        fin = np.isfinite(v)
+        assert np.array_equal(np.sign(u[np.isinf(v)]), np.sign(v[np.isinf(v)]))
+        assert not fin.any() or tu.maxrel(u[fin], v[fin]) < 1e-5
+    a.close()
+    ref.close()
