@@ -38,7 +38,6 @@
 #include "sb_umma.h"
 #include "sb_tcgen05.cuh"
 
-#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -2725,28 +2724,11 @@ static double plan_cost(int bn, int s, int n_cols, long m_tiles, int k_iters)
     const double mb_us = 0.5;
     return waves * (cdiv_i(k_iters, s) * t_iter * (per_sm > 1.0 ? 1.6 : 1.0) + 3.0) + (s > 1 ? 4.0 + mb_us * partial_mb : 0.0);
 }
-static TilePlan plan_tiles(int n_cols, long m_tiles, int k_iters, bool backward, bool force_pair, int fc_rows = 0)
+static TilePlan plan_tiles(int n_cols, long m_tiles, int k_iters, bool backward, bool force_pair, bool fc = false)
 {
     TilePlan t;
     int best_bn = 64, best_s = 1;
-    // FC forward over weights that stream from memory (64 MB and more; one M tile): time is their bytes at the 5.4 TB/s that 120 CTAs or
-    // more reach, or both operands' bytes at the 10.5 TB/s of L2 -> SM, whichever is longer, and the split sums.  25088 -> 4096 at batch
-    // 128: 256 columns in 8 splits 47.9 us, 128 in 4 (half the partial sums) 43.9; 256 in 4 (64 CTAs) 59.5.
-    const double w_mb = (double)n_cols * k_iters * 128.0 / 1e6;
-    bool planned = false;
-    if (fc_rows > 0 && !backward && !force_pair && m_tiles == 1 && w_mb >= 64.0) {
-        double best = 1e300;
-        for (int bn : {128, 256}) {      // (64 columns keep too few bytes in flight: batch 16 46 us against 39)
-            const long tiles = cdiv_i(n_cols, bn);
-            for (int s = 1; s <= 32 && k_iters / s >= 4 && tiles * s <= 148; ++s) {
-                const double hbm = w_mb / 5.4, l2 = w_mb * (1.0 + (double)fc_rows / bn) / 10.5;
-                const double c = std::max(hbm * std::max(1.0, 120.0 / (double)(tiles * s)), l2) + (s > 1 ? 2.5 + 0.5 * s * 128.0 * n_cols * 4e-6 : 0.0);
-                if (c < best - 1e-9) { best = c; best_bn = bn; best_s = s; }
-            }
-        }
-        planned = best < 1e299;             // (more tiles than SMs: the model below)
-    }
-    if (!planned) {
+    {
         double best = 1e300;
         for (int bn : {64, 128, 192, 256}) {
             if (bn > 64 && bn / 2 >= n_cols) break;      // never wider than the columns need
@@ -2776,7 +2758,7 @@ static TilePlan plan_tiles(int n_cols, long m_tiles, int k_iters, bool backward,
     // (the data gradient of an FC layer in one wave keeps its ring and with it one CTA per SM: two of 128 CTAs on some SMs and none on
     // others made 4096 -> 4096 at batch 32 take 15 us where 9 do, depending on which SMs the kernel before it left free; only the narrow
     // layer's small blocks run beside it)
-    const bool one_wave = fc_rows > 0 && tiles * t.splits <= 148;
+    const bool one_wave = fc && tiles * t.splits <= 148;
     if ((backward || fwd_too) && !one_wave && bwd_cohabit() && t.bn != 192 && tiles * t.splits >= cohabit_min && st > cohabit_stages(t.bn)) st = cohabit_stages(t.bn);
     // Grids of more than one CTA per SM: measured, the co-residency of CTAs (their set-up, first loads and
     // epilogues overlap one another's main loops) is worth more than ring depth -- the 1024-CTA 64-wide layer runs
@@ -3188,8 +3170,8 @@ static FcGeom fc_geom(const LayerView& lv, int B, bool force_pair)
 {
     FcGeom g;
     g.m_tiles = cdiv_i(B, 128);
-    g.fwd = plan_tiles(lv.out_f, g.m_tiles, cdiv_i(lv.in_f, 64), false, force_pair, B);
-    g.dgrad = plan_tiles(lv.in_f, g.m_tiles, cdiv_i(lv.out_f, 64), true, force_pair, B);
+    g.fwd = plan_tiles(lv.out_f, g.m_tiles, cdiv_i(lv.in_f, 64), false, force_pair);
+    g.dgrad = plan_tiles(lv.in_f, g.m_tiles, cdiv_i(lv.out_f, 64), true, force_pair, true);
     return g;
 }
 
