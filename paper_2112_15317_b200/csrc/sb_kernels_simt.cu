@@ -1163,12 +1163,15 @@ template <> struct Vec8<__nv_bfloat16> { static constexpr int N = 8; typedef uin
 
 // Forward.  Block = one batch row, a warp per output: the kernel is pure latency, so every lane has eight 16-byte loads in flight and
 // the code is one short loop.  (Two rows a block, the reduction in four slices and all outputs in a lane's registers: 6.5 us for
-// 4096 -> 10 at batch 128 in the replayed VGG-16 iteration; here 4.9 with the softmax.)
+// 4096 -> 10 at batch 128 in the replayed VGG-16 iteration; here 4.9 with the softmax.)  A lane keeps a sum for each of its four loads of
+// a step: one chain over all of its in_f / 32 products carried twice the rounding (float, 2-norm against 64-bit sums: 4096 inputs
+// 1.5e-7 where four give 1.0e-7, 25088 inputs 4.1e-7 and 2.2e-7).  Two blocks an SM: left alone the compiler fits the float form into 32
+// registers, too few for the loads (25088 -> 10 at batch 96, whole call 43 us, 26 so).
 // XENT: softmax cross-entropy of the row by warp 0, with the operations of softmax_xent_kernel in its order, without that kernel's
 // 4.3 us on the chain (most of them the last block's wait for every row loss).
 struct HeadArgs { PtrTab labels; int b_per_rep; float* row_loss; void* dZ; int scale_B; };
 template <typename T, bool TAB, bool VEC, bool XENT>
-__global__ void __launch_bounds__(32 * NARROW_MAX)
+__global__ void __launch_bounds__(32 * NARROW_MAX, 2)
 fc_narrow_fwd_kernel(const T* __restrict__ X, PtrTab tab, int tab_b, const T* __restrict__ Wt, const float* __restrict__ bias,
                      T* __restrict__ Y, float* __restrict__ Y32, int in_f, int out_f, int relu, const __grid_constant__ HeadArgs head)
 {
@@ -1181,8 +1184,9 @@ fc_narrow_fwd_kernel(const T* __restrict__ X, PtrTab tab, int tab_b, const T* __
     const T* wr = Wt + (size_t)j * in_f;
     int label = 0;
     if (XENT && j == 0) label = ((const int32_t*)head.labels.p[g / head.b_per_rep])[g % head.b_per_rep];
-    float acc = 0.f;
+    float acc;
     if (VEC) {
+        float part[4] = {0.f, 0.f, 0.f, 0.f};
         // (the host only selects this variant when every row starts 16-byte aligned)
 #pragma unroll 1
         for (int k0 = lane * VN; k0 < in_f; k0 += 128 * VN) {
@@ -1198,9 +1202,11 @@ fc_narrow_fwd_kernel(const T* __restrict__ X, PtrTab tab, int tab_b, const T* __
             for (int u = 0; u < 4; ++u)
                 if (k0 + u * 32 * VN < in_f)
 #pragma unroll
-                    for (int i = 0; i < VN; ++i) acc = fmaf(ldf((const T*)&xv[u] + i), ldf((const T*)&wv[u] + i), acc);
+                    for (int i = 0; i < VN; ++i) part[u] = fmaf(ldf((const T*)&xv[u] + i), ldf((const T*)&wv[u] + i), part[u]);
         }
+        acc = (part[0] + part[1]) + (part[2] + part[3]);
     } else {
+        acc = 0.f;
         for (int k = lane; k < in_f; k += 32) acc = fmaf(ldf(xr + k), ldf(wr + k), acc);
     }
 #pragma unroll

@@ -30,8 +30,8 @@ def _logits_error(m, layer, x, in_f):
     _view(m, sb.SB_T_BIAS, layer).zero_()
     m.refresh_shadow()
     B, out = x.shape[0], w.numel() // in_f
-    xs, ys = [x], [torch.zeros(B, dtype=torch.int32, device="cuda")]
-    m.forward_layers(layer, layer, xs, ys)
+    m.forward_layers(layer, layer, [torch.zeros(B, m.cfg.H, m.cfg.W, m.cfg.C, dtype=x.dtype, device="cuda")] if layer else [x],
+                     [torch.zeros(B, dtype=torch.int32, device="cuda")])
     want = x.reshape(B, in_f).double() @ (w.to(torch.bfloat16) if m.bf16 else w).double().reshape(out, in_f).T
     return ((_view(m, sb.SB_T_ACT, layer).reshape(B, out).double() - want).norm() / want.norm()).item()
 
@@ -47,4 +47,26 @@ def test_streamed_fc_forward(in_f, out, B):
     # result.  The chains are 3136 and 2048 terms long (2.4e-6 and 1.5e-6 measured, 5.3e-6 and 3.2e-6 over twice that length).
     chain = {25088: 3136, 8192: 2048}[in_f]
     assert _logits_error(m, 0, x, in_f) < chain / 16 * 2.0 ** -25 * 2 / 3
+    m.close()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "bf16"])
+@pytest.mark.parametrize("B", [2, 96])
+@pytest.mark.parametrize("side,channels", [(16, 16), (56, 8)])      # 4096 and 25088 inputs
+def test_narrow_logits(side, channels, B, precision):
+    import torch
+
+    from paper_2112_15317_b200 import binding as sb
+    m = sb.Model([(sb.SB_CONV3X3_RELU, channels), (sb.SB_FC, 10), (sb.SB_SOFTMAX_XENT, 10)], side, side, 4, B, 1, 1,
+                 sb.SB_FP32 if precision == "fp32" else sb.SB_BF16)
+    in_f = side * side * channels
+    act = _view(m, sb.SB_T_ACT, 0)
+    act.copy_(torch.randn(act.shape, generator=torch.Generator(device="cuda").manual_seed(B), device="cuda").relu())
+    # Chains of n = in_f / 128 products of either sign: every addition rounds by 2^-25 of a sum that grows with the root of its length, which
+    # adds up to 2^-25 sqrt(n / 2) of the result; the seven levels of additions across chains and lanes and the bias's make it n / 2 + 8.
+    # Products of bf16 operands have 16 bits and short sums of them are exact: half over long rows.  (Measured: 4096 inputs 1.1e-7 and
+    # 0.9e-7, 25088 2.4e-7 and 1.0e-7; in one chain a lane 1.5 to 2.2e-7, 4.0 to 4.2e-7 and 1.7e-7.)
+    bound = 2.0 ** -25 * math.sqrt(in_f / 128 / 2 + 8) * (1.0 if precision == "fp32" or in_f < 10000 else 0.5)
+    err = _logits_error(m, 1, act, in_f)
+    assert err < bound, (err, bound)
     m.close()
