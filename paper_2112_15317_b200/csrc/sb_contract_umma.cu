@@ -39,7 +39,7 @@
 // 45 / 47; 4096 -> 1024 30 / 27 / 23 -> 17 / 16 / 18. The 7-conv / 3-FC net: 2.54 -> 0.91 ms an iteration.
 //
 // Non-finite operands: infinity - infinity in the splitting makes the terms NaN where a float multiply-add would give an infinity, so
-// elements that come out as NaN are computed again with plain multiply-adds.
+// results that come out as NaN are looked at again behind the CTA's last unit, when no other warp waits (repair_unit).
 #include "sb_umma.h"
 #include "sb_tcgen05.cuh"
 
@@ -161,34 +161,22 @@ __device__ __forceinline__ void umma_ta(uint32_t d_tmem, uint32_t a_tmem, uint32
         ::"r"(d_tmem), "r"(a_tmem), "r"(blo), "r"(bhi), "r"(idesc), "r"(accumulate), "r"(elected)
         : "memory");
 }
-// Element (m, n) with plain multiply-adds over reduction steps k, k + step, ... below k1, up to `most` of them or the first NaN.
-// (Places outside the image are zeros that are multiplied, as in contract_kernel: 0 x infinity is NaN.)
+// Which taps of output pixel m fall inside the image (a bit each)
 template <int MODE>
-__device__ __noinline__ float plain_sum(const SplitParams& p, int m, int n, int k, int k1, int step, int most)
+__device__ __forceinline__ uint32_t taps_inside(const SplitParams& p, int m)
 {
-    const int HW = p.H * p.W;
-    float s = 0.f;
-    if (MODE == CMODE_WGRAD) {
-        const int t = n / p.Cin, c = n - t * p.Cin, dr = p.taps == 9 ? t / 3 - 1 : 0, ds = p.taps == 9 ? t % 3 - 1 : 0;
-        for (; k < k1 && most > 0 && s == s; k += step, --most) {
-            const int r = k % HW, h = r / p.W + dr, w = r % p.W + ds;
-            const bool in = (unsigned)h < (unsigned)p.H && (unsigned)w < (unsigned)p.W;
-            s = fmaf(p.dy[(size_t)k * p.Cout + m], in ? p.act[((long)k + (long)dr * p.W + ds) * p.Cin + c] : 0.f, s);
-        }
-        return s;
+    uint32_t in = 0u;
+    if (m >= p.M) return in;
+    if (p.taps == 1) return 1u;
+    const int HW = p.H * p.W, n = div_rcp(m, p.rcp_hw, HW), w = m - n * HW, h = div_rcp(w, p.rcp_w, p.W), x = w - h * p.W;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const int er = MODE == CMODE_FWD ? i / 3 - 1 : 1 - i / 3, es = MODE == CMODE_FWD ? i % 3 - 1 : 1 - i % 3;
+        if ((unsigned)(h + er) < (unsigned)p.H && (unsigned)(x + es) < (unsigned)p.W) in |= 1u << i;
     }
-    const int Cred = MODE == CMODE_DGRAD ? p.Cout : p.Cin, r = m % HW, h0 = r / p.W, w0 = r % p.W;
-    for (; k < k1 && most > 0 && s == s; k += step, --most) {
-        const int t = k / Cred, c = k - t * Cred;
-        int dr = p.taps == 9 ? t / 3 - 1 : 0, ds = p.taps == 9 ? t % 3 - 1 : 0;
-        if (MODE == CMODE_DGRAD) { dr = -dr; ds = -ds; }
-        const bool in = (unsigned)(h0 + dr) < (unsigned)p.H && (unsigned)(w0 + ds) < (unsigned)p.W;
-        const float a = in ? (MODE == CMODE_FWD ? p.act : p.dy)[((long)m + (long)dr * p.W + ds) * Cred + c] : 0.f;
-        s = fmaf(a, MODE == CMODE_FWD ? p.wt[(size_t)n * p.K + k] : p.wt[((size_t)c * p.taps + t) * p.Cin + n], s);
-    }
-    return s;
+    return in;
 }
-// Eight results of a row: bias and ReLU, or the ReLU mask (NaN -> 0, as everywhere)
+// Eight results of a row: bias and ReLU, or the ReLU mask.  A NaN stays one here: it is looked at again (repair_unit).
 template <int MODE>
 __device__ __forceinline__ void finish8(const SplitParams& p, float (&f)[8], size_t at, int n)
 {
@@ -199,11 +187,12 @@ __device__ __forceinline__ void finish8(const SplitParams& p, float (&f)[8], siz
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         if (MODE == CMODE_FWD) {
-            f[j] += e[j];
-            if (p.relu && !(f[j] > 0.f)) f[j] = 0.f;
-        } else if (!(e[j] > 0.f)) f[j] = 0.f;
+            const float y = f[j] + e[j];
+            f[j] = p.relu && !(y > 0.f) && f[j] == f[j] ? 0.f : y;
+        } else if (!(e[j] > 0.f) && f[j] == f[j]) f[j] = 0.f;
     }
 }
+// One result (NaN -> 0 behind a ReLU or a mask, as everywhere)
 
 template <int MODE>
 __device__ __forceinline__ float finish1(const SplitParams& p, float f, size_t at, int n)
@@ -230,6 +219,207 @@ __device__ __forceinline__ Unit unit_at(const SplitParams& p, int u)
     t.chunk0 = z * p.cps;
     t.n_iters = min(p.cps, p.chunks - t.chunk0);
     return t;
+}
+// Results of a unit that came out as NaN, by one warp for the 32 rows that it has stored (NaN and unfinished): what plain multiply-adds
+// give.  A NaN operand makes its whole row or column NaN (places outside the image are zeros that are multiplied, as in
+// contract_kernel: NaN x 0 and infinity x 0 are NaN), so the operands are searched for those first, and the search ends when they
+// explain every such result: a run that has diverged costs one look at the operands.  What is left has infinite or large operands
+// in its sum: the steps that hold any (in 1024 groups, a bit each, 32 to a lane) are summed, a lane per column; only where that is finite
+// does the sum run over all steps.
+// (a predicate, not a branch, so that the loads of several steps are under way together)
+__device__ __forceinline__ float load_if(const float* p, bool there)
+{
+    float v;
+    asm("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\tmov.b32 %0, 0;\n\t@p ld.global.f32 %0, [%1];\n\t}" : "=f"(v) : "l"(p), "r"((int)there));
+    return v;
+}
+template <int MODE> struct Step {      // a reduction step's tap and channel; WGRAD: its pixel's row and column
+    int k, tap, c;
+    __device__ __forceinline__ Step(const SplitParams& p, int k_) : k(k_)
+    {
+        if (MODE == CMODE_WGRAD) {
+            const int HW = p.H * p.W, r = k - div_rcp(k, p.rcp_hw, HW) * HW;
+            tap = div_rcp(r, p.rcp_w, p.W); c = r - tap * p.W;
+        } else {
+            const int cred = MODE == CMODE_DGRAD ? p.Cout : p.Cin;
+            tap = k / cred; c = k - tap * cred;
+        }
+    }
+    __device__ __forceinline__ void next(const SplitParams& p)
+    {
+        ++k;
+        if (++c == (MODE == CMODE_WGRAD ? p.W : MODE == CMODE_DGRAD ? p.Cout : p.Cin)) {
+            c = 0;
+            if (++tap == p.H && MODE == CMODE_WGRAD) tap = 0;
+        }
+    }
+};
+template <int MODE> struct Column {    // of the result; WGRAD: its tap's shift
+    const float* at;
+    int dr = 0, ds = 0;
+    bool in;
+    Column() = default;
+    __device__ __forceinline__ Column(const SplitParams& p, int n) : in(n < p.N)
+    {
+        n = in ? n : 0;
+        if (MODE == CMODE_WGRAD) {
+            const int t = n / p.Cin;
+            if (p.taps == 9) { dr = t / 3 - 1; ds = t % 3 - 1; }
+            at = p.act + ((long)dr * p.W + ds) * p.Cin + (n - t * p.Cin);
+        } else at = MODE == CMODE_FWD ? p.wt + (size_t)n * p.K : p.wt + n;
+    }
+    __device__ __forceinline__ float operand(const SplitParams& p, const Step<MODE>& s, bool there = true) const
+    {
+        bool ok = in && there;
+        const float* a = at;
+        if (MODE == CMODE_FWD) a += s.k;
+        else if (MODE == CMODE_DGRAD) a += ((size_t)s.c * p.taps + s.tap) * p.Cin;
+        else {
+            a += (size_t)s.k * p.Cin;
+            ok = ok && (unsigned)(s.tap + dr) < (unsigned)p.H && (unsigned)(s.c + ds) < (unsigned)p.W;
+        }
+        return load_if(a, ok);
+    }
+};
+template <int MODE>
+__device__ __forceinline__ float row_operand(const SplitParams& p, int m, uint32_t inside, const Step<MODE>& s, bool there = true)
+{
+    const float* a = MODE == CMODE_FWD ? p.act : p.dy;
+    if (MODE == CMODE_WGRAD) return load_if(a + (size_t)s.k * p.Cout + m, there && m < p.M);
+    const int shift = p.taps == 9 ? (s.tap / 3 - 1) * p.W + s.tap % 3 - 1 : 0;
+    a += ((long)m + (MODE == CMODE_FWD ? shift : -shift)) * (MODE == CMODE_FWD ? p.Cin : p.Cout) + s.c;
+    return load_if(a, there && ((inside >> s.tap) & 1u) != 0u);      // (no tap of a row past the last is inside)
+}
+// All operands of the 32 steps from k on (below k1) to the warp's rows and the unit's columns: a lane per step where an operand lies
+// along the reduction in memory, else a lane per line.  f(value, line, step, whether it is a column's): line or step is the lane's own.
+template <int MODE, int BN, typename F>
+__device__ __forceinline__ void visit(const SplitParams& p, const Column<MODE> (&col)[BN / 32], int row0, int n0, uint32_t inside, int k, int k1, F f)
+{
+    const int lane = threadIdx.x % 32;
+    const Step<MODE> mine(p, k + lane);
+    if (MODE == CMODE_FWD) {
+#pragma unroll 16
+        for (int i = 0; i < BN; ++i) f(Column<MODE>(p, n0 + i).operand(p, mine, k + lane < k1), i, lane, true);
+    } else {
+        Step<MODE> s(p, k);
+#pragma unroll 8
+        for (int i = 0; i < 32; ++i, s.next(p))
+#pragma unroll
+            for (int b = 0; b < BN / 32; ++b) f(col[b].operand(p, s, k + i < k1), 32 * b + lane, i, true);
+    }
+    if (MODE == CMODE_WGRAD) {
+        Step<MODE> s(p, k);
+#pragma unroll 16
+        for (int i = 0; i < 32; ++i, s.next(p)) f(row_operand<MODE>(p, row0 + lane, 0u, s, k + i < k1), lane, i, false);
+    } else {
+#pragma unroll 16
+        for (int i = 0; i < 32; ++i) f(row_operand<MODE>(p, row0 + i, __shfl_sync(0xffffffffu, inside, i), mine, k + lane < k1), i, lane, false);
+    }
+}
+// The sum of row m and the lane's column: over the groups of steps that hold large operands or, where that is finite, over all of them
+template <int MODE>
+__device__ __noinline__ float sum_again(const SplitParams& p, int m, uint32_t inside, const Column<MODE> col, bool left, int k0, int k1, int group, uint32_t large)
+{
+    auto add = [&](float sum, int from, int to) {      // (up to the first NaN of all lanes)
+        Step<MODE> s(p, from);
+        while (s.k < to && __any_sync(0xffffffffu, left && sum == sum)) {
+            const int stop = min(s.k + 32, to);
+#pragma unroll 8
+            for (; s.k < stop; s.next(p)) sum = fmaf(row_operand<MODE>(p, m, inside, s), col.operand(p, s, left), sum);
+        }
+        return sum;
+    };
+    float s = 0.f;
+    for (int l = 0; l < 32; ++l)
+        for (uint32_t w = __shfl_sync(0xffffffffu, large, l); w != 0u; w &= w - 1u) {
+            const int from = k0 + (32 * l + __ffs(w) - 1) * group;
+            s = add(s, from, min(from + group, k1));
+        }
+    if (__any_sync(0xffffffffu, left && s - s == 0.f)) {
+        const float whole = add(0.f, k0, k1);
+        if (s - s == 0.f) s = whole;
+    }
+    return s;
+}
+template <int MODE, int BN>
+__device__ __forceinline__ void repair_unit(const SplitParams& p, int u, int q)
+{
+    constexpr uint32_t ALL = 0xffffffffu;
+    constexpr int CB = BN / 32;
+    const Unit t = unit_at<BN>(p, u);
+    const int lane = threadIdx.x % 32, row0 = t.m0 + 32 * q;
+    const int k0 = t.chunk0 * 64, k1 = min(p.K, (t.chunk0 + t.n_iters) * 64), group = (k1 - k0 + 1023) / 1024;
+    const bool raw_sums = MODE == CMODE_WGRAD || p.splits > 1;
+    volatile float* const base = raw_sums ? p.part + (size_t)t.split * p.split_stride : p.out;
+    const uint32_t inside = MODE == CMODE_WGRAD ? 0u : taps_inside<MODE>(p, row0 + lane);      // (of row `lane`)
+    Column<MODE> col[CB];
+#pragma unroll
+    for (int b = 0; b < CB; ++b) col[b] = Column<MODE>(p, t.n0 + 32 * b + lane);
+    uint32_t rows = 0u, cols[CB], row_nan = 0u, col_nan[CB], large = 0u;
+#pragma unroll
+    for (int b = 0; b < CB; ++b) cols[b] = col_nan[b] = 0u;
+    for (int r = 0; r < 32 && row0 + r < p.M; ++r)
+#pragma unroll
+        for (int b = 0; b < CB; ++b) {
+            const int n = t.n0 + 32 * b + lane;
+            const float v = n < p.N ? base[(size_t)(row0 + r) * p.N + n] : 0.f;
+            const uint32_t nan = __ballot_sync(ALL, v != v);
+            cols[b] |= nan;
+            if (nan != 0u) rows |= 1u << r;
+        }
+    auto explained = [&] {
+        uint32_t c = 0u;
+#pragma unroll
+        for (int b = 0; b < CB; ++b) c |= cols[b] & ~col_nan[b];
+        return c == 0u || (rows & ~row_nan) == 0u;
+    };
+    for (int k = k0; k < k1 && !explained(); k += 32) {
+        // (products of operands below 2^53 are below 2^106: no sum of them overflows)
+        constexpr uint32_t LARGE = 0x5a000000u, INF = 0x7f800000u;
+        uint32_t top = 0u;
+        visit<MODE, BN>(p, col, row0, t.n0, inside, k, k1, [&](float v, int, int, bool) { top = max(top, __float_as_uint(v) & 0x7fffffffu); });
+        if (!__any_sync(ALL, top >= LARGE)) continue;
+        uint32_t rn = 0u, cn[CB], steps = 0u;
+#pragma unroll
+        for (int b = 0; b < CB; ++b) cn[b] = 0u;
+        visit<MODE, BN>(p, col, row0, t.n0, inside, k, k1, [&](float v, int line, int step, bool of_col) {
+            const uint32_t a = __float_as_uint(v) & 0x7fffffffu;
+            if (a >= LARGE && a <= INF) steps |= 1u << step;
+            if (a > INF && !of_col) rn |= 1u << line;
+#pragma unroll
+            for (int b = 0; b < CB; ++b)
+                if (a > INF && of_col && line / 32 == b) cn[b] |= 1u << (line % 32);
+        });
+        row_nan |= __reduce_or_sync(ALL, rn);
+#pragma unroll
+        for (int b = 0; b < CB; ++b) col_nan[b] |= __reduce_or_sync(ALL, cn[b]);
+        for (steps = __reduce_or_sync(ALL, steps); steps != 0u; steps &= steps - 1u) {
+            const int g = (k + __ffs(steps) - 1 - k0) / group;
+            if (lane == g >> 5) large |= 1u << (g & 31);
+        }
+    }
+    for (; rows != 0u; rows &= rows - 1u) {
+        const int r = __ffs(rows) - 1, m = row0 + r;
+        const uint32_t in = __shfl_sync(ALL, inside, r);
+#pragma unroll
+        for (int b = 0; b < CB; ++b) {
+            const int n = t.n0 + 32 * b + lane;
+            const size_t at = (size_t)m * p.N + n;
+            float sum = n < p.N ? base[at] : 0.f;
+            const bool mine = sum != sum;
+            const bool left = mine && !((row_nan >> r) & 1u) && !((col_nan[b] >> lane) & 1u);
+            if (__any_sync(ALL, left)) {
+                const float s = sum_again<MODE>(p, m, in, col[b], left, k0, k1, group, large);
+                if (left) sum = s;
+            }
+            if (mine) base[at] = raw_sums ? sum : finish1<MODE>(p, sum, at, n);
+        }
+    }
+}
+template <int MODE, int BN>
+__device__ __noinline__ void repair_units(const SplitParams& p, int q)
+{
+    for (int u = blockIdx.x; u < p.units; u += gridDim.x) repair_unit<MODE, BN>(p, u, q);
 }
 // slot of a ring and the parity of its current use
 struct Ring {
@@ -421,6 +611,7 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
         constexpr int LD = WT ? 2 : 1;      // loads per wait: what the registers allow
         Ring lead, rest;
         bool ok = true;
+        bool nan = false;      // one of this thread's sums is or was (rows past the last too: repair_unit leaves those out)
         for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
             const Unit t = unit_at<BN>(p, u);
             float acc[BN];
@@ -458,7 +649,8 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
             if (!ok) break;
             const int m = t.m0 + q * 32 + lane;
             float* const base = raw_sums ? p.part + (size_t)t.split * p.split_stride : p.out;
-            bool bad = false;
+#pragma unroll
+            for (int j = 0; j < BN; ++j) nan = nan || acc[j] != acc[j];
             if (m < p.M) {
                 const size_t row = (size_t)m * p.N;
 #pragma unroll
@@ -466,49 +658,16 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
                     if (t.n0 + c >= p.N) continue;
                     float f[8];
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        f[j] = acc[c + j];
-                        bad = bad || f[j] != f[j];
-                    }
+                    for (int j = 0; j < 8; ++j) f[j] = acc[c + j];
                     if (!raw_sums) finish8<MODE>(p, f, row + t.n0 + c, t.n0 + c);
                     float4* d = (float4*)(base + row + t.n0 + c);
                     d[0] = make_float4(f[0], f[1], f[2], f[3]);
                     d[1] = make_float4(f[4], f[5], f[6], f[7]);
                 }
             }
-            if (__any_sync(0xffffffffu, bad)) {
-                // What is NaN in plain arithmetic too has been stored as such.  Each lane sorts out of its row what 32 multiply-adds show
-                // to be (all of it where a whole operand is NaN); the warp then shares the reduction of every element that is left, so
-                // that one long row does not outlast the other warps' bounded waits.
-                const int k0 = t.chunk0 * 64, k1 = min(p.K, (t.chunk0 + t.n_iters) * 64);
-#pragma unroll
-                for (int c = 0; c < BN; c += 32) {
-                    uint32_t nan = 0u;
-#pragma unroll
-                    for (int j = 0; j < 32; ++j)
-                        if (acc[c + j] != acc[c + j] && m < p.M && t.n0 + c + j < p.N) nan |= 1u << j;
-                    uint32_t left = 0u;
-                    for (; nan != 0u; nan &= nan - 1u) {
-                        const int j = __ffs(nan) - 1;
-                        const float s = plain_sum<MODE>(p, m, t.n0 + c + j, k0, k1, 1, 32);
-                        if (s == s) left |= 1u << j;
-                    }
-                    __syncwarp();
-                    for (uint32_t rows = __ballot_sync(0xffffffffu, left != 0u); rows != 0u; rows &= rows - 1u) {
-                        const int src = __ffs(rows) - 1, mr = t.m0 + q * 32 + src;
-                        for (uint32_t b = __shfl_sync(0xffffffffu, left, src); b != 0u; b &= b - 1u) {
-                            const int n = t.n0 + c + __ffs(b) - 1;
-                            float s = plain_sum<MODE>(p, mr, n, k0 + lane, k1, 32, 1 << 30);
-                            __syncwarp();
-#pragma unroll
-                            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                            const size_t at = (size_t)mr * p.N + n;
-                            if (lane == src) base[at] = raw_sums ? s : finish1<MODE>(p, s, at, n);
-                        }
-                    }
-                }
-            }
         }
+        // (behind the last unit: no wait of the other warps depends on how long this takes)
+        if (__any_sync(0xffffffffu, nan) && ok) repair_units<MODE, BN>(p, q);
         if (!ok && lane == 0) { *abort_flag = 1; atomicMax(p.status, (uint32_t)DEV_TIMEOUT_EPI); }
     } else {
         // =========================== converters ==================================================================================
@@ -539,18 +698,6 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
         int b_shift[NB];                            // the float it starts at relative to the pixel's first
         const int step_h = (64 / p.W) % p.H, step_w = 64 % p.W;       // WGRAD: one chunk on, in rows and columns
 
-        auto taps_inside = [&](int m) {
-            uint32_t in = 0u;
-            if (m >= p.M) return in;
-            if (p.taps == 1) return 1u;
-            const int n = div_rcp(m, p.rcp_hw, HW), w = m - n * HW, h = div_rcp(w, p.rcp_w, p.W), x = w - h * p.W;
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                const int er = MODE == CMODE_FWD ? i / 3 - 1 : 1 - i / 3, es = MODE == CMODE_FWD ? i % 3 - 1 : 1 - i % 3;
-                if ((unsigned)(h + er) < (unsigned)p.H && (unsigned)(x + es) < (unsigned)p.W) in |= 1u << i;
-            }
-            return in;
-        };
         // the first chunk of a unit
         auto first_chunk = [&](const Unit& un) {
             kpos = un.chunk0 * 64;
@@ -579,7 +726,7 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
                 const int k = kpos + 16 * quarter, m = un.m0 + row;
                 a_tap = k / Cred; a_c = k - a_tap * Cred;
                 a_px = (MODE == CMODE_FWD ? p.act : p.dy) + (size_t)m * Cred;
-                a_px_in = taps_inside(m);
+                a_px_in = taps_inside<MODE>(p, m);
             }
         };
         auto next_chunk = [&] {
@@ -629,7 +776,7 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
             const bool do_bias = MODE == CMODE_WGRAD && un.n0 == 0;
             float bsum = 0.f;
             if (TMA && MODE != CMODE_WGRAD) {
-                a_in = taps_inside(un.m0 + row);
+                a_in = taps_inside<MODE>(p, un.m0 + row);
                 a_tap = un.chunk0 * 64 / Cred; a_c = un.chunk0 * 64 - a_tap * Cred;
             }
             for (int it = 0; it < un.n_iters && ok; ++it, ++chunk) {

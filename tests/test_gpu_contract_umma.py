@@ -150,3 +150,101 @@ def test_non_finite_operands_over_long_reductions(where):
         assert not fin.any() or tu.maxrel(u[fin], v[fin]) < 1e-5
     a.close()
     ref.close()
+
+
+def _same(u, v):
+    assert np.array_equal(np.isnan(u), np.isnan(v)) and np.array_equal(np.isinf(u), np.isinf(v))
+    assert np.array_equal(np.sign(u[np.isinf(v)]), np.sign(v[np.isinf(v)]))
+    fin = np.isfinite(v)
+    assert not fin.any() or tu.maxrel(u[fin], v[fin]) < 1e-5
+
+
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan, 3.4e38, 1e30])      # (1e30: products overflow, no operand is infinite)
+@pytest.mark.parametrize("layer", [1, 2])
+@pytest.mark.parametrize("H,W,c0,c1,width,b", [
+    (9, 7, 24, 72, 64, 40),       # chunks that cross taps, ragged rows and columns
+    (16, 16, 64, 64, 136, 96),    # conv: 192 row tiles, more than one unit a CTA
+])
+def test_non_finite_operands_of_all_forms(H, W, c0, c1, width, b, layer, bad):
+    """Convolution and FC layers, with and without whole taps a chunk: one bad input, weight and output gradient at a time."""
+    from paper_2112_15317_b200 import binding as sb
+    wl, params, batch = _net(H, W, c0, c1, width, b, 1)
+    xs, ys = tu.device_batch(wl, *batch, False)
+    got, ran = [], []
+    for flags in (sb.SB_FLAG_PROFILE_LAYERS, sb.SB_FLAG_FORCE_SIMT):
+        m = tu.gpu_model(wl, params, sb.SB_FP32, flags)
+        m.forward(xs, ys)
+        act, w = (m.read(what, li, 0, squeeze=False) for what, li in ((sb.SB_T_ACT, layer - 1), (sb.SB_T_WEIGHT, layer)))
+        dy = np.random.default_rng(7).normal(0.0, 0.01, m.read(sb.SB_T_DACT, layer).size).astype(np.float32)
+        out = []
+        for turn in range(3):
+            t = [act.copy(), w.copy(), dy.copy()]
+            t[turn].reshape(-1)[int(0.37 * t[turn].size)] = bad
+            if turn == 0:
+                t[0].reshape(-1)[-1] = bad
+            m.write(sb.SB_T_ACT, layer - 1, 0, t[0])
+            m.write(sb.SB_T_WEIGHT, layer, 0, t[1])
+            m.write(sb.SB_T_DACT, layer, 0, t[2])
+            m.profile_begin()
+            m.forward_layers(layer, layer)
+            out.append(m.read(sb.SB_T_ACT, layer))
+            m.backward_layers(layer, layer)
+            ran += [e["name"] for e in m.profile_end() if "f32_umma" in e["name"]]
+            m.loss()       # raises if a bounded wait ran out
+            out += [m.read(sb.SB_T_GRAD_W, layer), m.read(sb.SB_T_GRAD_B, layer), m.read(sb.SB_T_DACT, layer - 1)]
+        assert m.debug_check_guards()[0] == 0
+        got.append(out)
+        m.close()
+    assert len(ran) >= 6, ran
+    for u, v in zip(*got):
+        _same(u, v)
+
+
+@pytest.mark.parametrize("where", ["gradients of the last image NaN", "one image infinite", "all weights NaN"])
+def test_non_finite_operands_do_not_stall(where):
+    """512 -> 1024 channels at 28x28, batch 64: several units a CTA and 50176 pixels in one reduction.  The results of plain multiply-adds,
+    no wait that runs out, and passes that take a few times as long as on finite data, not hundreds."""
+    import torch
+
+    from paper_2112_15317_b200 import binding as sb
+    wl = si.Workload("stall", [(si.CONV3X3_RELU, 512), (si.CONV3X3_RELU, 1024), (si.FC, 10), (si.SOFTMAX_XENT, 10)], 28, 28, 4, 64, 1, 1)
+    x, y = torch.randn(64, 28, 28, 4, device="cuda"), torch.zeros(64, dtype=torch.int32, device="cuda")
+    got, ms = [], []
+    for flags in (0, sb.SB_FLAG_FORCE_SIMT):
+        m = sb.Model.from_workload(wl, precision=sb.SB_FP32, flags=flags)
+
+        def view(what, layer, shape):
+            off = m.tensor_info(what, layer)[0] - m.arena.data_ptr()
+            return m.arena[off:off + 4 * int(np.prod(shape))].view(torch.float32).view(shape)
+        g = torch.Generator(device="cuda").manual_seed(1)
+        act, w, dy = view(sb.SB_T_ACT, 0, (64, 28, 28, 512)), view(sb.SB_T_WEIGHT, 1, (1024, 9, 512)), view(sb.SB_T_DACT, 1, (64, 28, 28, 1024))
+        for t, std in ((act, 1.0), (w, 0.02), (dy, 0.01)):
+            t.copy_(torch.randn(t.shape, generator=g, device="cuda") * std)
+        act.relu_()
+        view(sb.SB_T_BIAS, 1, (1024,)).zero_()
+        m.forward_layers(0, 0, [x], [y])      # (binds the inputs; its output is replaced)
+        act.copy_(torch.randn(act.shape, generator=g, device="cuda").relu())
+
+        def passes():
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            e[0].record()
+            m.forward_layers(1, 1)
+            m.backward_layers(1, 1)
+            e[1].record()
+            torch.cuda.synchronize()
+            ms.append(e[0].elapsed_time(e[1]))
+        passes()
+        passes()
+        if where == "all weights NaN":
+            w.fill_(float("nan"))
+        elif where == "one image infinite":
+            act[37] = float("inf")
+        else:
+            dy[63] = float("nan")
+        passes()
+        m.loss()       # raises if a bounded wait ran out
+        got.append([t.cpu().numpy() for t in (view(sb.SB_T_ACT, 1, (64, 28, 28, 1024)), view(sb.SB_T_GRAD_W, 1, (1024, 9, 512)), view(sb.SB_T_DACT, 0, (64, 28, 28, 512)))])
+        m.close()
+    for u, v in zip(*got):
+        _same(u, v)
+    assert ms[2] < 15.0 * ms[1], ms
