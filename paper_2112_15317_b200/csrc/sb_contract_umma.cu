@@ -11,7 +11,8 @@
 // Precision.  The tensor core adds into its float accumulator with truncation, so a long chain in it would lose more than the
 // rounded multiply-adds of the CUDA cores.  The leading products a0 b0 are therefore accumulated over 64 reduction steps only (four
 // instructions) and then added to a rounded running sum in registers; the remaining products, 2^-9 times smaller, stay in an
-// accumulator of their own until the end.  Error against 64-bit sums (2-norm; half-normal x, normal w and dy), CUDA cores -> here:
+// accumulator of their own for 64 such chunks: at most 1280 truncated additions to a sum of 2^-8 of the result, 1.5e-7 of it if they all
+// have one sign (over 784 chunks, a weight gradient at 28x28 and batch 64, 2.1e-6).  Error against 64-bit sums (2-norm; half-normal x, normal w and dy), CUDA cores -> here:
 //   3x3, 64 channels at 32x32, batch 96    forward 3.0e-7 -> 0.9e-7   input gradient 4.2e-7 -> 0.9e-7   weight gradient 4.6e-7 -> 1.9e-7
 //   3x3, 256 channels at 8x8, batch 96             3.4e-7 -> 0.9e-7                  4.8e-7 -> 1.0e-7                   3.3e-7 -> 1.1e-7
 //   4096 -> 1024, batch 96                         1.8e-7 -> 1.0e-7                  2.1e-7 -> 0.9e-7                   1.3e-7 -> 0.5e-7
@@ -74,6 +75,7 @@ static_assert(Roles<true>::REGS_ISSUE < 128 && Roles<true>::REGS_CONV > 128 && R
 static_assert(Roles<false>::REGS_ISSUE < 80 && Roles<false>::REGS_CONV < 80 && Roles<false>::REGS_ISSUE + Roles<false>::REGS_SUMS + 4 * Roles<false>::REGS_CONV <= 6 * 80, "");
 constexpr int CONV0 = 256;
 constexpr int STAGES = 2, RAWS = 2, RAW = 32768, CTRL = 8192;
+constexpr int REST_CHUNKS = 64;      // after which the accumulator of the other products is emptied
 // PLANE: one term of the B tile, BN rows of 128 bytes (FWD) or 64-column boxes of 64 rows.  RAW: a chunk of A as floats, 32-column
 // boxes of 128-byte swizzled rows.  Tensor memory columns: buffers of leading products, buffers of the other products, then the
 // terms of A (2 stages x 3 x 32).  PAIRED (64 wide): the other products lie side by side, a0 b1 + a1 b0 and a0 b2 + a1 b1 + a2 b0, so
@@ -448,7 +450,7 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
     uint64_t* raw_empty = raw_full + RAWS;          // [RAWS] ... and is in registers: one arrival per converter warp
     uint64_t* lead_full = raw_empty + RAWS;         // [LEADS] leading products of a chunk complete
     uint64_t* lead_empty = lead_full + C::LEADS;    // [LEADS] ... and taken over: one arrival per summing warp
-    uint64_t* rest_full = lead_empty + C::LEADS;    // [RESTS] everything of a unit complete
+    uint64_t* rest_full = lead_empty + C::LEADS;    // [RESTS] the other products of REST_CHUNKS chunks, or of a unit's last ones, complete
     uint64_t* rest_empty = rest_full + C::RESTS;    // [RESTS] ... and taken over
     uint32_t* tmem_slot = (uint32_t*)(rest_empty + C::RESTS);
     volatile uint32_t* abort_flag = tmem_slot + 1;
@@ -487,11 +489,11 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
             const uint64_t dB = make_desc(smem_u32(smem), B_MN ? 8192u : 16u);
             const uint32_t b_hi = (uint32_t)(dB >> 32);
             Ring st, lead, rest;
-            int chunk = 0, unit = 0;      // (a buffer's first use needs no wait)
+            int chunk = 0;      // (a buffer's first use needs no wait)
             bool ok = true, ready = false;      // ready: the next chunk's terms and its buffer of leading products were seen to be
-            for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x, ++unit) {
-                const int n_iters = unit_at<BN>(p, u).n_iters;
-                for (int it = 0; it < n_iters; ++it, ++chunk) {
+            for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
+                const uint32_t n_iters = (uint32_t)unit_at<BN>(p, u).n_iters;
+                for (uint32_t it = 0; it < n_iters; ++it, ++chunk) {
                     if (!ready) {
                         bool w = mbar_wait(&full[st.i], st.ph);
                         if (chunk >= C::LEADS) w = w && mbar_wait(&lead_empty[lead.i], lead.ph ^ 1u);
@@ -504,7 +506,7 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk) umma_ta(d0, a + kk * A_STEP, b + kk * B_STEP, b_hi, idesc, kk > 0 ? 1u : 0u, elected);
                     if (elected) umma_commit(&lead_full[lead.i]);
-                    if (it == 0 && unit >= C::RESTS) {
+                    if (it % REST_CHUNKS == 0) {      // (a fresh barrier reports the phase before its first as complete)
                         ok = __all_sync(0xffffffffu, mbar_wait(&rest_empty[rest.i], rest.ph ^ 1u) ? 1 : 0) != 0;
                         if (!ok) break;
                         tc_fence_after();
@@ -514,7 +516,7 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
                     lead.next(C::LEADS);
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk) {
-                        const uint32_t ak = a + kk * A_STEP, bk = b + kk * B_STEP, acc = (it > 0 || kk > 0) ? 1u : 0u;
+                        const uint32_t ak = a + kk * A_STEP, bk = b + kk * B_STEP, acc = (it % REST_CHUNKS > 0 || kk > 0) ? 1u : 0u;
                         if (kk == 3) {      // behind the instructions still queued, not after them
                             bool w = mbar_test(&full[st.i], st.ph);
                             if (chunk + 1 >= C::LEADS) w = w && mbar_test(&lead_empty[lead.i], lead.ph ^ 1u);
@@ -533,10 +535,12 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
                         }
                     }
                     if (elected) umma_commit(&empty[st_now]);
-                    if (elected && it + 1 == n_iters) umma_commit(&rest_full[rest.i]);
+                    if ((it + 1) % REST_CHUNKS == 0 || it + 1 == n_iters) {
+                        if (elected) umma_commit(&rest_full[rest.i]);
+                        rest.next(C::RESTS);
+                    }
                     __syncwarp();
                 }
-                rest.next(C::RESTS);
             }
             if (!ok && lane == 0) { *abort_flag = 1; atomicMax(p.status, (uint32_t)DEV_TIMEOUT_MMA); }
             __syncwarp();
@@ -617,14 +621,14 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
             float acc[BN];
 #pragma unroll
             for (int j = 0; j < BN; ++j) acc[j] = 0.f;
-            for (int it = 0; it <= t.n_iters; ++it) {
-                // the leading products chunk by chunk, then the others
-                const bool last = it == t.n_iters;
-                uint64_t* in = last ? &rest_full[rest.i] : &lead_full[lead.i];
-                ok = __all_sync(0xffffffffu, mbar_wait(in, last ? rest.ph : lead.ph) ? 1 : 0) != 0;
+            bool others = false;
+            for (int it = 0; it < t.n_iters || others;) {
+                // the leading products chunk by chunk, the others whenever their accumulator is emptied
+                uint64_t* in = others ? &rest_full[rest.i] : &lead_full[lead.i];
+                ok = __all_sync(0xffffffffu, mbar_wait(in, others ? rest.ph : lead.ph) ? 1 : 0) != 0;
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t from = taddr + (last ? C::COL_REST + (uint32_t)rest.i * C::REST : (uint32_t)lead.i * BN);
+                const uint32_t from = taddr + (others ? C::COL_REST + (uint32_t)rest.i * C::REST : (uint32_t)lead.i * BN);
                 auto add = [&](uint32_t at) {
 #pragma unroll
                     for (int c = 0; c < BN; c += 16 * LD) {
@@ -639,12 +643,18 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
                     }
                 };
                 add(from);
-                if (C::PAIRED && last) add(from + BN);
+                if (C::PAIRED && others) add(from + BN);
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(last ? &rest_empty[rest.i] : &lead_empty[lead.i]));
-                if (last) rest.next(C::RESTS);
-                else lead.next(C::LEADS);
+                if (lane == 0) mbar_arrive(smem_u32(others ? &rest_empty[rest.i] : &lead_empty[lead.i]));
+                if (others) {
+                    rest.next(C::RESTS);
+                    others = false;
+                } else {
+                    lead.next(C::LEADS);
+                    ++it;
+                    others = it % REST_CHUNKS == 0 || it == t.n_iters;
+                }
             }
             if (!ok) break;
             const int m = t.m0 + q * 32 + lane;

@@ -12,7 +12,8 @@ import sb_testutil as tu
 pytestmark = pytest.mark.gpu
 
 # Bound on the 2-norm: products left out 2^-26, truncation of the leading products over 64 steps 4 x 2^-25, the rounded running sum
-# 2^-25 sqrt(chunks) of up to 60 chunks: below 4e-7 in all; the largest measured over a sweep of 25 layers is 2.1e-7.
+# 2^-25 sqrt(chunks) of up to 60 chunks: below 4e-7 in all; the largest measured over a sweep of 25 layers is 2.1e-7.  The other products
+# of 64 chunks take part with up to 1280 truncated additions to a sum of 2^-8 of the result: 1.5e-7 where all of them have one sign.
 BOUND = 5e-7
 
 
@@ -150,6 +151,31 @@ def test_non_finite_operands_over_long_reductions(where):
         assert not fin.any() or tu.maxrel(u[fin], v[fin]) < 1e-5
     a.close()
     ref.close()
+
+
+def test_long_reduction_of_one_sign():
+    """784 chunks in one split (512 -> 1024 channels at 28x28, batch 64), all terms of all operands positive: what the accumulators cut off
+    adds up.  The leading products are exact here (ones)."""
+    import torch
+
+    from paper_2112_15317_b200 import binding as sb
+    m = sb.Model([(si.CONV3X3_RELU, 512), (si.CONV3X3_RELU, 1024), (si.FC, 10), (si.SOFTMAX_XENT, 10)], 28, 28, 4, 64, 1, 1, sb.SB_FP32, sb.SB_FLAG_PROFILE_LAYERS)
+
+    def view(what, layer, shape):
+        off = m.tensor_info(what, layer)[0] - m.arena.data_ptr()
+        return m.arena[off:off + 4 * int(np.prod(shape))].view(torch.float32).view(shape)
+    act, dy = view(sb.SB_T_ACT, 0, (64, 784, 512)), view(sb.SB_T_DACT, 1, (64, 784, 1024))
+    g = torch.Generator(device="cuda").manual_seed(1)
+    m.forward_layers(0, 0, [torch.zeros(64, 28, 28, 4, device="cuda")], [torch.zeros(64, dtype=torch.int32, device="cuda")])
+    for t in (act, dy):
+        t.copy_(1.0 + 2.0 ** -8 * (0.25 + 0.7 * torch.rand(t.shape, generator=g, device="cuda")))      # (rounds to 1 in bf16)
+    m.profile_begin()
+    m.backward_layers(1, 1)
+    assert any(e["name"].startswith("conv_wgrad_f32_umma") for e in m.profile_end())
+    want = dy.reshape(-1, 1024)[:, :64].double().T @ act.reshape(-1, 512).double()      # (the middle tap, 64 of the output channels)
+    got = view(sb.SB_T_GRAD_W, 1, (1024, 9, 512))[:64, 4].double()
+    assert ((got - want).norm() / want.norm()).item() < 2e-7
+    m.close()
 
 
 def _same(u, v):
