@@ -1116,15 +1116,20 @@ static sb_status chain_bwd(sb_model* m, int i, cudaStream_t st, int part)
     return s;
 }
 
-// The conv weights as bf16 terms, at the beginning of every call that reads them so (layers first .. last): the weights may have changed
-// since the last one.  4 us for the 7-conv net's 1.7 M parameters.
+// The conv weights as bf16 terms, at the beginning of every call that reads them so: those from the first to the last layer of first ..
+// last that does.  The weights may have changed since the last call.  4 us for the 7-conv net's 1.7 M parameters.
 static sb_status split_weights(sb_model* m, int first, int last, bool fwd, bool dgrad, cudaStream_t st)
 {
-    bool any = false;
-    for (int i = first; i <= last; ++i) any = any || (fwd && wants_terms(m->L[i], CMODE_FWD)) || (dgrad && wants_terms(m->L[i], CMODE_DGRAD));
-    if (!any) return SB_OK;
+    size_t lo = m->t_n, hi = 0;
+    for (int i = first; i <= last; ++i) {
+        const Layer& l = m->L[i];
+        if (!(fwd && wants_terms(l, CMODE_FWD)) && !(dgrad && wants_terms(l, CMODE_DGRAD))) continue;
+        lo = std::min(lo, l.p_w);
+        hi = std::max(hi, l.p_w + align_up(l.n_w, 64));
+    }
+    if (hi == 0) return SB_OK;
     m->cur_layer = -1;
-    L_TRY("split_weights", 0.0, 10.0 * m->t_n, launch_split_weights(m->Wm, m->Tm, m->t_n, m->t_n, st));
+    L_TRY("split_weights", 0.0, 10.0 * (hi - lo), launch_split_weights(m->Wm + lo, m->Tm + lo, hi - lo, m->t_n, st));
     return SB_OK;
 }
 

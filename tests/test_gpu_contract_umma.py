@@ -153,6 +153,24 @@ def test_non_finite_operands_over_long_reductions(where):
     ref.close()
 
 
+def test_weights_split_for_the_layers_of_a_call():
+    """Every call takes apart the weights that it reads as terms, and no others."""
+    from paper_2112_15317_b200 import binding as sb
+    convs = [64, 64, 128, 256]
+    wl = si.Workload("split_weights", [(si.CONV3X3_RELU, c) for c in convs] + [(si.FC, 10), (si.SOFTMAX_XENT, 10)], 16, 16, 4, 32, 1, 1)
+    m = tu.gpu_model(wl, si.make_params(wl), sb.SB_FP32)
+    xs, ys = tu.device_batch(wl, *si.make_batch(wl), False)
+    m.forward(xs, ys)
+    n = [0, 64 * 9 * 64, 128 * 9 * 64, 256 * 9 * 128]      # (layer 0 reads images)
+    bias = [64, 64, 128]                                   # (between them in memory)
+    for first, last, want in [(0, 0, 0), (1, 1, n[1]), (2, 2, n[2]), (3, 3, n[3]), (2, 3, n[2] + bias[2] + n[3]), (0, 3, sum(n) + bias[1] + bias[2]), (4, 5, 0)]:
+        for run in (lambda: m.forward_layers(first, last), lambda: m.backward_layers(last, first)):
+            m.profile_begin()
+            run()
+            assert sum(e["bytes"] for e in m.profile_end() if e["name"] == "split_weights") == 10.0 * want, (first, last)
+    m.close()
+
+
 def test_long_reduction_of_one_sign():
     """784 chunks in one split (512 -> 1024 channels at 28x28, batch 64), all terms of all operands positive: what the accumulators cut off
     adds up.  The leading products are exact here (ones)."""
