@@ -110,7 +110,7 @@ struct sb_model {
     // stream, or (mean_aside) left to the backward pass, which enqueues it beside the chain.
     bool head_ok = false, mean_aside = false, mean_pending = false;
     int xent_by_fc = -1;
-    int bwd_lo = 1 << 30;      // lowest layer of the backward call that is being enqueued
+    int fwd_hi = -1, bwd_lo = 1 << 30;      // highest layer of the forward, lowest of the backward call that is being enqueued
     int unpooled = -1;         // index of the pool layer whose input gradient the layer above has already written (same backward call)
     int pooled_by_conv = -1;   // index of the pool layer whose output the conv kernel just before it has already written (same forward call)
     // Set by the multi-stream backward pass while it enqueues the weight side of one conv layer: the layer's split
@@ -514,11 +514,11 @@ XentArgs xent_args(sb_model* m, int i)
 }
 
 // The pool layer above conv layer i (its split reduction may pool in the same pass), or below layer i (whose split data gradient may
-// lead on through it: only where the pool layer belongs to the same backward call); p / dx == nullptr: there is none.
+// lead on through it), where the pool layer belongs to the same call; p / dx == nullptr: there is none.
 SplitPool pool_above(sb_model* m, int i)
 {
     SplitPool o{};
-    if (i + 1 < m->n_layers && m->L[i + 1].kind == SB_MAXPOOL2) {
+    if (i + 1 <= m->fwd_hi && m->L[i + 1].kind == SB_MAXPOOL2) {
         const Layer& pl = m->L[i + 1];
         o.H = pl.H; o.W = pl.W; o.C = pl.Cin; o.p = pl.act; o.idx = pl.idx;
     }
@@ -1143,15 +1143,13 @@ sb_status sb_forward_layers(sb_model* m, int32_t first, int32_t last, const void
     }
     m->pooled_by_conv = -1;     // a pool layer run on its own (or first in the range) computes its output itself
     m->st_clean = false;
-    const sb_status ss = split_weights(m, first, last, true, false, (cudaStream_t)stream);
-    if (ss != SB_OK) return ss;
-    for (int i = first; i <= last; ++i) {
-        sb_status s = chain_fwd(m, i, (cudaStream_t)stream);
-        if (s != SB_OK) return s;
-    }
+    m->fwd_hi = last;
+    sb_status s = split_weights(m, first, last, true, false, (cudaStream_t)stream);
+    for (int i = first; i <= last && s == SB_OK; ++i) s = chain_fwd(m, i, (cudaStream_t)stream);
+    m->fwd_hi = -1;
     m->st_clean = false;
     m->pooled_by_conv = -1;
-    return SB_OK;
+    return s;
 }
 
 sb_status sb_backward_layers(sb_model* m, int32_t last, int32_t first, void* stream)
@@ -1252,9 +1250,11 @@ static sb_status forward_pass(sb_model* m, cudaStream_t st, bool by_itself)
     m->xent_by_fc = -1;
     m->st_clean = false;
     m->head_ok = true;
+    m->fwd_hi = m->n_layers - 1;
     sb_status s = split_weights(m, 0, m->n_layers - 1, true, !by_itself, st);
     for (int i = 0; i < m->n_layers && s == SB_OK; ++i) s = chain_fwd(m, i, st);
     m->head_ok = false;
+    m->fwd_hi = -1;
     m->st_clean = false;
     m->pooled_by_conv = -1;
     return s;
@@ -1491,11 +1491,11 @@ static sb_status modulo_step_direct(sb_model* m, const void* const* x, const int
     const int ff = m->first_fc, K = m->cfg.K, R = m->cfg.R, b = m->cfg.batch_per_replica, Bk = m->B / K;
     const size_t D = (size_t)m->L[ff].in_f;
     m->st_clean = false;
-    if ((s = split_weights(m, 0, ff - 1, true, true, st)) != SB_OK) return s;
-    for (int i = 0; i < ff; ++i) {
-        s = chain_fwd(m, i, st);
-        if (s != SB_OK) return s;
-    }
+    m->fwd_hi = ff - 1;
+    s = split_weights(m, 0, ff - 1, true, true, st);
+    for (int i = 0; i < ff && s == SB_OK; ++i) s = chain_fwd(m, i, st);
+    m->fwd_hi = -1;
+    if (s != SB_OK) return s;
     m->cur_layer = ff;
     {
         ModuloCopyArgs a{m->L[ff - 1].act, m->mod_x, D * m->esz, R, b, K, 0, &m->label_tab, m->mod_labels};

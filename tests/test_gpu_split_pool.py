@@ -39,5 +39,12 @@ def test_pool_in_split_reduce(bf16, H, W, c0, c1, b, R, fwd, bwd):
         alone = [read(sb.SB_T_ACT, pool), read(sb.SB_T_POOL_IDX, pool), read(sb.SB_T_DACT, pool - 1)]
         for u, v in zip(whole, alone):
             assert np.array_equal(u, v)
+    # a conv layer run by itself leaves the pool layer above it alone
+    left = 7.0 * np.ones((b,) + m.tensor_info(sb.SB_T_ACT, 3, 0)[1][1:], np.float32)
+    for r in range(R):
+        m.write(sb.SB_T_ACT, 3, r, left)
+        m.write(sb.SB_T_POOL_IDX, 3, r, (left + 2).astype(np.uint8))
+    m.forward_layers(2, 2)
+    assert np.all(read(sb.SB_T_ACT, 3) == 7.0) and np.all(read(sb.SB_T_POOL_IDX, 3) == 9)
     assert m.debug_check_guards()[0] == 0
     m.close()
