@@ -736,29 +736,6 @@ sb_status backward_layer(sb_model* m, int i, cudaStream_t st, int part = SIDE_BO
             }
             break;
         }
-        auto data_side = [&]() -> sb_status {
-            if (!want_in_grad || !(part & SIDE_D)) return SB_OK;
-            // shard-layer / modulo-layer backward: dX = sum_j dY_j W_j, rows stay with their replica
-            const double bytes = act_bytes + (double)l.n_w * e + (below_relu ? (double)B * l.in_f * e : 0.0);
-            SplitPool offer = pool_below(m, i);
-            split_pool() = offer.dx ? &offer : nullptr;
-            if (l.um.dgrad.enabled) {
-                fs = [&]() -> sb_status { U_TRY("fc_dgrad_umma", flops, bytes, umma_fc_dgrad(m, i, st)); return SB_OK; }();
-                ++m->launches;
-            } else {
-                fs = contract_dgrad(m, i, "fc_dgrad_simt", flops, bytes, d_below, below_relu ? layer_input(m, i) : nullptr, st);
-            }
-            split_pool() = nullptr;
-            if (fs != SB_OK) return fs;
-            if (offer.done) m->unpooled = i - 1;
-            return SB_OK;
-        };
-        // Up to 128 rows (one row tile: the weights are read once a pass) the data side goes first: where both sides run on one stream, right
-        // after the layer's forward pass, it reads what L2 still holds of the weights before the stored gradient replaces it. 25088 -> 4096,
-        // forward + backward, data side first / last: batch 128 183 / 184 us (input gradient 39 / 50, but the write-back of the gradient falls
-        // to the next forward pass), 129 193 / 185 - 188, 143 202 / 194 - 202, 160 203 / 199, 224 213 / 215 (runs differ by up to 10).
-        const bool data_first = B <= 128;
-        if (data_first && (fs = data_side()) != SB_OK) return fs;
         if (!(part & SIDE_W)) {
         } else if (l.um.wgrad.enabled && m->fuse.on && !(part & SIDE_D) && umma_fc_wgrad_can_update(m, i)) {
             // fused pass: the update is applied by the weight-gradient kernel's epilogue (after the layer's input-gradient
@@ -775,7 +752,21 @@ sb_status backward_layer(sb_model* m, int i, cudaStream_t st, int part = SIDE_BO
             if ((fs = contract_wgrad("fc_wgrad_simt", flops, act_bytes + (double)l.n_w * 4.0, &S)) != SB_OK) return fs;
             if ((fs = finish_both(ws_w, S)) != SB_OK) return fs;
         }
-        if (!data_first && (fs = data_side()) != SB_OK) return fs;
+        if (want_in_grad && (part & SIDE_D)) {
+            // shard-layer / modulo-layer backward: dX = sum_j dY_j W_j, rows stay with their replica
+            const double bytes = act_bytes + (double)l.n_w * e + (below_relu ? (double)B * l.in_f * e : 0.0);
+            SplitPool offer = pool_below(m, i);
+            split_pool() = offer.dx ? &offer : nullptr;
+            if (l.um.dgrad.enabled) {
+                fs = [&]() -> sb_status { U_TRY("fc_dgrad_umma", flops, bytes, umma_fc_dgrad(m, i, st)); return SB_OK; }();
+                ++m->launches;
+            } else {
+                fs = contract_dgrad(m, i, "fc_dgrad_simt", flops, bytes, d_below, below_relu ? layer_input(m, i) : nullptr, st);
+            }
+            split_pool() = nullptr;
+            if (fs != SB_OK) return fs;
+            if (offer.done) m->unpooled = i - 1;
+        }
         break;
     }
     case SB_DROPOUT: {
