@@ -1,5 +1,5 @@
-// Float contractions on the tensor cores: every float operand element is taken apart into three bf16 terms that add up to it
-// (8 + 8 + 8 significant bits), and the products of the terms are accumulated in float.
+// Float contractions on the tensor cores: every float operand element (times 2^16, see OPERAND_SCALE_X2) is taken apart into three bf16
+// terms that add up to it (8 + 8 + 8 significant bits), and the products of the terms are accumulated in float.
 //
 //   a = a0 + a1 + a2,  |a1| <= 2^-9 |a|,  |a2| <= 2^-18 |a|           (b likewise)
 //   a * b = a0 b0  +  (a0 b1 + a1 b0)  +  (a0 b2 + a1 b1 + a2 b0)  +  terms below 2^-26 |a b| that are left out
@@ -40,7 +40,7 @@
 // 45 / 47; 4096 -> 1024 30 / 27 / 23 -> 17 / 16 / 18. The 7-conv / 3-FC net: 2.54 -> 0.91 ms an iteration.
 //
 // Non-finite operands: infinity - infinity in the splitting makes the terms NaN where a float multiply-add would give an infinity, so
-// results that come out as NaN are looked at again behind the CTA's last unit, when no other warp waits (repair_unit).
+// results that are not finite are looked at again behind the CTA's last unit, when no other warp waits (repair_unit).
 #include "sb_umma.h"
 #include "sb_tcgen05.cuh"
 
@@ -75,6 +75,11 @@ static_assert(Roles<true>::REGS_ISSUE < 128 && Roles<true>::REGS_CONV > 128 && R
 static_assert(Roles<false>::REGS_ISSUE < 80 && Roles<false>::REGS_CONV < 80 && Roles<false>::REGS_ISSUE + Roles<false>::REGS_SUMS + 4 * Roles<false>::REGS_CONV <= 6 * 80, "");
 constexpr int CONV0 = 256;
 constexpr int STAGES = 2, RAWS = 2, RAW = 32768, CTRL = 8192;
+// Both operands are multiplied by 2^16 before they are taken apart, so that the last term of the smallest float is still a bf16 number
+// (unscaled, operands below 2^-110 lost bits: 2e-6 of the result at 2^-116, 2e-3 at 2^-126), and the results by 2^-32.  Results that
+// overflow meanwhile (2^96 and more) are looked at again, as NaNs are.
+constexpr unsigned long long OPERAND_SCALE_X2 = 0x4780000047800000ull;
+constexpr float RESULT_SCALE = 0x1p-32f;
 constexpr int REST_CHUNKS = 64;      // after which the accumulator of the other products is emptied
 // PLANE: one term of the B tile, BN rows of 128 bytes (FWD) or 64-column boxes of 64 rows.  RAW: a chunk of A as floats, 32-column
 // boxes of 128-byte swizzled rows.  Tensor memory columns: buffers of leading products, buffers of the other products, then the
@@ -130,12 +135,21 @@ __device__ __forceinline__ uint32_t take_term(float& a, float& b)
     asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(d));
     return u;
 }
+// two floats, times OPERAND_SCALE
+__device__ __forceinline__ void scale_pair(float& a, float& b)
+{
+    unsigned long long d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+    asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(d) : "l"(OPERAND_SCALE_X2));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(d));
+}
 // the three terms of eight floats
 __device__ __forceinline__ void take_terms(const F8& f, uint32_t* t0, uint32_t* t1, uint32_t* t2)
 {
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         float a = f.v[2 * j], b = f.v[2 * j + 1];
+        scale_pair(a, b);
         t0[j] = take_term(a, b);
         t1[j] = take_term(a, b);
         const __nv_bfloat162 t = __floats2bfloat162_rn(a, b);
@@ -178,7 +192,8 @@ __device__ __forceinline__ uint32_t taps_inside(const SplitParams& p, int m)
     }
     return in;
 }
-// Eight results of a row: bias and ReLU, or the ReLU mask.  A NaN stays one here: it is looked at again (repair_unit).
+__device__ __forceinline__ bool finite(float f) { return fabsf(f) < INFINITY; }
+// Eight results of a row: bias and ReLU, or the ReLU mask.  What is not finite stays so here: it is looked at again (repair_unit).
 template <int MODE>
 __device__ __forceinline__ void finish8(const SplitParams& p, float (&f)[8], size_t at, int n)
 {
@@ -190,8 +205,8 @@ __device__ __forceinline__ void finish8(const SplitParams& p, float (&f)[8], siz
     for (int j = 0; j < 8; ++j) {
         if (MODE == CMODE_FWD) {
             const float y = f[j] + e[j];
-            f[j] = p.relu && !(y > 0.f) && f[j] == f[j] ? 0.f : y;
-        } else if (!(e[j] > 0.f) && f[j] == f[j]) f[j] = 0.f;
+            f[j] = p.relu && !(y > 0.f) && finite(f[j]) ? 0.f : y;
+        } else if (!(e[j] > 0.f) && finite(f[j])) f[j] = 0.f;
     }
 }
 // One result (NaN -> 0 behind a ReLU or a mask, as everywhere)
@@ -222,8 +237,8 @@ __device__ __forceinline__ Unit unit_at(const SplitParams& p, int u)
     t.n_iters = min(p.cps, p.chunks - t.chunk0);
     return t;
 }
-// Results of a unit that came out as NaN, by one warp for the 32 rows that it has stored (NaN and unfinished): what plain multiply-adds
-// give.  A NaN operand makes its whole row or column NaN (places outside the image are zeros that are multiplied, as in
+// Results of a unit that came out as NaN or infinite, by one warp for the 32 rows that it has stored (those unfinished): what plain
+// multiply-adds give.  A NaN operand makes its whole row or column NaN (places outside the image are zeros that are multiplied, as in
 // contract_kernel: NaN x 0 and infinity x 0 are NaN), so the operands are searched for those first, and the search ends when they
 // explain every such result: a run that has diverged costs one look at the operands.  What is left has infinite or large operands
 // in its sum: the steps that hold any (in 1024 groups, a bit each, 32 to a lane) are summed, a lane per column; only where that is finite
@@ -365,9 +380,9 @@ __device__ __forceinline__ void repair_unit(const SplitParams& p, int u, int q)
         for (int b = 0; b < CB; ++b) {
             const int n = t.n0 + 32 * b + lane;
             const float v = n < p.N ? base[(size_t)(row0 + r) * p.N + n] : 0.f;
-            const uint32_t nan = __ballot_sync(ALL, v != v);
-            cols[b] |= nan;
-            if (nan != 0u) rows |= 1u << r;
+            const uint32_t odd = __ballot_sync(ALL, !finite(v));
+            cols[b] |= odd;
+            if (odd != 0u) rows |= 1u << r;
         }
     auto explained = [&] {
         uint32_t c = 0u;
@@ -408,7 +423,7 @@ __device__ __forceinline__ void repair_unit(const SplitParams& p, int u, int q)
             const int n = t.n0 + 32 * b + lane;
             const size_t at = (size_t)m * p.N + n;
             float sum = n < p.N ? base[at] : 0.f;
-            const bool mine = sum != sum;
+            const bool mine = n < p.N && !finite(sum);
             const bool left = mine && !((row_nan >> r) & 1u) && !((col_nan[b] >> lane) & 1u);
             if (__any_sync(ALL, left)) {
                 const float s = sum_again<MODE>(p, m, in, col[b], left, k0, k1, group, large);
@@ -615,7 +630,7 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
         constexpr int LD = WT ? 2 : 1;      // loads per wait: what the registers allow
         Ring lead, rest;
         bool ok = true;
-        bool nan = false;      // one of this thread's sums is or was (rows past the last too: repair_unit leaves those out)
+        bool odd = false;      // one of this thread's sums is or was not finite (rows past the last too: repair_unit leaves those out)
         for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
             const Unit t = unit_at<BN>(p, u);
             float acc[BN];
@@ -660,7 +675,7 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
             const int m = t.m0 + q * 32 + lane;
             float* const base = raw_sums ? p.part + (size_t)t.split * p.split_stride : p.out;
 #pragma unroll
-            for (int j = 0; j < BN; ++j) nan = nan || acc[j] != acc[j];
+            for (int j = 0; j < BN; ++j) odd = odd || !finite(acc[j]);
             if (m < p.M) {
                 const size_t row = (size_t)m * p.N;
 #pragma unroll
@@ -668,7 +683,7 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
                     if (t.n0 + c >= p.N) continue;
                     float f[8];
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) f[j] = acc[c + j];
+                    for (int j = 0; j < 8; ++j) f[j] = RESULT_SCALE * acc[c + j];
                     if (!raw_sums) finish8<MODE>(p, f, row + t.n0 + c, t.n0 + c);
                     float4* d = (float4*)(base + row + t.n0 + c);
                     d[0] = make_float4(f[0], f[1], f[2], f[3]);
@@ -677,7 +692,7 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
             }
         }
         // (behind the last unit: no wait of the other warps depends on how long this takes)
-        if (__any_sync(0xffffffffu, nan) && ok) repair_units<MODE, BN>(p, q);
+        if (__any_sync(0xffffffffu, odd) && ok) repair_units<MODE, BN>(p, q);
         if (!ok && lane == 0) { *abort_flag = 1; atomicMax(p.status, (uint32_t)DEV_TIMEOUT_EPI); }
     } else {
         // =========================== converters ==================================================================================
@@ -924,6 +939,8 @@ split_weights_kernel(const float4* __restrict__ w, uint2* __restrict__ terms, si
     pdl_prologue();
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
         float4 v = __ldg(w + i);
+        scale_pair(v.x, v.y);
+        scale_pair(v.z, v.w);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             uint2 t;

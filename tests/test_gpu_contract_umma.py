@@ -153,6 +153,42 @@ def test_non_finite_operands_over_long_reductions(where):
     ref.close()
 
 
+@pytest.mark.parametrize("exps", [(-126, 40, 40), (40, -126, 40), (40, 40, -126), (-60, -58, 50), (60, 58, -50), (-145, 60, 60)])
+@pytest.mark.parametrize("c0", [64, 24])
+def test_operands_of_all_magnitudes(c0, exps):
+    """Inputs, weights and output gradients down to the smallest normal (and to subnormal) floats, results up to 2^124."""
+    import torch
+    import torch.nn.functional as F
+
+    from paper_2112_15317_b200 import binding as sb
+    wl, params, batch = _net(8, 8, c0, 128, 128, 24, 1)
+    m = tu.gpu_model(wl, params, sb.SB_FP32, sb.SB_FLAG_PROFILE_LAYERS)
+    m.forward(*tu.device_batch(wl, *batch, False))
+    rng = np.random.default_rng(5)
+    x, w, dy = (np.ldexp(rng.uniform(0.5, 1.0, s) * rng.choice([-1.0, 1.0], s), e).astype(np.float32)
+                for s, e in zip(((24, 8, 8, c0), (128, 3, 3, c0), (24, 8, 8, 128)), exps))
+    x = np.abs(x)
+    for what, li, a in ((sb.SB_T_ACT, 0, x), (sb.SB_T_WEIGHT, 1, w), (sb.SB_T_DACT, 1, dy), (sb.SB_T_BIAS, 1, np.zeros(128, np.float32))):
+        m.write(what, li, 0, a)
+    m.profile_begin()
+    m.forward_layers(1, 1)
+    y = m.read(sb.SB_T_ACT, 1, 0, squeeze=False)
+    m.backward_layers(1, 1)
+    assert sum("f32_umma" in e["name"] for e in m.profile_end()) >= 2
+    t = lambda a: torch.from_numpy(a).double().permute(0, 3, 1, 2).requires_grad_()  # noqa: E731
+    xt, wt = t(x), t(w)
+    want = F.conv2d(xt, wt, padding=1)
+    want.backward(t(dy).detach())
+    checks = tu.Checks()
+    for name, got, ref in (("forward", y, want.detach().relu()), ("input gradient", m.read(sb.SB_T_DACT, 0, 0, squeeze=False), xt.grad),
+                           ("weight gradient", m.read(sb.SB_T_GRAD_W, 1, 0, squeeze=False), wt.grad)):
+        ref = ref.permute(0, 2, 3, 1).numpy()
+        assert np.isfinite(got).all()
+        checks.le(name, np.linalg.norm(got.astype(np.float64) / np.abs(ref).max() - ref / np.abs(ref).max()) / np.linalg.norm(ref / np.abs(ref).max()), BOUND)
+    checks.finish()
+    m.close()
+
+
 def test_weights_split_for_the_layers_of_a_call():
     """Every call takes apart the weights that it reads as terms, and no others."""
     from paper_2112_15317_b200 import binding as sb
