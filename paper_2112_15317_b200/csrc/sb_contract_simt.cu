@@ -8,8 +8,9 @@
 // A fully-connected layer is the same thing with one tap and 1x1 images (pixel = batch row).
 //
 // Large enough float layers whose channel counts are multiples of eight run on the tensor cores instead (sb_contract_umma.cu): the plan
-// takes whichever the two cost models below say is faster.  3x3 over 64 channels at 32x32, batch 96: 180 us here, 66 there; 256
-// channels at 8x8: 157 and 50; 16 -> 32 channels at 16x16, batch 8, forward: 8.0 and 7.3; 4096 -> 1024 weight gradient at batch 8: 6.8 and 14.
+// takes whichever the two cost models below say is faster.  Forward, us between events, 3x3 over 64 channels at 32x32, batch 96: 183 here,
+// 58 there; 256 channels at 8x8: 159 and 46; 16 -> 32 channels at 16x16, batch 8: 12.9 and 12.5.  4096 -> 1024 weight gradient at batch
+// 8, the kernel alone: 6.8 and 14.
 //
 // What bounds it: the FFMA pipe (measured 70 TFLOP/s of packed fma.rn.f32x2 on registers, 68 of scalar FFMA).  A block of
 // BM x BN outputs gives every thread an 8 x 8 square, so that 16 shared-memory words feed 64 multiply-adds; the packed form

@@ -12,11 +12,14 @@
 // rounded multiply-adds of the CUDA cores.  The leading products a0 b0 are therefore accumulated over 64 reduction steps only (four
 // instructions) and then added to a rounded running sum in registers; the remaining products, 2^-9 times smaller, stay in an
 // accumulator of their own for 64 such chunks: at most 1280 truncated additions to a sum of 2^-8 of the result, 1.5e-7 of it if they all
-// have one sign (over 784 chunks, a weight gradient at 28x28 and batch 64, 2.1e-6).  Error against 64-bit sums (2-norm; half-normal x, normal w and dy), CUDA cores -> here:
-//   3x3, 64 channels at 32x32, batch 96    forward 3.0e-7 -> 0.9e-7   input gradient 4.2e-7 -> 0.9e-7   weight gradient 4.6e-7 -> 1.9e-7
+// have one sign (over 784 chunks, a weight gradient at 28x28 and batch 64, 2.1e-6).  Floats as sums of bf16 terms: G. Henry, P. T. P. Tang
+// and A. Heinecke, "Leveraging the bfloat16 artificial intelligence datatype for higher-precision computations" (2019); sums kept out of
+// the truncating accumulator: H. Ootomo and R. Yokota, "Recovering single precision accuracy from tensor cores" (2022).
+// Error against 64-bit sums (2-norm; half-normal x, normal w and dy), CUDA cores -> here:
+//   3x3, 64 channels at 32x32, batch 96    forward 2.9e-7 -> 0.8e-7   input gradient 4.3e-7 -> 1.0e-7   weight gradient 3.9e-7 -> 1.8e-7
 //   3x3, 256 channels at 8x8, batch 96             3.4e-7 -> 0.9e-7                  4.8e-7 -> 1.0e-7                   3.3e-7 -> 1.1e-7
 //   4096 -> 1024, batch 96                         1.8e-7 -> 1.0e-7                  2.1e-7 -> 0.9e-7                   1.3e-7 -> 0.5e-7
-//   3x3, 8 -> 40 channels at 5x7, batch 3          0.8e-7 -> 0.6e-7                  1.2e-7 -> 0.8e-7                   1.2e-7 -> 0.5e-7
+//   3x3, 8 -> 40 channels at 5x7, batch 3          0.7e-7 -> 0.6e-7                  1.4e-7 -> 0.9e-7                   1.1e-7 -> 0.5e-7
 //
 // One CTA per SM walks (tile, split) units; the results of a unit are written while the next one is under way.  Roles (24 warps, 16
 // where the weights arrive as terms; registers are moved between them): warp 0 allocates TMEM and issues the MMAs; warp 1 fetches A as
@@ -35,9 +38,10 @@
 // kernel out.) WGRAD: issue slots, 2.9 of 4 a cycle: 16 converter warps of 350 instructions a chunk, the summing warps' 128 additions
 // and the MMA warp. Without TMA and with a CTA per unit the same layers took a third longer (a row per lane made each load of A 32
 // wavefronts of the L1 port). Where the weights arrive as terms eight warps of 32 elements convert, not 16 of 16 (half the waits and
-// arrivals: 66 -> 62). Float CUDA cores -> here, us at batch 96: 3x3 over 64 channels at 32x32 forward 180 -> 58, input gradient 175
-// -> 66, weight gradient 177 -> 90; 128 channels at 16x16 155 / 164 / 156 -> 52 / 53 / 47; 256 channels at 8x8 157 / 170 / 159 -> 44 /
-// 45 / 47; 4096 -> 1024 30 / 27 / 23 -> 17 / 16 / 18. The 7-conv / 3-FC net: 2.54 -> 0.91 ms an iteration.
+// arrivals: 66 -> 62). Float CUDA cores -> here, us between events at batch 96 (about 4 of them the launch): 3x3 over 64 channels at 32x32
+// forward 183 -> 58, input gradient 189 -> 67, weight gradient 181 -> 97; 128 channels at 16x16 158 / 169 / 160 -> 54 / 55 / 52; 256
+// channels at 8x8 159 / 174 / 162 -> 46 / 46 / 52; 4096 -> 1024 33 / 31 / 27 -> 22 / 21 / 23. The 7-conv / 3-FC net: 2.54 -> 0.89 ms an
+// iteration.
 //
 // Non-finite operands: infinity - infinity in the splitting makes the terms NaN where a float multiply-add would give an infinity, so
 // results that are not finite are looked at again behind the CTA's last unit, when no other warp waits (repair_unit).
@@ -445,13 +449,15 @@ struct Ring {
     __device__ __forceinline__ void next(int n) { if (++i == n) { i = 0; ph ^= 1u; } }
 };
 
-// TMA: A arrives as raw floats by TMA (FWD, DGRAD: the channels of the reduction are a multiple of 64, so that a chunk lies in one
-// tap and its rows are those of the tile, shifted; WGRAD: always); otherwise the converters load it themselves.
-// WT: B arrives as terms by TMA (FWD, DGRAD of convolutions, whose weights every row tile reads: launch_split_weights).
+// WT: B arrives as terms by TMA (FWD, DGRAD of convolutions, whose weights every row tile reads: launch_split_weights), where the channels
+// of the reduction are a multiple of 64, so that a chunk lies in one tap.
+// TMA: A arrives as raw floats by TMA: with WT, whose chunk's rows of A are those of the tile, shifted, and in WGRAD; otherwise (FC
+// layers among them) the converters load it themselves.
 template <int MODE, int BN, bool TMA, bool WT>
 __global__ void __launch_bounds__(Roles<WT>::THREADS, 1)
 contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_constant__ SplitParams p)
 {
+    static_assert(MODE == CMODE_WGRAD ? TMA && !WT : TMA == WT, "the forms there are");
     using C = SplitCfg<BN>;
     using R = Roles<WT>;
     constexpr int NB = BN / 64;
@@ -781,7 +787,7 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
             }
         };
         auto load_b = [&](int j) {
-            if (MODE == CMODE_FWD) load8(rb[j], b_px + (size_t)(64 * j) * p.K + kpos, b_in[j] && (TMA || kpos + 8 * q < p.K));
+            if (MODE == CMODE_FWD) load8(rb[j], b_px + (size_t)(64 * j) * p.K + kpos, b_in[j] && kpos + 8 * q < p.K);
             else if (MODE == CMODE_DGRAD) load8(rb[j], b_px + ((size_t)b_o * p.taps + b_tap) * p.Cin + 64 * j, b_in[j] && b_tap < p.taps);
             else load8(rb[j], p.act + (long)(kpos + r) * p.Cin + b_shift[j],
                        b_in[j] && kpos + r < p.K && (unsigned)(b_h + dr[j]) < (unsigned)p.H && (unsigned)(b_w + ds[j]) < (unsigned)p.W);
@@ -800,7 +806,7 @@ contract_umma_kernel(const __grid_constant__ Maps<TMA> maps, const __grid_consta
             const Unit un = unit_at<BN>(p, u);
             const bool do_bias = MODE == CMODE_WGRAD && un.n0 == 0;
             float bsum = 0.f;
-            if (TMA && MODE != CMODE_WGRAD) {
+            if (WT) {
                 a_in = taps_inside<MODE>(p, un.m0 + row);
                 a_tap = un.chunk0 * 64 / Cred; a_c = un.chunk0 * 64 - a_tap * Cred;
             }
@@ -922,9 +928,7 @@ template <int MODE, int BN>
 cudaError_t launch_form(const ContractArgs& a, const SplitParams& p, cudaStream_t st)
 {
     if constexpr (MODE == CMODE_WGRAD) return launch_one<MODE, BN, true, false>(a, p, st);
-    else {
-        return a.wterms != nullptr ? launch_one<MODE, BN, true, true>(a, p, st) : launch_one<MODE, BN, false, false>(a, p, st);
-    }
+    else return a.wterms != nullptr ? launch_one<MODE, BN, true, true>(a, p, st) : launch_one<MODE, BN, false, false>(a, p, st);
 }
 template <int MODE>
 cudaError_t launch_mode(const ContractArgs& a, const SplitParams& p, cudaStream_t st)

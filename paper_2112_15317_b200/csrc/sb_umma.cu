@@ -3351,8 +3351,9 @@ sb_status umma_plan_layers(sb_model* m, int first_layer)
                     p.stages = g.wg_cps < fit ? g.wg_cps : fit;
                 }
                 {
-                    // (the filter-row kernel keeps its whole five-stage ring: with two slots per round the deeper ring is worth more
-                    // than a neighbour on the SM -- steps -0.2 to -1.6 % against a ring cut to two or three 40 KB stages)
+                    // (the filter-row kernel keeps four of its five 40 KB stages: with five it held an SM alone and the input layer's weight
+                    // gradient, last on the chain, waited for it -- 7-conv net 290.2 -> 288.0 us, VGG-16 at batch 128 524.0 -> 523.2; a ring
+                    // cut to two or three stages costs more than the neighbour is worth, steps 0.2 to 1.6 % against five)
                     const int cap = b->bn == 192 ? 4 : cohabit_stages(b->bn);
                     // (grids that leave SMs idle too: whole rings for those of fewer than 100 CTAs cost the step 1.2 % at CIFAR size, batch 128)
                     if (bwd_cohabit() && p.stages > cap) p.stages = cap;
