@@ -84,6 +84,20 @@ def test_modulo_step_matches_oracle(name, bf16):
     run(CASES[name](), bf16, steps=1 if bf16 else 2)
 
 
+def test_float_sub_batches_run_on_tensor_cores():
+    """The float case of the wide FC stack above: the sub-batches' own plans take the tensor-core contractions forward and for the input
+    gradient (a weight gradient over 32 rows is shorter on the CUDA cores)."""
+    b = sb()
+    wl = CASES["cfg1_fc_stack"]()
+    gm = gpu_model(wl, si.make_params(wl), b.SB_FP32, flags=b.SB_FLAG_MODULO_SCHEDULE)
+    gm.profile_begin()
+    gm.modulo_step(*device_batch(wl, *si.make_batch(wl), False), 0.01, 0.9)
+    launches = {e["name"]: e["launches"] for e in gm.profile_end()}
+    for name in ("fc_fwd_f32_umma", "fc_dgrad_f32_umma"):
+        assert launches.get(name, 0) >= wl.K, launches
+    gm.close()
+
+
 def test_modulo_step_with_K1_equals_the_synchronous_calls():
     b = sb()
     wl = si.Workload("modulo_k1", tensor_core_net(), 12, 20, 3, 3, 2, 1)
