@@ -245,14 +245,21 @@ __device__ __forceinline__ Unit unit_at(const SplitParams& p, int u)
 // multiply-adds give.  A NaN operand makes its whole row or column NaN (places outside the image are zeros that are multiplied, as in
 // contract_kernel: NaN x 0 and infinity x 0 are NaN), so the operands are searched for those first, and the search ends when they
 // explain every such result: a run that has diverged costs one look at the operands.  What is left has infinite or large operands
-// in its sum: the steps that hold any (in 1024 groups, a bit each, 32 to a lane) are summed, a lane per column; only where that is finite
-// does the sum run over all steps.
+// in its sum, or is too large: the blocks of 32 steps that hold large operands (in 1024 groups, a bit each, 32 to a lane) are summed, a lane
+// to two or four columns of as many rows, and all of them only where that is finite.
 // (a predicate, not a branch, so that the loads of several steps are under way together)
 __device__ __forceinline__ float load_if(const float* p, bool there)
 {
     float v;
     asm("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\tmov.b32 %0, 0;\n\t@p ld.global.f32 %0, [%1];\n\t}" : "=f"(v) : "l"(p), "r"((int)there));
     return v;
+}
+__device__ __forceinline__ void load8_if(F8& f, const float* p, bool there)      // (at a 16-byte boundary)
+{
+#pragma unroll
+    for (int h = 0; h < 8; h += 4)
+        asm("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %5, 0;\n\tmov.b32 %0, 0;\n\tmov.b32 %1, 0;\n\tmov.b32 %2, 0;\n\tmov.b32 %3, 0;\n\t"
+            "@p ld.global.v4.f32 {%0, %1, %2, %3}, [%4];\n\t}" : "=f"(f.v[h]), "=f"(f.v[h + 1]), "=f"(f.v[h + 2]), "=f"(f.v[h + 3]) : "l"(p + h), "r"((int)there));
 }
 template <int MODE> struct Step {      // a reduction step's tap and channel; WGRAD: its pixel's row and column
     int k, tap, c;
@@ -311,8 +318,60 @@ __device__ __forceinline__ float row_operand(const SplitParams& p, int m, uint32
     a += ((long)m + (MODE == CMODE_FWD ? shift : -shift)) * (MODE == CMODE_FWD ? p.Cin : p.Cout) + s.c;
     return load_if(a, there && ((inside >> s.tap) & 1u) != 0u);      // (no tap of a row past the last is inside)
 }
+// The eight reduction steps from k on (below k1), a multiple of eight: one tap's channels, or WGRAD: pixels (a bit each: steps that there
+// are, and those with an image row or column before and behind them)
+template <int MODE> struct Eight {
+    int k, tap = 0, c = 0;
+    uint32_t all, up = 0u, down = 0u, left = 0u, right = 0u;
+    __device__ __forceinline__ Eight(const SplitParams& p, int k_, int k1) : k(k_), all(k_ >= k1 ? 0u : k_ + 8 <= k1 ? 0xffu : (1u << (k1 - k_)) - 1u)
+    {
+        Step<MODE> s(p, k);
+        if constexpr (MODE == CMODE_WGRAD) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                up |= (s.tap > 0 ? 1u : 0u) << i; down |= (s.tap + 1 < p.H ? 1u : 0u) << i;
+                left |= (s.c > 0 ? 1u : 0u) << i; right |= (s.c + 1 < p.W ? 1u : 0u) << i;
+                s.next(p);
+            }
+        } else {
+            tap = s.tap; c = s.c;
+        }
+    }
+    __device__ __forceinline__ void row(const SplitParams& p, F8& f, int m, uint32_t inside) const
+    {
+        if constexpr (MODE == CMODE_WGRAD) {
+            const float* from = p.dy + (size_t)k * p.Cout + m;
+            const uint32_t there = m < p.M ? all : 0u;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) f.v[i] = load_if(from + (size_t)i * p.Cout, (there >> i) & 1u);
+        } else {
+            const int shift = p.taps == 9 ? (tap / 3 - 1) * p.W + tap % 3 - 1 : 0;
+            const float* from = MODE == CMODE_FWD ? p.act + ((long)m + shift) * p.Cin + c : p.dy + ((long)m - shift) * p.Cout + c;
+            load8_if(f, from, all != 0u && ((inside >> tap) & 1u) != 0u);      // (channel counts are multiples of eight)
+        }
+    }
+    __device__ __forceinline__ void column(const SplitParams& p, F8& f, const Column<MODE>& col) const
+    {
+        if constexpr (MODE == CMODE_FWD) {
+            load8_if(f, col.at + k, col.in && all != 0u);
+        } else {
+            uint32_t there = col.in ? all : 0u;
+            size_t stride = p.Cin;
+            const float* from = col.at + (size_t)k * p.Cin;
+            if constexpr (MODE == CMODE_DGRAD) {
+                stride = (size_t)p.taps * p.Cin;
+                from = col.at + ((size_t)c * p.taps + tap) * p.Cin;
+            } else {
+                if (col.dr != 0) there &= col.dr < 0 ? up : down;
+                if (col.ds != 0) there &= col.ds < 0 ? left : right;
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) f.v[i] = load_if(from + i * stride, (there >> i) & 1u);
+        }
+    }
+};
 // All operands of the 32 steps from k on (below k1) to the warp's rows and the unit's columns: a lane per step where an operand lies
-// along the reduction in memory, else a lane per line.  f(value, line, step, whether it is a column's): line or step is the lane's own.
+// along the reduction in memory, else a lane per line.  f(value, line, whether it is a column's)
 template <int MODE, int BN, typename F>
 __device__ __forceinline__ void visit(const SplitParams& p, const Column<MODE> (&col)[BN / 32], int row0, int n0, uint32_t inside, int k, int k1, F f)
 {
@@ -320,47 +379,22 @@ __device__ __forceinline__ void visit(const SplitParams& p, const Column<MODE> (
     const Step<MODE> mine(p, k + lane);
     if (MODE == CMODE_FWD) {
 #pragma unroll 16
-        for (int i = 0; i < BN; ++i) f(Column<MODE>(p, n0 + i).operand(p, mine, k + lane < k1), i, lane, true);
+        for (int i = 0; i < BN; ++i) f(Column<MODE>(p, n0 + i).operand(p, mine, k + lane < k1), i, true);
     } else {
         Step<MODE> s(p, k);
 #pragma unroll 8
         for (int i = 0; i < 32; ++i, s.next(p))
 #pragma unroll
-            for (int b = 0; b < BN / 32; ++b) f(col[b].operand(p, s, k + i < k1), 32 * b + lane, i, true);
+            for (int b = 0; b < BN / 32; ++b) f(col[b].operand(p, s, k + i < k1), 32 * b + lane, true);
     }
     if (MODE == CMODE_WGRAD) {
         Step<MODE> s(p, k);
 #pragma unroll 16
-        for (int i = 0; i < 32; ++i, s.next(p)) f(row_operand<MODE>(p, row0 + lane, 0u, s, k + i < k1), lane, i, false);
+        for (int i = 0; i < 32; ++i, s.next(p)) f(row_operand<MODE>(p, row0 + lane, 0u, s, k + i < k1), lane, false);
     } else {
 #pragma unroll 16
-        for (int i = 0; i < 32; ++i) f(row_operand<MODE>(p, row0 + i, __shfl_sync(0xffffffffu, inside, i), mine, k + lane < k1), i, lane, false);
+        for (int i = 0; i < 32; ++i) f(row_operand<MODE>(p, row0 + i, __shfl_sync(0xffffffffu, inside, i), mine, k + lane < k1), i, false);
     }
-}
-// The sum of row m and the lane's column: over the groups of steps that hold large operands or, where that is finite, over all of them
-template <int MODE>
-__device__ __noinline__ float sum_again(const SplitParams& p, int m, uint32_t inside, const Column<MODE> col, bool left, int k0, int k1, int group, uint32_t large)
-{
-    auto add = [&](float sum, int from, int to) {      // (up to the first NaN of all lanes)
-        Step<MODE> s(p, from);
-        while (s.k < to && __any_sync(0xffffffffu, left && sum == sum)) {
-            const int stop = min(s.k + 32, to);
-#pragma unroll 8
-            for (; s.k < stop; s.next(p)) sum = fmaf(row_operand<MODE>(p, m, inside, s), col.operand(p, s, left), sum);
-        }
-        return sum;
-    };
-    float s = 0.f;
-    for (int l = 0; l < 32; ++l)
-        for (uint32_t w = __shfl_sync(0xffffffffu, large, l); w != 0u; w &= w - 1u) {
-            const int from = k0 + (32 * l + __ffs(w) - 1) * group;
-            s = add(s, from, min(from + group, k1));
-        }
-    if (__any_sync(0xffffffffu, left && s - s == 0.f)) {
-        const float whole = add(0.f, k0, k1);
-        if (s - s == 0.f) s = whole;
-    }
-    return s;
 }
 template <int MODE, int BN>
 __device__ __forceinline__ void repair_unit(const SplitParams& p, int u, int q)
@@ -369,7 +403,7 @@ __device__ __forceinline__ void repair_unit(const SplitParams& p, int u, int q)
     constexpr int CB = BN / 32;
     const Unit t = unit_at<BN>(p, u);
     const int lane = threadIdx.x % 32, row0 = t.m0 + 32 * q;
-    const int k0 = t.chunk0 * 64, k1 = min(p.K, (t.chunk0 + t.n_iters) * 64), group = (k1 - k0 + 1023) / 1024;
+    const int k0 = t.chunk0 * 64, k1 = min(p.K, (t.chunk0 + t.n_iters) * 64), group = 32 * ((k1 - k0 + 32 * 1024 - 1) / (32 * 1024));
     const bool raw_sums = MODE == CMODE_WGRAD || p.splits > 1;
     volatile float* const base = raw_sums ? p.part + (size_t)t.split * p.split_stride : p.out;
     const uint32_t inside = MODE == CMODE_WGRAD ? 0u : taps_inside<MODE>(p, row0 + lane);      // (of row `lane`)
@@ -398,14 +432,15 @@ __device__ __forceinline__ void repair_unit(const SplitParams& p, int u, int q)
         // (products of operands below 2^53 are below 2^106: no sum of them overflows)
         constexpr uint32_t LARGE = 0x5a000000u, INF = 0x7f800000u;
         uint32_t top = 0u;
-        visit<MODE, BN>(p, col, row0, t.n0, inside, k, k1, [&](float v, int, int, bool) { top = max(top, __float_as_uint(v) & 0x7fffffffu); });
+        visit<MODE, BN>(p, col, row0, t.n0, inside, k, k1, [&](float v, int, bool) { top = max(top, __float_as_uint(v) & 0x7fffffffu); });
         if (!__any_sync(ALL, top >= LARGE)) continue;
-        uint32_t rn = 0u, cn[CB], steps = 0u;
+        uint32_t rn = 0u, cn[CB];
+        bool any = false;
 #pragma unroll
         for (int b = 0; b < CB; ++b) cn[b] = 0u;
-        visit<MODE, BN>(p, col, row0, t.n0, inside, k, k1, [&](float v, int line, int step, bool of_col) {
+        visit<MODE, BN>(p, col, row0, t.n0, inside, k, k1, [&](float v, int line, bool of_col) {
             const uint32_t a = __float_as_uint(v) & 0x7fffffffu;
-            if (a >= LARGE && a <= INF) steps |= 1u << step;
+            any = any || (a >= LARGE && a <= INF);
             if (a > INF && !of_col) rn |= 1u << line;
 #pragma unroll
             for (int b = 0; b < CB; ++b)
@@ -414,32 +449,83 @@ __device__ __forceinline__ void repair_unit(const SplitParams& p, int u, int q)
         row_nan |= __reduce_or_sync(ALL, rn);
 #pragma unroll
         for (int b = 0; b < CB; ++b) col_nan[b] |= __reduce_or_sync(ALL, cn[b]);
-        for (steps = __reduce_or_sync(ALL, steps); steps != 0u; steps &= steps - 1u) {
-            const int g = (k + __ffs(steps) - 1 - k0) / group;
-            if (lane == g >> 5) large |= 1u << (g & 31);
-        }
+        const int g = (k - k0) / group;
+        if (__any_sync(ALL, any) && lane == g >> 5) large |= 1u << (g & 31);
     }
-    for (; rows != 0u; rows &= rows - 1u) {
-        const int r = __ffs(rows) - 1, m = row0 + r;
-        const uint32_t in = __shfl_sync(ALL, inside, r);
+    constexpr int R = BN == 64 ? 4 : 2;
+#pragma unroll 1
+    for (int r0 = 0; r0 < 32; r0 += R) {
+        if (((rows >> r0) & ((1u << R) - 1u)) == 0u) continue;
+        float sum[R][CB];
+        uint32_t in[R], mine = 0u, left = 0u;      // (a bit per result of the lane)
 #pragma unroll
-        for (int b = 0; b < CB; ++b) {
-            const int n = t.n0 + 32 * b + lane;
-            const size_t at = (size_t)m * p.N + n;
-            float sum = n < p.N ? base[at] : 0.f;
-            const bool mine = n < p.N && !finite(sum);
-            const bool left = mine && !((row_nan >> r) & 1u) && !((col_nan[b] >> lane) & 1u);
-            if (__any_sync(ALL, left)) {
-                const float s = sum_again<MODE>(p, m, in, col[b], left, k0, k1, group, large);
-                if (left) sum = s;
+        for (int r = 0; r < R; ++r) {
+            in[r] = __shfl_sync(ALL, inside, r0 + r);
+#pragma unroll
+            for (int b = 0; b < CB; ++b) {
+                const int n = t.n0 + 32 * b + lane;
+                sum[r][b] = n < p.N && row0 + r0 + r < p.M ? base[(size_t)(row0 + r0 + r) * p.N + n] : 0.f;
+                if (finite(sum[r][b])) continue;
+                mine |= 1u << (r * CB + b);
+                if (!((row_nan >> (r0 + r)) & 1u) && !((col_nan[b] >> lane) & 1u)) left |= 1u << (r * CB + b);
             }
-            if (mine) base[at] = raw_sums ? sum : finish1<MODE>(p, sum, at, n);
+        }
+        // over the blocks with large operands, then, if some were left out and for what is finite, over all
+#pragma unroll 1
+        for (int pass = 0; pass < 2 && __any_sync(ALL, left != 0u); ++pass) {
+            float again[R][CB];
+            bool whole = true, alive = true;
+#pragma unroll
+            for (int j = 0; j < R * CB; ++j) again[j / CB][j % CB] = 0.f;
+#pragma unroll 1
+            for (int k = k0; k < k1 && __any_sync(ALL, alive); k += 32) {
+                const int g = (k - k0) / group;
+                if (pass == 0 && !((__shfl_sync(ALL, large, g >> 5) >> (g & 31)) & 1u)) {
+                    whole = false;
+                    continue;
+                }
+                float part[R][CB];
+#pragma unroll
+                for (int j = 0; j < R * CB; ++j) part[j / CB][j % CB] = 0.f;
+#pragma unroll 1
+                for (int i0 = 0; i0 < 32; i0 += 8) {
+                    const Eight<MODE> e(p, k + i0, k1);
+                    F8 a[R], c[CB];
+#pragma unroll
+                    for (int r = 0; r < R; ++r) e.row(p, a[r], row0 + r0 + r, in[r]);
+#pragma unroll
+                    for (int b = 0; b < CB; ++b) e.column(p, c[b], col[b]);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+#pragma unroll
+                        for (int j = 0; j < R * CB; ++j) part[j / CB][j % CB] = fmaf(a[j / CB].v[i], c[j % CB].v[i], part[j / CB][j % CB]);
+                }
+                alive = false;      // (a NaN stays one)
+#pragma unroll
+                for (int j = 0; j < R * CB; ++j) {
+                    again[j / CB][j % CB] += part[j / CB][j % CB];
+                    alive = alive || (((left >> j) & 1u) != 0u && again[j / CB][j % CB] == again[j / CB][j % CB]);
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < R * CB; ++j) {
+                if (!((left >> j) & 1u)) continue;
+                sum[j / CB][j % CB] = again[j / CB][j % CB];
+                if (whole || !finite(again[j / CB][j % CB])) left &= ~(1u << j);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < R * CB; ++j) {
+            const int m = row0 + r0 + j / CB, n = t.n0 + 32 * (j % CB) + lane;
+            const size_t at = (size_t)m * p.N + n;
+            if ((mine >> j) & 1u) base[at] = raw_sums ? sum[j / CB][j % CB] : finish1<MODE>(p, sum[j / CB][j % CB], at, n);
         }
     }
 }
 template <int MODE, int BN>
 __device__ __noinline__ void repair_units(const SplitParams& p, int q)
 {
+    __syncwarp();      // (lanes read what others have stored)
     for (int u = blockIdx.x; u < p.units; u += gridDim.x) repair_unit<MODE, BN>(p, u, q);
 }
 // slot of a ring and the parity of its current use
